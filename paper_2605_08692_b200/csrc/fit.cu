@@ -1,13 +1,18 @@
 // The fit rounds (Algorithm 1 lines 6-16).  With n_inner = 1 a round is the assignment step
 // (Eq. 8) and the activation-weighted centroid update (Eq. 11) in a single pass over W, and all
 // rounds of a layer run in ONE persistent kernel (one block per SM, cooperative launch): after
-// its pass every block adds its sums, as 96-bit fixed-point integers, into 65 global accumulators;
-// every 64-bit accumulator word also counts, in its upper 16 bits, the blocks that have added to
-// it, so a block knows that a total is complete by reading the total itself -- no separate
+// its pass every block adds its sums, as fixed-point integers of two 40-bit limbs, into 65 global
+// accumulators; every 64-bit accumulator word also counts, in its upper bits, the blocks that have
+// added to it, so a block knows that a total is complete by reading the total itself -- no separate
 // barrier, no fence between the sums and an arrival counter -- and every block ends up with the
 // same new tables without a relaunch (integer addition does not depend on the order in which the
 // blocks arrive, so the result is bitwise reproducible).  The wait for the totals is bounded: if
 // it runs out, the kernel sets AAAC_DEV_TIMEOUT in the device status word and returns.
+// What a round costs besides its pass (block sums, exchange, new tables) is latency: about 11k
+// cycles, kept short by leaving the small steps to one warp that needs no block barrier, by
+// lookups and conversions chosen for it (see below), and by having the first rows of the next pass
+// in flight meanwhile.  A pass of a 512 x 512 layer took 11.4 us with 19k cycles of it and whole
+// items, 6.9 us now; 4096 x 4096, 27.4 -> 25.0 us.
 // With n_inner > 1 the assignment pass (which is also the first inner iteration) stores the
 // selection bits, one word per row and 256-column slab, and the remaining n_inner - 1 inner
 // iterations are passes of a second instance of the kernel that reads those bits instead of
@@ -62,12 +67,13 @@
 // in the same copy, and a weight above the bin's breakpoint adds the distance to the next
 // interval's entry), the bins once per lane.
 //
-// Thread mapping.  A block of NW warps works on items of 4 NW rows x 256 columns, dealt to
+// Thread mapping.  A block of 16 warps works on items of 64 rows (32 or 16 in layers that have too
+// few items for the blocks) x 256 columns, dealt to
 // blocks as contiguous ranges (slab-major), so every sum has a fixed order and results are
 // bitwise reproducible.  A warp takes 4 rows; each lane 8 adjacent columns (one 128-bit load
 // per row), so its eight importances stay in registers.  A group is 2 lanes (g = 16) or 16
 // lanes (g = 128).  A row's registers are refilled from the next item right after the row is unpacked.
-#include <type_traits>
+#include <algorithm>
 
 #include "lookup.cuh"
 
@@ -82,7 +88,7 @@ struct FitParams {
     const float* rinv;            // INT4 reciprocal scales
     const float* I;
     Ctrl* ctrl;
-    unsigned long long* acc;      // [3][kUsed][3] words, 128 bytes apart: fixed-point sums over the blocks, one buffer per pass in rotation
+    unsigned long long* acc;      // [3][kAccBuffer] words: fixed-point sums over the blocks, one buffer per pass in rotation
     double* err_trace;            // [n_rounds] or null
     float* T01_out;               // [2][16] or null: the tables after the launch's last pass, as FP32
     uint32_t* dev_status;         // or null
@@ -92,26 +98,29 @@ struct FitParams {
     unsigned bar_base;            // passes of the layer's earlier launches (the sum buffers rotate per pass)
     unsigned arrivals;            // blocks whose sums a total must hold before it is read (the grid size)
     unsigned spin_limit;          // polls of a total before the wait is given up
-    int items, per_block, nrb;    // (4 NW)-row x 256-column items, items per block, row blocks per slab
+    int rows;                     // rows per warp of an item: 4, or 2 or 1 for layers that have too few items of 4
+    int items, per_block, nrb;    // items of (16 rows) x 256 columns, items per block, row blocks per slab
     int tail_item0, tail_quarters;   // items from tail_item0 on are dealt out a quarter (one row per warp) per block
 };
 
 constexpr uint32_t kLut1At = 65536;                    // shared address of the bin table (see fit_rounds_body)
-constexpr int kMaxFitBlocks = 1024;                   // grid limit: block sums are added as 32-bit limbs, the arrivals counted in 16 bits
-constexpr int kLimbs = 3;                             // a sum is a 96-bit two's-complement fixed-point number
-constexpr unsigned kDefaultSpinLimit = 1u << 23;      // polls of >= 32 ns each: several seconds
-constexpr int kAccStride = 16;                        // accumulator words lie 128 bytes apart: one cache line each, so that the
-                                                      // blocks' atomics on different sums do not queue behind one another
-constexpr int kAccBuffer = kUsed * kLimbs * kAccStride;   // 64-bit words of one pass's buffer
-constexpr int kCountShift = 48;                       // an accumulator word: limb sum below, arrivals above
+constexpr int kFitWarps = 16;
+constexpr int kMaxFitBlocks = 1023;                   // grid limit: the arrivals are counted in 14 bits, the limbs' sums have 10 bits of room
+constexpr int kLimbs = 2;                             // a sum is a fixed-point number of two 40-bit limbs
+constexpr int kLimbBits = 40;
+constexpr unsigned kDefaultSpinLimit = 1u << 23;      // polls of several hundred ns each: seconds
+// An accumulator buffer: per cell the limbs of the residual sum and of the weight sum, 32 bytes next to one
+// another (four lanes add them with one request, a reader takes them with two loads), cells 128 bytes apart
+// so that the blocks' atomics on different cells do not queue behind one another; then the objective's.
+constexpr int kAccStride = 16;
+constexpr int kAccBuffer = (kCells + 1) * kAccStride;  // 64-bit words of one pass's buffer
+constexpr int kCountShift = 50;                       // an accumulator word: limb sum below, arrivals above
 constexpr unsigned long long kLimbMask = (1ull << kCountShift) - 1ull;
 constexpr unsigned long long kOneArrival = 1ull << kCountShift;
-constexpr long long kTopBias = 1ll << 31;             // added to the (signed) top limb so that every block adds a non-negative number
+constexpr long long kTopBias = 1ll << (kLimbBits - 1);   // added to the (signed) top limb so that every block adds a non-negative number
 
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
+__device__ __forceinline__ void ld_relaxed_2xu64(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
+    asm volatile("ld.relaxed.gpu.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
 }
 __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
     unsigned v;
@@ -229,23 +238,43 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
     return esum;
 }
 
+// Integers of up to 51 bits travel to and from doubles by an addition (the 64-bit conversion instructions
+// run at a small fraction of the double-precision rate).
+constexpr double kIntMagic = 0x1.8p52;
+
+struct FitShared {
+    FitTables t;
+    double wsum[kFitWarps][2 * kCells + 2];   // the warps' sums of a pass: residuals, weights, objective
+    double fix_scale, fix_unscale;   // fixed-point scale of the sums over the blocks and its inverse
+    int failed;
+};
+
+// Double value of FP32 bits times 2^-896: the float's fields moved into a double's (zeros and denormals
+// included: their double is a denormal of the same scale, and double-precision hardware handles those at
+// full speed).  Three integer instructions instead of the slow conversion; the caller multiplies its sum
+// by 2^896.
+__device__ __forceinline__ double scaled_double(float f) {
+    const int u = __float_as_int(f);
+    return __hiloint2double((u >> 3) & (int)0x8FFFFFFFu, u << 29);
+}
+
 // SEL is the selection group size S (Sec. 3.1): the weights that share one codebook choice; the
 // scale group g is fixed by the format.
 // The passes of one layer, run by the nblk blocks bid = 0 .. nblk - 1 (a whole grid, or the part
 // of a grid that a batch of layers gives to this layer).
-template <int MODE, int SEL, int NW, int REP, int KIND>
+template <int MODE, int SEL, int KIND>
 __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsigned bid, const unsigned nblk) {
-    constexpr int NB = AAAC_FIT_BINS;
+    constexpr int NW = kFitWarps, NB = kNBins, REP = kRep;
+    constexpr unsigned kAll = 0xFFFFFFFFu;
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;      // scale group
     constexpr int LPG = SEL / 8;                         // lanes per selection group
     constexpr int R = kRowsPerWarp;
-    constexpr int kRowsPerItem = R * NW;
+    const int rows = p.rows;                             // rows per warp of an item (R or fewer)
     constexpr int NT = NW * 32;
-    constexpr int kLut1Bytes = REP * NB * 8;
     constexpr int kBinBytes = kBinSlots * kSlotBytes;        // per warp
-    static_assert(kLut1Bytes >= NW * kPartStride * 8, "the per-warp partials reuse the first table's space");
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ FitTables S;
+    __shared__ FitShared sh;
+    FitTables& S = sh.t;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // 32-bit shared addresses.  The bin table sits at a shared address that is a multiple of its own
@@ -254,7 +283,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     // warps' bins, the {P, Q} table and the near-tie lists follow it.  Slot offsets carry the address of
     // this lane's column of the {P, Q} table, so a lookup there needs no further arithmetic.
     static_assert(kLut1Bytes == (int)kLut1At, "the bin table spans exactly the alignment of its address");
-    const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(dyn);
+    const uint32_t dyn_at = (uint32_t)__cvta_generic_to_shared(dyn);
+    const uint32_t sm_base = (dyn_at + 255u) & ~255u;        // (a bin slot is 256 bytes: its lanes' offsets can be formed by xor)
     uint32_t dyn_size;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_size));
     const uint32_t gap = kLut1At - sm_base;                                            // bytes of the dynamic region below the table
@@ -262,20 +292,17 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     const uint32_t hi_base = kLut1At + kLut1Bytes;
     const uint32_t lut2_addr = hi_base + (uint32_t)(NW - n_low) * kBinBytes;           // the {P, Q} table
     const uint32_t lists_at = lut2_addr + kLut2Bytes;
-    if (sm_base > kLut1At || lists_at + NW * (kDeferCap * 8) > sm_base + dyn_size) {
+    if (sm_base > kLut1At || lists_at + NW * (kDeferCap * 8) > dyn_at + dyn_size) {
         // the layout does not fit the shared memory this launch was given (the same for every block, so
         // all of them leave before any of them waits): reported like a wait that ran out -- no valid result
         if (bid == 0 && threadIdx.x == 0 && p.dev_status) atomicOr(p.dev_status, AAAC_DEV_TIMEOUT);
         return;
     }
-    unsigned char* const lut1_mem = dyn + gap;
-    unsigned char* const lut2_mem = dyn + (lut2_addr - sm_base);
     const uint32_t lut1_or = kLut1At | ((lane & (REP - 1)) * 8);                        // table base | this lane's copy of a bin's entry; | bin * REP * 8
     const uint32_t bins_warp = warp < n_low ? sm_base + warp * kBinBytes : hi_base + (uint32_t)(warp - n_low) * kBinBytes;
     const uint32_t bins_lane = bins_warp + lane * 8;                                   // + cell * 256
     const uint32_t spare_lane = bins_lane + kSpareSlot * kSlotBytes;                   // sink of the near-tie groups' rows
     const uint32_t list_addr = lists_at + warp * (kDeferCap * 8);
-    double* wsum = reinterpret_cast<double*>(lut1_mem);    // [NW][kPartStride], over the first table
 
     // 32-bit index arithmetic throughout (N, K < 2^31); only the final element offsets are 64-bit
     const int N = (int)p.N, K = (int)p.K;
@@ -290,102 +317,119 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     const int tail_item = p.tail_item0 + ((int)bid >> 2), tail_u = (int)bid & 3;
     static_assert(R == 4, "a tail quarter is one of the four rows of a warp");
 
-    if (tid < 2 * kM) S.Td[tid] = p.ctrl->T[tid];
+    // Row registers of the item being processed; a row's registers are refilled with the same row
+    // of the next item as soon as the row has been unpacked, so the load has about an item's time
+    // to arrive and no second buffer is needed.  After the last item of a pass the next is the first
+    // one again: its rows, and the importances as long as the slab stays the same, are there when the
+    // next pass starts (a layer of one item per block waits for no load at all).
+    uint4 v[R];
+    uint32_t sc[R];           // NVFP4: scale byte; INT4: bits of the reciprocal scale
+    uint32_t sgw[R];          // inner iteration: the row's stored selection bits
+    constexpr bool INNER = KIND == kInner;
+    constexpr bool keep_sigma = KIND == kAssignKeep;
+#pragma unroll
+    for (int u = 0; u < R; ++u) { v[u] = make_uint4(0, 0, 0, 0); sc[u] = 0u; sgw[u] = 0u; }
+    // Offsets of the item being loaded (element offsets fit 32 bits: the entry points refuse layers of 2^32
+    // elements and more) and how many of its rows this lane may read.
+    unsigned nwo = 0u, ngo = 0u, nso = 0u;
+    int nlim = 0;
+    auto aim = [&](int slab, int rb) {
+        const int col0 = slab * 256 + lane * 8, row = (rb * NW + warp) * rows;
+        nwo = (unsigned)row * (unsigned)p.ldw + (unsigned)col0;
+        ngo = (unsigned)row * (unsigned)Gr + (unsigned)col0 / G;
+        if (INNER) nso = (unsigned)row * (unsigned)slabs + (unsigned)slab;
+        nlim = col0 < K ? min(N - row, rows) : 0;
+    };
+    auto load_row = [&](int u) {
+        v[u] = make_uint4(0, 0, 0, 0);
+        sc[u] = 0u;
+        if (INNER) sgw[u] = 0u;
+        if (u < nlim) {
+            v[u] = __ldcs(reinterpret_cast<const uint4*>(p.W + (nwo + (unsigned)u * (unsigned)p.ldw)));
+            const unsigned gi = ngo + (unsigned)u * (unsigned)Gr;
+            if (MODE == AAAC_NVFP4) sc[u] = p.scales[gi];          // masked at use: nothing waits on the load here
+            else sc[u] = __float_as_uint(__ldg(p.rinv + gi));
+            if (INNER) sgw[u] = __ldcg(p.sigw + (nso + (unsigned)u * (unsigned)slabs));
+        }
+    };
+    int cur_slab = -1;
+    uint64_t II[4];           // importances of the lane's eight columns, in pairs
+    float isum_raw = 0.f;     // sum of I over the lane's group (rounded up a little)
+    bool col_ok = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) II[j] = 0ull;
+    auto Ic = [&](int j) { return (j & 1) ? hi2(II[j >> 1]) : lo2(II[j >> 1]); };
+
+    // (slab, row block) of the current item and of the one being loaded
+    const int n_main = max(it1 - it0, 0), n_items = n_main + (has_tail ? 1 : 0);
+    const int first = n_main > 0 ? it0 : tail_item;
+    const int first_slab = first / p.nrb, first_rb = first - first_slab * p.nrb;
+    int slab = first_slab, rb = first_rb;
+    int nslab = slab, nrb = rb;
+    if (n_items > 0) {
+        aim(slab, rb);
+#pragma unroll
+        for (int u = 0; u < R; ++u) load_row(u);
+    }
+
     if (MODE == AAAC_NVFP4 && tid >= 64 && tid < 192) {
         const int c = tid - 64;
         const float sv = __fmul_rn(e4m3_value((uint32_t)c), p.ctrl->s_t);
         S.rlut[c] = c ? __frcp_rn(sv) : 0.f;
     }
-    __syncthreads();
 
-    // Fixed-point scale of the sums over the blocks.  Every sum of a pass is bounded by
-    // B = 256 N K max_k I_k (|w~ - c| < 16), so with 2^e > B the value v 2^(94 - e) fits 96 bits; what
-    // is dropped lies 2^-86 below B.  Integer addition is order-independent, so the totals do not
-    // depend on the order in which the blocks arrive (max is order-independent too).
+    // Fixed-point scale of the sums over the blocks.  Every sum of a pass is below B = 256 N sum_k I_k
+    // (|w~ - c| < 16), so with 2^e > B the value v 2^(78 - e) fits the limbs; what is dropped lies 2^-78
+    // below B, far below the rounding of a block's own sums.  Integer addition is order-independent, so
+    // the totals do not depend on the order in which the blocks arrive.
     {
-        float mx = 0.f;
-        for (int k = tid; k < K; k += NT) mx = fmaxf(mx, fabsf(__ldg(p.I + k)));
+        float sum = 0.f;
+        for (int k = tid; k < K; k += NT) sum = __fadd_ru(sum, fabsf(__ldg(p.I + k)));
 #pragma unroll
-        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-        float* red = reinterpret_cast<float*>(lut1_mem);
-        if (lane == 0) red[warp] = mx;
+        for (int o = 16; o; o >>= 1) sum = __fadd_ru(sum, __shfl_xor_sync(kAll, sum, o));
+        if (lane == 0) sh.wsum[warp][0] = (double)sum;
         __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < NW; ++w) mx = fmaxf(mx, red[w]);
-            const double B = 256.0 * (double)N * (double)K * (double)mx;
-            int e = 0;
-            if (B > 0.0 && B < 1e300) e = ilogb(B) + 1;
-            S.fix_scale = scalbn(1.0, 94 - e);
-            S.fix_unscale = scalbn(1.0, e - 94);
+        if (warp == 0) {
+            double B = sh.wsum[lane & 15][0];
+#pragma unroll
+            for (int o = 8; o; o >>= 1) B += __shfl_xor_sync(kAll, B, o);
+            B *= 257.0 * (double)N;
+            if (lane == 0) {
+                const int e = B > 0.0 && B < 1e300 ? ilogb(B) + 1 : 0;
+                sh.fix_scale = scalbn(1.0, 78 - e);
+                sh.fix_unscale = scalbn(1.0, e - 78);
+                sh.failed = 0;
+            }
+            derive_tables(S, lane, p.ctrl->T[lane]);
         }
-        __syncthreads();
     }
+    for (int b = 0; b < kBinSlots; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
+    __syncthreads();
+    write_tables<NT>(S, tid, kLut1At, lut2_addr);
+    __syncthreads();
 
     // bin arithmetic: the masked mantissa of fl32(kBinsPerUnit x + kMagic) is bin * (REP * 8)
     constexpr float kBinsPerUnit = (float)(NB / 16);
     constexpr float kMagic = (float)(NB / 2) + 1.5f * (float)(1 << 23) / (float)(REP * 8);
     constexpr uint32_t kBinMask = (uint32_t)(NB - 1) * (REP * 8);
 
-    for (int b = 0; b < kCells; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
   for (int round = 0; round < p.n_rounds; ++round) {
     const unsigned pass_no = p.bar_base + (unsigned)round;
     // block 0 clears the buffer of the next pass: it was the buffer of two passes ago, and every block
     // finished reading it before it added to the previous pass's buffer, whose totals block 0 has seen
-    static_assert(NT >= 256 + kUsed * kLimbs, "threads 256.. of block 0 clear the next buffer");
-    if (bid == 0 && tid >= 256 && tid < 256 + kUsed * kLimbs) {
-        p.acc[(size_t)((pass_no + 1u) % 3u) * kAccBuffer + (size_t)(tid - 256) * kAccStride] = 0ull;
+    static_assert(NT >= 256 + kCells * 4 + kLimbs, "threads 256.. of block 0 clear the next buffer");
+    if (bid == 0 && tid >= 256 && tid < 256 + kCells * 4 + kLimbs) {
+        const int w = tid - 256;
+        p.acc[(size_t)((pass_no + 1u) % 3u) * kAccBuffer + (size_t)(w >> 2) * kAccStride + (w & 3)] = 0ull;
         __threadfence();
     }
-    build_tables<MODE, NW, REP, NB>(S, lut1_mem, lut2_mem);
     // near-tie bound: sqrt(a b) <= (kappa a + b / kappa) / 2, so the bound of the header comment is at
     // most g1 * (E0 + E1) + g2 * sum I, with kappa = 1/8 (about the usual |w~ - entry|)
     const float g1 = 0x1p-24f * __fmaf_ru(S.tmax283, 4.f, 16.f), g2 = 0x1p-24f * __fmul_ru(S.tmax283, 0.0625f);
     double Eacc = 0.0;
 
-   auto pass = [&](auto inner_tag) {
-    constexpr bool INNER = decltype(inner_tag)::value;
-    constexpr bool keep_sigma = KIND == kAssignKeep;
-    // Row registers of the item being processed; a row's registers are refilled with the same row
-    // of the next item as soon as the row has been unpacked, so the load has about an item's time
-    // to arrive and no second buffer is needed.
-    uint4 v[R];
-    uint32_t sc[R];           // NVFP4: scale byte; INT4: bits of the reciprocal scale
-    uint32_t sgw[R];          // inner iteration: the row's stored selection bits
-    // (An unguarded form with clamped indices was measured too: faster for some instantiations, slower
-    // for others, depending on what else the kernel held; the guarded form is the one kept.)
-    auto load_row = [&](int u, int slab, int rb) {
-        const int col0 = slab * 256 + lane * 8;
-        const int row = rb * kRowsPerItem + warp * R + u;
-        v[u] = make_uint4(0, 0, 0, 0);
-        sc[u] = 0u;
-        if (INNER) sgw[u] = 0u;
-        if (col0 < K && row < N) {
-            // element offsets fit 32 bits (the entry points refuse layers of 2^32 elements and more)
-            v[u] = __ldcs(reinterpret_cast<const uint4*>(p.W + ((unsigned)row * (unsigned)p.ldw + (unsigned)col0)));
-            const unsigned gi = (unsigned)row * (unsigned)Gr + (unsigned)col0 / G;
-            if (MODE == AAAC_NVFP4) sc[u] = p.scales[gi];          // masked at use: nothing waits on the load here
-            else sc[u] = __float_as_uint(__ldg(p.rinv + gi));
-            if (INNER) sgw[u] = __ldcg(p.sigw + (size_t)row * (size_t)slabs + slab);
-        }
-    };
-
-    int cur_slab = -1;
     int ndefer = 0;           // groups on the warp's list (the same in every lane)
-    uint64_t II[8];           // {I, I} of the lane's eight columns
-    float isum = 0.f;         // g2 * sum of I over the lane's group (rounded up a little)
-    bool col_ok = false;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) II[j] = 0ull;
-
-    // (slab, row block) of the current item and of the one being loaded
-    const int n_main = max(it1 - it0, 0), n_items = n_main + (has_tail ? 1 : 0);
-    const int first = n_main > 0 ? it0 : tail_item;
-    int slab = first / p.nrb, rb = first - slab * p.nrb;
-    int nslab = slab, nrb = rb;
-    if (n_items > 0) {
-#pragma unroll
-        for (int u = 0; u < R; ++u) load_row(u, slab, rb);
-    }
+    float isum = __fmul_ru(isum_raw, g2);
     for (int i = 0; i < n_items; ++i) {
         slab = nslab;
         rb = nrb;
@@ -395,17 +439,17 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             nslab = tail_item / p.nrb;
             nrb = tail_item - nslab * p.nrb;
         }
-        // After the last item nothing follows: its own rows are fetched once more (in bounds, unused), so
-        // that the loads of the next item's rows stand in the row pipeline without a branch around them
-        // (with one, the compiler kept them from moving: 799 -> 835 Gweights/s on the benchmark layers).
-        if (i + 1 >= n_items) { nslab = slab; nrb = rb; }
+        // (the loads of the next item's rows stand in the row pipeline without a branch around them: with
+        // one, the compiler kept them from moving, 835 -> 799 Gweights/s)
+        if (i + 1 >= n_items) { nslab = first_slab; nrb = first_rb; }
+        aim(nslab, nrb);
         const bool whole = i < n_main;                     // else: row tail_u of every warp only
 
         if (slab != cur_slab) {
             cur_slab = slab;
             const int col0 = slab * 256 + lane * 8;
             col_ok = col0 < K;
-            isum = 0.f;
+            isum_raw = 0.f;
             float Iv[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) Iv[j] = 0.f;
@@ -416,13 +460,16 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 Iv[4] = b.x; Iv[5] = b.y; Iv[6] = b.z; Iv[7] = b.w;
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { isum += Iv[j]; II[j] = pack2(Iv[j], Iv[j]); }
+            for (int j = 0; j < 8; ++j) isum_raw += Iv[j];
 #pragma unroll
-            for (int o = LPG / 2; o; o >>= 1) isum += __shfl_xor_sync(0xFFFFFFFFu, isum, o);
-            isum = __fmul_ru(isum * 1.0001f, g2);
+            for (int j = 0; j < 4; ++j) II[j] = pack2(Iv[2 * j], Iv[2 * j + 1]);
+#pragma unroll
+            for (int o = LPG / 2; o; o >>= 1) isum_raw += __shfl_xor_sync(0xFFFFFFFFu, isum_raw, o);
+            isum_raw *= 1.0001f;
+            isum = __fmul_ru(isum_raw, g2);
         }
-        const int row0 = rb * kRowsPerItem + warp * R;
-        const int nrows = min(R, N - row0);                // rows of this warp inside the layer (may be <= 0)
+        const int row0 = (rb * NW + warp) * rows;
+        const int nrows = min(rows, N - row0);                // rows of this warp inside the layer (may be <= 0)
 
         // The rows of the item go through three stages, written out in the order in which the
         // shared-memory operations are to be issued, so that the read-modify-write chain on the
@@ -440,18 +487,21 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             if (INNER) sg_row = (sgw[u] >> lane) & 1u;
             const float rinv = MODE == AAAC_NVFP4 ? S.rlut[sc[u] & 0x7Fu] : __uint_as_float(sc[u]);
             const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+            const uint64_t rr = pack2(rinv, rinv);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                x[j] = __fmul_rn((j & 1) ? bf16_hi(w[j >> 1]) : bf16_lo(w[j >> 1]), rinv);
-                // (bin bits | lane's copy) is one three-input logic instruction, and the table's base, the
-                // same for every lane, can ride in the load's address: no add per weight
-                e1v[j] = lds_table_u2(((uint32_t)__float_as_int(__fmaf_rn(x[j], kBinsPerUnit, kMagic)) & kBinMask) | lut1_or);
+            for (int j = 0; j < 4; ++j) {
+                const uint64_t xx = mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr);
+                const uint64_t bb = fma2(xx, pack2(kBinsPerUnit, kBinsPerUnit), pack2(kMagic, kMagic));
+                unpack2(xx, x[2 * j], x[2 * j + 1]);
+                // (bin bits | lane's copy | table base) is one three-input logic instruction: no add per weight
+                e1v[2 * j] = lds_table_u2((__float_as_uint(lo2(bb)) & kBinMask) | lut1_or);
+                e1v[2 * j + 1] = lds_table_u2((__float_as_uint(hi2(bb)) & kBinMask) | lut1_or);
             }
         };
         // same, then refill the row's registers from the next item
         auto L1n = [&](int u) {
             L1(u);
-            load_row(u, nslab, nrb);
+            load_row(u);
         };
         auto L2 = [&]() {
 #pragma unroll
@@ -468,14 +518,14 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                     float cP, cQ;
                     unpack2(pq[j], cP, cQ);
                     c[j] = sg ? cQ : cP;
-                    mt_o[j] = __fmul_rn(lo2(II[j]), __fsub_rn(x[j], c[j]));
+                    mt_o[j] = __fmul_rn(Ic(j), __fsub_rn(x[j], c[j]));
                     chk += mt_o[j];
                 }
                 const bool bad = !(chk == chk);
                 if (__any_sync(0xFFFFFFFFu, bad)) {
                     Row8 r;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) { r.x[j] = x[j]; r.I[j] = lo2(II[j]); r.hint[j] = kNoHint; }
+                    for (int j = 0; j < 8; ++j) { r.x[j] = x[j]; r.I[j] = Ic(j); r.hint[j] = kNoHint; }
                     const Exact8 ex = exact_groups<LPG>(&S, r, (int)bad);
                     if (bad) {
 #pragma unroll
@@ -483,7 +533,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                             float cP, cQ;
                             unpack2(lds_table_b64(pq_entry_addr(lut2_addr, ex.J[j], lane)), cP, cQ);
                             c[j] = sg ? cQ : cP;
-                            mt_o[j] = __fmul_rn(lo2(II[j]), __fsub_rn(x[j], c[j]));
+                            mt_o[j] = __fmul_rn(Ic(j), __fsub_rn(x[j], c[j]));
                         }
                     }
                 }
@@ -492,15 +542,22 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 for (int j = 0; j < 8; ++j) ba_o[j] = base + (__float_as_uint(c[j]) & kIdxMask) * kSlotBytes;
                 return;
             }
-            uint64_t m[8];                                 // {I (x - P), I (x - Q)}
-            uint64_t e01 = 0ull;
+            // (pairs of columns rather than pairs of tables: eight registers of importances instead of sixteen)
+            uint64_t m0[4], m1[4];                         // I (x - P), I (x - Q)
+            uint64_t s0 = 0ull, s1 = 0ull;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint64_t u01 = diff2(x[j], pq[j]);
-                m[j] = mul2(II[j], u01);
-                e01 = fma2(m[j], u01, e01);
+            for (int j = 0; j < 4; ++j) {
+                float Pa, Qa, Pb, Qb;
+                unpack2(pq[2 * j], Pa, Qa);
+                unpack2(pq[2 * j + 1], Pb, Qb);
+                const uint64_t u0 = pack2(__fsub_rn(x[2 * j], Pa), __fsub_rn(x[2 * j + 1], Pb));
+                const uint64_t u1 = pack2(__fsub_rn(x[2 * j], Qa), __fsub_rn(x[2 * j + 1], Qb));
+                m0[j] = mul2(II[j], u0);
+                m1[j] = mul2(II[j], u1);
+                s0 = fma2(m0[j], u0, s0);
+                s1 = fma2(m1[j], u1, s1);
             }
-            float e0 = lo2(e01), e1 = hi2(e01);
+            float e0 = lo2(s0) + hi2(s0), e1 = lo2(s1) + hi2(s1);
 #pragma unroll
             for (int s = LPG / 2; s; s >>= 1) {
                 e0 += __shfl_xor_sync(0xFFFFFFFFu, e0, s);
@@ -532,10 +589,10 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             // cell = entry index (low bits of the centre constant) under the chosen table
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                float m0, m1, cP, cQ;
-                unpack2(m[j], m0, m1);
+                const float a0 = (j & 1) ? hi2(m0[j >> 1]) : lo2(m0[j >> 1]), a1 = (j & 1) ? hi2(m1[j >> 1]) : lo2(m1[j >> 1]);
+                float cP, cQ;
                 unpack2(pq[j], cP, cQ);
-                mt_o[j] = sg ? m1 : m0;
+                mt_o[j] = sg ? a1 : a0;
                 ba_o[j] = base + (__float_as_uint(sg ? cQ : cP) & idx_mask) * kSlotBytes;
             }
         };
@@ -544,7 +601,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             for (int j = j0; j < j1; ++j) {
                 float2 a = lds_bin(ba_i[j]);
                 a.x += mt_i[j];
-                a.y += lo2(II[j]);
+                a.y += Ic(j);
                 sts_bin(ba_i[j], a);
             }
         };
@@ -565,8 +622,18 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 M(row0 + u, mt[cur], ba[cur]);
             }
             B(mt[(R - 1) & 1], ba[(R - 1) & 1], 0, 8);
+        } else if (nrows == 2 && rows == 2) {
+            L1n(0);
+            L2();
+            M(row0, mt[0], ba[0]);
+            L1n(1);
+            B(mt[0], ba[0], 0, 2);
+            L2();
+            B(mt[0], ba[0], 2, 8);
+            M(row0 + 1, mt[1], ba[1]);
+            B(mt[1], ba[1], 0, 8);
         } else {
-            // ragged last row block of the layer: row by row, then refill all rows
+            // ragged last row block of the layer, quarter items, items of one row: row by row, then refill all rows
             uint4 vr[R];
             uint32_t sr[R], gr[R];
 #pragma unroll
@@ -583,7 +650,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 B(mt[0], ba[0], 0, 8);
             }
 #pragma unroll
-            for (int t = 0; t < R; ++t) load_row(t, nslab, nrb);
+            for (int t = 0; t < R; ++t) load_row(t);
         }
         Eacc += (double)eitem;
         if (!INNER && ndefer > kDeferCap - R * (32 / LPG)) {    // the next item could overflow the list
@@ -596,90 +663,115 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         __syncwarp();
         Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw}, list_addr, ndefer, bins_lane, lane);
     }
-   };
-    pass(std::integral_constant<bool, KIND == kInner>{});
 
-    // ---- block partial: lane c of a warp adds the 32 lane-private values of cell c (in a
-    //      rotated, fixed order that avoids bank conflicts); then the warps are added ----
-    __syncthreads();                                       // every warp is done with the lookup tables
+    // ---- the warp's sums: lane c adds the 32 lane-private values of cell c (in an order of its own that
+    //      avoids bank conflicts, and a fixed one).  In double, 32 FP32 values are added without rounding
+    //      unless they are more than 2^24 apart.  Then the warp's bins start the next pass at zero ----
+    const bool trace = KIND != kInner && p.err_trace != nullptr;
+    __syncwarp();
     {
-        // four interleaved chains in double: 32 FP32 values go into 53 bits without rounding unless they
-        // are more than 2^24 apart, and then by less than 2^-52 of the sum
+        const uint32_t cell_addr = bins_warp + lane * (kSlotBytes + 8);
         double dx[4] = {0.0, 0.0, 0.0, 0.0}, dy[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+        for (uint32_t i = 0; i < 256; i += 32) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float2 a = lds_bin(bins_warp + lane * kSlotBytes + ((i + lane) & 31) * 8);
-            dx[i & 3] += (double)a.x;
-            dy[i & 3] += (double)a.y;
+            for (uint32_t t = 0; t < 4; ++t) {
+                const float2 a = lds_bin(cell_addr ^ (i + t * 8));
+                dx[t] += scaled_double(a.x);
+                dy[t] += __hiloint2double(__float_as_int(a.y) >> 3, __float_as_int(a.y) << 29);      // (weights are not negative)
+            }
         }
-        wsum[warp * kPartStride + lane] = (dx[0] + dx[1]) + (dx[2] + dx[3]);
-        wsum[warp * kPartStride + kCells + lane] = (dy[0] + dy[1]) + (dy[2] + dy[3]);
-        // the warp's bins start the next pass at zero (done here, ahead of the wait for the totals)
+        sh.wsum[warp][lane] = ((dx[0] + dx[1]) + (dx[2] + dx[3])) * 0x1p896;
+        sh.wsum[warp][kCells + lane] = ((dy[0] + dy[1]) + (dy[2] + dy[3])) * 0x1p896;
+        if (trace) {
+#pragma unroll
+            for (int s = 16; s; s >>= 1) Eacc += __shfl_xor_sync(kAll, Eacc, s);
+            if (lane == 0) sh.wsum[warp][2 * kCells] = Eacc;
+        }
         __syncwarp();
 #pragma unroll 8
         for (int b = 0; b < kCells; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
     }
+    __syncthreads();                                       // every warp is done with the lookup tables, its sums are there
+    unsigned long long* const acc = p.acc + (size_t)(pass_no % 3u) * kAccBuffer;
+    // ---- the block's sums: half-warp h of warp v adds cell 2 v + h, a lane per warp, pairwise ----
+    static_assert(NW == 16 && 2 * NW == kCells, "a half-warp per cell, a lane per warp");
+    {
+        const int sum_warp = lane & 15, sum_cell = 2 * warp + (lane >> 4);
+        double dxs = sh.wsum[sum_warp][sum_cell], dys = sh.wsum[sum_warp][kCells + sum_cell];
+        double de = 0.0;
+        const bool do_e = trace && warp == NW - 1;
+        if (do_e) de = sh.wsum[sum_warp][2 * kCells];
 #pragma unroll
-    for (int s = 16; s; s >>= 1) Eacc += __shfl_xor_sync(0xFFFFFFFFu, Eacc, s);
-    if (lane == 0) wsum[warp * kPartStride + 2 * kCells] = Eacc;
-    __syncthreads();
-    // this block's sums go into the pass's buffer as three 32-bit limbs of a 96-bit fixed-point number,
-    // each with one arrival in the word's upper bits
-    unsigned long long* acc = p.acc + (size_t)(pass_no % 3u) * kAccBuffer + (size_t)tid * (kLimbs * kAccStride);   // this thread's three words
-    const unsigned long long want = (unsigned long long)p.arrivals;
-    bool ok = true;
-    if (tid < kUsed) {
-        double ws_[NW];                                     // the warps' sums, added pairwise (a fixed order)
-#pragma unroll
-        for (int w = 0; w < NW; ++w) ws_[w] = wsum[w * kPartStride + tid];
-#pragma unroll
-        for (int stride = 1; stride < NW; stride *= 2)
-#pragma unroll
-            for (int w = 0; w + stride < NW; w += 2 * stride) ws_[w] += ws_[w + stride];
-        const double sd = ws_[0] * S.fix_scale;
-        const double t2 = floor(sd * 0x1p-64);             // in [-2^30, 2^30)
-        const double r = sd - t2 * 0x1p64;                 // exact, in [0, 2^64)
-        const double t1 = floor(r * 0x1p-32);
-        const double t0 = floor(r - t1 * 0x1p32);
-        atomicAdd(acc + 0 * kAccStride, (unsigned long long)t0 + kOneArrival);
-        atomicAdd(acc + 1 * kAccStride, (unsigned long long)t1 + kOneArrival);
-        atomicAdd(acc + 2 * kAccStride, (unsigned long long)((long long)t2 + kTopBias) + kOneArrival);
+        for (int s = 8; s; s >>= 1) {
+            dxs += __shfl_xor_sync(kAll, dxs, s);
+            dys += __shfl_xor_sync(kAll, dys, s);
+            if (do_e) de += __shfl_xor_sync(kAll, de, s);
+        }
+        // The sums go into the pass's buffer as two 40-bit limbs, each with one arrival in the word's upper
+        // bits: lanes 0-1 of the half-warp add the residual sum's limbs, 2-3 those of the weight sum, 4-5 of
+        // the last warp's first half those of the objective.
+        const int which = sum_warp >> 1;
+        const double sd = (which == 0 ? dxs : which == 1 ? dys : de) * sh.fix_scale;
+        const double topm = __dadd_rd(sd * 0x1p-40, kIntMagic);               // floor, as the low bits of a double near 1.5 2^52
+        const long long top = __double_as_longlong(topm) - __double_as_longlong(kIntMagic);          // in [-2^38, 2^38)
+        const double lowm = __dadd_rd(__fma_rn(-(topm - kIntMagic), 0x1p40, sd), kIntMagic);
+        const long long low = __double_as_longlong(lowm) - __double_as_longlong(kIntMagic);          // in [0, 2^40)
+        const unsigned long long add = (unsigned long long)((sum_warp & 1) ? top + kTopBias : low) + kOneArrival;
+        if (which < 2) atomicAdd(acc + sum_cell * kAccStride + sum_warp, add);
+        else if (do_e && lane < 6 && which == 2) atomicAdd(acc + kCells * kAccStride + (lane - 4), add);
     }
-    // ---- wait until every block's sums are in, then read the totals.  One thread of the block
-    //      polls one word (all blocks add all their words at about the same time; a crowd of
-    //      pollers on the accumulators' cache lines would hold the atomics up); after it every
-    //      thread checks the arrival counts of its own words and waits on if they are short ----
-#ifndef AAAC_FIT_POLL_ALL
-#define AAAC_FIT_POLL_ALL 0
-#endif
-#if !AAAC_FIT_POLL_ALL
-    if (tid == kUsed - 1) {
+    // ---- one warp waits until every block's sums are in and derives the new tables; lane c takes cell c ----
+    if (warp == 0) {
+        const unsigned long long want = (unsigned long long)p.arrivals;
+        const bool my_e = trace && bid == 0 && lane == 0;
+        bool ok = true;
+        unsigned long long x[2], y[2], e[2] = {0, 0};
         for (unsigned spins = 0;; ++spins) {
-            if ((ld_relaxed_u64(acc) >> kCountShift) >= want) break;
-            if (spins >= p.spin_limit || ld_relaxed_u32(&p.ctrl->abort)) { ok = false; break; }
-            __nanosleep(32);
+            ld_relaxed_2xu64(acc + lane * kAccStride, x[0], x[1]);
+            ld_relaxed_2xu64(acc + lane * kAccStride + 2, y[0], y[1]);
+            if (my_e) ld_relaxed_2xu64(acc + kCells * kAccStride, e[0], e[1]);
+            bool in = true;
+#pragma unroll
+            for (int l = 0; l < kLimbs; ++l)
+                in = in && (x[l] >> kCountShift) >= want && (y[l] >> kCountShift) >= want && (!my_e || (e[l] >> kCountShift) >= want);
+            if (__all_sync(kAll, in)) break;
+            if (__any_sync(kAll, spins >= p.spin_limit || ((spins & 15u) == 15u && ld_relaxed_u32(&p.ctrl->abort)))) { ok = false; break; }
+        }
+        if (!ok) {
+            if (lane == 0) sh.failed = 1;
+        } else {
+            auto total = [&](const unsigned long long (&w)[2]) {
+                const long long top = (long long)(w[1] & kLimbMask) - (long long)nblk * kTopBias;
+                const long long low = (long long)(w[0] & kLimbMask);
+                const double t = __longlong_as_double(top + __double_as_longlong(kIntMagic)) - kIntMagic;
+                const double l = __longlong_as_double(low + __double_as_longlong(kIntMagic)) - kIntMagic;
+                return __fma_rn(t, 0x1p40, l) * sh.fix_unscale;
+            };
+            // Eq. 11; cells of duplicate entries are empty: they keep their value
+            const double sx = total(x), wt = total(y);
+            double T = wt > 0.0 ? (double)S.centre[lane] + __ddiv_rn(sx, wt) : S.Td[lane];
+            // the trace holds the Eq. 8 objective of each assignment step
+            if (my_e) p.err_trace[p.trace_base + round] = total(e);
+            const double Tp = __shfl_up_sync(kAll, T, 1);
+            if (__any_sync(kAll, (lane & 15) != 0 && Tp > T)) {
+                // ascending order within the table by rank (ties by index)
+                int rank = 0;
+#pragma unroll 1
+                for (int i = 0; i < kM; ++i) {
+                    const double o = __shfl_sync(kAll, T, (lane & 16) + i);
+                    rank += (o < T) || (o == T && i < (lane & 15));
+                }
+                S.Td[(lane & 16) + rank] = T;
+                __syncwarp();
+                T = S.Td[lane];
+                __syncwarp();
+            }
+            derive_tables(S, lane, T);
         }
     }
     __syncthreads();
-#endif
-    if (tid < kUsed) {
-        unsigned long long w0, w1, w2;
-        for (unsigned spins = 0;; ++spins) {
-            w0 = ld_relaxed_u64(acc + 0 * kAccStride);
-            w1 = ld_relaxed_u64(acc + 1 * kAccStride);
-            w2 = ld_relaxed_u64(acc + 2 * kAccStride);
-            if ((w0 >> kCountShift) >= want && (w1 >> kCountShift) >= want && (w2 >> kCountShift) >= want) break;
-            if (spins >= p.spin_limit || ld_relaxed_u32(&p.ctrl->abort)) { ok = false; break; }
-            __nanosleep(64);
-        }
-        const long long l2 = (long long)(w2 & kLimbMask) - (long long)nblk * kTopBias;
-        __int128 v = ((__int128)l2 << 64) + ((__int128)(w1 & kLimbMask) << 32) + (__int128)(w0 & kLimbMask);
-        const bool neg = v < 0;
-        if (neg) v = -v;
-        const double mag = (double)(unsigned long long)(v >> 64) * 0x1p64 + (double)(unsigned long long)v;
-        S.tot[tid] = (neg ? -mag : mag) * S.fix_unscale;
-    }
-    if (!__syncthreads_and(ok)) {
+    if (sh.failed) {
         // a wait ran out (here or in another block): tell the others, report, leave
         if (tid == 0) {
             atomicExch(&p.ctrl->abort, 1u);
@@ -687,25 +779,10 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         }
         return;
     }
-    if (tid < 2 * kM) {
-        // cells of duplicate entries are empty: they keep their value
-        const double sx = S.tot[tid], wt = S.tot[kCells + tid];
-        S.tot[2 * kCells + 1 + tid] = (wt > 0.0) ? (double)S.centre[tid] + __ddiv_rn(sx, wt) : S.Td[tid];
+    if (round + 1 < p.n_rounds) {
+        write_tables<NT>(S, tid, kLut1At, lut2_addr);
+        __syncthreads();
     }
-    __syncthreads();
-    if (tid < 2 * kM) {
-        // ascending order within the table by rank (ties by index)
-        const double* tn = S.tot + 2 * kCells + 1 + (tid & 16);
-        const double t = tn[tid & 15];
-        int rank = 0;
-#pragma unroll 1
-        for (int i = 0; i < kM; ++i) rank += (tn[i] < t) || (tn[i] == t && i < (tid & 15));
-        S.Td[(tid & 16) + rank] = t;
-    }
-    // the trace holds the Eq. 8 objective of each assignment step
-    if (KIND != kInner && bid == 0 && tid == 0 && p.err_trace)
-        p.err_trace[p.trace_base + round] = S.tot[2 * kCells];
-    __syncthreads();
   }
     if (bid == 0 && tid < 2 * kM) {
         p.ctrl->T[tid] = S.Td[tid];
@@ -713,34 +790,22 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     }
 }
 
-template <int MODE, int SEL, int NW, int REP, int KIND>
-__global__ void __launch_bounds__(NW * 32, 1) fit_rounds_kernel(const FitParams p) {
-    fit_rounds_body<MODE, SEL, NW, REP, KIND>(p, blockIdx.x, gridDim.x);
-}
-
 // Several layers in one launch (the paper processes layers independently, Sec. 3.3): the grid is
 // cut into consecutive ranges of blocks, one per layer, and every range runs that layer's rounds
 // by itself -- its blocks wait only for each other, on the layer's own accumulators -- so the
 // per-round fixed cost (sums across blocks, new tables, table building) is paid once for the
 // whole batch instead of once per layer, and small layers no longer leave most of the GPU idle.
-// The parameters of every layer stay kernel arguments (one copy of the code per slot).
 constexpr int kMaxBatch = 8;
 struct FitBatch {
     FitParams L[kMaxBatch];
     unsigned first[kMaxBatch + 1];    // first block of every layer; first[n..] = grid size
 };
 
-template <int MODE, int SEL, int NW, int REP>
-__global__ void __launch_bounds__(NW * 32, 1) fit_batch_kernel(const FitBatch b) {
-    const unsigned bx = blockIdx.x;
-#define AAAC_BATCH_SLOT(i)                                                                              \
-    if (bx < b.first[i + 1]) {                                                                           \
-        fit_rounds_body<MODE, SEL, NW, REP, kRounds>(b.L[i], bx - b.first[i], b.first[i + 1] - b.first[i]); \
-        return;                                                                                          \
-    }
-    AAAC_BATCH_SLOT(0) AAAC_BATCH_SLOT(1) AAAC_BATCH_SLOT(2) AAAC_BATCH_SLOT(3)
-    AAAC_BATCH_SLOT(4) AAAC_BATCH_SLOT(5) AAAC_BATCH_SLOT(6) AAAC_BATCH_SLOT(7)
-#undef AAAC_BATCH_SLOT
+template <int MODE, int SEL, int KIND>
+__global__ void __launch_bounds__(kFitWarps * 32, 1) fit_kernel(const __grid_constant__ FitBatch b) {
+    int l = 0;
+    while (l + 1 < kMaxBatch && blockIdx.x >= b.first[l + 1]) ++l;
+    fit_rounds_body<MODE, SEL, KIND>(b.L[l], blockIdx.x - b.first[l], b.first[l + 1] - b.first[l]);
 }
 
 __global__ void export_tables_kernel(const Ctrl* ctrl, float* T01) {
@@ -761,18 +826,25 @@ cudaError_t fit_dynamic_smem(const void* kern, size_t* bytes) {
     return cudaSuccess;
 }
 
-template <int MODE, int SEL, int NW, int REP, int KIND>
-cudaError_t launch_variant(FitParams& p, unsigned grid, cudaStream_t st) {
-    auto kern = fit_rounds_kernel<MODE, SEL, NW, REP, KIND>;
+template <int MODE, int SEL, int KIND>
+cudaError_t launch_variant(FitBatch& b, unsigned grid, cudaStream_t st) {
+    auto kern = fit_kernel<MODE, SEL, KIND>;
     size_t smem = 0;
     cudaError_t e = fit_dynamic_smem(reinterpret_cast<const void*>(kern), &smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    void* args[] = {&p};
+    void* args[] = {&b};
     note_launch();
-    // cooperative: every block is resident, which the grid-wide barrier relies on
-    return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3(grid), dim3(NW * 32), args, smem, st);
+    // cooperative: the blocks of a layer wait for each other, so all of them must be resident
+    return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3(grid), dim3(kFitWarps * 32), args, smem, st);
+}
+
+template <int KIND>
+cudaError_t launch_kind(FitBatch& b, unsigned grid, int mode, int sel_group, cudaStream_t st) {
+    if (mode == AAAC_INT4 && sel_group == 16) return launch_variant<AAAC_INT4, 16, KIND>(b, grid, st);
+    if (mode == AAAC_INT4) return launch_variant<AAAC_INT4, 128, KIND>(b, grid, st);
+    return launch_variant<AAAC_NVFP4, 16, KIND>(b, grid, st);
 }
 
 }  // namespace
@@ -781,29 +853,42 @@ cudaError_t launch_variant(FitParams& p, unsigned grid, cudaStream_t st) {
 // shorter for the busiest block, a tail dealt out one row per warp (a quarter item) per block.
 // Returns the number of blocks actually used.
 static int64_t plan_layer(FitParams& p, int64_t N, int64_t K, int64_t blocks) {
-    const int64_t slabs = (K + 255) / 256;
-    constexpr int kRowsPerItem = kRowsPerWarp * AAAC_FIT_WARPS;
-    const int64_t nrb = (N + kRowsPerItem - 1) / kRowsPerItem, items = slabs * nrb;
-    int64_t grid = blocks;
-    if (grid > items) grid = items;
-    if (grid > kMaxFitBlocks) grid = kMaxFitBlocks;
-    int64_t per_block = (items + grid - 1) / grid;
+    const int64_t slabs = (K + 255) / 256, g = blocks < kMaxFitBlocks ? blocks : kMaxFitBlocks;
+    p.rows = kRowsPerWarp;
+    p.nrb = (int)((N + kRowsPerWarp * kFitWarps - 1) / (kRowsPerWarp * kFitWarps));
+    const int64_t items = slabs * p.nrb;
+    p.per_block = (int)((items + g - 1) / g);
     p.tail_item0 = (int)items;
     p.tail_quarters = 0;
+    int64_t grid = 0, cost = 10 * kRowsPerWarp * (int64_t)p.per_block;
     {
         // an even number of whole items per block plus a quarter-item tail, where that is shorter for
         // the busiest block (a tail row costs more than a quarter of a pipelined item: count it double)
-        const int64_t g = blocks < kMaxFitBlocks ? blocks : kMaxFitBlocks;
         const int64_t whole = items / g, rest = items - whole * g;
-        if (whole >= 4 && rest > 0 && 4 * rest <= g && 2 * whole + 1 < 2 * per_block) {
-            per_block = whole;
+        if (whole >= 4 && rest > 0 && 4 * rest <= g && 2 * whole + 1 < 2 * p.per_block) {
+            p.per_block = (int)whole;
             p.tail_item0 = (int)(whole * g);
             p.tail_quarters = (int)(4 * rest);
             grid = g;
         }
     }
-    if (p.tail_quarters == 0) grid = (items + per_block - 1) / per_block;
-    p.nrb = (int)nrb; p.items = (int)items; p.per_block = (int)per_block;
+    // Layers with few items per block: items of two rows or one row per warp, where that is shorter for the
+    // busiest block (a row of such an item counts for 1.2 and 1.6 rows of the four-row pipeline).  512 x 512:
+    // 16 blocks of one item, 8.5 us a pass -> 64 blocks of one row per warp, 6.9; 1531 x 2064: two items of
+    // four rows -> three of two, 11.4 -> 10.6 us.
+    for (int rows = 2; rows >= 1; --rows) {
+        const int64_t nrb = (N + rows * kFitWarps - 1) / (rows * kFitWarps), it = slabs * nrb, per = (it + g - 1) / g;
+        const int64_t c = per * (rows == 2 ? 24 : 16);
+        if (c < cost && p.tail_quarters == 0) {
+            cost = c;
+            p.rows = rows;
+            p.nrb = (int)nrb;
+            p.per_block = (int)per;
+            p.tail_item0 = (int)it;
+        }
+    }
+    p.items = (int)(slabs * p.nrb);
+    if (p.tail_quarters == 0) grid = (p.items + p.per_block - 1) / p.per_block;
     p.arrivals = (unsigned)grid + (unsigned)g_extra_arrivals;
     return grid;
 }
@@ -817,79 +902,21 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
     p.spin_limit = g_spin_limit;
     p.sigw = a.ws.qlist;            // the quantile selection's list is free once the start tables exist
     const int64_t slabs = (a.K + 255) / 256;
-    constexpr int kRowsPerItem = kRowsPerWarp * AAAC_FIT_WARPS;
-    const int64_t nrb = (a.N + kRowsPerItem - 1) / kRowsPerItem;
+    const int64_t nrb = (a.N + kFitWarps - 1) / kFitWarps;
     return !(a.N > 0x7FFFFFFF || a.K > 0x7FFFFFFF || slabs * nrb > 0x7FFFFFFF);
-}
-
-cudaError_t launch_fit_rounds(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, int sel_group, const void* scales,
-                              const float* I, int n_outer, int n_inner, double* err_trace, float* T01_out, uint32_t* dev_status,
-                              const Workspace& ws, cudaStream_t st) {
-    if (n_outer <= 0) return cudaSuccess;
-    if (n_inner < 1 || (int64_t)n_outer * n_inner > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    FitLayerArgs a{W, N, K, ldw, scales, I, err_trace, T01_out, ws};
-    FitParams p;
-    if (!fill_params(p, a, n_outer, dev_status)) return cudaErrorInvalidValue;
-    const int64_t grid = plan_layer(p, N, K, sm_count());
-    constexpr int NW = AAAC_FIT_WARPS, REP = AAAC_FIT_REP;
-    auto launch = [&](auto kind) {
-        constexpr int KIND = decltype(kind)::value;
-        if (mode == AAAC_INT4 && sel_group == 16) return launch_variant<AAAC_INT4, 16, NW, REP, KIND>(p, (unsigned)grid, st);
-        if (mode == AAAC_INT4) return launch_variant<AAAC_INT4, 128, NW, REP, KIND>(p, (unsigned)grid, st);
-        return launch_variant<AAAC_NVFP4, 16, NW, REP, KIND>(p, (unsigned)grid, st);
-    };
-    // the three rotating sum buffers start at zero
-    static_assert(sizeof(unsigned long long) * 3 * kAccBuffer <= sizeof(double) * kMaxBlocks * kPartStride, "the sum buffers live in the block-partial region");
-    cudaError_t em = cudaMemsetAsync(p.acc, 0, sizeof(unsigned long long) * 3 * kAccBuffer, st);
-    if (em != cudaSuccess) return em;
-    if (n_inner == 1) return launch(std::integral_constant<int, kRounds>{});
-    for (int outer = 0; outer < n_outer; ++outer) {
-        p.n_rounds = 1; p.trace_base = outer;
-        cudaError_t e = launch(std::integral_constant<int, kAssignKeep>{});
-        if (e != cudaSuccess) return e;
-        p.bar_base += 1u;
-        p.n_rounds = n_inner - 1;
-        e = launch(std::integral_constant<int, kInner>{});
-        if (e != cudaSuccess) return e;
-        p.bar_base += (unsigned)(n_inner - 1);
-    }
-    return cudaSuccess;
-}
-
-template <int MODE, int SEL>
-static cudaError_t launch_batch_variant(FitBatch& b, unsigned grid, cudaStream_t st) {
-    constexpr int NW = AAAC_FIT_WARPS, REP = AAAC_FIT_REP;
-    auto kern = fit_batch_kernel<MODE, SEL, NW, REP>;
-    size_t smem = 0;
-    cudaError_t e = fit_dynamic_smem(reinterpret_cast<const void*>(kern), &smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    void* args[] = {&b};
-    note_launch();
-    // cooperative: the blocks of a layer wait for each other, so all of them must be resident
-    return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3(grid), dim3(NW * 32), args, smem, st);
 }
 
 cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode, int sel_group, int n_outer, int n_inner,
                                     uint32_t* dev_status, cudaStream_t st) {
     if (n_outer <= 0 || n <= 0) return cudaSuccess;
     if (n_inner < 1 || (int64_t)n_outer * n_inner > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    static_assert(sizeof(unsigned long long) * 3 * kAccBuffer <= sizeof(double) * kMaxBlocks * kPartStride, "the sum buffers live in the block-partial region");
     const int sms = sm_count();
     for (int at = 0; at < n;) {
-        const int m = (n - at) < kMaxBatch ? (n - at) : kMaxBatch;
-        if (m == 1 || n_inner > 1 || m > sms) {
-            // single layers and inner refinement go through the one-layer launches
-            const FitLayerArgs& a = layers[at];
-            cudaError_t e = launch_fit_rounds(a.W, a.N, a.K, a.ldw, mode, sel_group, a.scales, a.I, n_outer, n_inner,
-                                              a.err_trace, a.T01_out, dev_status, a.ws, st);
-            if (e != cudaSuccess) return e;
-            at += 1;
-            continue;
-        }
+        const int m = std::min({n - at, kMaxBatch, sms});
         FitBatch b{};
         int64_t items[kMaxBatch], share[kMaxBatch];
-        constexpr int kRowsPerItem = kRowsPerWarp * AAAC_FIT_WARPS;
+        constexpr int kRowsPerItem = kRowsPerWarp * kFitWarps;
         for (int l = 0; l < m; ++l) {
             const FitLayerArgs& a = layers[at + l];
             if (!fill_params(b.L[l], a, n_outer, dev_status)) return cudaErrorInvalidValue;
@@ -902,7 +929,7 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             int64_t load = 0;
             for (int l = 0; l < m; ++l) {
                 const int64_t per = (items[l] + share[l] - 1) / share[l];
-                if (share[l] < items[l] && share[l] < kMaxFitBlocks && per > load) { load = per; best = l; }
+                if (share[l] < kRowsPerWarp * items[l] && share[l] < kMaxFitBlocks && per > load) { load = per; best = l; }
             }
             if (best < 0) break;
             ++share[best];
@@ -916,10 +943,18 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             if (em != cudaSuccess) return em;
         }
         for (int l = m; l <= kMaxBatch; ++l) b.first[l] = grid;
-        cudaError_t e;
-        if (mode == AAAC_INT4 && sel_group == 16) e = launch_batch_variant<AAAC_INT4, 16>(b, grid, st);
-        else if (mode == AAAC_INT4) e = launch_batch_variant<AAAC_INT4, 128>(b, grid, st);
-        else e = launch_batch_variant<AAAC_NVFP4, 16>(b, grid, st);
+        cudaError_t e = cudaSuccess;
+        if (n_inner == 1) {
+            e = launch_kind<kRounds>(b, grid, mode, sel_group, st);
+        } else {
+            for (int outer = 0; outer < n_outer && e == cudaSuccess; ++outer) {
+                for (int l = 0; l < m; ++l) { b.L[l].n_rounds = 1; b.L[l].trace_base = outer; }
+                e = launch_kind<kAssignKeep>(b, grid, mode, sel_group, st);
+                for (int l = 0; l < m; ++l) { b.L[l].bar_base += 1u; b.L[l].n_rounds = n_inner - 1; }
+                if (e == cudaSuccess) e = launch_kind<kInner>(b, grid, mode, sel_group, st);
+                for (int l = 0; l < m; ++l) b.L[l].bar_base += (unsigned)(n_inner - 1);
+            }
+        }
         if (e != cudaSuccess) return e;
         at += m;
     }

@@ -16,17 +16,6 @@ constexpr int kQBins = 16384;     // first-level histogram bins of the quantile 
 constexpr int kQReq = 64;         // order statistics requested (2 per table entry)
 constexpr int kActMaxSplits = 32;   // row strips of the activation statistics (the second kernel adds them one after the other)
 
-// shape of the fit-round kernel: warps per block, copies of the {J_low, thr} table
-#ifndef AAAC_FIT_WARPS
-#define AAAC_FIT_WARPS 16
-#endif
-#ifndef AAAC_FIT_REP
-#define AAAC_FIT_REP 16           // one copy per lane of a half-warp: an 8-byte lookup has no bank conflicts
-#endif
-#ifndef AAAC_FIT_BINS
-#define AAAC_FIT_BINS 512         // uniform bins of the {J_low, thr} table on (-8, 8): width 1/32
-#endif
-
 // ---- control block at the start of the workspace (device memory) ----
 struct Ctrl {
     double T[2 * kM];               // current tables (double between rounds)
@@ -127,10 +116,7 @@ cudaError_t launch_init(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, in
                         const void* scales, const float* T01_user, uint32_t* dev_status, const Workspace& ws, cudaStream_t st,
                         bool hist_done = false);
 int act_splits_max(int64_t K);    // most row strips launch_act_stats uses for K input channels (sizes its partials)
-cudaError_t launch_fit_rounds(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, int sel_group, const void* scales,
-                              const float* I, int n_outer, int n_inner, double* err_trace, float* T01_out, uint32_t* dev_status,
-                              const Workspace& ws, cudaStream_t st);
-// the same for several layers of one mode in a single launch (n_inner = 1; otherwise layer by layer)
+// the rounds of several layers of one mode, up to eight in a launch
 struct FitLayerArgs {
     const uint16_t* W;
     int64_t N, K, ldw;

@@ -8,18 +8,18 @@
 namespace aaac {
 
 constexpr int kRowsPerWarp = 4;
-constexpr int kNBins = 1024;                       // default number of uniform bins on (-8, 8): width 1/64
+constexpr int kNBins = 512;                        // uniform bins of the per-bin table on (-8, 8): width 1/32
+constexpr int kRep = 16;                           // copies of the per-bin table: one per lane of a half-warp, so an 8-byte lookup has no bank conflicts
 constexpr int kJSlots = 32;                        // 31 intervals + the poisoned slot
 constexpr int kSlotBytes = 32 * 8;                 // bytes of a lane-private bin slot (one 8-byte entry per lane)
-// The {P, Q} table: one 256-byte pair per interval J -- entry J in 16 columns of 8 bytes, then
-// entry J + 1 in 16 columns -- so that a bin's table entry can name the address of its lower
-// interval and a weight above the bin's breakpoint adds kPairHalf to it.  Lane l uses column
-// l mod 16: an 8-byte load is served a half-warp at a time, so lanes l and l + 16 never meet.
-constexpr int kPairBytes = 256;
-constexpr int kPairHalf = 128;
+// The {P, Q} table: one row per interval J, 16 columns of 8 bytes, so that a bin's table entry can
+// name the row of its lower interval and a weight above the bin's breakpoint adds one row.  Lane l
+// uses column l mod 16: an 8-byte load is served a half-warp at a time, so lanes l and l + 16 never meet.
+constexpr int kPqRow = 128;
 constexpr int kPqCols = 16;
-constexpr int kPoison = kNJ * kPairBytes;          // byte offset of the poisoned pair (both halves NaN)
-constexpr int kLut2Bytes = kJSlots * kPairBytes;
+constexpr int kPoison = kNJ * kPqRow;              // byte offset of the poisoned row (NaN)
+constexpr int kLut1Bytes = kNBins * kRep * 8;
+constexpr int kLut2Bytes = kJSlots * kPqRow;
 constexpr int kCells = 2 * kM;                     // bins per lane: [sigma][entry]
 constexpr int kUsed = 2 * kCells + 1;              // [32] S, [32] Wt, E
 constexpr uint32_t kIdxMask = 15u;                 // low mantissa bits of a centre constant = entry index
@@ -88,7 +88,7 @@ __device__ __forceinline__ uint64_t diff2(float x, uint64_t pq) {
 
 // Address of the {P, Q} entry of a weight: `a` names the entry of the lower interval of the
 // weight's bin; a weight above the bin's breakpoint belongs to the next interval, whose entry
-// lies kPairHalf bytes further (one compare and one predicated add).
+// lies kPqRow bytes further (one compare and one predicated add).
 __device__ __forceinline__ uint32_t above_addr(uint32_t a, float x, uint32_t thr_bits) {
     asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
         : "+r"(a) : "f"(x), "f"(__uint_as_float(thr_bits)));
@@ -105,141 +105,123 @@ __device__ __forceinline__ void sts_bin(uint32_t addr, float2 v) {
 }
 
 struct FitTables {
-    double Td[2 * kM];
+    double Td[2 * kM];            // the tables
     double2 PQ[kJSlots];          // nearest entries of T0 / T1 on interval J, as double
     float bp[32];                 // sorted breakpoints, bp[30] = bp[31] = +inf
-    float tmp_b[32];
-    uint8_t tmp_src[32];
-    uint8_t src[32];              // table a breakpoint comes from
-    uint8_t tmp_exact[32], exact[32];   // the breakpoint is the exact midpoint of two different entries
-    float rlut[128];              // NVFP4: fl32(1 / s_eff) per E4M3 code
-    float2 pq32[kJSlots];         // {P, Q} of every interval before replication
+    float2 pq32[kJSlots];         // {P, Q} of every interval
+    float tmp_b[32];              // breakpoints by table
     float centre[2 * kM];         // centre constant of every entry (index in the low 4 mantissa bits)
+    float rlut[128];              // NVFP4: fl32(1 / s_eff) per E4M3 code
+    uint8_t src[32];              // table a breakpoint comes from
+    uint8_t exact[32];            // the breakpoint is the exact midpoint of two different entries
     float tmax283;                // 2.83 * 17 * max |entry|, rounded up
     int no_dup;                   // no table holds two equal entries: the interval of a weight is then the sum of its two entry indices
-    int is_last;
-    double tot[kPartStride];
-    double fix_scale, fix_unscale;   // fit rounds: fixed-point scale of the sums over the blocks and its inverse
 };
 
-// Builds every lookup table of the round from the current tables in S.Td.
-template <int MODE, int NW, int REP, int NB = kNBins>
-__device__ void build_tables(FitTables& S, unsigned char* lut1_mem, unsigned char* lut2_mem) {
-    constexpr int NT = NW * 32;
-    const int tid = threadIdx.x;
-    if (tid < kNBP) {
-        const int r = tid / 15, i = tid % 15;
-        const double mid = (S.Td[r * kM + i] + S.Td[r * kM + i + 1]) * 0.5;
-        const float f = f32_round_down(mid);
-        S.tmp_b[tid] = f;
-        S.tmp_src[tid] = (uint8_t)r;
-        S.tmp_exact[tid] = (uint8_t)(((double)f == mid) && (S.Td[r * kM + i] != S.Td[r * kM + i + 1]));
-    }
-    if (tid >= 30 && tid < 32) S.bp[tid] = __int_as_float(0x7F800000);
-    if (tid >= 32 && tid < 32 + 2 * kM) {
-        // centre constant: close to the FP32 rounding of the entry, with the entry's canonical
-        // (lowest duplicate) index in the low mantissa bits
-        const int t = tid - 32, r = t & 16;
-        int i = t & 15;
-        while (i > 0 && S.Td[r + i - 1] == S.Td[r + i]) --i;
-        // the float nearest to the FP32 rounding of the entry whose low 4 mantissa bits are i
-        // (at most 8 units in the last place away)
-        const uint32_t b = __float_as_uint((float)S.Td[t]);
-        const int mag = (int)(b & 0x7FFFFFFFu);
-        const int tt = mag + 8 - i;
-        const uint32_t mag2 = tt < 0 ? (uint32_t)i : (uint32_t)((tt & ~15) + i);
-        S.centre[t] = __uint_as_float((b & 0x80000000u) | mag2);
-        const bool all_distinct = __all_sync(0xFFFFFFFFu, i == (t & 15));      // threads 32..63 are one warp
-        if (t == 0) S.no_dup = all_distinct;
-    }
-    __syncthreads();
-    if (tid < kNBP) {
-        const float b = S.tmp_b[tid];
-        int rank = 0;
-        for (int j = 0; j < kNBP; ++j) rank += (S.tmp_b[j] < b) || (S.tmp_b[j] == b && j < tid);
-        S.bp[rank] = b;
-        S.src[rank] = S.tmp_src[tid];
-        S.exact[rank] = S.tmp_exact[tid];
-    }
-    __syncthreads();
-    float2* lut2 = reinterpret_cast<float2*>(lut2_mem);
-    if (tid < kJSlots) {
-        float P = __int_as_float(0x7FC00000), Q = P;
-        if (tid < kNJ) {
-            // entries of T0 / T1 whose upper midpoint lies below interval tid
-            const unsigned from1 = __ballot_sync(0x7FFFFFFFu, tid < kNBP && S.src[tid] == 1);
-            int i1 = __popc(from1 & ((1u << tid) - 1u)), i0 = tid - i1;
-            while (i0 > 0 && S.Td[i0 - 1] == S.Td[i0]) --i0;
-            while (i1 > 0 && S.Td[kM + i1 - 1] == S.Td[kM + i1]) --i1;
-            S.PQ[tid] = make_double2(S.Td[i0], S.Td[kM + i1]);
-            P = S.centre[i0];
-            Q = S.centre[kM + i1];
-        } else {
-            S.PQ[tid] = make_double2(0.0, 0.0);
-        }
-        double tm = fabs(S.Td[tid]);                     // 32 entries, one per lane of warp 0
+// number of breakpoints below x (sorted list): the interval of x
+__device__ __forceinline__ int find_interval(const float* bp, float x) {
+    int J = 0;
 #pragma unroll
-        for (int o = 16; o; o >>= 1) tm = fmax(tm, __shfl_xor_sync(0xFFFFFFFFu, tm, o));
-        if (tid == 0) S.tmax283 = __double2float_ru(tm * (2.83 * 17.0));
-        S.pq32[tid] = make_float2(P, Q);
-    }
-    // {slot address, thr} per bin.  With s = NB / 16 bins per unit, bin b holds the x with s x + NB / 2 in
-    // [b - h, b + 1 - h], h = half of the rounding step 1 / (8 REP) of the bin arithmetic.  The breakpoints are sorted, so those
-    // inside a bin are the first ones not below its lower edge.  The entries are first written
-    // once per bin (into the space of the {P, Q} table, which is filled afterwards) and then
-    // replicated REP times by consecutive lanes writing consecutive addresses: both steps are free
-    // of bank conflicts (one thread writing the REP copies of its bin would serialise 32-fold).
-    static_assert(NB * 8 <= kLut2Bytes, "the per-bin entries are staged in the {P, Q} table's space");
-    static_assert(REP == kPqCols, "copy c of a bin's entry carries the address of column c of the {P, Q} table");
-    uint2* binval = reinterpret_cast<uint2*>(lut2_mem);
-    const uint32_t lut2_addr = (uint32_t)__cvta_generic_to_shared(lut2_mem);
-    constexpr float h = 0.5f / (float)(REP * 8);
-    constexpr float kHalf = (float)(NB / 2), kWidth = 16.f / (float)NB;
-    for (int b = tid; b < NB; b += NT) {
-        const float lo = ((float)b - kHalf - h) * kWidth, hi = ((float)b - (kHalf - 1.f) - h) * kWidth;
-        int below = 0;                                   // number of breakpoints < lo (binary search)
-#pragma unroll
-        for (int step = 16; step; step >>= 1)
-            if (below + step <= kNBP && S.bp[below + step - 1] < lo) below += step;
-        const float v0 = S.bp[below], v1 = S.bp[below + 1];     // bp[30], bp[31] = +inf
-        uint2 e;
-        if (!(v1 <= hi)) {                               // at most one breakpoint inside
-            e.x = lut2_addr + (uint32_t)(below * kPairBytes);
-            e.y = v0 <= hi ? __float_as_uint(v0) : 0x7F800000u;
-        } else {
-            e.x = lut2_addr + (uint32_t)kPoison;
-            e.y = 0x7F800000u;
-        }
-        binval[b] = e;
-    }
-    __syncthreads();
-    {
-        uint4* lut1v = reinterpret_cast<uint4*>(lut1_mem);    // two copies (columns 2 i mod REP and the next) per store
-        for (int i = tid; i < NB * REP / 2; i += NT) {
-            const uint2 e = binval[(2 * i) / REP];
-            const uint32_t col = (uint32_t)((2 * i) % REP) * 8u;
-            lut1v[i] = make_uint4(e.x + col, e.y, e.x + col + 8u, e.y);
-        }
-    }
-    __syncthreads();
-    // pair J = {entry J, entry J + 1}, 16 columns each; the pair after the last interval is the poisoned one
-    for (int i = tid; i < kJSlots * 32; i += NT) {
-        const int pair = i >> 5, half = (i >> 4) & 1;
-        const int J = pair < kNJ ? min(pair + half, kNJ - 1) : kNJ;      // kNJ: the NaN entry
-        lut2[i] = S.pq32[J];
-    }
-    __syncthreads();
+    for (int step = 16; step; step >>= 1)
+        if (J + step <= kNBP && bp[J + step - 1] < x) J += step;
+    return J;
 }
 
-// the two tables one after the other in one buffer
-template <int MODE, int NW, int REP, int NB = kNBins>
-__device__ __forceinline__ void build_tables(FitTables& S, unsigned char* dyn) {
-    build_tables<MODE, NW, REP, NB>(S, dyn, dyn + (size_t)REP * NB * 8);
+// Everything that follows from the tables and is small: the merged breakpoints, the nearest entries of
+// every interval, the centre constants, the near-tie bound.  One warp, lane t with entry t in T, and no
+// block barrier: there are only 32 values of each, and what it costs is latency (0.4 us; the version that
+// used the block's threads and four barriers took 1.8 us of every round).
+__device__ __forceinline__ void derive_tables(FitTables& S, const int lane, const double T) {
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const int r = lane >> 4, i = lane & 15;
+    S.Td[lane] = T;
+    const double Tn = __shfl_down_sync(kAll, T, 1), Tp = __shfl_up_sync(kAll, T, 1);
+    const unsigned dup = __ballot_sync(kAll, i > 0 && Tp == T);          // equal to its predecessor
+    const bool sorted = !__any_sync(kAll, i > 0 && !(Tp <= T));
+    const double mid = (T + Tn) * 0.5;
+    const float b = i < 15 ? f32_round_down(mid) : __int_as_float(0x7F800000);
+    // place in the merged list (equal breakpoints: table 0 first, then by index), found by binary search in
+    // the other table's list; tables given by the caller may be out of order: count
+    S.tmp_b[lane] = b;
+    __syncwarp();
+    const float* other = S.tmp_b + (r ? 0 : 16);
+    int rank = 0;
+    if (sorted) {
+#pragma unroll
+        for (int step = 8; step; step >>= 1) {
+            const float ob = other[rank + step - 1];
+            if (r ? ob <= b : ob < b) rank += step;                      // (15 entries: index 14 at most)
+        }
+        rank += i;
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < 15; ++j) {
+            const float ob = other[j], own = S.tmp_b[(lane & 16) + j];
+            rank += (r ? ob <= b : ob < b) + ((own < b) || (own == b && j < i));
+        }
+    }
+    if (i == 15) rank = 30 + r;
+    S.bp[rank] = b;
+    S.src[rank] = (uint8_t)(i == 15 ? 0 : r);
+    S.exact[rank] = (uint8_t)(i < 15 && (double)b == mid && T != Tn);
+    // lowest index of the entries equal to entry k of table t
+    auto canonical = [&](int t, int k) { return 31 - __clz(~(t ? dup >> 16 : dup & 0xFFFFu) & ((2u << k) - 1u)); };
+    // centre constant: the float nearest to the FP32 rounding of the entry whose low 4 mantissa bits are
+    // the entry's canonical index (at most 8 units in the last place away)
+    const uint32_t bits = __float_as_uint((float)T);
+    const int ci = canonical(r, i), tt = (int)(bits & 0x7FFFFFFFu) + 8 - ci;
+    S.centre[lane] = __uint_as_float((bits & 0x80000000u) | (tt < 0 ? (uint32_t)ci : (uint32_t)((tt & ~15) + ci)));
+    __syncwarp();
+    // entries of T0 / T1 whose upper midpoint lies below interval `lane`
+    const unsigned from1 = __ballot_sync(kAll, S.src[lane] == 1);
+    int i1 = min(__popc(from1 & ((1u << lane) - 1u)), 15), i0 = max(0, min(lane - i1, 15));
+    i0 = canonical(0, i0);
+    i1 = canonical(1, i1);
+    const float nan = __int_as_float(0x7FC00000);
+    S.PQ[lane] = lane < kNJ ? make_double2(S.Td[i0], S.Td[kM + i1]) : make_double2(0.0, 0.0);
+    S.pq32[lane] = lane < kNJ ? make_float2(S.centre[i0], S.centre[kM + i1]) : make_float2(nan, nan);
+    const uint32_t tm = __reduce_max_sync(kAll, __float_as_uint(__double2float_ru(fabs(T))));
+    if (lane == 0) {
+        S.tmax283 = __fmul_ru(__uint_as_float(tm), 2.83f * 17.f);
+        S.no_dup = dup == 0u;
+    }
+}
+
+// The two lookup tables, written by the whole block (no barrier inside).  Bin b of width 1/32 holds the x
+// with 32 x + 256 in [b - h, b + 1 - h], h = half of the rounding step 1 / 128 of the bin arithmetic.  The
+// breakpoints are sorted, so those inside a bin are the first ones not below its lower edge.  A thread
+// writes the 16 copies of its bin, two per store, in an order rotated by its lane, so that the eight
+// lanes that a 16-byte store is served for meet in no bank.
+template <int NT>
+__device__ __forceinline__ void write_tables(const FitTables& S, const int tid, const uint32_t lut1_addr, const uint32_t lut2_addr) {
+    static_assert(kNBins % NT == 0, "whole bins per thread");
+    constexpr float h = 0.5f / (float)(kRep * 8);
+    constexpr float kHalf = (float)(kNBins / 2), kWidth = 16.f / (float)kNBins;
+#pragma unroll
+    for (int b = tid; b < kNBins; b += NT) {
+        const float lo = ((float)b - kHalf - h) * kWidth, hi = ((float)b - (kHalf - 1.f) - h) * kWidth;
+        const int below = find_interval(S.bp, lo);
+        const float v0 = S.bp[below], v1 = S.bp[below + 1];     // bp[30], bp[31] = +inf
+        const bool poison = v1 <= hi;                            // two breakpoints or more
+        const uint32_t a = lut2_addr + (poison ? (uint32_t)kPoison : (uint32_t)(below * kPqRow));
+        const uint32_t t = !poison && v0 <= hi ? __float_as_uint(v0) : 0x7F800000u;
+        const uint32_t at = lut1_addr + (uint32_t)b * (kRep * 8);
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const uint32_t c = (uint32_t)((s + tid) & 7) * 16u;
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %2};" :: "r"(at + c), "r"(a + c), "r"(t), "r"(a + c + 8u) : "memory");
+        }
+    }
+    static_assert(kLut2Bytes / 16 <= NT, "one store per thread");
+    if (tid < kLut2Bytes / 16) {
+        const float2 v = S.pq32[tid >> 3];
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %1, %2};" :: "r"(lut2_addr + (uint32_t)tid * 16u), "f"(v.x), "f"(v.y) : "memory");
+    }
 }
 
 // address of column (lane mod 16) of interval J's entry in the {P, Q} table that starts at lut2_addr
 __device__ __forceinline__ uint32_t pq_entry_addr(uint32_t lut2_addr, int J, int lane) {
-    return lut2_addr + (uint32_t)(J * kPairBytes) + (uint32_t)(lane & (kPqCols - 1)) * 8u;
+    return lut2_addr + (uint32_t)(J * kPqRow) + (uint32_t)(lane & (kPqCols - 1)) * 8u;
 }
 
 // hint[j] < kNJ names the interval of weight j where the caller knows it, else the interval is searched

@@ -36,7 +36,6 @@ namespace {
 #define AAAC_PACK_WARPS 8
 #endif
 constexpr int pack_warps(int) { return AAAC_PACK_WARPS; }
-constexpr int kPackRep = 16;          // one copy of the {J_low, thr} table per lane of a half-warp: no conflicts
 
 struct PackParams {
     const uint16_t* W;
@@ -108,47 +107,46 @@ __device__ __noinline__ Rare8 rare_groups(const FitTables* S, Row8 r, int flags)
     return out;
 }
 
-constexpr int kPackBins = 512;        // uniform bins of the per-bin table on (-8, 8): width 1/32
 constexpr int kPackBlocksPerSM = 2;
 
-template <int MODE, int SEL, int NW, int REP>
+template <int MODE, int SEL, int NW>
 __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const PackParams p) {
-    constexpr int NB = kPackBins;
+    constexpr int NB = kNBins, REP = kRep;
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;      // scale group
     constexpr int LPG = SEL / 8;                         // lanes per selection group
     static_assert(SEL == G || SEL == 16, "separate selection bits are laid out for groups of 16");
-    constexpr int kLut1Bytes = REP * NB * 8;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ FitTables S;
     __shared__ float slut[128];                      // NVFP4: s_eff per E4M3 code
     __shared__ double wsum[NW][2];
+    __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    // ---- BF16 tables (Algorithm 1 line 17), sorted
-    float tb = 0.f;
-    if (tid < 2 * kM) {
-        tb = __uint_as_float(f32_to_bf16_rne(p.T01_f32[tid]) << 16);
-        S.tot[tid] = (double)tb;
-    }
+    // ---- BF16 tables (Algorithm 1 line 17), sorted, and the lookup tables they give
     if (MODE == AAAC_NVFP4 && tid >= 64 && tid < 192) {
         const int c = tid - 64;
         const float sv = __fmul_rn(e4m3_value((uint32_t)c), p.tensor_scale[0]);
         slut[c] = sv;
         S.rlut[c] = c ? __frcp_rn(sv) : 0.f;
     }
-    __syncthreads();
-    if (tid < 2 * kM) {
-        const int r = tid & 16;
+    if (warp == 0) {
+        const float tb = __uint_as_float(f32_to_bf16_rne(p.T01_f32[lane]) << 16);
         int rank = 0;
+#pragma unroll 4
         for (int i = 0; i < kM; ++i) {
-            const double ti = S.tot[r + i];
-            rank += (ti < (double)tb) || (ti == (double)tb && i < (tid & 15));
+            const float ti = __shfl_sync(0xFFFFFFFFu, tb, (lane & 16) + i);
+            rank += (ti < tb) || (ti == tb && i < (lane & 15));
         }
-        S.Td[r + rank] = (double)tb;
+        S.Td[(lane & 16) + rank] = (double)tb;
+        __syncwarp();
+        const double T = S.Td[lane];
+        __syncwarp();
+        if (blockIdx.x == 0) p.T01_bf16[lane] = (uint16_t)(__float_as_uint((float)T) >> 16);
+        derive_tables(S, lane, T);
     }
     __syncthreads();
-    if (blockIdx.x == 0 && tid < 2 * kM) p.T01_bf16[tid] = (uint16_t)(__float_as_uint((float)S.Td[tid]) >> 16);
-    build_tables<MODE, NW, REP, NB>(S, dyn);
+    write_tables<NW * 32>(S, tid, (uint32_t)__cvta_generic_to_shared(dyn), (uint32_t)__cvta_generic_to_shared(dyn) + kLut1Bytes);
+    __syncthreads();
 
     const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(dyn);
     const uint32_t lut1_copy = (lane & (REP - 1)) * 8;             // this lane's copy of a bin's entry
@@ -345,9 +343,9 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) S.is_last = (atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1);
+    if (tid == 0) is_last = (atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1);
     __syncthreads();
-    if (!S.is_last) return;
+    if (!is_last) return;
     __threadfence();
     // the last block to finish adds the block partials in block order and hands the results out
     if (tid < 2) {
@@ -365,9 +363,9 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
 
 template <int MODE, int SEL>
 cudaError_t launch_pack_variant(const PackParams& p, unsigned grid, cudaStream_t st) {
-    constexpr size_t smem = (size_t)kPackRep * kPackBins * 8 + kLut2Bytes;
+    constexpr size_t smem = (size_t)kLut1Bytes + kLut2Bytes;
     constexpr int kPackWarps = pack_warps(MODE);
-    auto kern = pack_kernel<MODE, SEL, kPackWarps, kPackRep>;
+    auto kern = pack_kernel<MODE, SEL, kPackWarps>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, kPackWarps * 32, smem, st>>>(p);
