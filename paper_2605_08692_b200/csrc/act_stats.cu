@@ -2,11 +2,13 @@
 //
 // Layout: X is [T x K] BF16 row-major.  A block covers 256 adjacent columns (each lane owns
 // 8 of them = one 128-bit load per row) and a strip of rows; its 8 warps take rows
-// round-robin.  The square of a BF16 value is exact in FP32 (16 significant bits); a thread adds
-// its squares error-free into an FP32 pair (two-sum), because double-precision arithmetic runs
-// at a small fraction of the FP32 rate on this GPU.  The pairs become doubles once per thread,
-// so the result differs from an index-order double sum only by rounding at the 2^-48 level; a
-// second kernel adds the strip partials in strip order and rounds once to FP32.
+// round-robin.  The sums are kept in double: a BF16 magnitude becomes a double by two integer
+// instructions (its fields moved, the exponent rebased), and one double-precision multiply-add
+// squares it -- exactly -- and adds it, so a sum is off by a few 2^-53.  That is three
+// instructions an element where error-free FP32 pairs took nine, and leaves the pass to the
+// memory (16384 x 14336: 4.2 -> 5.9 TB/s with the launch geometry below).  A second kernel adds
+// the strip partials in a fixed order and rounds once to FP32.
+#include <algorithm>
 #include <mutex>
 
 #include "internal.cuh"
@@ -17,26 +19,24 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kUnroll = 4;
+constexpr int kBlocksPerSM = 4;          // resident blocks: 64 KB of loads in flight per SM
 
-// hi + lo += v without rounding error (Knuth's two-sum; intrinsics so that nothing is re-associated)
-__device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
-    const float s = __fadd_rn(hi, v);
-    const float bb = __fsub_rn(s, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb));
-    hi = s;
-    lo = __fadd_rn(lo, err);
-}
-__device__ __forceinline__ void add_squares(float (&hi)[8], float (&lo)[8], uint4 v) {
+// |a| of a BF16 value as a double (upper word; the lower is zero).  A zero or a denormal reads as some
+// 2^-127 <= |a| < 2^-126, whose square is below 2^-252 and vanishes in an FP32 sum; Inf and NaN read as
+// 2^128 and more, whose square makes the FP32 sum infinite.
+__device__ __forceinline__ double abs_lo(uint32_t w) { return __hiloint2double((int)((w & 0x7FFFu) * 8192u + 0x38000000u), 0); }
+__device__ __forceinline__ double abs_hi(uint32_t w) { return __hiloint2double((int)(((w & 0x7FFF0000u) >> 3) + 0x38000000u), 0); }
+__device__ __forceinline__ void add_squares(double (&s)[8], uint4 v) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float a = bf16_lo(w[j]), b = bf16_hi(w[j]);
-        two_sum(hi[2 * j], lo[2 * j], __fmul_rn(a, a));
-        two_sum(hi[2 * j + 1], lo[2 * j + 1], __fmul_rn(b, b));
+        const double a = abs_lo(w[j]), b = abs_hi(w[j]);
+        s[2 * j] = __fma_rn(a, a, s[2 * j]);
+        s[2 * j + 1] = __fma_rn(b, b, s[2 * j + 1]);
     }
 }
 
-__global__ void __launch_bounds__(kWarps * 32)
+__global__ void __launch_bounds__(kWarps * 32, kBlocksPerSM)
 act_sumsq_kernel(const uint16_t* __restrict__ X, int64_t T, int64_t K, int64_t ldx,
                  double* __restrict__ part, int rows_per_split) {
     __shared__ double sm[kWarps][256];
@@ -45,9 +45,11 @@ act_sumsq_kernel(const uint16_t* __restrict__ X, int64_t T, int64_t K, int64_t l
     const bool active = col0 < K;
     const int64_t t_begin = (int64_t)blockIdx.y * rows_per_split;
     const int64_t t_end = min(T, t_begin + rows_per_split);
-    float hi[8], lo[8];
+    chain_next();
+    chain_wait();
+    double s8[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { hi[j] = 0.f; lo[j] = 0.f; }
+    for (int j = 0; j < 8; ++j) s8[j] = 0.0;
 
     if (active) {
         const uint16_t* base = X + col0;
@@ -58,12 +60,12 @@ act_sumsq_kernel(const uint16_t* __restrict__ X, int64_t T, int64_t K, int64_t l
             for (int u = 0; u < kUnroll; ++u)
                 v[u] = __ldcs(reinterpret_cast<const uint4*>(base + (t + u * kWarps) * ldx));
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) add_squares(hi, lo, v[u]);
+            for (int u = 0; u < kUnroll; ++u) add_squares(s8, v[u]);
         }
-        for (; t < t_end; t += kWarps) add_squares(hi, lo, __ldcs(reinterpret_cast<const uint4*>(base + t * ldx)));
+        for (; t < t_end; t += kWarps) add_squares(s8, __ldcs(reinterpret_cast<const uint4*>(base + t * ldx)));
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sm[warp][lane * 8 + j] = (double)hi[j] + (double)lo[j];
+    for (int j = 0; j < 8; ++j) sm[warp][lane * 8 + j] = s8[j];
     __syncthreads();
     const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (col < K) {
@@ -74,12 +76,26 @@ act_sumsq_kernel(const uint16_t* __restrict__ X, int64_t T, int64_t K, int64_t l
     }
 }
 
-__global__ void act_final_kernel(const double* __restrict__ part, int splits, int64_t K,
-                                 float* __restrict__ I, int accumulate, uint32_t* dev_status) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
+// A block takes 32 columns; warp w adds the strips w, w + 8, ... of its columns, and the eight partial sums
+// are added in order.
+__global__ void __launch_bounds__(kWarps * 32)
+act_final_kernel(const double* __restrict__ part, int splits, int64_t K,
+                 float* __restrict__ I, int accumulate, uint32_t* dev_status) {
+    __shared__ double sm[kWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t k = (int64_t)blockIdx.x * 32 + lane;
     double s = 0.0;
-    for (int p = 0; p < splits; ++p) s += part[(int64_t)p * K + k];
+    chain_next();
+    chain_wait();
+    if (k < K) {
+#pragma unroll 4
+        for (int p = warp; p < splits; p += kWarps) s += part[(int64_t)p * K + k];
+    }
+    sm[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || k >= K) return;
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) s += sm[w][lane];
     float v = (float)s;
     if (accumulate) v += I[k];
     I[k] = v;
@@ -88,31 +104,36 @@ __global__ void act_final_kernel(const double* __restrict__ part, int splits, in
 
 }  // namespace
 
+// Row strips for K input channels: one wave of resident blocks (a second, partly filled one costs more than
+// shorter strips give back).
 int act_splits_max(int64_t K) {
-    const int64_t bx = (K + 255) / 256;
-    int64_t want = ((int64_t)sm_count() * 8 + bx - 1) / (bx > 0 ? bx : 1);
-    if (want < 1) want = 1;
-    return (int)(want > kActMaxSplits ? kActMaxSplits : want);
+    const int64_t bx = K > 0 ? (K + 255) / 256 : 1;
+    const int64_t want = (int64_t)sm_count() * kBlocksPerSM / bx;
+    return (int)(want < 1 ? 1 : want > kActMaxSplits ? kActMaxSplits : want);
 }
 
-cudaError_t launch_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate,
-                             uint32_t* dev_status, const Workspace& ws, cudaStream_t st) {
+namespace {
+// the two launches; `part` holds [max_splits][K] doubles
+cudaError_t run_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate, uint32_t* dev_status,
+                          double* part, int64_t splits, cudaStream_t st) {
     const int bx = (int)((K + 255) / 256);
-    int64_t want = act_splits_max(K);
-    int64_t max_by_rows = (T + kWarps - 1) / kWarps;
-    int64_t splits = want < 1 ? 1 : want;
+    const int64_t max_by_rows = (T + kWarps - 1) / kWarps;
     if (splits > max_by_rows) splits = max_by_rows;
-    if (splits > kActMaxSplits) splits = kActMaxSplits;
     int64_t rows = (T + splits - 1) / splits;
     rows = (rows + kWarps - 1) / kWarps * kWarps;
     splits = (T + rows - 1) / rows;
-    act_sumsq_kernel<<<dim3(bx, (unsigned)splits), kWarps * 32, 0, st>>>(X, T, K, ldx, ws.act_part, (int)rows);
+    cudaError_t e = launch_chained(act_sumsq_kernel, dim3(bx, (unsigned)splits), kWarps * 32, 0, st, X, T, K, ldx, part, (int)rows);
     note_launch();
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    act_final_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(ws.act_part, (int)splits, K, I, accumulate, dev_status);
+    // every partial that the second kernel reads is written by the first: nothing has to be cleared
     note_launch();
-    return cudaGetLastError();
+    return launch_chained(act_final_kernel, (unsigned)((K + 31) / 32), kWarps * 32, 0, st, part, (int)splits, K, I, accumulate, dev_status);
+}
+}  // namespace
+
+cudaError_t launch_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate,
+                             uint32_t* dev_status, const Workspace& ws, cudaStream_t st) {
+    return run_act_stats(X, T, K, ldx, I, accumulate, dev_status, ws.act_part, act_splits_max(K), st);
 }
 
 }  // namespace aaac
@@ -167,21 +188,7 @@ extern "C" int aaac_act_stats_noalloc(const void* X, int64_t T, int64_t K, int64
     double* part = nullptr;
     if (noalloc_scratch(&part) != cudaSuccess) return AAAC_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int bx = (int)((K + 255) / 256);
-    int64_t splits = ((int64_t)sm_count() * 8 + bx - 1) / bx;
-    const int64_t max_by_rows = (T + kWarps - 1) / kWarps;
-    if (splits > max_by_rows) splits = max_by_rows;
-    if (splits > kNoAllocSplits) splits = kNoAllocSplits;
-    if (splits < 1) splits = 1;
-    int64_t rows = (T + splits - 1) / splits;
-    rows = (rows + kWarps - 1) / kWarps * kWarps;
-    splits = (T + rows - 1) / rows;
-    // every partial that the second kernel reads is written by the first: nothing has to be cleared
-    act_sumsq_kernel<<<dim3(bx, (unsigned)splits), kWarps * 32, 0, st>>>(static_cast<const uint16_t*>(X), T, K, ldx,
-                                                                        part, (int)rows);
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return AAAC_ERR_CUDA;
-    act_final_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(part, (int)splits, K, I, accumulate, dev_status);
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? AAAC_OK : AAAC_ERR_CUDA;
+    const int64_t splits = std::min<int64_t>(act_splits_max(K), kNoAllocSplits);
+    if (run_act_stats(static_cast<const uint16_t*>(X), T, K, ldx, I, accumulate, dev_status, part, splits, st) != cudaSuccess) return AAAC_ERR_CUDA;
+    return AAAC_OK;
 }

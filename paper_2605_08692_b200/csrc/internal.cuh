@@ -14,7 +14,7 @@ constexpr int kPartStride = 128;  // doubles per block partial (pack: [2][31] S,
 constexpr int kMaxBlocks = 2048;  // upper bound on fit-kernel grid size
 constexpr int kQBins = 16384;     // first-level histogram bins of the quantile selection
 constexpr int kQReq = 64;         // order statistics requested (2 per table entry)
-constexpr int kActMaxSplits = 32;   // row strips of the activation statistics (the second kernel adds them one after the other)
+constexpr int kActMaxSplits = 128;  // row strips of the activation statistics
 
 // ---- control block at the start of the workspace (device memory) ----
 struct Ctrl {
@@ -140,6 +140,28 @@ cudaError_t launch_dequant(const uint8_t* codes, const void* scales, const uint8
 
 cudaError_t launch_prescale(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, const float* a, uint16_t* Wout,
                             int64_t ldo, const float* I, float* Iout, uint32_t* dev_status, cudaStream_t st);
+
+// Kernels of a call follow one another with a programmatic dependency: the next one's blocks are put on the
+// SMs as the previous one's leave them and wait inside (chain_wait, before the kernel's first access to
+// global memory), so that launching them is not added to the chain.  A kernel that waits for the previous
+// grid's end has waited for everything before it too.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// the next kernel of the chain may take its place on the SMs from here on
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 int sm_count();
 void note_launch(int n = 1);      // counts kernel launches (aaac_launch_count)
