@@ -100,11 +100,16 @@ def _check(rc: int):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# The raw handle of the current stream: building a Stream object for it would take longer than all the
+# rest of a small call's host work.
+_raw_stream = torch._C._cuda_getCurrentRawStream
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(torch.cuda.current_device())
 
 
 def group_of(mode: int) -> int:

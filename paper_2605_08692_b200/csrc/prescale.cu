@@ -4,7 +4,9 @@
 // nearest even -- and I'_k = I_k / a_k^2 (the layer's input is divided by a_k in exchange),
 // formed in double and rounded once.  A pure stream: 2 bytes in, 2 bytes out per weight; each
 // thread handles 8 adjacent columns of four rows per step (four 128-bit loads in flight), so its
-// eight multipliers stay in registers.
+// eight multipliers stay in registers; the blocks of the first row strip form I' on the way (a kernel of
+// its own for K elements cost a tenth of the call).  4096 x 14336: 45.1 -> 39.0 us (5.2 -> 6.0 TB/s),
+// 4096 x 4096: 18.7 -> 12.8 us.
 #include "internal.cuh"
 
 namespace aaac {
@@ -13,12 +15,25 @@ namespace {
 
 __global__ void __launch_bounds__(256)
 prescale_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, const float* __restrict__ a,
-                uint16_t* __restrict__ Wout, int64_t ldo, int rows_per_block) {
+                uint16_t* __restrict__ Wout, int64_t ldo, int rows_per_block, const float* __restrict__ I,
+                float* __restrict__ Iout, uint32_t* dev_status) {
     const int64_t col = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
     if (col >= K) return;
+    chain_next();
+    chain_wait();
     const float4 a0 = __ldg(reinterpret_cast<const float4*>(a + col));
     const float4 a1 = __ldg(reinterpret_cast<const float4*>(a + col + 4));
     const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    if (blockIdx.y == 0) {
+        // the first strip's blocks also look the multipliers over and form I'
+        bool bad = false;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            bad |= !(av[j] > 0.f) || !(av[j] < __int_as_float(0x7F800000));          // zero, negative, infinite or NaN
+            if (I) Iout[col + j] = (float)__ddiv_rn((double)I[col + j], __dmul_rn((double)av[j], (double)av[j]));
+        }
+        if (bad && dev_status) atomicOr(dev_status, AAAC_DEV_NONFINITE);
+    }
     const int64_t r0 = (int64_t)blockIdx.y * rows_per_block;
     const int64_t r1 = min(N, r0 + rows_per_block);
     for (int64_t row = r0; row < r1; row += 4) {
@@ -42,17 +57,6 @@ prescale_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ld
     }
 }
 
-__global__ void prescale_importance_kernel(const float* __restrict__ a, int64_t K, const float* __restrict__ I,
-                                           float* __restrict__ Iout, uint32_t* dev_status) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const float ak = a[k];
-    if (!(ak > 0.f) || !(ak < __int_as_float(0x7F800000))) {           // zero, negative, infinite or NaN
-        if (dev_status) atomicOr(dev_status, AAAC_DEV_NONFINITE);
-    }
-    if (I && Iout) Iout[k] = (float)__ddiv_rn((double)I[k], __dmul_rn((double)ak, (double)ak));
-}
-
 }  // namespace
 
 cudaError_t launch_prescale(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, const float* a, uint16_t* Wout,
@@ -66,13 +70,8 @@ cudaError_t launch_prescale(const uint16_t* W, int64_t N, int64_t K, int64_t ldw
     int64_t rows = (N + strips - 1) / strips;
     rows = (rows + 3) / 4 * 4;
     strips = (N + rows - 1) / rows;
-    prescale_kernel<<<dim3(bx, (unsigned)strips), 256, 0, st>>>(W, N, K, ldw, a, Wout, ldo, (int)rows);
     note_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    prescale_importance_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(a, K, I, Iout, dev_status);
-    note_launch();
-    return cudaGetLastError();
+    return launch_chained(prescale_kernel, dim3(bx, (unsigned)strips), 256, 0, st, W, N, K, ldw, a, Wout, ldo, (int)rows, I, Iout, dev_status);
 }
 
 }  // namespace aaac
