@@ -1,6 +1,7 @@
 // C ABI of the library: argument validation, workspace carving, launch sequencing.
 #include <algorithm>
 #include <atomic>
+#include <cstddef>
 #include <mutex>
 
 #include "internal.cuh"
@@ -57,11 +58,12 @@ Workspace carve(void* base, int mode, int64_t N, int64_t K, size_t ws_bytes = 0,
     const int g = mode == AAAC_INT4 ? 128 : 16;
     const int64_t K8 = (K + 7) / 8 * 8;
     w.ctrl = static_cast<Ctrl*>(take(sizeof(Ctrl)));
+    w.acc = static_cast<unsigned long long*>(take(sizeof(unsigned long long) * kFitAccWords));
+    w.qhist = static_cast<uint32_t*>(take(sizeof(uint32_t) * kQBins));
     w.part = static_cast<double*>(take(sizeof(double) * kMaxBlocks * kPartStride));
     w.rinv = static_cast<float*>(take(sizeof(float) * (size_t)(mode == AAAC_INT4 && N > 0 && K > 0 ? N * (K / g + 1) : 1)));
     w.I = static_cast<float*>(take(sizeof(float) * (size_t)(K8 > 0 ? K8 : 8)));
     w.act_part = static_cast<double*>(take(sizeof(double) * (size_t)act_splits_max(K) * (size_t)(K8 > 0 ? K8 : 8)));
-    w.qhist = static_cast<uint32_t*>(take(sizeof(uint32_t) * kQBins));
     w.qslot_of_bin = static_cast<uint8_t*>(take(kQBins));
     const size_t nk = (size_t)(N > 0 && K > 0 ? N * K : 1);
     size_t cap = full ? nk : default_qcap(N, K);
@@ -114,7 +116,6 @@ struct Timing {
 // caller's stream and joined back to it: the small latency-bound kernels of one layer (plan,
 // selection, the tails of the streaming passes) then run under the bandwidth-bound passes of another.
 constexpr int kSideStreams = 7;
-constexpr int kMaxDevices = 64;
 struct SideStreams {
     bool tried = false, ok = false;
     cudaStream_t s[kSideStreams];
@@ -274,16 +275,16 @@ int importance_owner(const aaac_layer* layers, int l) {
 int prepare_fit_layer(const aaac_layer& L, int mode, int init, uint32_t* dev_status, const Workspace& w, cudaStream_t st,
                       const float* shared_I, const float** I_used) {
     const uint16_t* Wp = static_cast<const uint16_t*>(L.W);
-    if (cudaMemsetAsync(w.ctrl, 0, sizeof(Ctrl), st) != cudaSuccess) return AAAC_ERR_CUDA;
+    const bool fused = init == AAAC_INIT_QUANTILE;      // the scales pass counts the quantile start's histogram on its way
+    if (cudaMemsetAsync(w.ctrl, 0, w.zero_bytes(fused), st) != cudaSuccess) return AAAC_ERR_CUDA;
     const float* I = L.I ? L.I : shared_I;
     if (!I) {
         if (launch_act_stats(static_cast<const uint16_t*>(L.X), L.T, L.K, L.ldx, w.I, 0, dev_status, w, st) != cudaSuccess)
             return AAAC_ERR_CUDA;
         I = w.I;
     }
-    const bool fused = init == AAAC_INIT_QUANTILE;      // the scales pass counts the quantile start's histogram on its way
     if (launch_scales(Wp, L.N, L.K, L.ldw, mode, L.scales, L.tensor_scale, dev_status, w, st, fused) != cudaSuccess) return AAAC_ERR_CUDA;
-    if (launch_init(Wp, L.N, L.K, L.ldw, mode, init, L.scales, L.T01, dev_status, w, st, fused) != cudaSuccess) return AAAC_ERR_CUDA;
+    if (launch_init(Wp, L.N, L.K, L.ldw, mode, init, L.scales, L.T01, dev_status, w, st) != cudaSuccess) return AAAC_ERR_CUDA;
     *I_used = I;
     return AAAC_OK;
 }
@@ -348,17 +349,15 @@ int aaac_fit_layer_sel(const void* W, int64_t N, int64_t K, int64_t ldw, int mod
 }
 
 namespace {
-// the pack pass of one layer on `st`; arguments already checked
+// The pack pass of one layer on `st`; arguments already checked.  It uses the block counter and its own
+// result fields of the control block, which a fit leaves at zero; `fresh` says that one has just run.
 int enqueue_pack(const void* W, int64_t N, int64_t K, int64_t ldw, int mode, int sel_group,
                  const float* I, const float* T01_f32, uint16_t* T01_bf16,
                  void* scales, const float* tensor_scale, uint8_t* codes, uint8_t* sigma_bits,
-                 double* err_out, uint64_t* stats, void* ws, size_t ws_bytes, cudaStream_t stream) {
+                 double* err_out, uint64_t* stats, void* ws, size_t ws_bytes, bool fresh, cudaStream_t stream) {
     Workspace w = carve(ws, mode, N, K, ws_bytes);
     cudaStream_t st = stream;
-    // the pack pass uses only the block counter and its own result fields of the control block
-    if (cudaMemsetAsync(&w.ctrl->done, 0, sizeof(uint32_t), st) != cudaSuccess) return AAAC_ERR_CUDA;
-    if (cudaMemsetAsync(w.ctrl->pack_err, 0, sizeof(double) * 2 + sizeof(unsigned long long) * 4, st) != cudaSuccess)
-        return AAAC_ERR_CUDA;
+    if (!fresh && cudaMemsetAsync(w.ctrl->pack_err, 0, sizeof(Ctrl) - offsetof(Ctrl, pack_err), st) != cudaSuccess) return AAAC_ERR_CUDA;
     return launch_pack(static_cast<const uint16_t*>(W), N, K, ldw, mode, sel_group, I, T01_f32, T01_bf16, scales,
                        tensor_scale, codes, sigma_bits, err_out, reinterpret_cast<unsigned long long*>(stats), w, st) == cudaSuccess
                ? AAAC_OK : AAAC_ERR_CUDA;
@@ -390,7 +389,7 @@ int aaac_pack_sel(const void* W, int64_t N, int64_t K, int64_t ldw, int mode, in
     rc = check_ws(ws, ws_bytes, carve(nullptr, mode, N, K).bytes);
     if (rc) return rc;
     return enqueue_pack(W, N, K, ldw, mode, sel_group, I, T01_f32, T01_bf16, scales, tensor_scale, codes, sigma_bits,
-                        err_out, stats, ws, ws_bytes, static_cast<cudaStream_t>(stream));
+                        err_out, stats, ws, ws_bytes, false, static_cast<cudaStream_t>(stream));
 }
 
 int aaac_quantize_layers(const aaac_layer* layers, const aaac_layer_out* outs, int n_layers, int mode, int group,
@@ -421,7 +420,7 @@ int aaac_quantize_layers(const aaac_layer* layers, const aaac_layer_out* outs, i
         const float* I = L.I ? L.I : carve(Lo.ws, mode, Lo.N, Lo.K, Lo.ws_bytes).I;
         uint8_t* sg = sel_group == group ? nullptr : O.sigma_bits;
         rc = enqueue_pack(L.W, L.N, L.K, L.ldw, mode, sel_group, I, L.T01, O.T01_bf16, L.scales, L.tensor_scale, O.codes, sg,
-                          O.err_out, O.stats, L.ws, L.ws_bytes, lanes.of(l));
+                          O.err_out, O.stats, L.ws, L.ws_bytes, true, lanes.of(l));
         if (rc == AAAC_OK && O.What &&
             launch_dequant(O.codes, L.scales, sg, L.tensor_scale, O.T01_bf16, L.N, L.K, mode, static_cast<uint16_t*>(O.What),
                            O.ldo, lanes.of(l)) != cudaSuccess)

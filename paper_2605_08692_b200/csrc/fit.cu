@@ -814,26 +814,25 @@ __global__ void export_tables_kernel(const Ctrl* ctrl, float* T01) {
 
 // The fit kernels place their tables at fixed shared addresses and take all the shared memory a block
 // may have beyond their static part (one block per SM either way); the kernel checks that its layout fits.
-cudaError_t fit_dynamic_smem(const void* kern, size_t* bytes) {
-    cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, kern);
-    if (e != cudaSuccess) return e;
-    int dev = 0, optin = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-    if ((size_t)optin <= a.sharedSizeBytes) return cudaErrorInvalidValue;
-    *bytes = (size_t)optin - a.sharedSizeBytes;
-    return cudaSuccess;
-}
-
 template <int MODE, int SEL, int KIND>
 cudaError_t launch_variant(FitBatch& b, unsigned grid, cudaStream_t st) {
     auto kern = fit_kernel<MODE, SEL, KIND>;
-    size_t smem = 0;
-    cudaError_t e = fit_dynamic_smem(reinterpret_cast<const void*>(kern), &smem);
+    static std::atomic<size_t> ready[kMaxDevices];          // dynamic shared memory, once it is set up on a device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    size_t smem = ready[dev].load(std::memory_order_relaxed);
+    if (smem == 0) {
+        cudaFuncAttributes a;
+        int optin = 0;
+        if ((e = cudaFuncGetAttributes(&a, reinterpret_cast<const void*>(kern))) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+        if ((size_t)optin <= a.sharedSizeBytes) return cudaErrorInvalidValue;
+        smem = (size_t)optin - a.sharedSizeBytes;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        ready[dev].store(smem, std::memory_order_relaxed);
+    }
     void* args[] = {&b};
     note_launch();
     // cooperative: the blocks of a layer wait for each other, so all of them must be resident
@@ -897,7 +896,7 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
     p = FitParams{};
     p.W = a.W; p.N = a.N; p.K = a.K; p.ldw = a.ldw;
     p.scales = static_cast<const uint8_t*>(a.scales); p.rinv = a.ws.rinv; p.I = a.I;
-    p.ctrl = a.ws.ctrl; p.acc = reinterpret_cast<unsigned long long*>(a.ws.part); p.err_trace = a.err_trace; p.T01_out = a.T01_out; p.dev_status = dev_status;
+    p.ctrl = a.ws.ctrl; p.acc = a.ws.acc; p.err_trace = a.err_trace; p.T01_out = a.T01_out; p.dev_status = dev_status;
     p.n_rounds = n_outer; p.trace_base = 0; p.bar_base = 0u;
     p.spin_limit = g_spin_limit;
     p.sigw = a.ws.qlist;            // the quantile selection's list is free once the start tables exist
@@ -910,7 +909,7 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
                                     uint32_t* dev_status, cudaStream_t st) {
     if (n_outer <= 0 || n <= 0) return cudaSuccess;
     if (n_inner < 1 || (int64_t)n_outer * n_inner > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    static_assert(sizeof(unsigned long long) * 3 * kAccBuffer <= sizeof(double) * kMaxBlocks * kPartStride, "the sum buffers live in the block-partial region");
+    static_assert(kFitAccWords == 3 * kAccBuffer, "the workspace holds three sum buffers");
     const int sms = sm_count();
     for (int at = 0; at < n;) {
         const int m = std::min({n - at, kMaxBatch, sms});
@@ -939,8 +938,6 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             const FitLayerArgs& a = layers[at + l];
             b.first[l] = grid;
             grid += (unsigned)plan_layer(b.L[l], a.N, a.K, share[l]);
-            cudaError_t em = cudaMemsetAsync(b.L[l].acc, 0, sizeof(unsigned long long) * 3 * kAccBuffer, st);
-            if (em != cudaSuccess) return em;
         }
         for (int l = m; l <= kMaxBatch; ++l) b.first[l] = grid;
         cudaError_t e = cudaSuccess;

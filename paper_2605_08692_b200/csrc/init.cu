@@ -3,8 +3,8 @@
 // Quantile initialisation (Eq. 9, Eq. 10): T0[i] = Quantile_{i/15}, T1[i] = Quantile_{d + (1-d) i/15},
 // d = 1/30, of all N*K normalised weights, with linear interpolation at position q (n - 1).
 // That needs up to 64 exact order statistics of n values.  They are selected without sorting:
-//   1. histogram of every w~ over 16384 uniform bins on [-8, 8) (shared-memory histogram per
-//      block, merged with integer atomics);
+//   1. histogram of every w~ over 16384 uniform bins on [-8, 8): counted by the scales pass
+//      (scales_hist_kernel);
 //   2. one block turns the histogram into a prefix sum, finds the bin and the rank inside the
 //      bin of every requested order statistic, and gives each distinct bin a slot;
 //   3. a second pass over W appends the (order-preserving integer keys of the) values that fall
@@ -33,63 +33,6 @@ constexpr uint32_t kSlotOver = 0x40u;      // bin -> slot table: the slot's cand
 __device__ __forceinline__ float key_float(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
-// reciprocal of the group's scale for the 8 weights a lane holds
-template <int MODE>
-__device__ __forceinline__ float group_rinv(const void* scales, int64_t gi, float s_t) {
-    if (MODE == AAAC_INT4) {
-        const uint32_t b = reinterpret_cast<const uint16_t*>(scales)[gi] & 0x7FFFu;
-        return __frcp_rn(__uint_as_float(b << 16));
-    }
-    const uint32_t c = reinterpret_cast<const uint8_t*>(scales)[gi] & 0x7Fu;
-    return __frcp_rn(__fmul_rn(e4m3_value(c), s_t));
-}
-
-// Step 1: histogram of every w~ (shared-memory counters per block, merged with integer atomics).
-// A warp takes four 256-column pieces per iteration so that four loads are in flight.
-template <int MODE>
-__global__ void __launch_bounds__(512, 3)
-quantile_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
-                     const void* __restrict__ scales, const Ctrl* ctrl, uint32_t* __restrict__ hist) {
-    constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
-    extern __shared__ uint32_t sm[];                      // kQBins counters
-    const int lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < kQBins; i += blockDim.x) sm[i] = 0;
-    __syncthreads();
-    const float s_t = ctrl->s_t;
-    const int64_t slabs = (K + 255) / 256, Gr = K / G;
-    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    SlabWalk it(warp0, nwarps, slabs);
-    while (it.row < N) {
-        uint4 v[4];
-        float r[4];
-        bool ok[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int64_t row = it.row, col = (int64_t)it.slab * 256 + lane * 8;
-            ok[h] = row < N && col < K;
-            v[h] = make_uint4(0, 0, 0, 0);
-            r[h] = 0.f;
-            if (ok[h]) {
-                v[h] = __ldg(reinterpret_cast<const uint4*>(W + row * ldw + col));
-                r[h] = group_rinv<MODE>(scales, row * Gr + col / G, s_t);
-            }
-            it.next();
-        }
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            if (!ok[h]) continue;
-            const uint32_t w[4] = {v[h].x, v[h].y, v[h].z, v[h].w};
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                atomicAdd(&sm[qbin(__fmul_rn((j & 1) ? bf16_hi(w[j >> 1]) : bf16_lo(w[j >> 1]), r[h]))], 1u);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kQBins; i += blockDim.x)
-        if (sm[i]) atomicAdd(&hist[i], sm[i]);
-}
-
 // Step 3: candidates of the slotted bins, staged per block.
 constexpr int kStageCap = 4096;                  // staged candidates per block
 constexpr int kStageEvery = 4;                   // loop iterations between two looks at the stage's fill
@@ -110,6 +53,8 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
     __shared__ uint32_t okmin[kQReq], okmax[kQReq];       // smallest / largest key of the slots without list space
     __shared__ float rl[128];                             // NVFP4: reciprocal of the effective scale per E4M3 code
     const int tid = threadIdx.x, lane = tid & 31;
+    chain_next();
+    chain_wait();
     const float s_t = ctrl->s_t;
     if (MODE == AAAC_NVFP4 && tid < 128) rl[tid] = __frcp_rn(__fmul_rn(e4m3_value((uint32_t)tid), s_t));
     {
@@ -160,7 +105,7 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
     // walks only its candidates (one, nearly always), found by a bit scan of the packed bytes, and
     // recomputes w~ of that weight alone.
     auto take = [&](const uint4& v, uint32_t ss) {
-        // the reciprocal group_rinv would give for these scale bits
+        // fl32(1 / s) for these scale bits
         const float r = MODE == AAAC_INT4 ? __frcp_rn(__uint_as_float((ss & 0x7FFFu) << 16)) : rl[ss & 0x7Fu];
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
         uint32_t sl[8], all = 0x80u;
@@ -246,6 +191,8 @@ quantile_plan_kernel(Ctrl* ctrl, const uint32_t* __restrict__ hist, uint8_t* __r
     __shared__ int req_first[kQReq];
     __shared__ unsigned long long wtot[32];
     const int tid = threadIdx.x;
+    chain_next();
+    chain_wait();
     constexpr int per = kQBins / 1024;
     static_assert(per == 16, "a thread's chunk is four 16-byte loads");
     uint32_t h[per];
@@ -564,6 +511,8 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
 __global__ void __launch_bounds__(1024)
 quantile_select_kernel(Ctrl* ctrl, const uint32_t* __restrict__ list, uint32_t* dev_status) {
     __shared__ int last;
+    chain_next();
+    chain_wait();
     select_slot(ctrl, list);
     __threadfence();
     __syncthreads();
@@ -584,6 +533,8 @@ quantile_select_kernel(Ctrl* ctrl, const uint32_t* __restrict__ list, uint32_t* 
 
 __global__ void grid_init_kernel(Ctrl* ctrl, int mode, const float* T01_user) {
     const int t = threadIdx.x;
+    chain_next();
+    chain_wait();
     if (t >= 2 * kM) return;
     if (T01_user) {
         ctrl->T[t] = (double)T01_user[t];
@@ -599,12 +550,10 @@ __global__ void grid_init_kernel(Ctrl* ctrl, int mode, const float* T01_user) {
 }  // namespace
 
 cudaError_t launch_init(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, int init,
-                        const void* scales, const float* T01_user, uint32_t* dev_status, const Workspace& ws, cudaStream_t st,
-                        bool hist_done) {
+                        const void* scales, const float* T01_user, uint32_t* dev_status, const Workspace& ws, cudaStream_t st) {
     if (init != AAAC_INIT_QUANTILE) {
-        grid_init_kernel<<<1, 32, 0, st>>>(ws.ctrl, mode, init == AAAC_INIT_USER ? T01_user : nullptr);
         note_launch();
-        return cudaGetLastError();
+        return launch_chained(grid_init_kernel, 1, 32, 0, st, ws.ctrl, mode, init == AAAC_INIT_USER ? T01_user : nullptr);
     }
     // positions of the 32 quantiles, as the definition states them
     Requests rq;
@@ -622,33 +571,15 @@ cudaError_t launch_init(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, in
         rq.rank[2 * e + 1] = (unsigned long long)hi;
         rq.frac[e] = pos - lo;
     }
-    cudaError_t e;
-    const int blocks = sm_count() * 3;
-    const size_t sm0 = kQBins * sizeof(uint32_t);
-    if (hist_done) {
-        // the scales pass has already counted the histogram (launch_scales with with_hist)
-    } else if ((e = cudaMemsetAsync(ws.qhist, 0, kQBins * sizeof(uint32_t), st)) != cudaSuccess) {
-        return e;
-    } else if (mode == AAAC_INT4) {
-        if ((e = cudaFuncSetAttribute(quantile_hist_kernel<AAAC_INT4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm0)) != cudaSuccess) return e;
-        quantile_hist_kernel<AAAC_INT4><<<blocks, 512, sm0, st>>>(W, N, K, ldw, scales, ws.ctrl, ws.qhist);
-        note_launch();
-    } else {
-        if ((e = cudaFuncSetAttribute(quantile_hist_kernel<AAAC_NVFP4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm0)) != cudaSuccess) return e;
-        quantile_hist_kernel<AAAC_NVFP4><<<blocks, 512, sm0, st>>>(W, N, K, ldw, scales, ws.ctrl, ws.qhist);
-        note_launch();
-    }
-    quantile_plan_kernel<<<1, 1024, 0, st>>>(ws.ctrl, ws.qhist, ws.qslot_of_bin, (unsigned long long)ws.qcap, rq);
+    cudaError_t e = launch_chained(quantile_plan_kernel, 1, 1024, 0, st, ws.ctrl, ws.qhist, ws.qslot_of_bin, (unsigned long long)ws.qcap, rq);
     note_launch();
-    const int blocks1 = sm_count() * 4;
-    if (mode == AAAC_INT4)
-        quantile_collect_kernel<AAAC_INT4><<<blocks1, 256, kQBins, st>>>(W, N, K, ldw, scales, ws.ctrl, ws.qslot_of_bin, ws.qlist);
-    else
-        quantile_collect_kernel<AAAC_NVFP4><<<blocks1, 256, kQBins, st>>>(W, N, K, ldw, scales, ws.ctrl, ws.qslot_of_bin, ws.qlist);
+    if (e != cudaSuccess) return e;
+    auto collect = mode == AAAC_INT4 ? quantile_collect_kernel<AAAC_INT4> : quantile_collect_kernel<AAAC_NVFP4>;
+    e = launch_chained(collect, sm_count() * 4, 256, kQBins, st, W, N, K, ldw, scales, ws.ctrl, ws.qslot_of_bin, ws.qlist);
     note_launch();
-    quantile_select_kernel<<<kQReq, 1024, 0, st>>>(ws.ctrl, ws.qlist, dev_status);
+    if (e != cudaSuccess) return e;
     note_launch();
-    return cudaGetLastError();
+    return launch_chained(quantile_select_kernel, kQReq, 1024, 0, st, ws.ctrl, ws.qlist, dev_status);
 }
 
 }  // namespace aaac

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/aaac.h"
 
 namespace aaac {
@@ -10,23 +12,22 @@ namespace aaac {
 constexpr int kM = 16;            // entries per table
 constexpr int kNBP = 30;          // merged breakpoints: 15 midpoints of T0 + 15 of T1
 constexpr int kNJ = 31;           // merged intervals
-constexpr int kPartStride = 128;  // doubles per block partial (pack: [2][31] S, Wt, E; fit: [32] S, [32] Wt, E)
-constexpr int kMaxBlocks = 2048;  // upper bound on fit-kernel grid size
+constexpr int kPartStride = 2;    // doubles per block partial of the pack pass
+constexpr int kMaxBlocks = 2048;  // upper bound on its grid
 constexpr int kQBins = 16384;     // first-level histogram bins of the quantile selection
 constexpr int kQReq = 64;         // order statistics requested (2 per table entry)
 constexpr int kActMaxSplits = 128;  // row strips of the activation statistics
 
 // ---- control block at the start of the workspace (device memory) ----
+// It, the fit's sum buffers and the start's histogram follow one another in the workspace, so that one
+// memset brings them to zero at the start of a fit.
 struct Ctrl {
     double T[2 * kM];               // current tables (double between rounds)
     float s_t;                      // NVFP4 tensor scale
     uint32_t absmax_bits;           // layer max |w| as float bits (atomicMax on non-negative floats)
-    uint32_t done;                  // blocks that have written their partial this round
     uint32_t nonfinite;             // set if a non-finite weight was seen
-    uint32_t bar;                   // (unused)
     uint32_t abort;                 // set when a block's wait for the totals of a pass ran out
     // quantile selection
-    unsigned long long rank[kQReq]; // requested 0-based ranks (host-written via kernel args)
     double frac[2 * kM];            // interpolation fraction per table entry
     float rank_val[kQReq];          // selected order statistics
     uint32_t req_slot[kQReq];       // slot of each request
@@ -37,22 +38,29 @@ struct Ctrl {
     uint32_t slot_over[kQReq];      // the slot's candidates did not fit the list: only their smallest and largest key are kept
     uint32_t slot_kmin[kQReq], slot_kmax[kQReq];
     uint32_t scratch_short;         // an order statistic could not be found within the scratch given
-    // pack results
+    // pack results, and the counter of finished blocks that the selection and pack kernels use (zero between them)
     double pack_err[2];
     unsigned long long pack_stats[4];
+    uint32_t done;
 };
+
+constexpr int kFitAccWords = 3 * (2 * kM + 1) * 16;     // the fit rounds' sum buffers (see fit.cu)
 
 struct Workspace {
     Ctrl* ctrl;
-    double* part;            // [kMaxBlocks][kPartStride]: the pack pass's block partials; the fit rounds' sum buffers
+    unsigned long long* acc; // [kFitAccWords]
+    uint32_t* qhist;         // [kQBins]
+    double* part;            // [kMaxBlocks][kPartStride]: the pack pass's block partials
     float* rinv;             // [N*K/g]  INT4 reciprocal scales (one element in NVFP4 mode)
     float* I;                // [K] importance computed from X
-    double* act_part;        // [kActMaxSplits][K]
-    uint32_t* qhist;         // [kQBins]
+    double* act_part;        // row strip partials of the activation statistics
     uint8_t* qslot_of_bin;   // [kQBins]
     uint32_t* qlist;         // [qcap] candidates of the quantile selection; afterwards the fit's selection bits [N][ceil(K/256)]
     size_t qcap;             // entries of qlist
     size_t bytes;
+    size_t zero_bytes(bool with_hist) const {
+        return (size_t)(reinterpret_cast<char*>(qhist) - reinterpret_cast<char*>(ctrl)) + (with_hist ? sizeof(uint32_t) * kQBins : 0);
+    }
 };
 
 // ---- formats ----
@@ -109,12 +117,11 @@ __device__ __forceinline__ float f32_round_down(double d) { return __double2floa
 cudaError_t launch_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate,
                              uint32_t* dev_status, const Workspace& ws, cudaStream_t st);
 // with_hist: the scales pass also counts the 16384-bin histogram of the normalised weights (the quantile
-// start's first pass over W) into ws.qhist; launch_init is then told so
+// start's first pass over W) into ws.qhist, which is zero before
 cudaError_t launch_scales(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, void* scales,
                           float* tensor_scale, uint32_t* dev_status, const Workspace& ws, cudaStream_t st, bool with_hist = false);
 cudaError_t launch_init(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, int init,
-                        const void* scales, const float* T01_user, uint32_t* dev_status, const Workspace& ws, cudaStream_t st,
-                        bool hist_done = false);
+                        const void* scales, const float* T01_user, uint32_t* dev_status, const Workspace& ws, cudaStream_t st);
 int act_splits_max(int64_t K);    // most row strips launch_act_stats uses for K input channels (sizes its partials)
 // the rounds of several layers of one mode, up to eight in a launch
 struct FitLayerArgs {
@@ -162,6 +169,19 @@ cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // the next kernel of the chain may take its place on the SMs from here on
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Raises a kernel's dynamic shared memory limit, once per device.
+constexpr int kMaxDevices = 64;
+template <typename K>
+cudaError_t allow_smem(K kern, size_t bytes, std::atomic<size_t> (&done)[kMaxDevices]) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && dev >= 0 && dev < kMaxDevices) done[dev].store(bytes, std::memory_order_relaxed);
+    return e;
+}
 
 int sm_count();
 void note_launch(int n = 1);      // counts kernel launches (aaac_launch_count)

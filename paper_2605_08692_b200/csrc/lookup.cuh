@@ -21,7 +21,6 @@ constexpr int kPoison = kNJ * kPqRow;              // byte offset of the poisone
 constexpr int kLut1Bytes = kNBins * kRep * 8;
 constexpr int kLut2Bytes = kJSlots * kPqRow;
 constexpr int kCells = 2 * kM;                     // bins per lane: [sigma][entry]
-constexpr int kUsed = 2 * kCells + 1;              // [32] S, [32] Wt, E
 constexpr uint32_t kIdxMask = 15u;                 // low mantissa bits of a centre constant = entry index
 
 // Shared-memory accesses of the hot loop with explicit 32-bit addresses.  All are volatile asm,

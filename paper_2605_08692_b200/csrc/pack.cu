@@ -24,7 +24,7 @@
 // on, the other's load is in flight and nothing is copied -- with 32-bit element offsets advanced by
 // the row stride and no branch around the loads; a lane takes 8 adjacent columns (one 128-bit load per row, one 32-bit store of 8 codes); the two errors travel
 // as one packed FP32 pair.
-// Error sums go through one partial per block, added in block order by the last block to finish.
+// Error sums go through one partial per block, added by the last block to finish.
 #include "lookup.cuh"
 
 namespace aaac {
@@ -122,6 +122,8 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
     __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
+    chain_next();
+    chain_wait();
     // ---- BF16 tables (Algorithm 1 line 17), sorted, and the lookup tables they give
     if (MODE == AAAC_NVFP4 && tid >= 64 && tid < 192) {
         const int c = tid - 64;
@@ -347,12 +349,17 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    // the last block to finish adds the block partials in block order and hands the results out
-    if (tid < 2) {
+    // The last block to finish adds the block partials (a fixed order: lane by lane, then pairwise) and hands
+    // the results out.  A warp per sum: two threads walking the partials one after the other took 10-25 us.
+    if (warp < 2) {
         double s = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) s += __ldcg(p.part + (size_t)b * kPartStride + tid);
-        p.ctrl->pack_err[tid] = s;
-        if (p.err_out) p.err_out[tid] = s;
+        for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(p.part + (size_t)b * kPartStride + warp);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+        if (lane == 0) {
+            p.ctrl->pack_err[warp] = s;
+            if (p.err_out) p.err_out[warp] = s;
+        }
     }
     if (tid < 4) {
         if (p.stats) p.stats[tid] = __ldcg(&p.ctrl->pack_stats[tid]);
@@ -366,11 +373,11 @@ cudaError_t launch_pack_variant(const PackParams& p, unsigned grid, cudaStream_t
     constexpr size_t smem = (size_t)kLut1Bytes + kLut2Bytes;
     constexpr int kPackWarps = pack_warps(MODE);
     auto kern = pack_kernel<MODE, SEL, kPackWarps>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<size_t> ready[kMaxDevices];
+    const cudaError_t e = allow_smem(kern, smem, ready);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kPackWarps * 32, smem, st>>>(p);
     note_launch();
-    return cudaGetLastError();
+    return launch_chained(kern, grid, kPackWarps * 32, smem, st, p);
 }
 
 }  // namespace

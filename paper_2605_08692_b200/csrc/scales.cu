@@ -29,6 +29,8 @@ __device__ __forceinline__ uint32_t absmax16(uint4 v) {
 
 __global__ void __launch_bounds__(256)
 absmax_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, Ctrl* ctrl, uint32_t* dev_status) {
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t slabs = (K + 255) / 256;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -65,6 +67,8 @@ scales_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
               float* __restrict__ rinv, float* __restrict__ tensor_scale, Ctrl* ctrl, uint32_t* dev_status) {
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
     constexpr int LPG = G / 8;                         // lanes per group
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t slabs = (K + 255) / 256, Gr = K / G;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -145,7 +149,9 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
     constexpr int LPG = G / 8;                         // lanes per group
     extern __shared__ uint32_t sm[];                   // kQBins counters
+    chain_next();
     for (int i = threadIdx.x; i < kQBins; i += blockDim.x) sm[i] = 0;
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t slabs = (K + 255) / 256, Gr = K / G;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -228,31 +234,22 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
 cudaError_t launch_scales(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, void* scales,
                           float* tensor_scale, uint32_t* dev_status, const Workspace& ws, cudaStream_t st, bool with_hist) {
     const int blocks = sm_count() * 8;
+    cudaError_t e = cudaSuccess;
     if (mode == AAAC_NVFP4) {
-        absmax_kernel<<<blocks, 256, 0, st>>>(W, N, K, ldw, ws.ctrl, dev_status);
         note_launch();
+        if ((e = launch_chained(absmax_kernel, blocks, 256, 0, st, W, N, K, ldw, ws.ctrl, dev_status)) != cudaSuccess) return e;
     }
-    if (with_hist) {
-        cudaError_t e = cudaMemsetAsync(ws.qhist, 0, kQBins * sizeof(uint32_t), st);
-        if (e != cudaSuccess) return e;
-        const int hb = sm_count() * AAAC_SH_BLOCKS;
-        const size_t sm0 = kQBins * sizeof(uint32_t);
-        if (mode == AAAC_NVFP4) {
-            if ((e = cudaFuncSetAttribute(scales_hist_kernel<AAAC_NVFP4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm0)) != cudaSuccess) return e;
-            scales_hist_kernel<AAAC_NVFP4><<<hb, 512, sm0, st>>>(W, N, K, ldw, scales, nullptr, tensor_scale, ws.ctrl, dev_status, ws.qhist);
-        } else {
-            if ((e = cudaFuncSetAttribute(scales_hist_kernel<AAAC_INT4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm0)) != cudaSuccess) return e;
-            scales_hist_kernel<AAAC_INT4><<<hb, 512, sm0, st>>>(W, N, K, ldw, scales, ws.rinv, tensor_scale, ws.ctrl, dev_status, ws.qhist);
-        }
-        note_launch();
-    } else if (mode == AAAC_NVFP4) {
-        scales_kernel<AAAC_NVFP4><<<blocks, 256, 0, st>>>(W, N, K, ldw, scales, nullptr, tensor_scale, ws.ctrl, dev_status);
-        note_launch();
-    } else {
-        scales_kernel<AAAC_INT4><<<blocks, 256, 0, st>>>(W, N, K, ldw, scales, ws.rinv, tensor_scale, ws.ctrl, dev_status);
-        note_launch();
+    note_launch();
+    float* const rinv = mode == AAAC_NVFP4 ? nullptr : ws.rinv;
+    if (!with_hist) {
+        auto kern = mode == AAAC_NVFP4 ? scales_kernel<AAAC_NVFP4> : scales_kernel<AAAC_INT4>;
+        return launch_chained(kern, blocks, 256, 0, st, W, N, K, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status);
     }
-    return cudaGetLastError();
+    static std::atomic<size_t> ready[2][kMaxDevices];
+    const size_t smem = kQBins * sizeof(uint32_t);
+    auto kern = mode == AAAC_NVFP4 ? scales_hist_kernel<AAAC_NVFP4> : scales_hist_kernel<AAAC_INT4>;
+    if ((e = allow_smem(kern, smem, ready[mode == AAAC_NVFP4])) != cudaSuccess) return e;
+    return launch_chained(kern, sm_count() * AAAC_SH_BLOCKS, 512, smem, st, W, N, K, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status, ws.qhist);
 }
 
 }  // namespace aaac
