@@ -36,14 +36,23 @@ __device__ __forceinline__ void add_squares(double (&s)[8], uint4 v) {
     }
 }
 
+__device__ __forceinline__ void finish(float* I, int64_t k, double s, int accumulate, uint32_t* dev_status) {
+    float v = (float)s;
+    if (accumulate) v += I[k];
+    I[k] = v;
+    if (dev_status && !isfinite(v)) atomicOr(dev_status, AAAC_DEV_NONFINITE);
+}
+
 __global__ void __launch_bounds__(kWarps * 32, kBlocksPerSM)
 act_sumsq_kernel(const uint16_t* __restrict__ X, int64_t T, int64_t K, int64_t ldx,
-                 double* __restrict__ part, int rows_per_split) {
+                 double* __restrict__ part, int rows_per_split, int strip0, float* __restrict__ I, int accumulate,
+                 uint32_t* dev_status) {
     __shared__ double sm[kWarps][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t col0 = (int64_t)blockIdx.x * 256 + lane * 8;
     const bool active = col0 < K;
-    const int64_t t_begin = (int64_t)blockIdx.y * rows_per_split;
+    const int strip = strip0 + blockIdx.y;
+    const int64_t t_begin = (int64_t)strip * rows_per_split;
     const int64_t t_end = min(T, t_begin + rows_per_split);
     chain_next();
     chain_wait();
@@ -72,7 +81,8 @@ act_sumsq_kernel(const uint16_t* __restrict__ X, int64_t T, int64_t K, int64_t l
         double s = 0.0;
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) s += sm[w][threadIdx.x];
-        part[(int64_t)blockIdx.y * K + col] = s;
+        if (I) finish(I, col, s, accumulate, dev_status);          // the only strip
+        else part[(int64_t)strip * K + col] = s;
     }
 }
 
@@ -96,10 +106,7 @@ act_final_kernel(const double* __restrict__ part, int splits, int64_t K,
     if (warp != 0 || k >= K) return;
 #pragma unroll
     for (int w = 1; w < kWarps; ++w) s += sm[w][lane];
-    float v = (float)s;
-    if (accumulate) v += I[k];
-    I[k] = v;
-    if (dev_status && !isfinite(v)) atomicOr(dev_status, AAAC_DEV_NONFINITE);
+    finish(I, k, s, accumulate, dev_status);
 }
 
 }  // namespace
@@ -112,22 +119,37 @@ int act_splits_max(int64_t K) {
     return (int)(want < 1 ? 1 : want > kActMaxSplits ? kActMaxSplits : want);
 }
 
+ActPlan act_plan(int64_t T, int64_t K, int max_splits) {
+    // up to 256 rows a strip more costs less than the second kernel
+    int64_t splits = T <= 256 ? 1 : std::min<int64_t>(max_splits, (T + kWarps - 1) / kWarps);
+    ActPlan p;
+    p.rows = ((T + splits - 1) / splits + kWarps - 1) / kWarps * kWarps;
+    p.strips = (int)((T + p.rows - 1) / p.rows);
+    return p;
+}
+
+cudaError_t launch_act_strips(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, const ActPlan& plan, int first, int count,
+                              float* I, int accumulate, uint32_t* dev_status, double* part, cudaStream_t st) {
+    note_launch();
+    return launch_chained(act_sumsq_kernel, dim3((unsigned)((K + 255) / 256), (unsigned)count), kWarps * 32, 0, st, X, T, K, ldx, part,
+                          (int)plan.rows, first, plan.strips == 1 ? I : nullptr, accumulate, dev_status);
+}
+
+cudaError_t launch_act_finish(int64_t K, const ActPlan& plan, float* I, int accumulate, uint32_t* dev_status, const double* part,
+                              cudaStream_t st) {
+    if (plan.strips == 1) return cudaSuccess;              // the strip kernel has finished the sums itself
+    note_launch();
+    return launch_chained(act_final_kernel, (unsigned)((K + 31) / 32), kWarps * 32, 0, st, part, plan.strips, K, I, accumulate, dev_status);
+}
+
 namespace {
-// the two launches; `part` holds [max_splits][K] doubles
+// both launches; `part` holds [max_splits][K] doubles.  Every partial that the second kernel reads is written
+// by the first: nothing has to be cleared.
 cudaError_t run_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate, uint32_t* dev_status,
-                          double* part, int64_t splits, cudaStream_t st) {
-    const int bx = (int)((K + 255) / 256);
-    const int64_t max_by_rows = (T + kWarps - 1) / kWarps;
-    if (splits > max_by_rows) splits = max_by_rows;
-    int64_t rows = (T + splits - 1) / splits;
-    rows = (rows + kWarps - 1) / kWarps * kWarps;
-    splits = (T + rows - 1) / rows;
-    cudaError_t e = launch_chained(act_sumsq_kernel, dim3(bx, (unsigned)splits), kWarps * 32, 0, st, X, T, K, ldx, part, (int)rows);
-    note_launch();
-    if (e != cudaSuccess) return e;
-    // every partial that the second kernel reads is written by the first: nothing has to be cleared
-    note_launch();
-    return launch_chained(act_final_kernel, (unsigned)((K + 31) / 32), kWarps * 32, 0, st, part, (int)splits, K, I, accumulate, dev_status);
+                          double* part, int max_splits, cudaStream_t st) {
+    const ActPlan plan = act_plan(T, K, max_splits);
+    const cudaError_t e = launch_act_strips(X, T, K, ldx, plan, 0, plan.strips, I, accumulate, dev_status, part, st);
+    return e != cudaSuccess ? e : launch_act_finish(K, plan, I, accumulate, dev_status, part, st);
 }
 }  // namespace
 
@@ -188,7 +210,7 @@ extern "C" int aaac_act_stats_noalloc(const void* X, int64_t T, int64_t K, int64
     double* part = nullptr;
     if (noalloc_scratch(&part) != cudaSuccess) return AAAC_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int64_t splits = std::min<int64_t>(act_splits_max(K), kNoAllocSplits);
+    const int splits = std::min(act_splits_max(K), kNoAllocSplits);
     if (run_act_stats(static_cast<const uint16_t*>(X), T, K, ldx, I, accumulate, dev_status, part, splits, st) != cudaSuccess) return AAAC_ERR_CUDA;
     return AAAC_OK;
 }

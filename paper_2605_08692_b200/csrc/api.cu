@@ -120,6 +120,8 @@ struct SideStreams {
     bool tried = false, ok = false;
     cudaStream_t s[kSideStreams];
     cudaEvent_t fork, join[kSideStreams];
+    cudaEvent_t step;              // what one stream of a host-buffer call waits for on the other (re-recorded, see HostLanes)
+    unsigned next_copy = 0;        // the side stream the next host-buffer call copies on
 };
 std::mutex g_side_mu;                  // held while a call queues work on the side streams
 SideStreams g_side[kMaxDevices];
@@ -131,7 +133,8 @@ SideStreams* side_streams() {
     SideStreams& p = g_side[dev];
     if (!p.tried) {
         p.tried = true;
-        bool ok = cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess;
+        bool ok = cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&p.step, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < kSideStreams && ok; ++i)
             ok = cudaStreamCreateWithFlags(&p.s[i], cudaStreamNonBlocking) == cudaSuccess &&
                  cudaEventCreateWithFlags(&p.join[i], cudaEventDisableTiming) == cudaSuccess;
@@ -177,6 +180,31 @@ private:
     cudaStream_t st_;
     int lanes_ = 1;
     bool ok_ = true;
+};
+
+// The two streams of a host-buffer call: the caller's, with the kernels, and one for the copies (a side
+// stream, taken in turn; or the caller's own, where overlapping is not worth the events).  to_kernels() /
+// to_copies() make the one stream wait for what the other holds so far: a wait takes the event as it was
+// recorded last, so one event serves all of them.
+class HostLanes {
+public:
+    HostLanes(cudaStream_t st, bool overlap) : lk_(g_side_mu, std::defer_lock), st_(st), cp_(st) {
+        if (!overlap) return;
+        lk_.lock();
+        side_ = side_streams();
+        if (side_) cp_ = side_->s[side_->next_copy++ % kSideStreams];
+    }
+    cudaStream_t copies() const { return cp_; }
+    bool overlapped() const { return cp_ != st_; }
+    bool to_copies() { return pass(st_, cp_); }
+    bool to_kernels() { return pass(cp_, st_); }
+private:
+    bool pass(cudaStream_t from, cudaStream_t to) {
+        return from == to || (cudaEventRecord(side_->step, from) == cudaSuccess && cudaStreamWaitEvent(to, side_->step, 0) == cudaSuccess);
+    }
+    std::unique_lock<std::mutex> lk_;
+    SideStreams* side_ = nullptr;
+    cudaStream_t st_, cp_;
 };
 
 }  // namespace
@@ -288,6 +316,23 @@ int prepare_fit_layer(const aaac_layer& L, int mode, int init, uint32_t* dev_sta
     *I_used = I;
     return AAAC_OK;
 }
+// the rounds of a batch (up to eight layers in a launch), bracketed by the optional timing's events
+int enqueue_rounds(const FitLayerArgs* args, int n_layers, int mode, int sel_group, int n_outer, int n_inner, uint32_t* dev_status,
+                   cudaStream_t st) {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (n_outer > 0) {
+        std::lock_guard<std::mutex> lk(g_timing.mu);
+        if (g_timing.on && g_timing.n < g_timing.cap) {
+            e0 = g_timing.ev[2 * g_timing.n];
+            e1 = g_timing.ev[2 * g_timing.n + 1];
+            ++g_timing.n;
+        }
+    }
+    if (e0) cudaEventRecord(e0, st);
+    const cudaError_t e = launch_fit_rounds_batch(args, n_layers, mode, sel_group, n_outer, n_inner, dev_status, st);
+    if (e1) cudaEventRecord(e1, st);
+    return e == cudaSuccess ? AAAC_OK : AAAC_ERR_CUDA;
+}
 }  // namespace
 
 int aaac_fit_layers(const aaac_layer* layers, int n_layers, int mode, int group, int sel_group,
@@ -317,21 +362,7 @@ int aaac_fit_layers(const aaac_layer* layers, int n_layers, int mode, int group,
         }
         if (!lanes.join() && rc == AAAC_OK) rc = AAAC_ERR_CUDA;
     }
-    if (rc == AAAC_OK) {
-        // all rounds run in one launch per batch; the optional timing brackets the launches of this call
-        cudaEvent_t e0 = nullptr, e1 = nullptr;
-        if (n_outer > 0) {
-            std::lock_guard<std::mutex> lk(g_timing.mu);
-            if (g_timing.on && g_timing.n < g_timing.cap) {
-                e0 = g_timing.ev[2 * g_timing.n];
-                e1 = g_timing.ev[2 * g_timing.n + 1];
-                ++g_timing.n;
-            }
-        }
-        if (e0) cudaEventRecord(e0, st);
-        if (launch_fit_rounds_batch(args, n_layers, mode, sel_group, n_outer, n_inner, dev_status, st) != cudaSuccess) rc = AAAC_ERR_CUDA;
-        if (e1) cudaEventRecord(e1, st);
-    }
+    if (rc == AAAC_OK) rc = enqueue_rounds(args, n_layers, mode, sel_group, n_outer, n_inner, dev_status, st);
     // with rounds to run the last fit launch writes the tables out itself; with none, a small kernel does
     for (int l = 0; l < n_layers && rc == AAAC_OK && n_outer == 0; ++l)
         if (launch_export_tables(layers[l].T01, args[l].ws, st) != cudaSuccess) rc = AAAC_ERR_CUDA;
@@ -531,33 +562,63 @@ int aaac_quantize_layer_host_async(const void* W_host, int64_t N, int64_t K, int
     const int g = group;
     const size_t scale_bytes = (size_t)N * (K / g) * (mode == AAAC_INT4 ? 2 : 1);
     uint32_t* dstatus = reinterpret_cast<uint32_t*>(d + h.status);
-    if (cudaMemsetAsync(dstatus, 0, 4, st) != cudaSuccess) return AAAC_ERR_CUDA;
-    if (cudaMemcpyAsync(d + h.X, X_host, (size_t)T * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess) return AAAC_ERR_CUDA;
-    if (cudaMemcpyAsync(d + h.W, W_host, (size_t)N * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess) return AAAC_ERR_CUDA;
-    void* lws = d + h.ws;
-    const size_t lws_bytes = ws_bytes - h.ws;
-    float* I = reinterpret_cast<float*>(d + h.I);
-    float* T01 = reinterpret_cast<float*>(d + h.T01);
-    rc = aaac_act_stats(d + h.X, T, K, K, I, 0, dstatus, lws, lws_bytes, stream);
-    if (rc) return rc;
-    rc = aaac_fit_layer(d + h.W, N, K, K, mode, group, I, nullptr, 0, 0, n_outer, 1, init, T01, d + h.scales,
-                        reinterpret_cast<float*>(d + h.ts), nullptr, dstatus, lws, lws_bytes, stream);
-    if (rc) return rc;
-    rc = aaac_pack(d + h.W, N, K, K, mode, group, I, T01, reinterpret_cast<uint16_t*>(d + h.Tb), d + h.scales,
-                   reinterpret_cast<float*>(d + h.ts), reinterpret_cast<uint8_t*>(d + h.codes),
-                   reinterpret_cast<double*>(d + h.err), nullptr, lws, lws_bytes, stream);
-    if (rc) return rc;
+    if ((unsigned long long)N * (unsigned long long)K >= (1ull << 32)) return AAAC_ERR_TOO_LARGE;
+    const Workspace w = carve(d + h.ws, mode, N, K, ws_bytes - h.ws);
+    const uint16_t* const W = reinterpret_cast<const uint16_t*>(d + h.W);
+    const uint16_t* const X = reinterpret_cast<const uint16_t*>(d + h.X);
+    float* const I = reinterpret_cast<float*>(d + h.I);
+    float* const T01 = reinterpret_cast<float*>(d + h.T01);
+    float* const ts = reinterpret_cast<float*>(d + h.ts);
+    // Copies on a stream of their own: the scales and start passes, which need W alone, run while X arrives, X is
+    // summed piece by piece as it does, and the codes of packed rows leave while the next rows are packed.  The
+    // events cost some 10 us of host time, which copies of 4 MB and more hide.
+    HostLanes lanes(st, (size_t)(N + T) * (size_t)K * 2 >= ((size_t)4 << 20));
+    cudaStream_t const cp = lanes.copies();
     cudaError_t e = cudaSuccess;
-    auto back = [&](void* dst, size_t off, size_t bytes) {
-        if (e == cudaSuccess && dst) e = cudaMemcpyAsync(dst, d + off, bytes, cudaMemcpyDeviceToHost, st);
+    auto run = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+    auto ok = [&](bool r) { if (!r) run(cudaErrorUnknown); };
+    auto back = [&](void* dst, size_t off, size_t bytes, cudaStream_t s) {
+        if (e == cudaSuccess && dst && bytes) run(cudaMemcpyAsync(dst, d + off, bytes, cudaMemcpyDeviceToHost, s));
     };
-    back(codes_host, h.codes, (size_t)N * K / 2);
-    back(scales_host, h.scales, scale_bytes);
-    back(T01_host, h.T01, 2 * kM * 4);
-    back(T01_bf16_host, h.Tb, 2 * kM * 2);
-    back(tensor_scale_host, h.ts, 4);
-    back(err_out_host, h.err, 16);
-    back(status_host, h.status, 4);
+    ok(lanes.to_copies());
+    run(cudaMemcpyAsync(d + h.W, W_host, (size_t)N * K * 2, cudaMemcpyHostToDevice, cp));
+    ok(lanes.to_kernels());
+    const bool hist = init == AAAC_INIT_QUANTILE;
+    run(cudaMemsetAsync(dstatus, 0, 4, st));
+    run(cudaMemsetAsync(w.ctrl, 0, w.zero_bytes(hist), st));
+    if (e == cudaSuccess) run(launch_scales(W, N, K, K, mode, d + h.scales, ts, dstatus, w, st, hist));
+    if (e == cudaSuccess) run(launch_init(W, N, K, K, mode, init, d + h.scales, T01, dstatus, w, st));
+    const ActPlan plan = act_plan(T, K, act_splits_max(K));
+    const int pieces = lanes.overlapped() ? std::min(4, plan.strips) : 1;
+    for (int c = 0; c < pieces; ++c) {
+        const int s0 = (int)((int64_t)plan.strips * c / pieces), s1 = (int)((int64_t)plan.strips * (c + 1) / pieces);
+        const int64_t t0 = s0 * plan.rows, t1 = std::min<int64_t>(T, s1 * plan.rows);
+        run(cudaMemcpyAsync(d + h.X + (size_t)t0 * K * 2, static_cast<const char*>(X_host) + (size_t)t0 * K * 2, (size_t)(t1 - t0) * K * 2,
+                            cudaMemcpyHostToDevice, cp));
+        ok(lanes.to_kernels());
+        if (e == cudaSuccess) run(launch_act_strips(X, T, K, K, plan, s0, s1 - s0, I, 0, dstatus, w.act_part, st));
+    }
+    if (e == cudaSuccess) run(launch_act_finish(K, plan, I, 0, dstatus, w.act_part, st));
+    const FitLayerArgs args{W, N, K, K, d + h.scales, I, nullptr, T01, w};
+    if (e == cudaSuccess && enqueue_rounds(&args, 1, mode, g, n_outer, 1, dstatus, st) != AAAC_OK) run(cudaErrorUnknown);
+    if (e == cudaSuccess && n_outer == 0) run(launch_export_tables(T01, w, st));
+    const int64_t range = lanes.overlapped() && N >= 64 * kPackRanges ? pack_range_rows(N) : N;
+    const size_t scale_row = scale_bytes / (size_t)N;
+    for (int64_t r0 = 0; r0 < N; r0 += range) {
+        const int64_t r1 = std::min(N, r0 + range);
+        if (e == cudaSuccess)
+            run(launch_pack(W, N, K, K, mode, g, I, T01, reinterpret_cast<uint16_t*>(d + h.Tb), d + h.scales, ts,
+                            reinterpret_cast<uint8_t*>(d + h.codes), nullptr, reinterpret_cast<double*>(d + h.err), nullptr, w, st, r0, r1));
+        ok(lanes.to_copies());
+        back(codes_host + (size_t)r0 * (K / 2), h.codes + (size_t)r0 * (K / 2), (size_t)(r1 - r0) * (K / 2), cp);
+        back(static_cast<char*>(scales_host) + r0 * scale_row, h.scales + r0 * scale_row, (size_t)(r1 - r0) * scale_row, cp);
+    }
+    back(T01_host, h.T01, 2 * kM * 4, st);
+    back(T01_bf16_host, h.Tb, 2 * kM * 2, st);
+    back(tensor_scale_host, h.ts, 4, st);
+    back(err_out_host, h.err, 16, st);
+    back(status_host, h.status, 4, st);
+    ok(lanes.to_kernels());
     return e == cudaSuccess ? AAAC_OK : AAAC_ERR_CUDA;
 }
 

@@ -116,6 +116,13 @@ __device__ __forceinline__ float f32_round_down(double d) { return __double2floa
 // ---- launchers (each enqueues on `st` and returns the launch status) ----
 cudaError_t launch_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate,
                              uint32_t* dev_status, const Workspace& ws, cudaStream_t st);
+// the same in pieces: strips [first, first + count) of the plan, then the sum over the strips
+struct ActPlan { int64_t rows; int strips; };
+ActPlan act_plan(int64_t T, int64_t K, int max_splits);
+cudaError_t launch_act_strips(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, const ActPlan& plan, int first, int count,
+                              float* I, int accumulate, uint32_t* dev_status, double* part, cudaStream_t st);
+cudaError_t launch_act_finish(int64_t K, const ActPlan& plan, float* I, int accumulate, uint32_t* dev_status, const double* part,
+                              cudaStream_t st);
 // with_hist: the scales pass also counts the 16384-bin histogram of the normalised weights (the quantile
 // start's first pass over W) into ws.qhist, which is zero before
 cudaError_t launch_scales(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, void* scales,
@@ -136,11 +143,13 @@ struct FitLayerArgs {
 cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode, int sel_group, int n_outer, int n_inner,
                                     uint32_t* dev_status, cudaStream_t st);
 cudaError_t launch_export_tables(float* T01, const Workspace& ws, cudaStream_t st);
+// row0, row1: only these rows (row0 a multiple of 64; the launches of a layer in order, the last one, with row1 = N,
+// hands the results out); the default is all of them.
 // sigma_bits: null when the selection group is the scale group (sigma in the scale's sign bit)
 cudaError_t launch_pack(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, int sel_group, const float* I,
                         const float* T01_f32, uint16_t* T01_bf16, void* scales, const float* tensor_scale,
                         uint8_t* codes, uint8_t* sigma_bits, double* err_out, unsigned long long* stats,
-                        const Workspace& ws, cudaStream_t st);
+                        const Workspace& ws, cudaStream_t st, int64_t row0 = 0, int64_t row1 = -1);
 cudaError_t launch_dequant(const uint8_t* codes, const void* scales, const uint8_t* sigma_bits,
                            const float* tensor_scale, const uint16_t* Tb, int64_t N, int64_t K, int mode,
                            uint16_t* What, int64_t ldo, cudaStream_t st);
@@ -182,6 +191,10 @@ cudaError_t allow_smem(K kern, size_t bytes, std::atomic<size_t> (&done)[kMaxDev
     if (e == cudaSuccess && dev >= 0 && dev < kMaxDevices) done[dev].store(bytes, std::memory_order_relaxed);
     return e;
 }
+
+// the row ranges in which the host-buffer call packs a layer, so that the codes of one travel while the next is packed
+constexpr int kPackRanges = 4;
+inline int64_t pack_range_rows(int64_t N) { return ((N + kPackRanges - 1) / kPackRanges + 63) / 64 * 64; }
 
 int sm_count();
 void note_launch(int n = 1);      // counts kernel launches (aaac_launch_count)

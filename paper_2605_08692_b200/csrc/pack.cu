@@ -25,6 +25,8 @@
 // the row stride and no branch around the loads; a lane takes 8 adjacent columns (one 128-bit load per row, one 32-bit store of 8 codes); the two errors travel
 // as one packed FP32 pair.
 // Error sums go through one partial per block, added by the last block to finish.
+#include <algorithm>
+
 #include "lookup.cuh"
 
 namespace aaac {
@@ -51,6 +53,7 @@ struct PackParams {
     uint8_t* sigma_bits;          // [N][K / 128] when the selection group is 16 inside a scale group of 128; else null
     double* err_out;              // [2] or null
     unsigned long long* stats;    // [4] or null
+    unsigned first_block, blocks; // this launch's place among the blocks of all launches of the layer, and their number (0: not the last launch)
 };
 
 // The rare path of a row, out of line so that the hot loop holds a single call: for the lanes that
@@ -143,7 +146,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
         __syncwarp();
         const double T = S.Td[lane];
         __syncwarp();
-        if (blockIdx.x == 0) p.T01_bf16[lane] = (uint16_t)(__float_as_uint((float)T) >> 16);
+        if (p.first_block + blockIdx.x == 0) p.T01_bf16[lane] = (uint16_t)(__float_as_uint((float)T) >> 16);
         derive_tables(S, lane, T);
     }
     __syncthreads();
@@ -341,10 +344,11 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
         double s = 0.0;
 #pragma unroll
         for (int w = 0; w < NW; ++w) s += wsum[w][tid];
-        p.part[(size_t)blockIdx.x * kPartStride + tid] = s;
+        p.part[(size_t)(p.first_block + blockIdx.x) * kPartStride + tid] = s;
     }
     __threadfence();
     __syncthreads();
+    if (p.blocks == 0) return;                             // (a later launch adds the sums)
     if (tid == 0) is_last = (atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1);
     __syncthreads();
     if (!is_last) return;
@@ -353,7 +357,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
     // the results out.  A warp per sum: two threads walking the partials one after the other took 10-25 us.
     if (warp < 2) {
         double s = 0.0;
-        for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(p.part + (size_t)b * kPartStride + warp);
+        for (unsigned b = lane; b < p.blocks; b += 32) s += __ldcg(p.part + (size_t)b * kPartStride + warp);
 #pragma unroll
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         if (lane == 0) {
@@ -385,21 +389,27 @@ cudaError_t launch_pack_variant(const PackParams& p, unsigned grid, cudaStream_t
 cudaError_t launch_pack(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, int sel_group, const float* I,
                         const float* T01_f32, uint16_t* T01_bf16, void* scales, const float* tensor_scale,
                         uint8_t* codes, uint8_t* sigma_bits, double* err_out, unsigned long long* stats,
-                        const Workspace& ws, cudaStream_t st) {
-    PackParams p{};
-    p.W = W; p.N = N; p.K = K; p.ldw = ldw;
-    p.scales = scales; p.I = I; p.tensor_scale = tensor_scale;
-    p.ctrl = ws.ctrl; p.part = ws.part; p.T01_f32 = T01_f32; p.T01_bf16 = T01_bf16; p.codes = codes;
-    p.sigma_bits = sigma_bits;
-    p.err_out = err_out; p.stats = stats;
+                        const Workspace& ws, cudaStream_t st, int64_t row0, int64_t row1) {
     if (N > 0x7FFFFFFF || K > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    if (row1 < 0) row1 = N;
     // two blocks per SM; no more warps than there are (row, slab) pieces of work
     const int64_t slabs = (K + 255) / 256;
-    int64_t grid = (int64_t)sm_count() * kPackBlocksPerSM;
-    const int64_t pieces = (N * slabs + pack_warps(mode) - 1) / pack_warps(mode);
-    if (grid > pieces) grid = pieces;
-    if (grid > kMaxBlocks) grid = kMaxBlocks;
-    if (grid < 1) grid = 1;
+    const int64_t most = std::min<int64_t>((int64_t)sm_count() * kPackBlocksPerSM, kMaxBlocks / kPackRanges);
+    auto grid_of = [&](int64_t rows) {
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(most, (rows * slabs + pack_warps(mode) - 1) / pack_warps(mode)));
+    };
+    const unsigned grid = grid_of(row1 - row0);
+    PackParams p{};
+    const int64_t g = mode == AAAC_INT4 ? 128 : 16;
+    p.W = W + row0 * ldw; p.N = row1 - row0; p.K = K; p.ldw = ldw;
+    p.scales = static_cast<char*>(scales) + row0 * (K / g) * (mode == AAAC_INT4 ? 2 : 1);
+    p.I = I; p.tensor_scale = tensor_scale;
+    p.ctrl = ws.ctrl; p.part = ws.part; p.T01_f32 = T01_f32; p.T01_bf16 = T01_bf16; p.codes = codes + row0 * (K / 2);
+    p.sigma_bits = sigma_bits ? sigma_bits + row0 * (K / 128) : nullptr;
+    p.err_out = err_out; p.stats = stats;
+    // (the ranges before the last are all of one size, see aaac_quantize_layer_host_async)
+    p.first_block = row0 ? (unsigned)(row0 / pack_range_rows(N)) * grid_of(pack_range_rows(N)) : 0u;
+    p.blocks = row1 == N ? p.first_block + grid : 0u;
     cudaError_t e;
     if (mode == AAAC_INT4 && sel_group == 16) e = launch_pack_variant<AAAC_INT4, 16>(p, (unsigned)grid, st);
     else if (mode == AAAC_INT4) e = launch_pack_variant<AAAC_INT4, 128>(p, (unsigned)grid, st);
