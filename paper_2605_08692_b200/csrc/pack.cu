@@ -22,8 +22,10 @@
 // than by a hand-built pipeline: a warp walks down the rows of one 256-column slab (so its eight
 // importances stay in registers), two rows per trip in registers of their own -- while one is worked
 // on, the other's load is in flight and nothing is copied -- with 32-bit element offsets advanced by
-// the row stride and no branch around the loads; a lane takes 8 adjacent columns (one 128-bit load per row, one 32-bit store of 8 codes); the two errors travel
-// as one packed FP32 pair.
+// the row stride and no branch around the loads; a lane takes 8 adjacent columns (one 128-bit load per row, one 32-bit store of 8 codes); the two
+// errors travel as pairs of columns.  27 instructions per weight, and at 16 warps per SM the loads bound the
+// pass as much as they do: the rows after next are asked for into L2 ahead of time.  14336 x 4096: NVFP4
+// 96 -> 79 us (0.75 Tweights/s), INT4 107 -> 91; 24 warps per SM (80 registers) spilled and took 100.
 // Error sums go through one partial per block, added by the last block to finish.
 #include <algorithm>
 
@@ -56,38 +58,33 @@ struct PackParams {
     unsigned first_block, blocks; // this launch's place among the blocks of all launches of the layer, and their number (0: not the last launch)
 };
 
-// The rare path of a row, out of line so that the hot loop holds a single call: for the lanes that
-// ask (flags != 0) the interval of every weight is found by binary search of the breakpoint list;
-// the groups flagged kNear are decided in double (Eq. 8 as a plain double-precision loop states
-// it, the lanes of a group combined by a shuffle tree); and for every asking lane the weights that
-// lie exactly half-way between two different entries of the chosen table are counted (x equals a
-// breakpoint that is an exact midpoint of that table).  Every lane of the warp calls.
-constexpr int kNear = 1, kTieCand = 2, kFastSigma = 4;
+// The near-tie path of a row, out of line so that the hot loop holds a single call: for the lanes that ask,
+// the interval of every weight is found by binary search of the breakpoint list, the groups are decided in
+// double (Eq. 8 as a plain double-precision loop states it, the lanes of a group combined by a shuffle
+// tree), and the weights that lie exactly half-way between two different entries of the chosen table are
+// counted (x equals a breakpoint that is an exact midpoint of that table).  Every lane of the warp calls.
 struct Rare8 { int J[8]; double emin; int sigma; int tie; int nties; };
 
+__device__ __forceinline__ int half_way(const FitTables* S, float x, int J, int sigma) {
+    for (int jj = J; jj < kNBP && S->bp[jj] == x; ++jj)                 // the breakpoints equal to x, if any
+        if (S->src[jj] == (uint8_t)sigma && S->exact[jj]) return 1;
+    return 0;
+}
+
 template <int LPG>
-__device__ __noinline__ Rare8 rare_groups(const FitTables* S, Row8 r, int flags) {
+__device__ __noinline__ Rare8 rare_groups(const FitTables* S, Row8 r, bool near) {
     Rare8 out;
-    const bool need = (flags & (kNear | kTieCand)) != 0, near = (flags & kNear) != 0;
     double e0 = 0.0, e1 = 0.0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         int J = 0;
-        if (need) {
-            if (r.hint[j] < (uint32_t)kNJ) {
-                J = (int)r.hint[j];
-            } else {
-#pragma unroll
-                for (int step = 16; step; step >>= 1)      // number of breakpoints below x (sorted list)
-                    if (J + step <= kNBP && S->bp[J + step - 1] < r.x[j]) J += step;
-            }
-            if (near) {
-                const double2 pq = S->PQ[J];
-                const double xd = (double)r.x[j], id = (double)r.I[j];
-                const double d0 = __dsub_rn(xd, pq.x), d1 = __dsub_rn(xd, pq.y);
-                e0 = __dadd_rn(e0, __dmul_rn(id, __dmul_rn(d0, d0)));
-                e1 = __dadd_rn(e1, __dmul_rn(id, __dmul_rn(d1, d1)));
-            }
+        if (near) {
+            J = r.hint[j] < (uint32_t)kNJ ? (int)r.hint[j] : find_interval(S->bp, r.x[j]);
+            const double2 pq = S->PQ[J];
+            const double xd = (double)r.x[j], id = (double)r.I[j];
+            const double d0 = __dsub_rn(xd, pq.x), d1 = __dsub_rn(xd, pq.y);
+            e0 = __dadd_rn(e0, __dmul_rn(id, __dmul_rn(d0, d0)));
+            e1 = __dadd_rn(e1, __dmul_rn(id, __dmul_rn(d1, d1)));
         }
         out.J[j] = J;
     }
@@ -96,18 +93,45 @@ __device__ __noinline__ Rare8 rare_groups(const FitTables* S, Row8 r, int flags)
         e0 = __dadd_rn(e0, __shfl_xor_sync(0xFFFFFFFFu, e0, s));
         e1 = __dadd_rn(e1, __shfl_xor_sync(0xFFFFFFFFu, e1, s));
     }
-    out.sigma = near ? (int)(e1 < e0) : ((flags & kFastSigma) != 0);
+    out.sigma = e1 < e0;
     out.tie = near && e0 == e1;
     out.emin = out.sigma ? e1 : e0;
     int n = 0;
-    if (need) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            for (int jj = out.J[j]; jj < kNBP && S->bp[jj] == r.x[j]; ++jj)     // the breakpoints equal to x, if any
-                if (S->src[jj] == (uint8_t)out.sigma && S->exact[jj]) { ++n; break; }
+    if (near) {
+#pragma unroll 1
+        for (int j = 0; j < 8; ++j) n += half_way(S, r.x[j], out.J[j], out.sigma);
     }
     out.nties = n;
     return out;
+}
+
+// Lanes that hold a weight equal to the breakpoint of its bin (a few per cent of the rows have one: BF16
+// weights times the reciprocal of a coarse scale hit BF16 midpoints) go on a short per-warp list, worked off
+// 32 at a time, an entry per lane: deciding them row by row made the whole warp run a rare path for one lane.
+constexpr int kTieCap = 64;
+template <int MODE>
+__device__ __noinline__ uint32_t count_ties(const FitTables* S, const uint16_t* W, unsigned ldw, unsigned Gr, const void* scales,
+                                            uint32_t list_addr, int count, int slab, int lane) {
+    constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
+    uint32_t n = 0;
+#pragma unroll 1
+    for (int e = lane; e < count; e += 32) {
+        uint32_t row, what;                                               // what: lane of the row, selection bit above
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(row), "=r"(what) : "r"(list_addr + (uint32_t)e * 8u) : "memory");
+        const unsigned col = (unsigned)slab * 256u + (what & 31u) * 8u;
+        const uint4 v = *reinterpret_cast<const uint4*>(W + (row * ldw + col));
+        const unsigned gi = row * Gr + col / G;
+        // (the sign bit may or may not have been set by now)
+        const float rinv = MODE == AAAC_NVFP4 ? S->rlut[reinterpret_cast<const uint8_t*>(scales)[gi] & 0x7Fu]
+                                              : __frcp_rn(__uint_as_float((uint32_t)(reinterpret_cast<const uint16_t*>(scales)[gi] & 0x7FFFu) << 16));
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float x = __fmul_rn((j & 1) ? bf16_hi(w[j >> 1]) : bf16_lo(w[j >> 1]), rinv);
+            n += half_way(S, x, find_interval(S->bp, x), (int)(what >> 5));
+        }
+    }
+    return n;
 }
 
 constexpr int kPackBlocksPerSM = 2;
@@ -122,6 +146,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
     __shared__ FitTables S;
     __shared__ float slut[128];                      // NVFP4: s_eff per E4M3 code
     __shared__ double wsum[NW][2];
+    __shared__ uint2 tie_list[NW][kTieCap];
     __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -156,6 +181,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
     const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(dyn);
     const uint32_t lut1_copy = (lane & (REP - 1)) * 8;             // this lane's copy of a bin's entry
     const uint32_t lut2_addr = sm_base + kLut1Bytes;                // the {P, Q} table
+    const uint32_t list_addr = (uint32_t)__cvta_generic_to_shared(&tie_list[warp][0]);
     constexpr float kBinsPerUnit = (float)(NB / 16);
     constexpr float kMagic = (float)(NB / 2) + 1.5f * (float)(1 << 23) / (float)(REP * 8);
     constexpr uint32_t kBinMask = (uint32_t)(NB - 1) * (REP * 8);
@@ -179,7 +205,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
         const int my = nw_total >= slabs ? gw / slabs : 0;
         const int col0 = slab * 256 + lane * 8;
         const bool col_ok = col0 < K;
-        uint64_t II[8];                       // {I, I} of the lane's eight columns
+        uint64_t II[4];                       // importances of the lane's eight columns, in pairs
         float isum = 0.f;                     // g2 * sum of I over the lane's selection group (rounded up a little)
         {
             float Iv[8];
@@ -192,7 +218,9 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
                 Iv[4] = b.x; Iv[5] = b.y; Iv[6] = b.z; Iv[7] = b.w;
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { isum += Iv[j]; II[j] = pack2(Iv[j], Iv[j]); }
+            for (int j = 0; j < 8; ++j) isum += Iv[j];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) II[j] = pack2(Iv[2 * j], Iv[2 * j + 1]);
 #pragma unroll
             for (int o = LPG / 2; o; o >>= 1) isum += __shfl_xor_sync(0xFFFFFFFFu, isum, o);
             isum = __fmul_ru(isum * 1.0001f, g2);
@@ -209,8 +237,13 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
             if (MODE == AAAC_NVFP4) sc = reinterpret_cast<const uint8_t*>(p.scales)[go];
             else sc = reinterpret_cast<const uint16_t*>(p.scales)[go];
         };
+        // the rows after next are asked for into L2 (one lane per 128 bytes): the load one row ahead covers the way
+        // from there, not the one from DRAM
+        auto ahead = [&](int row, unsigned wo) {
+            if (row < N && (lane & 7) == 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(Wp + wo));
+        };
+        int nlist = 0;                        // entries of the warp's tie list
         float ef = 0.f, eof = 0.f;            // the two error sums of up to 16 rows (one conversion to double per 16 rows)
-        int nrow = 0;
         // one row: v and scv were loaded before; (wo, go) are the row's offsets, co the byte offset of its codes
         auto do_row = [&](const uint4& v, uint32_t scv, int row, unsigned go, unsigned co) {
             const uint32_t sbits = MODE == AAAC_NVFP4 ? (scv & 0x7Fu) : (scv & 0x7FFFu);
@@ -226,18 +259,30 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
             float x[8];
             uint64_t pq[8];
             bool tcand = false;                             // some w~ equals the breakpoint of its bin
-            uint64_t e01 = 0ull;
+            const uint64_t rr = pack2(rinv, rinv);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                x[j] = __fmul_rn((j & 1) ? bf16_hi(w[j >> 1]) : bf16_lo(w[j >> 1]), rinv);
-                const uint32_t off = ((uint32_t)__float_as_int(__fmaf_rn(x[j], kBinsPerUnit, kMagic)) & kBinMask) | lut1_copy;
-                const uint2 e = lds_table_u2(sm_base + off);
-                tcand |= (x[j] == __uint_as_float(e.y));
-                pq[j] = lds_table_b64(above_addr(e.x, x[j], e.y));
-                const uint64_t u01 = diff2(x[j], pq[j]);
-                e01 = fma2(mul2(II[j], u01), u01, e01);
+            for (int j = 0; j < 4; ++j) {
+                const uint64_t xx = mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr);
+                const uint64_t bb = fma2(xx, pack2(kBinsPerUnit, kBinsPerUnit), pack2(kMagic, kMagic));
+                unpack2(xx, x[2 * j], x[2 * j + 1]);
+                const uint2 ea = lds_table_u2(sm_base + (((uint32_t)__float_as_int(lo2(bb)) & kBinMask) | lut1_copy));
+                const uint2 eb = lds_table_u2(sm_base + (((uint32_t)__float_as_int(hi2(bb)) & kBinMask) | lut1_copy));
+                tcand |= (x[2 * j] == __uint_as_float(ea.y)) | (x[2 * j + 1] == __uint_as_float(eb.y));
+                pq[2 * j] = lds_table_b64(above_addr(ea.x, x[2 * j], ea.y));
+                pq[2 * j + 1] = lds_table_b64(above_addr(eb.x, x[2 * j + 1], eb.y));
             }
-            float e0 = lo2(e01), e1 = hi2(e01);
+            uint64_t s0 = 0ull, s1 = 0ull;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float Pa, Qa, Pb, Qb;
+                unpack2(pq[2 * j], Pa, Qa);
+                unpack2(pq[2 * j + 1], Pb, Qb);
+                const uint64_t u0 = pack2(__fsub_rn(x[2 * j], Pa), __fsub_rn(x[2 * j + 1], Pb));
+                const uint64_t u1 = pack2(__fsub_rn(x[2 * j], Qa), __fsub_rn(x[2 * j + 1], Qb));
+                s0 = fma2(mul2(II[j], u0), u0, s0);
+                s1 = fma2(mul2(II[j], u1), u1, s1);
+            }
+            float e0 = lo2(s0) + hi2(s0), e1 = lo2(s1) + hi2(s1);
 #pragma unroll
             for (int s2 = LPG / 2; s2; s2 >>= 1) {
                 e0 += __shfl_xor_sync(0xFFFFFFFFu, e0, s2);
@@ -249,19 +294,35 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
             bool sg = e1 < e0;
             float emin = sg ? e1 : e0;
             if (__any_sync(0xFFFFFFFFu, near || tcand)) {
-                // near-ties, poisoned slots and weights that sit on a breakpoint (rare, out of line)
-                Row8 r;
+                if (__any_sync(0xFFFFFFFFu, near)) {
+                    // near-ties and poisoned slots (rare, out of line)
+                    Row8 r;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) { r.x[j] = x[j]; r.I[j] = lo2(II[j]); r.hint[j] = interval_hint(S, pq[j]); }
-                const Rare8 ex = rare_groups<LPG>(&S, r, (near ? kNear : 0) | (tcand ? kTieCand : 0) | (sg ? kFastSigma : 0));
-                if (near) {
+                    for (int j = 0; j < 8; ++j) { r.x[j] = x[j]; r.I[j] = (j & 1) ? hi2(II[j >> 1]) : lo2(II[j >> 1]); r.hint[j] = interval_hint(S, pq[j]); }
+                    const Rare8 ex = rare_groups<LPG>(&S, r, near);
+                    if (near) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) pq[j] = lds_table_b64(pq_entry_addr(lut2_addr, ex.J[j], lane));
-                    sg = ex.sigma != 0;
-                    emin = (float)ex.emin;
-                    if (col_ok && (lane % LPG) == 0) { ++n_exact; n_sig_tie += ex.tie; }
+                        for (int j = 0; j < 8; ++j) pq[j] = lds_table_b64(pq_entry_addr(lut2_addr, ex.J[j], lane));
+                        sg = ex.sigma != 0;
+                        emin = (float)ex.emin;
+                        if (col_ok) {
+                            n_idx_tie += ex.nties;
+                            if ((lane % LPG) == 0) { ++n_exact; n_sig_tie += ex.tie; }
+                        }
+                    }
                 }
-                if (col_ok) n_idx_tie += ex.nties;
+                const bool listed = tcand && !near && col_ok;
+                const unsigned lm = __ballot_sync(0xFFFFFFFFu, listed);
+                if (listed)
+                    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" :: "r"(list_addr + (uint32_t)(nlist + __popc(lm & ((1u << lane) - 1u))) * 8u),
+                                 "r"(row), "r"((uint32_t)lane | (sg ? 32u : 0u)) : "memory");
+                nlist += __popc(lm);
+                if (nlist > kTieCap - 32) {
+                    __syncwarp();
+                    n_idx_tie += count_ties<MODE>(&S, Wp, (unsigned)p.ldw, (unsigned)Gr, p.scales, list_addr, nlist, slab, lane);
+                    nlist = 0;
+                    __syncwarp();
+                }
             }
             if (SEL != G) {
                 // selection bits apart (Algorithm 1 line 20, S < g): group j of the row in bit j % 8 of
@@ -281,12 +342,13 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
                 eof = __fmaf_rn(emin, __fmul_rn(sval, sval), eof);
             }
             // codes (Eq. 6): the entry index rides in the low mantissa bits of the chosen constant
+            // (a funnel shift takes the lowest four bits of one constant after the other in from the top)
             uint32_t word = 0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 float cP, cQ;
                 unpack2(pq[j], cP, cQ);
-                word |= (__float_as_uint(sg ? cQ : cP) & kIdxMask) << (4 * j);
+                word = __funnelshift_r(word, __float_as_uint(sg ? cQ : cP), 4);
             }
             *reinterpret_cast<uint32_t*>(p.codes + co) = word;
             if (SEL == G && (lane % LPG) == 0) {
@@ -304,23 +366,36 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
             uint4 va, vb;
             uint32_t sa, sb;
             load(wo, go, va, sa);
-            for (int row = my; row < N; row += 2 * per_slab) {
-                const bool more1 = row + per_slab < N;
-                const unsigned wo1 = more1 ? wo + step_w : wo, go1 = more1 ? go + step_g : go;
-                load(wo1, go1, vb, sb);
-                do_row(va, sa, row, go, co);
-                if (!more1) break;
-                const bool more2 = row + 2 * per_slab < N;
-                const unsigned wo2 = more2 ? wo1 + step_w : wo1, go2 = more2 ? go1 + step_g : go1;
-                load(wo2, go2, va, sa);
-                do_row(vb, sb, row + per_slab, go1, co + step_c);
-                wo = wo2; go = go2; co += 2 * step_c;
-                nrow += 2;
-                if (nrow >= 16) { Eacc += (double)ef; Eout += (double)eof; ef = 0.f; eof = 0.f; nrow = 0; }
+            bool more = true;
+            for (int row = my; more;) {
+#pragma unroll 1
+                for (int trip = 0; trip < 8; ++trip) {
+                    const bool more1 = row + per_slab < N;
+                    ahead(row + 2 * per_slab, wo + 2 * step_w);
+                    ahead(row + 3 * per_slab, wo + 3 * step_w);
+                    const unsigned wo1 = more1 ? wo + step_w : wo, go1 = more1 ? go + step_g : go;
+                    load(wo1, go1, vb, sb);
+                    do_row(va, sa, row, go, co);
+                    if (!more1) { more = false; break; }
+                    const bool more2 = row + 2 * per_slab < N;
+                    const unsigned wo2 = more2 ? wo1 + step_w : wo1, go2 = more2 ? go1 + step_g : go1;
+                    load(wo2, go2, va, sa);
+                    do_row(vb, sb, row + per_slab, go1, co + step_c);
+                    wo = wo2; go = go2; co += 2 * step_c;
+                    row += 2 * per_slab;
+                    if (!more2) { more = false; break; }
+                }
+                Eacc += (double)ef;
+                Eout += (double)eof;
+                ef = 0.f;
+                eof = 0.f;
             }
         }
         Eacc += (double)ef;
         Eout += (double)eof;
+        __syncwarp();
+        if (nlist > 0) n_idx_tie += count_ties<MODE>(&S, Wp, (unsigned)p.ldw, (unsigned)Gr, p.scales, list_addr, nlist, slab, lane);
+        __syncwarp();
     }
 
     // ---- block partial of the two error sums; integer statistics by atomics ----
