@@ -51,12 +51,12 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
     __shared__ unsigned long long base[kQReq];
     __shared__ uint32_t nbuf;
     __shared__ uint32_t okmin[kQReq], okmax[kQReq];       // smallest / largest key of the slots without list space
-    __shared__ float rl[128];                             // NVFP4: reciprocal of the effective scale per E4M3 code
+    __shared__ float rl[128];                             // fl32(1 / s) per E4M3 code, or per mantissa of a BF16 scale
     const int tid = threadIdx.x, lane = tid & 31;
     chain_next();
     chain_wait();
     const float s_t = ctrl->s_t;
-    if (MODE == AAAC_NVFP4 && tid < 128) rl[tid] = __frcp_rn(__fmul_rn(e4m3_value((uint32_t)tid), s_t));
+    if (tid < 128) rl[tid] = MODE == AAAC_NVFP4 ? __frcp_rn(__fmul_rn(e4m3_value((uint32_t)tid), s_t)) : bf16_rcp_entry((uint32_t)tid);
     {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(slot_of_bin);
         for (int i = tid; i < kQBins / 4; i += blockDim.x) sm[i] = src[i];
@@ -106,14 +106,13 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
     // recomputes w~ of that weight alone.
     auto take = [&](const uint4& v, uint32_t ss) {
         // fl32(1 / s) for these scale bits
-        const float r = MODE == AAAC_INT4 ? __frcp_rn(__uint_as_float((ss & 0x7FFFu) << 16)) : rl[ss & 0x7Fu];
+        const float r = MODE == AAAC_INT4 ? bf16_rcp(rl, ss & 0x7FFFu) : rl[ss & 0x7Fu];
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        uint32_t sl[8], all = 0x80u;
+        uint32_t bin[8], sl[8];
+        qbins<1>(v, r, bin);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            sl[j] = sm_slot[qbin(__fmul_rn((j & 1) ? bf16_hi(w[j >> 1]) : bf16_lo(w[j >> 1]), r))];
-            all &= sl[j];
-        }
+        for (int j = 0; j < 8; ++j) sl[j] = sm_slot[bin[j]];
+        const uint32_t all = 0x80u & (sl[0] & sl[1] & sl[2]) & (sl[3] & sl[4] & sl[5]) & (sl[6] & sl[7]);
         if (all) return;
         const uint32_t lo = __byte_perm(__byte_perm(sl[0], sl[1], 0x0040), __byte_perm(sl[2], sl[3], 0x0040), 0x5410);
         const uint32_t hi = __byte_perm(__byte_perm(sl[4], sl[5], 0x0040), __byte_perm(sl[6], sl[7], 0x0040), 0x5410);
@@ -272,10 +271,13 @@ quantile_plan_kernel(Ctrl* ctrl, const uint32_t* __restrict__ hist, uint8_t* __r
     }
     __syncthreads();
     if (tid < kQReq) {
-        // a slot per distinct bin, in order of first appearance among the requests
+        // a slot per distinct bin, in order of first appearance among the requests (no early exit: the reads
+        // are then independent of one another)
         int first = tid;
-        for (int q = 0; q < tid; ++q)
-            if (req_bin[q] == req_bin[tid]) { first = q; break; }
+        const int mine = req_bin[tid];
+#pragma unroll 16
+        for (int q = kQReq - 1; q >= 0; --q)
+            if (req_bin[q] == mine) first = min(first, q);
         req_first[tid] = first;
     }
     __syncthreads();
@@ -288,11 +290,13 @@ quantile_plan_kernel(Ctrl* ctrl, const uint32_t* __restrict__ hist, uint8_t* __r
         uint32_t slot = 0, ns = 0;
         unsigned long long off = 0, tot = 0;
         const int first = req_first[tid];
+#pragma unroll 16
         for (int q = 0; q < kQReq; ++q) {
-            if (req_first[q] != q) continue;
-            if (q < first) { ++slot; off += req_cnt[q]; }
-            ++ns;
-            tot += req_cnt[q];
+            const bool lead = req_first[q] == q;
+            const unsigned long long c = lead ? req_cnt[q] : 0ull;
+            if (lead) ++ns;
+            tot += c;
+            if (q < first) { slot += lead; off += c; }
         }
         if (tid == 0) all_fit = tot <= qcap;
         if (tot <= qcap) {

@@ -89,12 +89,64 @@ __device__ __forceinline__ uint32_t e4m3_encode(float x) {
     return u > 0x7Eu ? 0x7Eu : u;
 }
 
-// bin = floor(1024 x + 8192): one multiply-add rounded down onto 1.5 * 2^23 (where floats are
-// spaced by 1) leaves the integer in the low mantissa bits; the mask keeps any input inside the
-// table (|w~| < 8 by the scale rules, so for finite weights it changes nothing)
-__device__ __forceinline__ int qbin(float x) {
-    return (int)(__float_as_uint(__fmaf_rd(x, 1024.f, 8192.f + 12582912.f)) & (uint32_t)(kQBins - 1));
+// Packed pairs of FP32 values in one 64-bit register and the two-wide FP32 instructions of
+// sm_100 on them (each half is rounded exactly like the scalar instruction).
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
 }
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float lo2(uint64_t v) { float lo, hi; unpack2(v, lo, hi); return lo; }
+__device__ __forceinline__ float hi2(uint64_t v) { float lo, hi; unpack2(v, lo, hi); return hi; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2_rd(uint64_t a, uint64_t b, uint64_t c) {      // rounded down
+    uint64_t r;
+    asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// The bins floor(1024 w~ + 8192) of the quantile start's histogram for a lane's eight normalised weights
+// w~ = fl32(w r), times UNIT (1, or 4 for byte offsets of counters): one multiply-add rounded down onto
+// 1.5 * 2^23 (where floats are spaced by 1) leaves the integer in the low mantissa bits, and the mask keeps
+// any input inside the table (|w~| < 8 by the scale rules, so for finite weights it changes nothing but the
+// low bits that UNIT = 4 leaves).  Two weights per instruction.
+template <int UNIT>
+__device__ __forceinline__ void qbins(const uint4& v, float r, uint32_t (&bin)[8]) {
+    constexpr float kScale = 1024.f * UNIT, kAdd = 8192.f * UNIT + 12582912.f;
+    constexpr uint32_t kMask = (uint32_t)(kQBins - 1) * UNIT;
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const uint64_t rr = pack2(r, r);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint64_t t = fma2_rd(mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr), pack2(kScale, kScale), pack2(kAdd, kAdd));
+        bin[2 * j] = __float_as_uint(lo2(t)) & kMask;
+        bin[2 * j + 1] = __float_as_uint(hi2(t)) & kMask;
+    }
+}
+
+// fl32(1 / s) of a positive BF16 scale, from fl32(1 / (1 + m / 128)) per mantissa m: a power of two more does
+// not change the rounding (scales are 2^-126 or more).
+__device__ __forceinline__ float bf16_rcp(const float* lut, uint32_t b) {
+    return __fmul_rn(lut[b & 0x7Fu], __uint_as_float((254u - ((b >> 7) & 0xFFu)) << 23));
+}
+__device__ __forceinline__ float bf16_rcp_entry(uint32_t m) { return __frcp_rn(1.f + (float)m * 0.0078125f); }
 
 // Walks the items first, first + stride, first + 2 stride, ... of an N x slabs grid (row-major)
 // without a division per step; row runs past N when the walk is over.

@@ -42,34 +42,6 @@ __device__ __forceinline__ uint64_t lds_table_b64(uint32_t addr) {
     return r;
 }
 
-// Packed pairs of FP32 values in one 64-bit register and the two-wide FP32 instructions of
-// sm_100 on them (each half is rounded exactly like the scalar instruction).
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ float lo2(uint64_t v) { float lo, hi; unpack2(v, lo, hi); return lo; }
-__device__ __forceinline__ float hi2(uint64_t v) { float lo, hi; unpack2(v, lo, hi); return hi; }
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // {x - P, x - Q}: each half one correctly rounded FP32 subtraction, either as two scalar
 // instructions writing a register pair or as one packed instruction on {x, x}
 #ifndef AAAC_SCALAR_SUB

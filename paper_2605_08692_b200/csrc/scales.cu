@@ -27,31 +27,43 @@ __device__ __forceinline__ uint32_t absmax16(uint4 v) {
     return m;
 }
 
+// Layer absmax.  Dense rows are one array of 16-byte pieces (no rows or columns to keep track of), eight in
+// flight per thread; rows with gaps are walked row by row.
+constexpr int kAbsLoads = 8;
+template <bool DENSE>
 __global__ void __launch_bounds__(256)
 absmax_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, Ctrl* ctrl, uint32_t* dev_status) {
     chain_next();
     chain_wait();
     const int lane = threadIdx.x & 31;
-    const int64_t slabs = (K + 255) / 256;
-    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     uint32_t m = 0;
-    // four independent loads in flight per thread
-    SlabWalk it(warp0, nwarps, slabs);
-    while (it.row < N) {
-        uint4 v[4];
+    if (DENSE) {
+        const uint4* __restrict__ src = reinterpret_cast<const uint4*>(W);
+        const int64_t n = N * (K / 8), step = (int64_t)gridDim.x * 256;
+        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += step * kAbsLoads) {
+            uint4 v[kAbsLoads];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            v[u] = make_uint4(0, 0, 0, 0);
-            const int64_t col = (int64_t)it.slab * 256 + lane * 8;
-            if (it.row < N && col < K) v[u] = __ldg(reinterpret_cast<const uint4*>(W + (int64_t)it.row * ldw + col));
-            it.next();
+            for (int u = 0; u < kAbsLoads; ++u) v[u] = __ldg(src + min(i + u * step, n - 1));
+#pragma unroll
+            for (int u = 0; u < kAbsLoads; ++u) m = max(m, absmax16(v[u]));
         }
+    } else {
+        const int64_t slabs = (K + 255) / 256;
+        SlabWalk it(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((int64_t)gridDim.x * blockDim.x) >> 5, slabs);
+        while (it.row < N) {
+            uint4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) m = max(m, absmax16(v[u]));
+            for (int u = 0; u < 4; ++u) {
+                v[u] = make_uint4(0, 0, 0, 0);
+                const int64_t col = (int64_t)it.slab * 256 + lane * 8;
+                if (it.row < N && col < K) v[u] = __ldg(reinterpret_cast<const uint4*>(W + (int64_t)it.row * ldw + col));
+                it.next();
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) m = max(m, absmax16(v[u]));
+        }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
     if (lane == 0 && m) {
         atomicMax(&ctrl->absmax_bits, m << 16);
         if (m >= 0x7F80u) {
@@ -59,6 +71,29 @@ absmax_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
             if (dev_status) atomicOr(dev_status, AAAC_DEV_NONFINITE);
         }
     }
+}
+
+// The two scale rules, with the division replaced by a multiplication by the reciprocal wherever that cannot
+// change the result: the product is within three units in the last place of the quotient, so the rounding
+// that follows (to BF16, to E4M3) gives the same unless the product lies that close to a half-way point.
+// Those few, and small quotients, take the division (it cost four instructions per weight of the pass).
+__device__ __forceinline__ uint32_t int4_scale_bits(float a) {
+    if (a == 0.f) return 0x3F80u;
+    float y = __fmul_rn(a, 1.f / 7.f);
+    if ((((__float_as_uint(y) + 0x8004u) & 0xFFFFu) <= 8u) || !(y >= 0x1p-100f)) y = __fdiv_rn(a, 7.f);
+    float s = __uint_as_float(f32_to_bf16_rne(y) << 16);
+    if (s < 0x1p-126f) s = 0x1p-126f;
+    return __float_as_uint(s) >> 16;
+}
+__device__ __forceinline__ uint32_t nvfp4_scale_code(float a, float d6, float inv6) {
+    const float y = __fmul_rn(a, inv6);
+    const uint32_t u = __float_as_uint(y);
+    if (y >= 0.0157f && y < 447.f && ((u + 0x80004u) & 0xFFFFFu) > 8u)            // normal codes: 3 mantissa bits
+        return ((u + 0x7FFFFu + ((u >> 20) & 1u)) >> 20) - 960u;
+    const float x = __fdiv_rn(a, d6);
+    uint32_t q = e4m3_encode(x);
+    if (q <= 1u) q = (x > 1.25f * 0x1p-9f) ? 2u : 1u;
+    return q;
 }
 
 template <int MODE>
@@ -74,12 +109,13 @@ scales_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
 
-    float s_t = 1.f, d6 = 6.f;
+    float s_t = 1.f, d6 = 6.f, inv6 = 1.f;
     if (MODE == AAAC_NVFP4) {
         const float A = __uint_as_float(ctrl->absmax_bits);
         s_t = (A == 0.f) ? 1.f : __fdiv_rn(A, 2688.f);
         if (s_t < 0x1p-96f) s_t = 0x1p-96f;
         d6 = __fmul_rn(6.f, s_t);
+        inv6 = __frcp_rn(d6);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctrl->s_t = s_t;
@@ -111,18 +147,11 @@ scales_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
             bad |= (m >= 0x7F80u);
             const int64_t gi = row * Gr + col / G;
             if (MODE == AAAC_INT4) {
-                float s = 1.f;
-                if (a != 0.f) {
-                    s = __uint_as_float(f32_to_bf16_rne(__fdiv_rn(a, 7.f)) << 16);
-                    if (s < 0x1p-126f) s = 0x1p-126f;
-                }
-                reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)(__float_as_uint(s) >> 16);
-                rinv[gi] = __frcp_rn(s);
+                const uint32_t b = int4_scale_bits(a);
+                reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)b;
+                rinv[gi] = __frcp_rn(__uint_as_float(b << 16));
             } else {
-                const float x = __fdiv_rn(a, d6);
-                uint32_t q = e4m3_encode(x);
-                if (q <= 1u) q = (x > 1.25f * 0x1p-9f) ? 2u : 1u;
-                reinterpret_cast<uint8_t*>(scales)[gi] = (uint8_t)q;
+                reinterpret_cast<uint8_t*>(scales)[gi] = (uint8_t)nvfp4_scale_code(a, d6, inv6);
             }
         }
       }
@@ -157,19 +186,21 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
 
-    float s_t = 1.f, d6 = 6.f;
+    float s_t = 1.f, d6 = 6.f, inv6 = 1.f;
     if (MODE == AAAC_NVFP4) {
         const float A = __uint_as_float(ctrl->absmax_bits);
         s_t = (A == 0.f) ? 1.f : __fdiv_rn(A, 2688.f);
         if (s_t < 0x1p-96f) s_t = 0x1p-96f;
         d6 = __fmul_rn(6.f, s_t);
+        inv6 = __frcp_rn(d6);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctrl->s_t = s_t;
         if (tensor_scale) tensor_scale[0] = s_t;
     }
-    __shared__ float rl[128];                          // NVFP4: fl32(1 / (E4M3 value * s_t)) per scale code, as the later passes form it
-    if (MODE == AAAC_NVFP4 && threadIdx.x < 128) rl[threadIdx.x] = __frcp_rn(__fmul_rn(e4m3_value(threadIdx.x), s_t));
+    __shared__ float rl[128];                          // fl32(1 / s) per E4M3 code, or per mantissa of a BF16 scale (bf16_rcp)
+    if (threadIdx.x < 128)
+        rl[threadIdx.x] = MODE == AAAC_NVFP4 ? __frcp_rn(__fmul_rn(e4m3_value(threadIdx.x), s_t)) : bf16_rcp_entry(threadIdx.x);
     __syncthreads();
     bool bad = false;
     SlabWalk it(warp0, nwarps, slabs);
@@ -197,27 +228,21 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
         const int64_t gi = row * Gr + col / G;
         float r;                                       // fl32(1 / s), as the later passes form it
         if (MODE == AAAC_INT4) {
-            float s = 1.f;
-            if (a != 0.f) {
-                s = __uint_as_float(f32_to_bf16_rne(__fdiv_rn(a, 7.f)) << 16);
-                if (s < 0x1p-126f) s = 0x1p-126f;
-            }
-            r = __frcp_rn(s);
+            const uint32_t b = int4_scale_bits(a);
+            r = bf16_rcp(rl, b);
             if ((lane % LPG) == 0) {
-                reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)(__float_as_uint(s) >> 16);
+                reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)b;
                 rinv[gi] = r;
             }
         } else {
-            const float x = __fdiv_rn(a, d6);
-            uint32_t q = e4m3_encode(x);
-            if (q <= 1u) q = (x > 1.25f * 0x1p-9f) ? 2u : 1u;
+            const uint32_t q = nvfp4_scale_code(a, d6, inv6);
             r = rl[q];
             if ((lane % LPG) == 0) reinterpret_cast<uint8_t*>(scales)[gi] = (uint8_t)q;
         }
-        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+        uint32_t off[8];
+        qbins<4>(v[u], r, off);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            atomicAdd(&sm[qbin(__fmul_rn((j & 1) ? bf16_hi(w[j >> 1]) : bf16_lo(w[j >> 1]), r))], 1u);
+        for (int j = 0; j < 8; ++j) atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(sm) + off[j]), 1u);
       }
     }
     if (bad) {
@@ -237,7 +262,7 @@ cudaError_t launch_scales(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, 
     cudaError_t e = cudaSuccess;
     if (mode == AAAC_NVFP4) {
         note_launch();
-        if ((e = launch_chained(absmax_kernel, blocks, 256, 0, st, W, N, K, ldw, ws.ctrl, dev_status)) != cudaSuccess) return e;
+        if ((e = launch_chained(ldw == K ? absmax_kernel<true> : absmax_kernel<false>, blocks, 256, 0, st, W, N, K, ldw, ws.ctrl, dev_status)) != cudaSuccess) return e;
     }
     note_launch();
     float* const rinv = mode == AAAC_NVFP4 ? nullptr : ws.rinv;
