@@ -37,9 +37,9 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 constexpr int kStageCap = 4096;                  // staged candidates per block
 constexpr int kStageEvery = 4;                   // loop iterations between two looks at the stage's fill
 
-template <int MODE>
+template <int MODE, bool DENSE>
 __global__ void __launch_bounds__(256)
-quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
+quantile_collect_kernel(const uint16_t* __restrict__ W, unsigned n_pieces, unsigned per_row, int64_t ldw,
                         const void* __restrict__ scales, Ctrl* ctrl, const uint8_t* __restrict__ slot_of_bin,
                         uint32_t* __restrict__ list) {
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
@@ -65,10 +65,9 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
     }
     __syncthreads();
     const uint8_t* sm_slot = reinterpret_cast<const uint8_t*>(sm);
-    const int64_t slabs = (K + 255) / 256, items = N * slabs, Gr = K / G;
-    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + tid) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t iters = (items + 2 * nwarps - 1) / (2 * nwarps);     // two items per warp and iteration
+    constexpr int LPG = G / 8;                            // lanes per scale group
+    const unsigned step = gridDim.x * blockDim.x;
+    const unsigned iters = (n_pieces + 2 * step - 1) / (2 * step);     // two pieces per thread and iteration
 
     auto flush = [&]() {                                  // called by the whole block, after a barrier
         const uint32_t n = min(nbuf, (uint32_t)kStageCap);
@@ -85,20 +84,16 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
         __syncthreads();
     };
 
-    SlabWalk it(warp0, nwarps, slabs);
-    // (the scale travels as its stored bits: nothing waits for the load before the row is worked on)
+    unsigned next = blockIdx.x * blockDim.x + tid;
+    // (the scale travels as its stored bits: nothing waits for the load before the piece is worked on)
     auto fetch = [&](uint4& vv, uint32_t& ss, bool& okk) {
-        const int64_t row = it.row, col = (int64_t)it.slab * 256 + lane * 8;
-        okk = row < N && col < K;
-        vv = make_uint4(0, 0, 0, 0);
-        ss = 0u;
+        okk = next < n_pieces;
         if (okk) {
-            vv = __ldg(reinterpret_cast<const uint4*>(W + row * ldw + col));
-            const int64_t gi = row * Gr + col / G;
-            if (MODE == AAAC_INT4) ss = reinterpret_cast<const uint16_t*>(scales)[gi];
-            else ss = reinterpret_cast<const uint8_t*>(scales)[gi];
+            vv = load_piece<DENSE>(W, next, per_row, ldw);
+            if (MODE == AAAC_INT4) ss = __ldg(reinterpret_cast<const uint16_t*>(scales) + next / LPG);
+            else ss = __ldg(reinterpret_cast<const uint8_t*>(scales) + next / LPG);
         }
-        it.next();
+        next += step;
     };
     // The slots of a lane's eight weights first.  A slot byte has bit 7 set where the bin is not asked
     // for, so the AND of the eight bytes tells whether the lane holds a candidate; a lane that does
@@ -144,17 +139,17 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, in
         }
     };
 
-    // Two items per warp are in flight: the loads of iteration k + 1 are issued before iteration k
+    // Two pieces per thread are in flight: the loads of iteration k + 1 are issued before iteration k
     // is processed.  The warps of a block meet only every kStageEvery iterations, to empty the
     // stage once it is half full (the vote makes the decision the same for every thread).
-    uint4 va, vb;
-    uint32_t ra, rb;
+    uint4 va{}, vb{};
+    uint32_t ra = 0, rb = 0;
     bool oka, okb;
     fetch(va, ra, oka);
     fetch(vb, rb, okb);
-    for (int64_t k = 0; k < iters; ++k) {
-        uint4 vna, vnb;
-        uint32_t rna, rnb;
+    for (unsigned k = 0; k < iters; ++k) {
+        uint4 vna{}, vnb{};
+        uint32_t rna = 0, rnb = 0;
         bool okna, oknb;
         fetch(vna, rna, okna);
         fetch(vnb, rnb, oknb);
@@ -578,8 +573,11 @@ cudaError_t launch_init(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, in
     cudaError_t e = launch_chained(quantile_plan_kernel, 1, 1024, 0, st, ws.ctrl, ws.qhist, ws.qslot_of_bin, (unsigned long long)ws.qcap, rq);
     note_launch();
     if (e != cudaSuccess) return e;
-    auto collect = mode == AAAC_INT4 ? quantile_collect_kernel<AAAC_INT4> : quantile_collect_kernel<AAAC_NVFP4>;
-    e = launch_chained(collect, sm_count() * 4, 256, kQBins, st, W, N, K, ldw, scales, ws.ctrl, ws.qslot_of_bin, ws.qlist);
+    const bool dense = ldw == K;
+    auto collect = mode == AAAC_INT4 ? (dense ? quantile_collect_kernel<AAAC_INT4, true> : quantile_collect_kernel<AAAC_INT4, false>)
+                                     : (dense ? quantile_collect_kernel<AAAC_NVFP4, true> : quantile_collect_kernel<AAAC_NVFP4, false>);
+    e = launch_chained(collect, sm_count() * 4, 256, kQBins, st, W, (unsigned)(N * (K / 8)), (unsigned)(K / 8), ldw, scales, ws.ctrl,
+                       ws.qslot_of_bin, ws.qlist);
     note_launch();
     if (e != cudaSuccess) return e;
     note_launch();

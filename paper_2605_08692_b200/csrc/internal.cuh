@@ -148,19 +148,15 @@ __device__ __forceinline__ float bf16_rcp(const float* lut, uint32_t b) {
 }
 __device__ __forceinline__ float bf16_rcp_entry(uint32_t m) { return __frcp_rn(1.f + (float)m * 0.0078125f); }
 
-// Walks the items first, first + stride, first + 2 stride, ... of an N x slabs grid (row-major)
-// without a division per step; row runs past N when the walk is over.
-struct SlabWalk {
-    int row, slab, drow, dslab, slabs;
-    __device__ SlabWalk(int64_t first, int64_t stride, int64_t slabs_)
-        : row((int)(first / slabs_)), slab((int)(first % slabs_)), drow((int)(stride / slabs_)),
-          dslab((int)(stride % slabs_)), slabs((int)slabs_) {}
-    __device__ void next() {
-        row += drow;
-        slab += dslab;
-        if (slab >= slabs) { slab -= slabs; ++row; }
-    }
-};
+// The passes before the fit take a layer as a list of 16-byte pieces (8 weights), piece i of a row-major
+// layer in group i / (g / 8): without gaps between the rows (DENSE) neither rows nor columns need to be
+// known, which is half of such a pass's instructions; with gaps the row is found by a division.
+template <bool DENSE>
+__device__ __forceinline__ uint4 load_piece(const uint16_t* __restrict__ W, unsigned i, unsigned per_row, int64_t ldw) {
+    if (DENSE) return __ldg(reinterpret_cast<const uint4*>(W) + i);
+    const unsigned row = i / per_row;
+    return __ldg(reinterpret_cast<const uint4*>(W + row * ldw + (i - row * per_row) * 8u));
+}
 
 // largest float <= d
 __device__ __forceinline__ float f32_round_down(double d) { return __double2float_rd(d); }

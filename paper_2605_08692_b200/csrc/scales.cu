@@ -7,7 +7,7 @@
 //                    subnormal step the code is raised so that |w / s| <= 7.5.
 // Both rules keep every normalised weight strictly inside (-8, 8).
 //
-// One warp handles 256 adjacent columns of one row (one 128-bit load per lane); the group
+// One warp handles 256 adjacent weights (one 128-bit load per lane); the group
 // maximum is a shuffle reduction over the 16 (INT4) or 2 (NVFP4) lanes of the group.
 #include "internal.cuh"
 
@@ -27,41 +27,22 @@ __device__ __forceinline__ uint32_t absmax16(uint4 v) {
     return m;
 }
 
-// Layer absmax.  Dense rows are one array of 16-byte pieces (no rows or columns to keep track of), eight in
-// flight per thread; rows with gaps are walked row by row.
+// Layer absmax, eight pieces in flight per thread.
 constexpr int kAbsLoads = 8;
 template <bool DENSE>
 __global__ void __launch_bounds__(256)
-absmax_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, Ctrl* ctrl, uint32_t* dev_status) {
+absmax_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row, int64_t ldw, Ctrl* ctrl, uint32_t* dev_status) {
     chain_next();
     chain_wait();
     const int lane = threadIdx.x & 31;
+    const unsigned step = gridDim.x * 256u;
     uint32_t m = 0;
-    if (DENSE) {
-        const uint4* __restrict__ src = reinterpret_cast<const uint4*>(W);
-        const int64_t n = N * (K / 8), step = (int64_t)gridDim.x * 256;
-        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += step * kAbsLoads) {
-            uint4 v[kAbsLoads];
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n; i += step * kAbsLoads) {
+        uint4 v[kAbsLoads];
 #pragma unroll
-            for (int u = 0; u < kAbsLoads; ++u) v[u] = __ldg(src + min(i + u * step, n - 1));
+        for (int u = 0; u < kAbsLoads; ++u) v[u] = load_piece<DENSE>(W, min(i + u * step, n - 1u), per_row, ldw);
 #pragma unroll
-            for (int u = 0; u < kAbsLoads; ++u) m = max(m, absmax16(v[u]));
-        }
-    } else {
-        const int64_t slabs = (K + 255) / 256;
-        SlabWalk it(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((int64_t)gridDim.x * blockDim.x) >> 5, slabs);
-        while (it.row < N) {
-            uint4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                v[u] = make_uint4(0, 0, 0, 0);
-                const int64_t col = (int64_t)it.slab * 256 + lane * 8;
-                if (it.row < N && col < K) v[u] = __ldg(reinterpret_cast<const uint4*>(W + (int64_t)it.row * ldw + col));
-                it.next();
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) m = max(m, absmax16(v[u]));
-        }
+        for (int u = 0; u < kAbsLoads; ++u) m = max(m, absmax16(v[u]));
     }
     m = __reduce_max_sync(0xFFFFFFFFu, m);
     if (lane == 0 && m) {
@@ -96,18 +77,16 @@ __device__ __forceinline__ uint32_t nvfp4_scale_code(float a, float d6, float in
     return q;
 }
 
-template <int MODE>
+template <int MODE, bool DENSE>
 __global__ void __launch_bounds__(256)
-scales_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, void* __restrict__ scales,
+scales_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row, int64_t ldw, void* __restrict__ scales,
               float* __restrict__ rinv, float* __restrict__ tensor_scale, Ctrl* ctrl, uint32_t* dev_status) {
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
     constexpr int LPG = G / 8;                         // lanes per group
     chain_next();
     chain_wait();
     const int lane = threadIdx.x & 31;
-    const int64_t slabs = (K + 255) / 256, Gr = K / G;
-    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const unsigned step = gridDim.x * blockDim.x;
 
     float s_t = 1.f, d6 = 6.f, inv6 = 1.f;
     if (MODE == AAAC_NVFP4) {
@@ -122,39 +101,34 @@ scales_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
         if (tensor_scale) tensor_scale[0] = s_t;
     }
     bool bad = false;
-    SlabWalk it(warp0, nwarps, slabs);
-    while (it.row < N) {
-      // four independent loads in flight per thread (the row of an item is the same in every lane)
-      uint4 v[4];
-      int rows[4], cols[4];
+    // four pieces in flight per thread; whole warps go round the loop (a group is 2 or 16 lanes, and n a
+    // multiple of that)
+    for (unsigned i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += 4 * step) {
+        uint4 v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-          v[u] = make_uint4(0, 0, 0, 0);
-          rows[u] = it.row;
-          cols[u] = it.slab * 256 + lane * 8;
-          if (it.row < N && cols[u] < K) v[u] = __ldg(reinterpret_cast<const uint4*>(W + (int64_t)it.row * ldw + cols[u]));
-          it.next();
-      }
+        for (int u = 0; u < 4; ++u) {
+            const unsigned i = i0 + u * step + lane;
+            v[u] = i < n ? load_piece<DENSE>(W, i, per_row, ldw) : make_uint4(0, 0, 0, 0);
+        }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (rows[u] >= N) break;                       // uniform over the warp
-        const int64_t row = rows[u], col = cols[u];
-        uint32_t m = absmax16(v[u]);
+        for (int u = 0; u < 4; ++u) {
+            const unsigned i = i0 + u * step + lane;
+            uint32_t m = absmax16(v[u]);
 #pragma unroll
-        for (int o = LPG / 2; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        if (col < K && (lane % LPG) == 0) {
-            const float a = __uint_as_float(m << 16);
-            bad |= (m >= 0x7F80u);
-            const int64_t gi = row * Gr + col / G;
-            if (MODE == AAAC_INT4) {
-                const uint32_t b = int4_scale_bits(a);
-                reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)b;
-                rinv[gi] = __frcp_rn(__uint_as_float(b << 16));
-            } else {
-                reinterpret_cast<uint8_t*>(scales)[gi] = (uint8_t)nvfp4_scale_code(a, d6, inv6);
+            for (int o = LPG / 2; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+            if (i < n && (lane % LPG) == 0) {
+                const float a = __uint_as_float(m << 16);
+                bad |= (m >= 0x7F80u);
+                const unsigned gi = i / LPG;
+                if (MODE == AAAC_INT4) {
+                    const uint32_t b = int4_scale_bits(a);
+                    reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)b;
+                    rinv[gi] = __frcp_rn(__uint_as_float(b << 16));
+                } else {
+                    reinterpret_cast<uint8_t*>(scales)[gi] = (uint8_t)nvfp4_scale_code(a, d6, inv6);
+                }
             }
         }
-      }
     }
     if (bad) {
         atomicOr(&ctrl->nonfinite, 1u);
@@ -170,9 +144,9 @@ scales_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw,
 #ifndef AAAC_SH_BLOCKS
 #define AAAC_SH_BLOCKS 2
 #endif
-template <int MODE>
+template <int MODE, bool DENSE>
 __global__ void __launch_bounds__(512, AAAC_SH_BLOCKS)
-scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, void* __restrict__ scales,
+scales_hist_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row, int64_t ldw, void* __restrict__ scales,
                    float* __restrict__ rinv, float* __restrict__ tensor_scale, Ctrl* ctrl, uint32_t* dev_status,
                    uint32_t* __restrict__ hist) {
     constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
@@ -182,9 +156,7 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
     for (int i = threadIdx.x; i < kQBins; i += blockDim.x) sm[i] = 0;
     chain_wait();
     const int lane = threadIdx.x & 31;
-    const int64_t slabs = (K + 255) / 256, Gr = K / G;
-    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const unsigned step = gridDim.x * blockDim.x;
 
     float s_t = 1.f, d6 = 6.f, inv6 = 1.f;
     if (MODE == AAAC_NVFP4) {
@@ -203,47 +175,40 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
         rl[threadIdx.x] = MODE == AAAC_NVFP4 ? __frcp_rn(__fmul_rn(e4m3_value(threadIdx.x), s_t)) : bf16_rcp_entry(threadIdx.x);
     __syncthreads();
     bool bad = false;
-    SlabWalk it(warp0, nwarps, slabs);
-    while (it.row < N) {
-      uint4 v[4];
-      int rows[4], cols[4];
+    for (unsigned i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += 4 * step) {
+        uint4 v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-          v[u] = make_uint4(0, 0, 0, 0);
-          rows[u] = it.row;
-          cols[u] = it.slab * 256 + lane * 8;
-          if (it.row < N && cols[u] < K) v[u] = __ldg(reinterpret_cast<const uint4*>(W + (int64_t)it.row * ldw + cols[u]));
-          it.next();
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (rows[u] >= N) break;                       // uniform over the warp
-        const int64_t row = rows[u], col = cols[u];
-        uint32_t m = absmax16(v[u]);
-#pragma unroll
-        for (int o = LPG / 2; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        if (col >= K) continue;
-        const float a = __uint_as_float(m << 16);
-        bad |= (m >= 0x7F80u);
-        const int64_t gi = row * Gr + col / G;
-        float r;                                       // fl32(1 / s), as the later passes form it
-        if (MODE == AAAC_INT4) {
-            const uint32_t b = int4_scale_bits(a);
-            r = bf16_rcp(rl, b);
-            if ((lane % LPG) == 0) {
-                reinterpret_cast<uint16_t*>(scales)[gi] = (uint16_t)b;
-                rinv[gi] = r;
-            }
-        } else {
-            const uint32_t q = nvfp4_scale_code(a, d6, inv6);
-            r = rl[q];
-            if ((lane % LPG) == 0) reinterpret_cast<uint8_t*>(scales)[gi] = (uint8_t)q;
+        for (int u = 0; u < 4; ++u) {
+            const unsigned i = i0 + u * step + lane;
+            v[u] = i < n ? load_piece<DENSE>(W, i, per_row, ldw) : make_uint4(0, 0, 0, 0);
         }
-        uint32_t off[8];
-        qbins<4>(v[u], r, off);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(sm) + off[j]), 1u);
-      }
+        for (int u = 0; u < 4; ++u) {
+            const unsigned i = i0 + u * step + lane;
+            uint32_t m = absmax16(v[u]);
+#pragma unroll
+            for (int o = LPG / 2; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+            if (i >= n) continue;
+            const float a = __uint_as_float(m << 16);
+            bad |= (m >= 0x7F80u);
+            float r;                                   // fl32(1 / s), as the later passes form it
+            if (MODE == AAAC_INT4) {
+                const uint32_t b = int4_scale_bits(a);
+                r = bf16_rcp(rl, b);
+                if ((lane % LPG) == 0) {
+                    reinterpret_cast<uint16_t*>(scales)[i / LPG] = (uint16_t)b;
+                    rinv[i / LPG] = r;
+                }
+            } else {
+                const uint32_t q = nvfp4_scale_code(a, d6, inv6);
+                r = rl[q];
+                if ((lane % LPG) == 0) reinterpret_cast<uint8_t*>(scales)[i / LPG] = (uint8_t)q;
+            }
+            uint32_t off[8];
+            qbins<4>(v[u], r, off);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(sm) + off[j]), 1u);
+        }
     }
     if (bad) {
         atomicOr(&ctrl->nonfinite, 1u);
@@ -259,22 +224,26 @@ scales_hist_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t
 cudaError_t launch_scales(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, int mode, void* scales,
                           float* tensor_scale, uint32_t* dev_status, const Workspace& ws, cudaStream_t st, bool with_hist) {
     const int blocks = sm_count() * 8;
+    const bool dense = ldw == K;
+    const unsigned n = (unsigned)(N * (K / 8)), per_row = (unsigned)(K / 8);       // (layers are below 2^32 elements)
     cudaError_t e = cudaSuccess;
     if (mode == AAAC_NVFP4) {
         note_launch();
-        if ((e = launch_chained(ldw == K ? absmax_kernel<true> : absmax_kernel<false>, blocks, 256, 0, st, W, N, K, ldw, ws.ctrl, dev_status)) != cudaSuccess) return e;
+        if ((e = launch_chained(dense ? absmax_kernel<true> : absmax_kernel<false>, blocks, 256, 0, st, W, n, per_row, ldw, ws.ctrl, dev_status)) != cudaSuccess) return e;
     }
     note_launch();
     float* const rinv = mode == AAAC_NVFP4 ? nullptr : ws.rinv;
     if (!with_hist) {
-        auto kern = mode == AAAC_NVFP4 ? scales_kernel<AAAC_NVFP4> : scales_kernel<AAAC_INT4>;
-        return launch_chained(kern, blocks, 256, 0, st, W, N, K, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status);
+        auto kern = mode == AAAC_NVFP4 ? (dense ? scales_kernel<AAAC_NVFP4, true> : scales_kernel<AAAC_NVFP4, false>)
+                                       : (dense ? scales_kernel<AAAC_INT4, true> : scales_kernel<AAAC_INT4, false>);
+        return launch_chained(kern, blocks, 256, 0, st, W, n, per_row, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status);
     }
-    static std::atomic<size_t> ready[2][kMaxDevices];
+    static std::atomic<size_t> ready[4][kMaxDevices];
     const size_t smem = kQBins * sizeof(uint32_t);
-    auto kern = mode == AAAC_NVFP4 ? scales_hist_kernel<AAAC_NVFP4> : scales_hist_kernel<AAAC_INT4>;
-    if ((e = allow_smem(kern, smem, ready[mode == AAAC_NVFP4])) != cudaSuccess) return e;
-    return launch_chained(kern, sm_count() * AAAC_SH_BLOCKS, 512, smem, st, W, N, K, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status, ws.qhist);
+    auto kern = mode == AAAC_NVFP4 ? (dense ? scales_hist_kernel<AAAC_NVFP4, true> : scales_hist_kernel<AAAC_NVFP4, false>)
+                                   : (dense ? scales_hist_kernel<AAAC_INT4, true> : scales_hist_kernel<AAAC_INT4, false>);
+    if ((e = allow_smem(kern, smem, ready[2 * (mode == AAAC_NVFP4) + dense])) != cudaSuccess) return e;
+    return launch_chained(kern, sm_count() * AAAC_SH_BLOCKS, 512, smem, st, W, n, per_row, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status, ws.qhist);
 }
 
 }  // namespace aaac
