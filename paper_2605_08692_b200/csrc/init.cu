@@ -11,7 +11,7 @@
 //      into a slotted bin to that slot's list -- the lists' sizes are known from step 1.  A block
 //      stages its candidates in shared memory and reserves list space once per slot, so the
 //      global counters see one atomic per block and slot instead of one per candidate;
-//   4. one block per slot selects the requested ranks of its list by an 8-bit radix select (the
+//   4. one block per slot selects the requested ranks of its list by an 11-bit radix select (the
 //      list is read once into registers when it is short enough, else streamed per pass);
 //   5. the table entries are interpolated in double and rounded to FP32.
 // Integer atomics only, so the result does not depend on scheduling.
@@ -338,16 +338,17 @@ quantile_plan_kernel(Ctrl* ctrl, const uint32_t* __restrict__ hist, uint8_t* __r
 //  - The first kKeep * 1024 keys of the list are read once and stay in registers for every sweep;
 //    only what is beyond them is streamed from memory, eight loads in flight per thread.
 //  - The keys of a slot lie in one narrow bin, so they share their leading bits: one sweep finds
-//    the bits on which all keys agree, and only the 8-bit digits below them need a radix pass.
-//    Within a pass equal digits within a warp are counted once (match), which keeps the
-//    shared-memory atomics apart.
+//    the bits on which all keys agree, and only the digits of 11 bits below them need a radix pass: two,
+//    mostly (8-bit digits took three, and combining equal digits within a warp before counting cost more
+//    than the counting).
 //  - The two neighbours that one table entry interpolates between are consecutive ranks: the
-//    second is the first's key again, or the smallest larger key -- one sweep instead of a
-//    second selection.
+//    second is the first's key again, or the next larger key, which the last pass's counters name
+//    unless it differs in a higher digit; then one sweep finds it.
 __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restrict__ list) {
-    __shared__ uint32_t hist[256];
-    __shared__ uint32_t sh_prefix, sh_mask;
-    __shared__ unsigned long long sh_k;
+    constexpr int kDigit = 11, kDigits = 1 << kDigit;
+    __shared__ uint32_t hist[kDigits];
+    __shared__ uint32_t wsum[32];
+    __shared__ uint32_t sh_digit, sh_left, sh_in, sh_next;
     __shared__ uint32_t req_slot[kQReq];
     __shared__ unsigned long long req_local[kQReq];
     __shared__ uint32_t sh_or, sh_and, sh_cnt, sh_min;
@@ -411,24 +412,27 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
         if (lane == 0) { atomicOr(&sh_or, o); atomicAnd(&sh_and, a); }
     }
     __syncthreads();
-    int first_shift = 24;
-    uint32_t first_prefix = 0u, first_mask = 0u;
+    int top = 31;                                          // highest bit on which keys of the list differ
+    uint32_t first_mask = 0u, first_prefix = 0u;           // ... and the bits above it, the same in all
     if (n > 0) {
         const uint32_t diff = sh_or ^ sh_and;
-        first_shift = diff ? ((31 - __clz(diff)) >> 3) << 3 : 0;
-        first_mask = first_shift == 24 ? 0u : ~((1u << (first_shift + 8)) - 1u);
+        top = diff ? 31 - __clz(diff) : 0;
+        first_mask = top == 31 ? 0u : ~((2u << top) - 1u);
         first_prefix = sh_and & first_mask;
     }
     bool have_prev = false;                                // rank and key of the request answered last
     unsigned long long prev_k = 0;
-    uint32_t prev_key = 0u;
+    uint32_t prev_key = 0u, prev_next = 0u;                // the next larger key, if the counters named it (else 0)
+    bool prev_last = false;                                // no further key equal to it comes after that rank
     for (int q = 0; q < kQReq; ++q) {
         if (req_slot[q] != slot) continue;                 // uniform across the block
         if (have_prev && (req_local[q] == prev_k || req_local[q] == prev_k + 1)) {
             // the same or the next order statistic: it equals the previous key unless every key
             // up to that one is already counted, in which case it is the smallest larger key
             uint32_t key = prev_key;
-            if (req_local[q] == prev_k + 1) {
+            if (req_local[q] == prev_k + 1 && prev_last && prev_next) {
+                key = prev_next;
+            } else if (req_local[q] == prev_k + 1 && prev_last) {
                 if (threadIdx.x == 0) { sh_cnt = 0u; sh_min = 0xFFFFFFFFu; }
                 __syncthreads();
                 uint32_t c = 0u, m = 0xFFFFFFFFu;
@@ -446,62 +450,62 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
                 __syncthreads();
             }
             if (threadIdx.x == 0) ctrl->rank_val[q] = key_float(key);
-            prev_k = req_local[q];
-            prev_key = key;
+            // (at most two consecutive ranks belong together; a third is selected anew)
+            have_prev = req_local[q] == prev_k;
             continue;
         }
-        if (threadIdx.x == 0) { sh_prefix = first_prefix; sh_mask = first_mask; sh_k = req_local[q]; }
-        __syncthreads();
-        for (int shift = first_shift; shift >= 0; shift -= 8) {
-            if (threadIdx.x < 256) hist[threadIdx.x] = 0;
+        uint32_t prefix = first_prefix, mask = first_mask;
+        uint32_t k_left = (uint32_t)min(req_local[q], (unsigned long long)0xFFFFFFFFu);     // rank among the keys with this prefix
+        for (int hi = top; hi >= 0;) {
+            const int shift = hi >= kDigit ? hi - (kDigit - 1) : 0;
+            const uint32_t width = (2u << (hi - shift)) - 1u;
+            for (int i = threadIdx.x; i < kDigits; i += blockDim.x) hist[i] = 0;
+            if (threadIdx.x == 0) { sh_digit = width; sh_left = 0u; sh_in = 1u; sh_next = 0xFFFFFFFFu; }   // (ranks beyond the list are never requested)
             __syncthreads();
-            const uint32_t prefix = sh_prefix, mask = sh_mask;
             for_each_key([&](uint32_t k, bool valid) {
-                const bool sel = valid && (k & mask) == prefix;
-                const unsigned act = __ballot_sync(0xFFFFFFFFu, sel);
-                if (sel) {
-                    const uint32_t d = (k >> shift) & 0xFFu;
-                    const unsigned peers = __match_any_sync(act, d);
-                    if (lane == __ffs(peers) - 1) atomicAdd(&hist[d], (uint32_t)__popc(peers));
-                }
+                if (valid && (k & mask) == prefix) atomicAdd(&hist[(k >> shift) & width], 1u);
             });
             __syncthreads();
-            if (threadIdx.x < 32) {
-                // digit that holds rank k: lane l owns digits 8 l .. 8 l + 7
-                uint32_t c[8], tot = 0;
+            // the digit that holds the rank: thread t owns digits 2 t and 2 t + 1
+            const uint32_t c0 = hist[2 * threadIdx.x], c1 = hist[2 * threadIdx.x + 1], tot = c0 + c1;
+            uint32_t incl = tot;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) { c[i] = hist[lane * 8 + i]; tot += c[i]; }
-                uint32_t incl = tot;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                    if (lane >= o) incl += t;
-                }
-                const unsigned long long k = sh_k;
-                const unsigned long long before = incl - tot;
-                const bool mine = k >= before && k < (unsigned long long)incl;
-                const unsigned who = __ballot_sync(0xFFFFFFFFu, mine);
-                // ranks beyond the list (never requested) fall to the last digit
-                const int owner = who ? __ffs(who) - 1 : 31;
-                if (lane == owner) {
-                    unsigned long long r = k - before;
-                    int i = 0;
-                    for (; i < 7; ++i) {
-                        if (r < c[i]) break;
-                        r -= c[i];
-                    }
-                    sh_k = r;
-                    sh_prefix = prefix | ((uint32_t)(lane * 8 + i) << shift);
-                    sh_mask = mask | (0xFFu << shift);
-                }
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane == 31) wsum[threadIdx.x >> 5] = incl;
+            __syncthreads();
+            uint32_t before = lane < (int)(threadIdx.x >> 5) ? wsum[lane] : 0u;
+            before = __reduce_add_sync(0xFFFFFFFFu, before) + incl - tot;
+            if (k_left >= before && k_left < before + tot) {
+                const bool second = k_left - before >= c0;
+                sh_digit = 2 * threadIdx.x + second;
+                sh_left = k_left - before - (second ? c0 : 0u);
+                sh_in = second ? c1 : c0;
             }
             __syncthreads();
+            const uint32_t digit = sh_digit;
+            if (shift == 0) {
+                // the next larger digit in use names the next larger key
+                const uint32_t d0 = 2 * threadIdx.x;
+                const uint32_t nx = d0 > digit && c0 ? d0 : d0 + 1 > digit && c1 ? d0 + 1 : 0xFFFFFFFFu;
+                const uint32_t wnx = __reduce_min_sync(0xFFFFFFFFu, nx);
+                if (lane == 0 && wnx != 0xFFFFFFFFu) atomicMin(&sh_next, wnx);
+                __syncthreads();
+                prev_last = sh_left + 1 >= sh_in;
+                prev_next = sh_next == 0xFFFFFFFFu ? 0u : prefix | sh_next;
+            }
+            k_left = sh_left;
+            prefix |= digit << shift;
+            mask |= width << shift;
+            hi = shift - 1;
+            __syncthreads();                               // (sh_* and hist are written again)
         }
-        if (threadIdx.x == 0) ctrl->rank_val[q] = key_float(sh_prefix);
+        if (threadIdx.x == 0) ctrl->rank_val[q] = key_float(prefix);
         have_prev = true;
         prev_k = req_local[q];
-        prev_key = sh_prefix;
-        __syncthreads();
+        prev_key = prefix;
     }
 }
 
