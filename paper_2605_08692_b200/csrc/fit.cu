@@ -31,14 +31,18 @@
 //     fl32(s x + NB / 2 + 1.5 * 2^(23-k)) holds (s x + NB / 2) * 2^k rounded to an integer; masked,
 //     it is the byte offset bin * 2^k of the bin's table entry (2^k = bytes per bin over all
 //     copies), bin = floor of s x + NB / 2 after rounding to a multiple of 2^-k.
-//     A table gives per bin {J_low, thr}: J_low breakpoints lie
-//     below the bin, thr is the one breakpoint inside it (+inf if none), J = J_low + (x > thr).
-//     Breakpoints are the rounded-down FP32 midpoints, for which x > thr <=> x > midpoint, so J
-//     is exact.  A bin that holds two or more breakpoints points at a poisoned slot (J = 31)
+//     A table gives per bin either {P, Q} of (b) itself, where no breakpoint lies in the bin (four
+//     fifths of the weights), or {thr, address}: thr is the one breakpoint inside, and the address
+//     names {P, Q} of the interval below it, the row after it that of the interval above.  Only the
+//     lanes with such a bin look up a second time, and a shared-memory load of a few lanes costs one
+//     cycle where a full 8-byte one costs two (9.8 -> 8.9 wavefronts per 32 weights; the shared-memory
+//     pipe was 93 % busy during a pass).
+//     Breakpoints are the rounded-down FP32 midpoints, for which x > thr <=> x > midpoint, so the
+//     interval is exact.  A bin that holds two or more breakpoints names a poisoned row (J = 31)
 //     whose entries are NaN: the group falls through to the exact path below, which searches J
 //     directly.  (Fitted tables keep their merged breakpoints apart -- the two codebooks
 //     specialise -- so such bins are rare outside degenerate starts.)
-// (b) Selection.  A second table gives {P, Q}: the FP32 roundings of the nearest entries of T0
+// (b) Selection.  {P, Q} are the FP32 roundings of the nearest entries of T0
 //     and T1 on interval J, moved by at most 8 units in the last place so that the low 4 mantissa
 //     bits equal the entry's index (so the
 //     same 8 bytes also say which cell the weight falls into).  u_r = x - T_r,
@@ -50,8 +54,8 @@
 //     |E0 - E1| <= 2^-24 (16 (E0 + E1) + 2.83 * 17 max|T| sqrt(sum I (E0 + E1))) (and NaN) are
 //     re-evaluated in double with the exact entries, so sigma is the double-precision decision
 //     (the kernel tests against the slightly larger bound that sqrt(a b) <= a / 16 + 4 b gives,
-//     which needs one multiply-add per group).  The two errors are carried as one packed
-//     FP32 pair per weight (sub / mul / fma.f32x2).
+//     which needs one multiply-add per group).  The errors are summed by pairs of columns
+//     (mul / fma.f32x2).
 // (c) Centroid sums, centred.  Lane-private shared-memory bins [sigma][entry] hold
 //     (sum I (x - c), sum I) with c the constant of (b) for the entry the weight is assigned to,
 //     so the new entry is c + sum I (x - c) / sum I.  The residual sums are small and of mixed
@@ -63,9 +67,7 @@
 //
 // Tables in shared memory are replicated against bank conflicts: the per-bin table and the
 // {P, Q} table 16 times (lane l uses copy l mod 16, so the 16 lanes that share a wavefront of an
-// 8-byte load never collide; a bin's entry holds the address of its lower interval's {P, Q} entry
-// in the same copy, and a weight above the bin's breakpoint adds the distance to the next
-// interval's entry), the bins once per lane.
+// 8-byte load never collide; an address in a bin's entry names the same copy), the bins once per lane.
 //
 // Thread mapping.  A block of 16 warps works on items of 64 rows (32 or 16 in layers that have too
 // few items for the blocks) x 256 columns, dealt to
@@ -327,30 +329,27 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     uint32_t sgw[R];          // inner iteration: the row's stored selection bits
     constexpr bool INNER = KIND == kInner;
     constexpr bool keep_sigma = KIND == kAssignKeep;
-#pragma unroll
-    for (int u = 0; u < R; ++u) { v[u] = make_uint4(0, 0, 0, 0); sc[u] = 0u; sgw[u] = 0u; }
     // Offsets of the item being loaded (element offsets fit 32 bits: the entry points refuse layers of 2^32
-    // elements and more) and how many of its rows this lane may read.
+    // elements and more).  Nothing guards the loads: rows past the item's last read that one again, lanes past
+    // K the row's last columns (their importances are zero).
     unsigned nwo = 0u, ngo = 0u, nso = 0u;
-    int nlim = 0;
+    int nlast = 0;
     auto aim = [&](int slab, int rb) {
-        const int col0 = slab * 256 + lane * 8, row = (rb * NW + warp) * rows;
-        nwo = (unsigned)row * (unsigned)p.ldw + (unsigned)col0;
-        ngo = (unsigned)row * (unsigned)Gr + (unsigned)col0 / G;
+        const int row = min((rb * NW + warp) * rows, N - 1);
+        const unsigned col = (unsigned)min(slab * 256 + lane * 8, K - 8);
+        nwo = (unsigned)row * (unsigned)p.ldw + col;
+        ngo = (unsigned)row * (unsigned)Gr + col / G;
         if (INNER) nso = (unsigned)row * (unsigned)slabs + (unsigned)slab;
-        nlim = col0 < K ? min(N - row, rows) : 0;
+        nlast = min(N - row, rows) - 1;
     };
+    // (volatile: the compiler would move these loads down to where the row is worked on, to save registers)
     auto load_row = [&](int u) {
-        v[u] = make_uint4(0, 0, 0, 0);
-        sc[u] = 0u;
-        if (INNER) sgw[u] = 0u;
-        if (u < nlim) {
-            v[u] = __ldcs(reinterpret_cast<const uint4*>(p.W + (nwo + (unsigned)u * (unsigned)p.ldw)));
-            const unsigned gi = ngo + (unsigned)u * (unsigned)Gr;
-            if (MODE == AAAC_NVFP4) sc[u] = p.scales[gi];          // masked at use: nothing waits on the load here
-            else sc[u] = __float_as_uint(__ldg(p.rinv + gi));
-            if (INNER) sgw[u] = __ldcg(p.sigw + (nso + (unsigned)u * (unsigned)slabs));
-        }
+        const unsigned m = (unsigned)min(u, nlast);
+        asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[u].x), "=r"(v[u].y), "=r"(v[u].z), "=r"(v[u].w)
+                     : "l"(p.W + (nwo + m * (unsigned)p.ldw)));
+        if (MODE == AAAC_NVFP4) asm volatile("ld.global.u8 %0, [%1];" : "=r"(sc[u]) : "l"(p.scales + (ngo + m * (unsigned)Gr)));   // masked at use
+        else asm volatile("ld.global.u32 %0, [%1];" : "=r"(sc[u]) : "l"(p.rinv + (ngo + m * (unsigned)Gr)));
+        if (INNER) asm volatile("ld.global.u32 %0, [%1];" : "=r"(sgw[u]) : "l"(p.sigw + (nso + m * (unsigned)slabs)));
     };
     int cur_slab = -1;
     uint64_t II[4];           // importances of the lane's eight columns, in pairs
@@ -478,8 +477,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         //   M(u):  errors, sigma, the centred terms and bin addresses;   B(u): bins += terms.
         float eitem = 0.f;                                 // objective of this item's groups led by this lane
         float x[8];                                        // w~ of the row in L1..M
-        uint2 e1v[8];                                      // {address of the lower interval's {P, Q} entry, thr}
-        uint64_t pq[8];                                    // {P, Q}, packed
+        uint64_t pq[8];                                    // the bins' entries, then {P, Q}
         float mt[2][8];                                    // chosen centred term I (x - c) of the rows in B / M
         uint32_t ba[2][8];                                 // its bin address
         bool sg_row = false;                               // inner iteration: this lane's stored selection bit
@@ -494,8 +492,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 const uint64_t bb = fma2(xx, pack2(kBinsPerUnit, kBinsPerUnit), pack2(kMagic, kMagic));
                 unpack2(xx, x[2 * j], x[2 * j + 1]);
                 // (bin bits | lane's copy | table base) is one three-input logic instruction: no add per weight
-                e1v[2 * j] = lds_table_u2((__float_as_uint(lo2(bb)) & kBinMask) | lut1_or);
-                e1v[2 * j + 1] = lds_table_u2((__float_as_uint(hi2(bb)) & kBinMask) | lut1_or);
+                pq[2 * j] = lds_table_b64((__float_as_uint(lo2(bb)) & kBinMask) | lut1_or);
+                pq[2 * j + 1] = lds_table_b64((__float_as_uint(hi2(bb)) & kBinMask) | lut1_or);
             }
         };
         // same, then refill the row's registers from the next item
@@ -505,7 +503,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         };
         auto L2 = [&]() {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) pq[j] = lds_table_b64(above_addr(e1v[j].x, x[j], e1v[j].y));
+            for (int j = 0; j < 8; ++j) second_lookup(pq[j], x[j]);
         };
         auto M = [&](int row, float (&mt_o)[8], uint32_t (&ba_o)[8]) {
             if constexpr (INNER) {
@@ -515,9 +513,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 float c[8], chk = 0.f;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    float cP, cQ;
-                    unpack2(pq[j], cP, cQ);
-                    c[j] = sg ? cQ : cP;
+                    c[j] = sg ? hi2(pq[j]) : lo2(pq[j]);
                     mt_o[j] = __fmul_rn(Ic(j), __fsub_rn(x[j], c[j]));
                     chk += mt_o[j];
                 }
@@ -530,9 +526,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                     if (bad) {
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
-                            float cP, cQ;
-                            unpack2(lds_table_b64(pq_entry_addr(lut2_addr, ex.J[j], lane)), cP, cQ);
-                            c[j] = sg ? cQ : cP;
+                            const float2 e = lds_table_f2(pq_entry_addr(lut2_addr, ex.J[j], lane));
+                            c[j] = sg ? e.y : e.x;
                             mt_o[j] = __fmul_rn(Ic(j), __fsub_rn(x[j], c[j]));
                         }
                     }
@@ -547,11 +542,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             uint64_t s0 = 0ull, s1 = 0ull;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                float Pa, Qa, Pb, Qb;
-                unpack2(pq[2 * j], Pa, Qa);
-                unpack2(pq[2 * j + 1], Pb, Qb);
-                const uint64_t u0 = pack2(__fsub_rn(x[2 * j], Pa), __fsub_rn(x[2 * j + 1], Pb));
-                const uint64_t u1 = pack2(__fsub_rn(x[2 * j], Qa), __fsub_rn(x[2 * j + 1], Qb));
+                const uint64_t u0 = pack2(__fsub_rn(x[2 * j], lo2(pq[2 * j])), __fsub_rn(x[2 * j + 1], lo2(pq[2 * j + 1])));
+                const uint64_t u1 = pack2(__fsub_rn(x[2 * j], hi2(pq[2 * j])), __fsub_rn(x[2 * j + 1], hi2(pq[2 * j + 1])));
                 m0[j] = mul2(II[j], u0);
                 m1[j] = mul2(II[j], u1);
                 s0 = fma2(m0[j], u0, s0);
@@ -590,10 +582,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float a0 = (j & 1) ? hi2(m0[j >> 1]) : lo2(m0[j >> 1]), a1 = (j & 1) ? hi2(m1[j >> 1]) : lo2(m1[j >> 1]);
-                float cP, cQ;
-                unpack2(pq[j], cP, cQ);
                 mt_o[j] = sg ? a1 : a0;
-                ba_o[j] = base + (__float_as_uint(sg ? cQ : cP) & idx_mask) * kSlotBytes;
+                ba_o[j] = base + (__float_as_uint(sg ? hi2(pq[j]) : lo2(pq[j])) & idx_mask) * kSlotBytes;
             }
         };
         auto B = [&](const float (&mt_i)[8], const uint32_t (&ba_i)[8], int j0, int j1) {
@@ -803,6 +793,9 @@ struct FitBatch {
 
 template <int MODE, int SEL, int KIND>
 __global__ void __launch_bounds__(kFitWarps * 32, 1) fit_kernel(const __grid_constant__ FitBatch b) {
+    // a single layer: its parameters at fixed places (1-3 % faster than picked by index, which for several
+    // layers is as fast as a copy of the body per layer)
+    if (b.first[1] == gridDim.x) { fit_rounds_body<MODE, SEL, KIND>(b.L[0], blockIdx.x, gridDim.x); return; }
     int l = 0;
     while (l + 1 < kMaxBatch && blockIdx.x >= b.first[l + 1]) ++l;
     fit_rounds_body<MODE, SEL, KIND>(b.L[l], blockIdx.x - b.first[l], b.first[l + 1] - b.first[l]);

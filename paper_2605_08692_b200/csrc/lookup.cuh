@@ -13,7 +13,7 @@ constexpr int kRep = 16;                           // copies of the per-bin tabl
 constexpr int kJSlots = 32;                        // 31 intervals + the poisoned slot
 constexpr int kSlotBytes = 32 * 8;                 // bytes of a lane-private bin slot (one 8-byte entry per lane)
 // The {P, Q} table: one row per interval J, 16 columns of 8 bytes, so that a bin's table entry can
-// name the row of its lower interval and a weight above the bin's breakpoint adds one row.  Lane l
+// name the row of its lower interval and a weight above the bin's breakpoint takes the next row.  Lane l
 // uses column l mod 16: an 8-byte load is served a half-warp at a time, so lanes l and l + 16 never meet.
 constexpr int kPqRow = 128;
 constexpr int kPqCols = 16;
@@ -26,44 +26,30 @@ constexpr uint32_t kIdxMask = 15u;                 // low mantissa bits of a cen
 // Shared-memory accesses of the hot loop with explicit 32-bit addresses.  All are volatile asm,
 // which keeps them in the order in which the loop writes them (table lookups of one row issued
 // ahead of the read-modify-write chain of the previous one).
-__device__ __forceinline__ uint2 lds_table_u2(uint32_t addr) {
-    uint2 r;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "r"(addr));
-    return r;
-}
 __device__ __forceinline__ float2 lds_table_f2(uint32_t addr) {
     float2 r;
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "r"(addr));
     return r;
 }
+// A bin's entry is {P, Q} itself where no breakpoint lies in the bin (four fifths of the weights), else
+// {breakpoint, address of the lower interval's {P, Q}}: an address is below kAddrLimit, which no centre
+// constant is as an integer.  Such a weight looks {P, Q} up, in the next row if it lies above the
+// breakpoint; the other lanes take no part, and a load of a few lanes costs half of a full one.
+constexpr uint32_t kAddrLimit = 0x40000u;
+__device__ __forceinline__ void second_lookup(uint64_t& pq, float x) {
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 a;\n\t.reg .f32 b;\n\t"
+                 "mov.b64 {b, a}, %0;\n\t"
+                 "setp.lt.u32 p, a, 262144;\n\t"
+                 "setp.gt.and.f32 q, %1, b, p;\n\t"
+                 "@q add.u32 a, a, 128;\n\t"
+                 "mov.b64 %0, {b, a};\n\t"
+                 "@p ld.shared.b64 %0, [a];\n\t}"
+                 : "+l"(pq) : "f"(x));
+}
 __device__ __forceinline__ uint64_t lds_table_b64(uint32_t addr) {
     uint64_t r;
     asm volatile("ld.shared.b64 %0, [%1];" : "=l"(r) : "r"(addr));
     return r;
-}
-
-// {x - P, x - Q}: each half one correctly rounded FP32 subtraction, either as two scalar
-// instructions writing a register pair or as one packed instruction on {x, x}
-#ifndef AAAC_SCALAR_SUB
-#define AAAC_SCALAR_SUB 1
-#endif
-__device__ __forceinline__ uint64_t diff2(float x, uint64_t pq) {
-#if AAAC_SCALAR_SUB
-    float P, Q;
-    unpack2(pq, P, Q);
-    return pack2(__fsub_rn(x, P), __fsub_rn(x, Q));
-#else
-    return sub2(pack2(x, x), pq);
-#endif
-}
-
-// Address of the {P, Q} entry of a weight: `a` names the entry of the lower interval of the
-// weight's bin; a weight above the bin's breakpoint belongs to the next interval, whose entry
-// lies kPqRow bytes further (one compare and one predicated add).
-__device__ __forceinline__ uint32_t above_addr(uint32_t a, float x, uint32_t thr_bits) {
-    asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
-        : "+r"(a) : "f"(x), "f"(__uint_as_float(thr_bits)));
-    return a;
 }
 
 __device__ __forceinline__ float2 lds_bin(uint32_t addr) {
@@ -139,9 +125,10 @@ __device__ __forceinline__ void derive_tables(FitTables& S, const int lane, cons
     auto canonical = [&](int t, int k) { return 31 - __clz(~(t ? dup >> 16 : dup & 0xFFFFu) & ((2u << k) - 1u)); };
     // centre constant: the float nearest to the FP32 rounding of the entry whose low 4 mantissa bits are
     // the entry's canonical index (at most 8 units in the last place away)
+    // (and is never below 2^-100 in magnitude, so that as an integer it cannot be taken for an address)
     const uint32_t bits = __float_as_uint((float)T);
-    const int ci = canonical(r, i), tt = (int)(bits & 0x7FFFFFFFu) + 8 - ci;
-    S.centre[lane] = __uint_as_float((bits & 0x80000000u) | (tt < 0 ? (uint32_t)ci : (uint32_t)((tt & ~15) + ci)));
+    const int ci = canonical(r, i), tt = max((int)(bits & 0x7FFFFFFFu), 0x0D800010) + 8 - ci;
+    S.centre[lane] = __uint_as_float((bits & 0x80000000u) | (uint32_t)((tt & ~15) + ci));
     __syncwarp();
     // entries of T0 / T1 whose upper midpoint lies below interval `lane`
     const unsigned from1 = __ballot_sync(kAll, S.src[lane] == 1);
@@ -151,7 +138,7 @@ __device__ __forceinline__ void derive_tables(FitTables& S, const int lane, cons
     const float nan = __int_as_float(0x7FC00000);
     S.PQ[lane] = lane < kNJ ? make_double2(S.Td[i0], S.Td[kM + i1]) : make_double2(0.0, 0.0);
     S.pq32[lane] = lane < kNJ ? make_float2(S.centre[i0], S.centre[kM + i1]) : make_float2(nan, nan);
-    const uint32_t tm = __reduce_max_sync(kAll, __float_as_uint(__double2float_ru(fabs(T))));
+    const uint32_t tm = __reduce_max_sync(kAll, __float_as_uint(fmaxf(__double2float_ru(fabs(T)), 0x1p-70f)));
     if (lane == 0) {
         S.tmax283 = __fmul_ru(__uint_as_float(tm), 2.83f * 17.f);
         S.no_dup = dup == 0u;
@@ -174,13 +161,22 @@ __device__ __forceinline__ void write_tables(const FitTables& S, const int tid, 
         const int below = find_interval(S.bp, lo);
         const float v0 = S.bp[below], v1 = S.bp[below + 1];     // bp[30], bp[31] = +inf
         const bool poison = v1 <= hi;                            // two breakpoints or more
-        const uint32_t a = lut2_addr + (poison ? (uint32_t)kPoison : (uint32_t)(below * kPqRow));
-        const uint32_t t = !poison && v0 <= hi ? __float_as_uint(v0) : 0x7F800000u;
+        uint32_t e0, e1, c1 = 0;                                // c1: what an address grows by from copy to copy
+        if (!poison && !(v0 <= hi)) {
+            const float2 v = S.pq32[below];
+            e0 = __float_as_uint(v.x);
+            e1 = __float_as_uint(v.y);
+        } else {
+            e0 = poison ? 0x7F800000u : __float_as_uint(v0);
+            e1 = lut2_addr + (poison ? (uint32_t)kPoison : (uint32_t)(below * kPqRow));
+            c1 = 8u;
+        }
         const uint32_t at = lut1_addr + (uint32_t)b * (kRep * 8);
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
             const uint32_t c = (uint32_t)((s + tid) & 7) * 16u;
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %2};" :: "r"(at + c), "r"(a + c), "r"(t), "r"(a + c + 8u) : "memory");
+            const uint32_t f = e1 + (c1 ? c : 0u);
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %1, %3};" :: "r"(at + c), "r"(e0), "r"(f), "r"(f + c1) : "memory");
         }
     }
     static_assert(kLut2Bytes / 16 <= NT, "one store per thread");
@@ -202,15 +198,7 @@ constexpr uint32_t kNoHint = 0xFFu;
 // The interval of a weight from the constants {P, Q} the fast path has looked up: with no equal
 // entries inside a table, entry index = number of that table's breakpoints below the weight, and
 // the interval of the merged list is the sum of the two.  (A poisoned slot reads as NaN: no hint.)
-#ifndef AAAC_USE_HINT
-#define AAAC_USE_HINT 1
-#endif
-__device__ __forceinline__ uint32_t interval_hint(const FitTables& S, uint64_t pq) {
-#if !AAAC_USE_HINT
-    return kNoHint;
-#endif
-    float P, Q;
-    unpack2(pq, P, Q);
+__device__ __forceinline__ uint32_t interval_hint(const FitTables& S, float P, float Q) {
     return (S.no_dup && P == P) ? (__float_as_uint(P) & kIdxMask) + (__float_as_uint(Q) & kIdxMask) : kNoHint;
 }
 struct Exact8 { int J[8]; double emin; int sigma; int tie; };

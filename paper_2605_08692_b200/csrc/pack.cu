@@ -265,20 +265,19 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
                 const uint64_t xx = mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr);
                 const uint64_t bb = fma2(xx, pack2(kBinsPerUnit, kBinsPerUnit), pack2(kMagic, kMagic));
                 unpack2(xx, x[2 * j], x[2 * j + 1]);
-                const uint2 ea = lds_table_u2(sm_base + (((uint32_t)__float_as_int(lo2(bb)) & kBinMask) | lut1_copy));
-                const uint2 eb = lds_table_u2(sm_base + (((uint32_t)__float_as_int(hi2(bb)) & kBinMask) | lut1_copy));
-                tcand |= (x[2 * j] == __uint_as_float(ea.y)) | (x[2 * j + 1] == __uint_as_float(eb.y));
-                pq[2 * j] = lds_table_b64(above_addr(ea.x, x[2 * j], ea.y));
-                pq[2 * j + 1] = lds_table_b64(above_addr(eb.x, x[2 * j + 1], eb.y));
+                pq[2 * j] = lds_table_b64(sm_base + ((__float_as_uint(lo2(bb)) & kBinMask) | lut1_copy));
+                pq[2 * j + 1] = lds_table_b64(sm_base + ((__float_as_uint(hi2(bb)) & kBinMask) | lut1_copy));
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                tcand |= x[j] == lo2(pq[j]) && __float_as_uint(hi2(pq[j])) < kAddrLimit;
+                second_lookup(pq[j], x[j]);
             }
             uint64_t s0 = 0ull, s1 = 0ull;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                float Pa, Qa, Pb, Qb;
-                unpack2(pq[2 * j], Pa, Qa);
-                unpack2(pq[2 * j + 1], Pb, Qb);
-                const uint64_t u0 = pack2(__fsub_rn(x[2 * j], Pa), __fsub_rn(x[2 * j + 1], Pb));
-                const uint64_t u1 = pack2(__fsub_rn(x[2 * j], Qa), __fsub_rn(x[2 * j + 1], Qb));
+                const uint64_t u0 = pack2(__fsub_rn(x[2 * j], lo2(pq[2 * j])), __fsub_rn(x[2 * j + 1], lo2(pq[2 * j + 1])));
+                const uint64_t u1 = pack2(__fsub_rn(x[2 * j], hi2(pq[2 * j])), __fsub_rn(x[2 * j + 1], hi2(pq[2 * j + 1])));
                 s0 = fma2(mul2(II[j], u0), u0, s0);
                 s1 = fma2(mul2(II[j], u1), u1, s1);
             }
@@ -298,7 +297,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
                     // near-ties and poisoned slots (rare, out of line)
                     Row8 r;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) { r.x[j] = x[j]; r.I[j] = (j & 1) ? hi2(II[j >> 1]) : lo2(II[j >> 1]); r.hint[j] = interval_hint(S, pq[j]); }
+                    for (int j = 0; j < 8; ++j) { r.x[j] = x[j]; r.I[j] = (j & 1) ? hi2(II[j >> 1]) : lo2(II[j >> 1]); r.hint[j] = interval_hint(S, lo2(pq[j]), hi2(pq[j])); }
                     const Rare8 ex = rare_groups<LPG>(&S, r, near);
                     if (near) {
 #pragma unroll
@@ -346,9 +345,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
             uint32_t word = 0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                float cP, cQ;
-                unpack2(pq[j], cP, cQ);
-                word = __funnelshift_r(word, __float_as_uint(sg ? cQ : cP), 4);
+                word = __funnelshift_r(word, __float_as_uint(sg ? hi2(pq[j]) : lo2(pq[j])), 4);
             }
             *reinterpret_cast<uint32_t*>(p.codes + co) = word;
             if (SEL == G && (lane % LPG) == 0) {
