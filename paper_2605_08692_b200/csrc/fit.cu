@@ -404,7 +404,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     }
     for (int b = 0; b < kBinSlots; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
     __syncthreads();
-    write_tables<NT>(S, tid, kLut1At, lut2_addr);
+    write_tables<NT, true>(S, tid, kLut1At, lut2_addr);
     __syncthreads();
 
     // bin arithmetic: the masked mantissa of fl32(kBinsPerUnit x + kMagic) is bin * (REP * 8)
@@ -770,7 +770,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         return;
     }
     if (round + 1 < p.n_rounds) {
-        write_tables<NT>(S, tid, kLut1At, lut2_addr);
+        write_tables<NT, true>(S, tid, kLut1At, lut2_addr);
         __syncthreads();
     }
   }

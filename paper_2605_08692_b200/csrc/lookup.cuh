@@ -31,11 +31,24 @@ __device__ __forceinline__ float2 lds_table_f2(uint32_t addr) {
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "r"(addr));
     return r;
 }
-// A bin's entry is {P, Q} itself where no breakpoint lies in the bin (four fifths of the weights), else
+// Two forms of a bin's entry.  The pack pass, which is bound by its instructions: {address of the lower
+// interval's {P, Q}, breakpoint}, and every weight looks {P, Q} up, a row further if it lies above the
+// breakpoint (one compare, one predicated add).
+__device__ __forceinline__ uint32_t above_addr(uint32_t a, float x, uint32_t thr_bits) {
+    asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
+        : "+r"(a) : "f"(x), "f"(__uint_as_float(thr_bits)));
+    return a;
+}
+__device__ __forceinline__ uint2 lds_table_u2(uint32_t addr) {
+    uint2 r;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "r"(addr));
+    return r;
+}
+
+// The fit rounds, bound by shared memory: {P, Q} itself where no breakpoint lies in the bin (four fifths of the weights), else
 // {breakpoint, address of the lower interval's {P, Q}}: an address is below kAddrLimit, which no centre
 // constant is as an integer.  Such a weight looks {P, Q} up, in the next row if it lies above the
 // breakpoint; the other lanes take no part, and a load of a few lanes costs half of a full one.
-constexpr uint32_t kAddrLimit = 0x40000u;
 __device__ __forceinline__ void second_lookup(uint64_t& pq, float x) {
     asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 a;\n\t.reg .f32 b;\n\t"
                  "mov.b64 {b, a}, %0;\n\t"
@@ -150,7 +163,8 @@ __device__ __forceinline__ void derive_tables(FitTables& S, const int lane, cons
 // breakpoints are sorted, so those inside a bin are the first ones not below its lower edge.  A thread
 // writes the 16 copies of its bin, two per store, in an order rotated by its lane, so that the eight
 // lanes that a 16-byte store is served for meet in no bank.
-template <int NT>
+// DIRECT: the fit rounds' form of the bins' entries.
+template <int NT, bool DIRECT>
 __device__ __forceinline__ void write_tables(const FitTables& S, const int tid, const uint32_t lut1_addr, const uint32_t lut2_addr) {
     static_assert(kNBins % NT == 0, "whole bins per thread");
     constexpr float h = 0.5f / (float)(kRep * 8);
@@ -162,7 +176,10 @@ __device__ __forceinline__ void write_tables(const FitTables& S, const int tid, 
         const float v0 = S.bp[below], v1 = S.bp[below + 1];     // bp[30], bp[31] = +inf
         const bool poison = v1 <= hi;                            // two breakpoints or more
         uint32_t e0, e1, c1 = 0;                                // c1: what an address grows by from copy to copy
-        if (!poison && !(v0 <= hi)) {
+        if (!DIRECT) {
+            e0 = lut2_addr + (poison ? (uint32_t)kPoison : (uint32_t)(below * kPqRow));
+            e1 = !poison && v0 <= hi ? __float_as_uint(v0) : 0x7F800000u;
+        } else if (!poison && !(v0 <= hi)) {
             const float2 v = S.pq32[below];
             e0 = __float_as_uint(v.x);
             e1 = __float_as_uint(v.y);
@@ -175,8 +192,12 @@ __device__ __forceinline__ void write_tables(const FitTables& S, const int tid, 
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
             const uint32_t c = (uint32_t)((s + tid) & 7) * 16u;
-            const uint32_t f = e1 + (c1 ? c : 0u);
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %1, %3};" :: "r"(at + c), "r"(e0), "r"(f), "r"(f + c1) : "memory");
+            if (DIRECT) {
+                const uint32_t f = e1 + (c1 ? c : 0u);
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %1, %3};" :: "r"(at + c), "r"(e0), "r"(f), "r"(f + c1) : "memory");
+            } else {
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %2};" :: "r"(at + c), "r"(e0 + c), "r"(e1), "r"(e0 + c + 8u) : "memory");
+            }
         }
     }
     static_assert(kLut2Bytes / 16 <= NT, "one store per thread");

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
         derive_tables(S, lane, T);
     }
     __syncthreads();
-    write_tables<NW * 32>(S, tid, (uint32_t)__cvta_generic_to_shared(dyn), (uint32_t)__cvta_generic_to_shared(dyn) + kLut1Bytes);
+    write_tables<NW * 32, false>(S, tid, (uint32_t)__cvta_generic_to_shared(dyn), (uint32_t)__cvta_generic_to_shared(dyn) + kLut1Bytes);
     __syncthreads();
 
     const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(dyn);
@@ -265,13 +265,11 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
                 const uint64_t xx = mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr);
                 const uint64_t bb = fma2(xx, pack2(kBinsPerUnit, kBinsPerUnit), pack2(kMagic, kMagic));
                 unpack2(xx, x[2 * j], x[2 * j + 1]);
-                pq[2 * j] = lds_table_b64(sm_base + ((__float_as_uint(lo2(bb)) & kBinMask) | lut1_copy));
-                pq[2 * j + 1] = lds_table_b64(sm_base + ((__float_as_uint(hi2(bb)) & kBinMask) | lut1_copy));
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                tcand |= x[j] == lo2(pq[j]) && __float_as_uint(hi2(pq[j])) < kAddrLimit;
-                second_lookup(pq[j], x[j]);
+                const uint2 ea = lds_table_u2(sm_base + ((__float_as_uint(lo2(bb)) & kBinMask) | lut1_copy));
+                const uint2 eb = lds_table_u2(sm_base + ((__float_as_uint(hi2(bb)) & kBinMask) | lut1_copy));
+                tcand |= (x[2 * j] == __uint_as_float(ea.y)) | (x[2 * j + 1] == __uint_as_float(eb.y));
+                pq[2 * j] = lds_table_b64(above_addr(ea.x, x[2 * j], ea.y));
+                pq[2 * j + 1] = lds_table_b64(above_addr(eb.x, x[2 * j + 1], eb.y));
             }
             uint64_t s0 = 0ull, s1 = 0ull;
 #pragma unroll
