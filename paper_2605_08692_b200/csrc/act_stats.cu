@@ -120,8 +120,8 @@ int act_splits_max(int64_t K) {
 }
 
 ActPlan act_plan(int64_t T, int64_t K, int max_splits) {
-    // up to 256 rows a strip more costs less than the second kernel
-    int64_t splits = T <= 256 ? 1 : std::min<int64_t>(max_splits, (T + kWarps - 1) / kWarps);
+    // up to 64 rows (two loop iterations of a block) one strip is shorter than a second kernel
+    int64_t splits = T <= 64 ? 1 : std::min<int64_t>(max_splits, (T + kWarps - 1) / kWarps);
     ActPlan p;
     p.rows = ((T + splits - 1) / splits + kWarps - 1) / kWarps * kWarps;
     p.strips = (int)((T + p.rows - 1) / p.rows);
