@@ -89,8 +89,7 @@ size_t aaac_workspace_bytes_full(int mode, int64_t N, int64_t K, int64_t T);
 
 /*
  * Activation importance, Eq. 7:  I[k] = sum_t X[t,k]^2.
- * The squares are exact in FP32 and are added without rounding error (an FP32 value pair per
- * column, strips combined in a fixed order in double); the sum is rounded once to FP32.
+ * The squares are exact and are added in double, in a fixed order; the sum is rounded once to FP32.
  * accumulate = 0 overwrites I; 1 adds to the existing I (FP32 add), so that the tokens can
  * be streamed in chunks.  Sets AAAC_DEV_NONFINITE if a sum is not finite.
  */

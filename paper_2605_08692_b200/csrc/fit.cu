@@ -26,8 +26,7 @@
 // (b) its two weighted squared errors, and (c) one accumulation into the centroid sums of cell
 // (sigma, J).
 //
-// (a) Interval.  NB uniform bins on (-8, 8) (512 of width 1/32 here; the pack pass, which has no
-//     bins to hold, uses 1024 of width 1/64): with s = NB / 16 the mantissa of
+// (a) Interval.  NB uniform bins on (-8, 8) (512 of width 1/32): with s = NB / 16 the mantissa of
 //     fl32(s x + NB / 2 + 1.5 * 2^(23-k)) holds (s x + NB / 2) * 2^k rounded to an integer; masked,
 //     it is the byte offset bin * 2^k of the bin's table entry (2^k = bytes per bin over all
 //     copies), bin = floor of s x + NB / 2 after rounding to a multiple of 2^-k.
