@@ -314,28 +314,33 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
     __shared__ uint32_t hist[kDigits];
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t sh_digit, sh_left, sh_in, sh_next;
-    __shared__ uint32_t req_slot[kQReq];
+    __shared__ uint32_t asked[kQReq / 32];                 // the requests that live in this slot
     __shared__ unsigned long long req_local[kQReq];
     __shared__ uint32_t sh_or, sh_and, sh_cnt, sh_min;
     const uint32_t slot = blockIdx.x;
-    if (slot >= ctrl->nslots) return;
-    if (ctrl->slot_over[slot]) {
+    // (read side by side: the launch is all latency for most lists)
+    const uint32_t nslots = ctrl->nslots, over = ctrl->slot_over[slot];
+    const unsigned long long begin = ctrl->slot_off[slot], n = ctrl->slot_off[slot + 1] - begin;
+    const uint32_t my_slot = threadIdx.x < kQReq ? ctrl->req_slot[threadIdx.x] : ~0u;
+    const unsigned long long my_local = threadIdx.x < kQReq ? ctrl->req_local[threadIdx.x] : 0ull;
+    if (slot >= nslots) return;
+    if (over) {
         // the bin's weights had no room in the list: if they all share one value, that value is every
         // order statistic of the bin; otherwise the scratch was too small for this layer
         const uint32_t kmin = ctrl->slot_kmin[slot], kmax = ctrl->slot_kmax[slot];
-        if (threadIdx.x < kQReq && ctrl->req_slot[threadIdx.x] == slot) {
+        if (my_slot == slot) {
             if (kmin == kmax) ctrl->rank_val[threadIdx.x] = key_float(kmin);
             else { ctrl->rank_val[threadIdx.x] = 0.f; ctrl->scratch_short = 1u; }
         }
         return;
     }
     if (threadIdx.x < kQReq) {
-        req_slot[threadIdx.x] = ctrl->req_slot[threadIdx.x];
-        req_local[threadIdx.x] = ctrl->req_local[threadIdx.x];
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, my_slot == slot);
+        if ((threadIdx.x & 31) == 0) asked[threadIdx.x >> 5] = m;
+        req_local[threadIdx.x] = my_local;
     }
     if (threadIdx.x == 0) { sh_or = 0u; sh_and = 0xFFFFFFFFu; }
-    const uint32_t* keys = list + ctrl->slot_off[slot];
-    const unsigned long long n = ctrl->slot_off[slot + 1] - ctrl->slot_off[slot];
+    const uint32_t* keys = list + begin;
     const unsigned long long n_up = (n + blockDim.x - 1) / blockDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     constexpr int kKeep = 24;
@@ -389,8 +394,9 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
     unsigned long long prev_k = 0;
     uint32_t prev_key = 0u, prev_next = 0u;                // the next larger key, if the counters named it (else 0)
     bool prev_last = false;                                // no further key equal to it comes after that rank
-    for (int q = 0; q < kQReq; ++q) {
-        if (req_slot[q] != slot) continue;                 // uniform across the block
+    unsigned long long todo = asked[1];
+    for (todo = todo << 32 | asked[0]; todo; todo &= todo - 1) {      // uniform across the block
+        const int q = __ffsll((long long)todo) - 1;
         if (have_prev && (req_local[q] == prev_k || req_local[q] == prev_k + 1)) {
             // the same or the next order statistic: it equals the previous key unless every key
             // up to that one is already counted, in which case it is the smallest larger key

@@ -215,8 +215,12 @@ scales_hist_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row,
         if (dev_status) atomicOr(dev_status, AAAC_DEV_NONFINITE);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kQBins; i += blockDim.x)
+    // every block starts elsewhere, so that they do not meet on the same counters
+    const unsigned first = threadIdx.x + blockIdx.x * blockDim.x;
+    for (unsigned k = 0; k < kQBins; k += blockDim.x) {
+        const unsigned i = (first + k) % kQBins;
         if (sm[i]) atomicAdd(&hist[i], sm[i]);
+    }
 }
 
 }  // namespace
