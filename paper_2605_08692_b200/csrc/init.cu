@@ -332,8 +332,9 @@ quantile_plan_kernel(Ctrl* ctrl, const uint32_t* __restrict__ hist, uint8_t* __r
 //    only what is beyond them is streamed from memory, eight loads in flight per thread.
 //  - The keys of a slot lie in one narrow bin, so they share their leading bits: one sweep finds
 //    the bits on which all keys agree, and only the digits of 11 bits below them need a radix pass: two,
-//    mostly (8-bit digits took three, and combining equal digits within a warp before counting cost more
-//    than the counting).
+//    mostly, or none where the keys are all equal (8-bit digits took three, and combining equal digits within a
+//    warp before counting cost more than the counting).  A thread counts its keys in 32 bits and tests nothing else
+//    about them: the longest lists of a layer hold some 60 000 keys and are bound by instructions.
 //  - The two neighbours that one table entry interpolates between are consecutive ranks: the
 //    second is the first's key again, or the next larger key, which the last pass's counters name
 //    unless it differs in a higher digit; then one sweep finds it.
@@ -343,14 +344,15 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t sh_digit, sh_left, sh_in, sh_next;
     __shared__ uint32_t asked[kQReq / 32];                 // the requests that live in this slot
-    __shared__ unsigned long long req_local[kQReq];
+    __shared__ uint32_t req_local[kQReq];
     __shared__ uint32_t sh_or, sh_and, sh_cnt, sh_min;
     const uint32_t slot = blockIdx.x;
     // (read side by side: the launch is all latency for most lists)
     const uint32_t nslots = ctrl->nslots, over = ctrl->slot_over[slot];
-    const unsigned long long begin = ctrl->slot_off[slot], n = ctrl->slot_off[slot + 1] - begin;
+    const unsigned long long begin = ctrl->slot_off[slot];
+    const uint32_t n = (uint32_t)(ctrl->slot_off[slot + 1] - begin);       // (a layer has fewer than 2^32 weights)
     const uint32_t my_slot = threadIdx.x < kQReq ? ctrl->req_slot[threadIdx.x] : ~0u;
-    const unsigned long long my_local = threadIdx.x < kQReq ? ctrl->req_local[threadIdx.x] : 0ull;
+    const uint32_t my_local = threadIdx.x < kQReq ? (uint32_t)ctrl->req_local[threadIdx.x] : 0u;
     if (slot >= nslots) return;
     if (over) {
         // the bin's weights had no room in the list: if they all share one value, that value is every
@@ -369,42 +371,36 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
     }
     if (threadIdx.x == 0) { sh_or = 0u; sh_and = 0xFFFFFFFFu; }
     const uint32_t* keys = list + begin;
-    const unsigned long long n_up = (n + blockDim.x - 1) / blockDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
-    constexpr int kKeep = 24;
-    const unsigned long long n_keep = min(n_up, (unsigned long long)kKeep * blockDim.x);   // a multiple of the block size
+    constexpr uint32_t kThreads = 1024;
+    constexpr int kKeep = 24, kAhead = 8;
+    const uint32_t* mine = keys + threadIdx.x;             // this thread's keys are kThreads apart
+    const uint32_t n_mine = threadIdx.x < n ? (n - threadIdx.x - 1) / kThreads + 1 : 0u;
     uint32_t kc[kKeep];
 #pragma unroll
-    for (int u = 0; u < kKeep; ++u) {
-        const unsigned long long i = threadIdx.x + (unsigned long long)u * blockDim.x;
-        kc[u] = i < n ? keys[i] : 0u;
-    }
-    // f(key, valid) for every key of the list; every thread of the block makes the same calls
+    for (int u = 0; u < kKeep; ++u) kc[u] = u < n_mine ? mine[u * kThreads] : 0u;
+    // f(key) for every key of this thread's part of the list
     auto for_each_key = [&](auto f) {
 #pragma unroll
         for (int u = 0; u < kKeep; ++u) {
-            if ((unsigned long long)u * blockDim.x >= n_keep) break;
-            f(kc[u], threadIdx.x + (unsigned long long)u * blockDim.x < n);
+            if (u >= n_mine) return;
+            f(kc[u]);
         }
-        for (unsigned long long i0 = n_keep + threadIdx.x; i0 < n_up; i0 += 8ull * blockDim.x) {
-            uint32_t kk[8];
+        const uint32_t* p = mine + kKeep * kThreads;
+        uint32_t left = n_mine - kKeep;
+        for (; left >= kAhead; left -= kAhead, p += kAhead * kThreads) {
+            uint32_t kk[kAhead];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const unsigned long long i = i0 + (unsigned long long)u * blockDim.x;
-                kk[u] = i < n ? keys[i] : 0u;
-            }
+            for (int u = 0; u < kAhead; ++u) kk[u] = p[u * kThreads];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const unsigned long long i = i0 + (unsigned long long)u * blockDim.x;
-                if (i >= n_up) break;
-                f(kk[u], i < n);
-            }
+            for (int u = 0; u < kAhead; ++u) f(kk[u]);
         }
+        for (; left; --left, p += kThreads) f(*p);
     };
     __syncthreads();
     {
         uint32_t o = 0u, a = 0xFFFFFFFFu;
-        for_each_key([&](uint32_t k, bool valid) { if (valid) { o |= k; a &= k; } });
+        for_each_key([&](uint32_t k) { o |= k; a &= k; });
         o = __reduce_or_sync(0xFFFFFFFFu, o);
         a = __reduce_and_sync(0xFFFFFFFFu, a);
         if (lane == 0) { atomicOr(&sh_or, o); atomicAnd(&sh_and, a); }
@@ -414,12 +410,16 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
     uint32_t first_mask = 0u, first_prefix = 0u;           // ... and the bits above it, the same in all
     if (n > 0) {
         const uint32_t diff = sh_or ^ sh_and;
-        top = diff ? 31 - __clz(diff) : 0;
+        if (!diff) {                                       // one value (many a bin of scaled BF16 weights)
+            if (my_slot == slot) ctrl->rank_val[threadIdx.x] = key_float(sh_and);
+            return;
+        }
+        top = 31 - __clz(diff);
         first_mask = top == 31 ? 0u : ~((2u << top) - 1u);
         first_prefix = sh_and & first_mask;
     }
     bool have_prev = false;                                // rank and key of the request answered last
-    unsigned long long prev_k = 0;
+    uint32_t prev_k = 0;
     uint32_t prev_key = 0u, prev_next = 0u;                // the next larger key, if the counters named it (else 0)
     bool prev_last = false;                                // no further key equal to it comes after that rank
     unsigned long long todo = asked[1];
@@ -435,17 +435,15 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
                 if (threadIdx.x == 0) { sh_cnt = 0u; sh_min = 0xFFFFFFFFu; }
                 __syncthreads();
                 uint32_t c = 0u, m = 0xFFFFFFFFu;
-                for_each_key([&](uint32_t k, bool valid) {
-                    if (valid) {
-                        if (k <= prev_key) ++c;
-                        else m = min(m, k);
-                    }
+                for_each_key([&](uint32_t k) {
+                    if (k <= prev_key) ++c;
+                    else m = min(m, k);
                 });
                 c = __reduce_add_sync(0xFFFFFFFFu, c);
                 m = __reduce_min_sync(0xFFFFFFFFu, m);
                 if (lane == 0) { atomicAdd(&sh_cnt, c); atomicMin(&sh_min, m); }
                 __syncthreads();
-                if (req_local[q] >= (unsigned long long)sh_cnt && sh_min != 0xFFFFFFFFu) key = sh_min;
+                if (req_local[q] >= sh_cnt && sh_min != 0xFFFFFFFFu) key = sh_min;
                 __syncthreads();
             }
             if (threadIdx.x == 0) ctrl->rank_val[q] = key_float(key);
@@ -454,15 +452,15 @@ __device__ __forceinline__ void select_slot(Ctrl* ctrl, const uint32_t* __restri
             continue;
         }
         uint32_t prefix = first_prefix, mask = first_mask;
-        uint32_t k_left = (uint32_t)min(req_local[q], (unsigned long long)0xFFFFFFFFu);     // rank among the keys with this prefix
+        uint32_t k_left = req_local[q];                    // rank among the keys with this prefix
         for (int hi = top; hi >= 0;) {
             const int shift = hi >= kDigit ? hi - (kDigit - 1) : 0;
             const uint32_t width = (2u << (hi - shift)) - 1u;
             for (int i = threadIdx.x; i < kDigits; i += blockDim.x) hist[i] = 0;
             if (threadIdx.x == 0) { sh_digit = width; sh_left = 0u; sh_in = 1u; sh_next = 0xFFFFFFFFu; }   // (ranks beyond the list are never requested)
             __syncthreads();
-            for_each_key([&](uint32_t k, bool valid) {
-                if (valid && (k & mask) == prefix) atomicAdd(&hist[(k >> shift) & width], 1u);
+            for_each_key([&](uint32_t k) {
+                if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & width], 1u);
             });
             __syncthreads();
             // the digit that holds the rank: thread t owns digits 2 t and 2 t + 1
