@@ -655,7 +655,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
 
     // ---- the warp's sums: lane c adds the 32 lane-private values of cell c (in an order of its own that
     //      avoids bank conflicts, and a fixed one).  In double, 32 FP32 values are added without rounding
-    //      unless they are more than 2^24 apart.  Then the warp's bins start the next pass at zero ----
+    //      unless they are more than 2^24 apart ----
     const bool trace = KIND != kInner && p.err_trace != nullptr;
     __syncwarp();
     {
@@ -677,9 +677,6 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             for (int s = 16; s; s >>= 1) Eacc += __shfl_xor_sync(kAll, Eacc, s);
             if (lane == 0) sh.wsum[warp][2 * kCells] = Eacc;
         }
-        __syncwarp();
-#pragma unroll 8
-        for (int b = 0; b < kCells; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
     }
     __syncthreads();                                       // every warp is done with the lookup tables, its sums are there
     unsigned long long* const acc = p.acc + (size_t)(pass_no % 3u) * kAccBuffer;
@@ -709,6 +706,16 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         const unsigned long long add = (unsigned long long)((sum_warp & 1) ? top + kTopBias : low) + kOneArrival;
         if (which < 2) atomicAdd(acc + sum_cell * kAccStride + sum_warp, add);
         else if (do_e && lane < 6 && which == 2) atomicAdd(acc + kCells * kAccStride + (lane - 4), add);
+    }
+    // ---- meanwhile the bins start the next pass at zero: behind the sums, which the other blocks wait for
+    //      (warp 1 clears those of warp 0, which waits) ----
+    if (warp) {
+#pragma unroll 8
+        for (int b = 0; b < kCells; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
+        if (warp == 1) {
+#pragma unroll 8
+            for (int b = 0; b < kCells; ++b) sts_bin((n_low > 0 ? sm_base : hi_base) + lane * 8 + b * kSlotBytes, make_float2(0.f, 0.f));
+        }
     }
     // ---- one warp waits until every block's sums are in and derives the new tables; lane c takes cell c ----
     if (warp == 0) {
