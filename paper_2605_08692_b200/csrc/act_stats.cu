@@ -119,9 +119,11 @@ int act_splits_max(int64_t K) {
     return (int)(want < 1 ? 1 : want > kActMaxSplits ? kActMaxSplits : want);
 }
 
-ActPlan act_plan(int64_t T, int64_t K, int max_splits) {
-    // up to 64 rows (two loop iterations of a block) one strip is shorter than a second kernel
-    int64_t splits = T <= 64 ? 1 : std::min<int64_t>(max_splits, (T + kWarps - 1) / kWarps);
+// A pass over few rows is one strip, which needs no second kernel: up to 64 rows (two loop iterations of a block) it is
+// shorter than that kernel, and up to 128 where a caller waits for this result alone and nothing runs beside it
+// (kActAlone; 128 x 512 3.0 -> 2.7 us, 128 x 4096 4.2 -> 2.8, but 256 x 512 3.0 -> 4.1).
+ActPlan act_plan(int64_t T, int64_t K, int max_splits, int64_t one_strip_rows) {
+    int64_t splits = T <= one_strip_rows ? 1 : std::min<int64_t>(max_splits, (T + kWarps - 1) / kWarps);
     ActPlan p;
     p.rows = ((T + splits - 1) / splits + kWarps - 1) / kWarps * kWarps;
     p.strips = (int)((T + p.rows - 1) / p.rows);
@@ -146,16 +148,16 @@ namespace {
 // both launches; `part` holds [max_splits][K] doubles.  Every partial that the second kernel reads is written
 // by the first: nothing has to be cleared.
 cudaError_t run_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate, uint32_t* dev_status,
-                          double* part, int max_splits, cudaStream_t st) {
-    const ActPlan plan = act_plan(T, K, max_splits);
+                          double* part, int max_splits, int64_t one_strip_rows, cudaStream_t st) {
+    const ActPlan plan = act_plan(T, K, max_splits, one_strip_rows);
     const cudaError_t e = launch_act_strips(X, T, K, ldx, plan, 0, plan.strips, I, accumulate, dev_status, part, st);
     return e != cudaSuccess ? e : launch_act_finish(K, plan, I, accumulate, dev_status, part, st);
 }
 }  // namespace
 
 cudaError_t launch_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate,
-                             uint32_t* dev_status, const Workspace& ws, cudaStream_t st) {
-    return run_act_stats(X, T, K, ldx, I, accumulate, dev_status, ws.act_part, act_splits_max(K), st);
+                             uint32_t* dev_status, const Workspace& ws, int64_t one_strip_rows, cudaStream_t st) {
+    return run_act_stats(X, T, K, ldx, I, accumulate, dev_status, ws.act_part, act_splits_max(K), one_strip_rows, st);
 }
 
 }  // namespace aaac
@@ -211,6 +213,6 @@ extern "C" int aaac_act_stats_noalloc(const void* X, int64_t T, int64_t K, int64
     if (noalloc_scratch(&part) != cudaSuccess) return AAAC_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int splits = std::min(act_splits_max(K), kNoAllocSplits);
-    if (run_act_stats(static_cast<const uint16_t*>(X), T, K, ldx, I, accumulate, dev_status, part, splits, st) != cudaSuccess) return AAAC_ERR_CUDA;
+    if (run_act_stats(static_cast<const uint16_t*>(X), T, K, ldx, I, accumulate, dev_status, part, splits, kActAlone, st) != cudaSuccess) return AAAC_ERR_CUDA;
     return AAAC_OK;
 }

@@ -253,7 +253,7 @@ int aaac_act_stats(const void* X, int64_t T, int64_t K, int64_t ldx, float* I, i
     if (rc) return rc;
     Workspace w = carve(ws, AAAC_NVFP4, 1, K, ws_bytes);
     return launch_act_stats(static_cast<const uint16_t*>(X), T, K, ldx, I, accumulate, dev_status, w,
-                            static_cast<cudaStream_t>(stream)) == cudaSuccess ? AAAC_OK : AAAC_ERR_CUDA;
+                            kActAlone, static_cast<cudaStream_t>(stream)) == cudaSuccess ? AAAC_OK : AAAC_ERR_CUDA;
 }
 
 int aaac_fit_layer(const void* W, int64_t N, int64_t K, int64_t ldw, int mode, int group,
@@ -307,7 +307,7 @@ int prepare_fit_layer(const aaac_layer& L, int mode, int init, uint32_t* dev_sta
     if (cudaMemsetAsync(w.ctrl, 0, w.zero_bytes(fused), st) != cudaSuccess) return AAAC_ERR_CUDA;
     const float* I = L.I ? L.I : shared_I;
     if (!I) {
-        if (launch_act_stats(static_cast<const uint16_t*>(L.X), L.T, L.K, L.ldx, w.I, 0, dev_status, w, st) != cudaSuccess)
+        if (launch_act_stats(static_cast<const uint16_t*>(L.X), L.T, L.K, L.ldx, w.I, 0, dev_status, w, kActBeside, st) != cudaSuccess)
             return AAAC_ERR_CUDA;
         I = w.I;
     }
@@ -588,7 +588,7 @@ int aaac_quantize_layer_host_async(const void* W_host, int64_t N, int64_t K, int
     run(cudaMemsetAsync(w.ctrl, 0, w.zero_bytes(hist), st));
     if (e == cudaSuccess) run(launch_scales(W, N, K, K, mode, d + h.scales, ts, dstatus, w, st, hist));
     if (e == cudaSuccess) run(launch_init(W, N, K, K, mode, init, d + h.scales, T01, dstatus, w, st));
-    const ActPlan plan = act_plan(T, K, act_splits_max(K));
+    const ActPlan plan = act_plan(T, K, act_splits_max(K), kActBeside);
     const int pieces = lanes.overlapped() ? std::min(4, plan.strips) : 1;
     for (int c = 0; c < pieces; ++c) {
         const int s0 = (int)((int64_t)plan.strips * c / pieces), s1 = (int)((int64_t)plan.strips * (c + 1) / pieces);

@@ -158,10 +158,11 @@ __device__ __forceinline__ float f32_round_down(double d) { return __double2floa
 
 // ---- launchers (each enqueues on `st` and returns the launch status) ----
 cudaError_t launch_act_stats(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, float* I, int accumulate,
-                             uint32_t* dev_status, const Workspace& ws, cudaStream_t st);
+                             uint32_t* dev_status, const Workspace& ws, int64_t one_strip_rows, cudaStream_t st);
 // the same in pieces: strips [first, first + count) of the plan, then the sum over the strips
 struct ActPlan { int64_t rows; int strips; };
-ActPlan act_plan(int64_t T, int64_t K, int max_splits);
+constexpr int64_t kActAlone = 128, kActBeside = 64;    // rows that make one strip (see act_stats.cu)
+ActPlan act_plan(int64_t T, int64_t K, int max_splits, int64_t one_strip_rows);
 cudaError_t launch_act_strips(const uint16_t* X, int64_t T, int64_t K, int64_t ldx, const ActPlan& plan, int first, int count,
                               float* I, int accumulate, uint32_t* dev_status, double* part, cudaStream_t st);
 cudaError_t launch_act_finish(int64_t K, const ActPlan& plan, float* I, int accumulate, uint32_t* dev_status, const double* part,

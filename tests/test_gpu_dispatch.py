@@ -68,7 +68,7 @@ def test_scales_over_the_whole_range_of_group_maxima(mode):
         assert np.array_equal(host(r["scales_pos"]), want) and host(r["tensor_scale"])[0] == ts[0]
 
 
-@pytest.mark.parametrize("T", [64, 65, 2049])
+@pytest.mark.parametrize("T", [64, 128, 129, 2049])
 def test_importances_in_one_strip_and_in_several(T):
     K = 264
     X = synth.activations(T, K, 3, f"strips/{T}", kind="loguniform", massive_frac=0.01)
