@@ -8,11 +8,11 @@
 // same new tables without a relaunch (integer addition does not depend on the order in which the
 // blocks arrive, so the result is bitwise reproducible).  The wait for the totals is bounded: if
 // it runs out, the kernel sets AAAC_DEV_TIMEOUT in the device status word and returns.
-// What a round costs besides its pass (block sums, exchange, new tables) is latency: about 11k
+// What a round costs besides its pass (block sums, exchange, new tables) is latency: about 8.5k
 // cycles, kept short by leaving the small steps to one warp that needs no block barrier, by
 // lookups and conversions chosen for it (see below), and by having the first rows of the next pass
-// in flight meanwhile.  A pass of a 512 x 512 layer took 11.4 us with 19k cycles of it and whole
-// items, 6.9 us now; 4096 x 4096, 27.4 -> 25.0 us.
+// in flight, and the bins being cleared, meanwhile.  A pass of a 512 x 512 layer took 11.4 us with 19k cycles of it and whole
+// items, 5.2 us now; 4096 x 4096, 27.4 -> 23.3 us.
 // With n_inner > 1 the assignment pass (which is also the first inner iteration) stores the
 // selection bits, one word per row and 256-column slab, and the remaining n_inner - 1 inner
 // iterations are passes of a second instance of the kernel that reads those bits instead of
