@@ -59,6 +59,7 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, unsigned n_pieces, unsig
     __shared__ float queue_r[8][kQueue];
     __shared__ uint32_t cnt[kQReq];
     __shared__ unsigned long long base[kQReq];
+    __shared__ uint32_t room[kQReq];                      // what a slot's list has left for the block's keys
     __shared__ uint32_t nbuf;
     __shared__ uint32_t okmin[kQReq], okmax[kQReq];       // smallest / largest key of the slots without list space
     __shared__ float rl[128];                             // fl32(1 / s) per E4M3 code, or per mantissa of a BF16 scale
@@ -79,16 +80,24 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, unsigned n_pieces, unsig
     const unsigned step = gridDim.x * blockDim.x;
     const unsigned iters = (n_pieces + 2 * step - 1) / (2 * step);     // two pieces per thread and iteration
 
+    // Reserves n places of slot s's list; returns how many of them the list has.  (All of them: its size was counted
+    // from the same weights.  The check keeps a layer that is written to meanwhile from spoiling other memory.)
+    auto reserve = [&](uint32_t s, uint32_t n, unsigned long long& at) {
+        const unsigned long long off = ctrl->slot_off[s];
+        const uint32_t size = (uint32_t)(ctrl->slot_off[s + 1] - off), before = atomicAdd(&ctrl->slot_fill[s], n);
+        at = off + before;
+        return before < size ? min(size - before, n) : 0u;
+    };
     auto flush = [&]() {                                  // called by the whole block, after a barrier
         const uint32_t n = min(nbuf, (uint32_t)kStageCap);
         if (tid < kQReq) cnt[tid] = 0;
         __syncthreads();
         for (uint32_t i = tid; i < n; i += blockDim.x) buf_pos[i] = (uint16_t)atomicAdd(&cnt[buf_slot[i]], 1u);
         __syncthreads();
-        if (tid < kQReq && cnt[tid])
-            base[tid] = ctrl->slot_off[tid] + atomicAdd(&ctrl->slot_fill[tid], cnt[tid]);
+        if (tid < kQReq && cnt[tid]) room[tid] = reserve(tid, cnt[tid], base[tid]);
         __syncthreads();
-        for (uint32_t i = tid; i < n; i += blockDim.x) list[base[buf_slot[i]] + buf_pos[i]] = buf_key[i];
+        for (uint32_t i = tid; i < n; i += blockDim.x)
+            if (buf_pos[i] < room[buf_slot[i]]) list[base[buf_slot[i]] + buf_pos[i]] = buf_key[i];
         __syncthreads();
         if (tid == 0) nbuf = 0;
         __syncthreads();
@@ -137,7 +146,8 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, unsigned n_pieces, unsig
                         buf_slot[pos] = (uint8_t)s;
                     } else {
                         // the stage is full until the block next looks at it: straight to the slot's list
-                        list[ctrl->slot_off[s] + atomicAdd(&ctrl->slot_fill[s], 1u)] = key;
+                        unsigned long long at;
+                        if (reserve(s, 1u, at)) list[at] = key;
                     }
                 }
             }
@@ -151,7 +161,7 @@ quantile_collect_kernel(const uint16_t* __restrict__ W, unsigned n_pieces, unsig
         // fl32(1 / s) for these scale bits
         const float r = MODE == AAAC_INT4 ? bf16_rcp(rl, ss & 0x7FFFu) : rl[ss & 0x7Fu];
         uint32_t bin[8], sl[8];
-        qbins<1>(v, r, bin);
+        qbins(v, r, bin);
 #pragma unroll
         for (int j = 0; j < 8; ++j) sl[j] = sm_slot[bin[j]];
         const uint32_t none = 0x80u & (sl[0] & sl[1] & sl[2]) & (sl[3] & sl[4] & sl[5]) & (sl[6] & sl[7]);

@@ -118,21 +118,19 @@ __device__ __forceinline__ uint64_t fma2_rd(uint64_t a, uint64_t b, uint64_t c) 
 }
 
 // The bins floor(1024 w~ + 8192) of the quantile start's histogram for a lane's eight normalised weights
-// w~ = fl32(w r), times UNIT (1, or 4 for byte offsets of counters): one multiply-add rounded down onto
-// 1.5 * 2^23 (where floats are spaced by 1) leaves the integer in the low mantissa bits, and the mask keeps
-// any input inside the table (|w~| < 8 by the scale rules, so for finite weights it changes nothing but the
-// low bits that UNIT = 4 leaves).  Two weights per instruction.
-template <int UNIT>
+// w~ = fl32(w r): one multiply-add rounded down onto 1.5 * 2^23 (where floats are spaced by 1) leaves the integer
+// in the low mantissa bits.  Two weights per instruction.  |w~| < 8 by the scale rules; in a group that holds a NaN
+// it may be anything, and the mask keeps it inside the table.  The pass that counts the bins and the one that
+// collects their weights both take them from here: a weight that they placed differently would have no room in its list.
 __device__ __forceinline__ void qbins(const uint4& v, float r, uint32_t (&bin)[8]) {
-    constexpr float kScale = 1024.f * UNIT, kAdd = 8192.f * UNIT + 12582912.f;
-    constexpr uint32_t kMask = (uint32_t)(kQBins - 1) * UNIT;
+    constexpr float kAdd = 8192.f + 12582912.f;
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     const uint64_t rr = pack2(r, r);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const uint64_t t = fma2_rd(mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr), pack2(kScale, kScale), pack2(kAdd, kAdd));
-        bin[2 * j] = __float_as_uint(lo2(t)) & kMask;
-        bin[2 * j + 1] = __float_as_uint(hi2(t)) & kMask;
+        const uint64_t t = fma2_rd(mul2(pack2(bf16_lo(w[j]), bf16_hi(w[j])), rr), pack2(1024.f, 1024.f), pack2(kAdd, kAdd));
+        bin[2 * j] = __float_as_uint(lo2(t)) & (uint32_t)(kQBins - 1);
+        bin[2 * j + 1] = __float_as_uint(hi2(t)) & (uint32_t)(kQBins - 1);
     }
 }
 

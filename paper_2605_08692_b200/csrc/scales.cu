@@ -204,10 +204,10 @@ scales_hist_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row,
                 r = rl[q];
                 if ((lane % LPG) == 0) reinterpret_cast<uint8_t*>(scales)[i / LPG] = (uint8_t)q;
             }
-            uint32_t off[8];
-            qbins<4>(v[u], r, off);
+            uint32_t bin[8];
+            qbins(v[u], r, bin);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(sm) + off[j]), 1u);
+            for (int j = 0; j < 8; ++j) atomicAdd(&sm[bin[j]], 1u);
         }
     }
     if (bad) {
