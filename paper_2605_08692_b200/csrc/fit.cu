@@ -88,6 +88,7 @@ struct FitParams {
     const uint8_t* scales;        // NVFP4 scale bytes
     const float* rinv;            // INT4 reciprocal scales
     const float* I;
+    const float* reach;           // what the caller's start tables add to the bound of the sums (a factor), or null
     Ctrl* ctrl;
     unsigned long long* acc;      // [3][kAccBuffer] words: fixed-point sums over the blocks, one buffer per pass in rotation
     double* err_trace;            // [n_rounds] or null
@@ -401,14 +402,16 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     }
 
     // Fixed-point scale of the sums over the blocks.  Every sum of a pass is below B = 256 N sum_k I_k
-    // (|w~ - c| < 16), so with 2^e > B the value v 2^(78 - e) fits the limbs; what is dropped lies 2^-78
-    // below B, far below the rounding of a block's own sums.  Integer addition is order-independent, so
-    // the totals do not depend on the order in which the blocks arrive.
+    // (|w~ - c| < 16, or more with tables of the caller's outside (-8, 8): then B is larger by that, squared), so
+    // with 2^e > B the value v 2^(78 - e) fits the limbs; what is dropped lies 2^-78 below B, far below the
+    // rounding of a block's own sums.  Integer addition is order-independent, so the totals do not depend on
+    // the order in which the blocks arrive.
     {
         float sum = 0.f;
         for (int k = tid; k < K; k += NT) sum = __fadd_ru(sum, fabsf(__ldg(p.I + k)));
 #pragma unroll
         for (int o = 16; o; o >>= 1) sum = __fadd_ru(sum, __shfl_xor_sync(kAll, sum, o));
+        if (p.reach) sum = __fmul_ru(sum, *p.reach);
         if (lane == 0) sh.wsum[warp][0] = (double)sum;
         __syncthreads();
         if (warp == 0) {
@@ -717,8 +720,11 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         // The sums go into the pass's buffer as two 40-bit limbs, each with one arrival in the word's upper
         // bits: lanes 0-1 of the half-warp add the residual sum's limbs, 2-3 those of the weight sum, 4-5 of
         // the last warp's first half those of the objective.
+        // A sum outside the limbs' range -- it cannot be right: an infinite or NaN weight or importance, reported by the
+        // passes that read them -- counts as none, so that it does not spill into the arrivals.
         const int which = sum_warp >> 1;
-        const double sd = (which == 0 ? dxs : which == 1 ? dys : de) * sh.fix_scale;
+        double sd = (which == 0 ? dxs : which == 1 ? dys : de) * sh.fix_scale;
+        if (!(fabs(sd) < 0x1p78)) sd = 0.0;
         const double topm = __dadd_rd(sd * 0x1p-40, kIntMagic);               // floor, as the low bits of a double near 1.5 2^52
         const long long top = __double_as_longlong(topm) - __double_as_longlong(kIntMagic);          // in [-2^38, 2^38)
         const double lowm = __dadd_rd(__fma_rn(-(topm - kIntMagic), 0x1p40, sd), kIntMagic);
@@ -914,7 +920,7 @@ static int64_t plan_layer(FitParams& p, int64_t N, int64_t K, int64_t blocks) {
 static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32_t* dev_status) {
     p = FitParams{};
     p.W = a.W; p.N = a.N; p.K = a.K; p.ldw = a.ldw;
-    p.scales = static_cast<const uint8_t*>(a.scales); p.rinv = a.ws.rinv; p.I = a.I;
+    p.scales = static_cast<const uint8_t*>(a.scales); p.rinv = a.ws.rinv; p.I = a.I; p.reach = a.reach;
     p.ctrl = a.ws.ctrl; p.acc = a.ws.acc; p.err_trace = a.err_trace; p.T01_out = a.T01_out; p.dev_status = dev_status;
     p.n_rounds = n_outer; p.trace_base = 0; p.bar_base = 0u;
     p.spin_limit = g_spin_limit;

@@ -547,7 +547,11 @@ __global__ void grid_init_kernel(Ctrl* ctrl, int mode, const float* T01_user) {
     chain_wait();
     if (t >= 2 * kM) return;
     if (T01_user) {
-        ctrl->T[t] = (double)T01_user[t];
+        const float T = T01_user[t];
+        const uint32_t tmax = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fabsf(T)));
+        const float reach = fmaxf(16.f, 8.f + __uint_as_float(tmax)) * 0.0625f;         // |w~| < 8; a round only brings entries in
+        ctrl->T[t] = (double)T;
+        if (t == 0) ctrl->reach = __fmul_ru(reach, reach);
         return;
     }
     const double e2m1[kM] = {-6, -4, -3, -2, -1.5, -1, -0.5, 0, 0, 0.5, 1, 1.5, 2, 3, 4, 6};

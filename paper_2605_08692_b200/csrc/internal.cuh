@@ -23,6 +23,7 @@ constexpr int kActMaxSplits = 128;  // row strips of the activation statistics
 // memset brings them to zero at the start of a fit.
 struct Ctrl {
     double T[2 * kM];               // current tables (double between rounds)
+    float reach;                    // INIT_USER: (how far from an entry a weight can be / 16) squared, 1 or more
     float s_t;                      // NVFP4 tensor scale
     uint32_t absmax_bits;           // layer max |w| as float bits (atomicMax on non-negative floats)
     uint32_t nonfinite;             // set if a non-finite weight was seen
@@ -181,6 +182,7 @@ struct FitLayerArgs {
     double* err_trace;
     float* T01_out;          // where the fitted tables go as FP32 (written by the last launch), or null
     Workspace ws;
+    const float* reach = nullptr;   // Ctrl::reach where the start tables are the caller's, else null
 };
 cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode, int sel_group, int n_outer, int n_inner,
                                     uint32_t* dev_status, cudaStream_t st);

@@ -45,3 +45,55 @@ def test_quantile_start_with_nan_groups_stays_inside_its_workspace():
     _, status = fit_only(dev_bf16(W.reshape(N, K)), INT4, torch.ones(K, device=DEV), 0, binding.INIT_QUANTILE, buf[:size])
     assert status & binding.DEV_NONFINITE
     assert bool((buf[size:] == 0xA5).all())
+
+
+def quantize_from_host(W, X, mode, rounds, init=binding.INIT_QUANTILE):
+    N, K, T = W.shape[0], W.shape[1], X.shape[0]
+    pin = lambda *a, **k: torch.empty(*a, **k).pin_memory()
+    out = dict(T01_host=pin(2, 16, dtype=torch.float32), T01_bf16_host=pin(2, 16, dtype=torch.int16),
+               scales_host=pin(N, K // binding.group_of(mode), dtype=torch.int16 if mode == INT4 else torch.uint8),
+               tensor_scale_host=pin(1, dtype=torch.float32), codes_host=pin(N, K // 2, dtype=torch.uint8),
+               err_out_host=pin(2, dtype=torch.float64))
+    ws = torch.empty(binding.host_workspace_bytes(mode, N, K, T), dtype=torch.uint8, device=DEV)
+    binding.quantize_layer_host(torch.from_numpy(W.view(np.int16)).pin_memory(), torch.from_numpy(X.view(np.int16)).pin_memory(), mode,
+                                n_outer=rounds, init=init, ws=ws, **out)
+    return out
+
+
+# (4096 x 1024 and 4096 x 512: a quarter and a half of the blocks share the column slab of the infinite importance)
+@pytest.mark.parametrize("mode,N,K", [(NVFP4, 4096, 1024), (NVFP4, 4096, 512), (INT4, 4096, 1024), (INT4, 64, 256)])
+@pytest.mark.parametrize("value", [0x7F80, 0xFF80, 0x7FC0])
+def test_nonfinite_activations_are_reported_as_such(mode, N, K, value):
+    """An infinite or NaN importance makes a cell's sums infinite: the blocks' exchange of sums has to end all the same."""
+    W, X = layer(mode, N, K, name=f"infact/{mode}/{N}x{K}")
+    X[5, 33] = value
+    r = binding.quantize_layer(dev_bf16(W), mode, X=dev_bf16(X), n_outer=5, init=binding.INIT_QUANTILE, want_trace=True)
+    torch.cuda.synchronize()
+    assert int(r["status"].item()) == binding.DEV_NONFINITE
+    with pytest.raises(binding.AaacError, match="Inf or NaN"):
+        quantize_from_host(W, X, mode, 5)
+
+
+@pytest.mark.parametrize("mode", [INT4, NVFP4])
+@pytest.mark.parametrize("n_inner", [1, 3])
+def test_nonfinite_weights_are_reported_after_rounds(mode, n_inner):
+    W, X = layer(mode, 300, 768, name=f"infw/{mode}")
+    W[7, 100], W[200, 5], W[31, 700] = 0x7F80, 0x7FC0, 0xFF80
+    r = binding.quantize_layer(dev_bf16(W), mode, X=dev_bf16(X), n_outer=3, n_inner=n_inner, init=binding.INIT_QUANTILE, want_trace=True)
+    torch.cuda.synchronize()
+    assert int(r["status"].item()) & (binding.DEV_NONFINITE | binding.DEV_TIMEOUT) == binding.DEV_NONFINITE
+
+
+@pytest.mark.parametrize("far", [30.0, 1000.0])
+def test_user_tables_far_outside_the_weights(far):
+    """Every weight is `far` and more away from its entry, and one block holds the whole layer: the first objective is the
+    largest sum a pass can have."""
+    W, X = layer(INT4, 16, 256, name="fartables")
+    T0 = np.stack([far + np.arange(16), far + 8 + np.arange(16)]).astype(np.float32)
+    o = oracle.fit_layer(W, INT4, 128, 2, X=X, init="user", T_init=T0)
+    r = binding.quantize_layer(dev_bf16(W), INT4, X=dev_bf16(X), n_outer=2, init=binding.INIT_USER, T01_init=torch.from_numpy(T0).to(DEV),
+                               want_trace=True)
+    torch.cuda.synchronize()
+    assert int(r["status"].item()) == 0
+    assert np.allclose(host(r["trace"]), o["trace"], rtol=1e-4)
+    assert table_close(host(r["T01"]), o["T"])[0]
