@@ -1,7 +1,7 @@
 // The fit rounds (Algorithm 1 lines 6-16).  With n_inner = 1 a round is the assignment step
 // (Eq. 8) and the activation-weighted centroid update (Eq. 11) in a single pass over W, and all
 // rounds of a layer run in ONE persistent kernel (one block per SM, cooperative launch): after
-// its pass every block adds its sums, as fixed-point integers of two 40-bit limbs, into 65 global
+// its pass every block adds its sums, as fixed-point integers of two 47-bit limbs, into 65 global
 // accumulators; every 64-bit accumulator word also counts, in its upper bits, the blocks that have
 // added to it, so a block knows that a total is complete by reading the total itself -- no separate
 // barrier, no fence between the sums and an arrival counter -- and every block ends up with the
@@ -107,16 +107,18 @@ struct FitParams {
 
 constexpr uint32_t kLut1At = 65536;                    // shared address of the bin table (see fit_rounds_body)
 constexpr int kFitWarps = 16;
-constexpr int kMaxFitBlocks = 1023;                   // grid limit: the arrivals are counted in 14 bits, the limbs' sums have 10 bits of room
-constexpr int kLimbs = 2;                             // a sum is a fixed-point number of two 40-bit limbs
-constexpr int kLimbBits = 40;
+constexpr int kMaxFitBlocks = 255;                    // grid limit: the limbs' sums have 8 bits of room, the arrivals are counted in the 9 above
+constexpr int kLimbs = 2;                             // a sum is a fixed-point number of two 47-bit limbs
+constexpr int kLimbBits = 47;
+constexpr double kLimb = (double)(1ll << kLimbBits);
+constexpr int kSumBits = 2 * kLimbBits - 1;           // a block's sum as an integer is below 2^kSumBits in magnitude
 constexpr unsigned kDefaultSpinLimit = 1u << 23;      // polls of several hundred ns each: seconds
 // An accumulator buffer: per cell the limbs of the residual sum and of the weight sum, 32 bytes next to one
 // another (four lanes add them with one request, a reader takes them with two loads), cells 128 bytes apart
 // so that the blocks' atomics on different cells do not queue behind one another; then the objective's.
 constexpr int kAccStride = 16;
 constexpr int kAccBuffer = (kCells + 1) * kAccStride;  // 64-bit words of one pass's buffer
-constexpr int kCountShift = 50;                       // an accumulator word: limb sum below, arrivals above
+constexpr int kCountShift = 55;                       // an accumulator word: limb sum below, arrivals above
 constexpr unsigned long long kLimbMask = (1ull << kCountShift) - 1ull;
 constexpr unsigned long long kOneArrival = 1ull << kCountShift;
 constexpr long long kTopBias = 1ll << (kLimbBits - 1);   // added to the (signed) top limb so that every block adds a non-negative number
@@ -401,11 +403,11 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         S.rlut[c] = c ? __frcp_rn(sv) : 0.f;
     }
 
-    // Fixed-point scale of the sums over the blocks.  Every sum of a pass is below B = 256 N sum_k I_k
-    // (|w~ - c| < 16, or more with tables of the caller's outside (-8, 8): then B is larger by that, squared), so
-    // with 2^e > B the value v 2^(78 - e) fits the limbs; what is dropped lies 2^-78 below B, far below the
-    // rounding of a block's own sums.  Integer addition is order-independent, so the totals do not depend on
-    // the order in which the blocks arrive.
+    // Fixed-point scale of the sums over the blocks.  The sums of a cell, and a sixteenth of the objective, are
+    // below B = 16 N sum_k I_k (|w~ - c| < 16, or more with tables of the caller's outside (-8, 8): then B is larger
+    // by that, squared), so with 2^e > B the value v 2^(93 - e) fits the limbs.  What is dropped lies 2^-93 below
+    // B: also a cell whose only weight has 10^-20 of the importances' sum moves its entry.  Integer addition is
+    // order-independent, so the totals do not depend on the order in which the blocks arrive.
     {
         float sum = 0.f;
         for (int k = tid; k < K; k += NT) sum = __fadd_ru(sum, fabsf(__ldg(p.I + k)));
@@ -418,11 +420,11 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             double B = sh.wsum[lane & 15][0];
 #pragma unroll
             for (int o = 8; o; o >>= 1) B += __shfl_xor_sync(kAll, B, o);
-            B *= 257.0 * (double)N;
+            B *= 257.0 / 16.0 * (double)N;
             if (lane == 0) {
                 const int e = B > 0.0 && B < 1e300 ? ilogb(B) + 1 : 0;
-                sh.fix_scale = scalbn(1.0, 78 - e);
-                sh.fix_unscale = scalbn(1.0, e - 78);
+                sh.fix_scale = scalbn(1.0, kSumBits - e);
+                sh.fix_unscale = scalbn(1.0, e - kSumBits);
                 sh.failed = 0;
             }
             derive_tables(S, lane, p.ctrl->T[lane]);
@@ -717,18 +719,18 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             dys += __shfl_xor_sync(kAll, dys, s);
             if (do_e) de += __shfl_xor_sync(kAll, de, s);
         }
-        // The sums go into the pass's buffer as two 40-bit limbs, each with one arrival in the word's upper
+        // The sums go into the pass's buffer as two 47-bit limbs, each with one arrival in the word's upper
         // bits: lanes 0-1 of the half-warp add the residual sum's limbs, 2-3 those of the weight sum, 4-5 of
         // the last warp's first half those of the objective.
         // A sum outside the limbs' range -- it cannot be right: an infinite or NaN weight or importance, reported by the
         // passes that read them -- counts as none, so that it does not spill into the arrivals.
         const int which = sum_warp >> 1;
-        double sd = (which == 0 ? dxs : which == 1 ? dys : de) * sh.fix_scale;
-        if (!(fabs(sd) < 0x1p78)) sd = 0.0;
-        const double topm = __dadd_rd(sd * 0x1p-40, kIntMagic);               // floor, as the low bits of a double near 1.5 2^52
-        const long long top = __double_as_longlong(topm) - __double_as_longlong(kIntMagic);          // in [-2^38, 2^38)
-        const double lowm = __dadd_rd(__fma_rn(-(topm - kIntMagic), 0x1p40, sd), kIntMagic);
-        const long long low = __double_as_longlong(lowm) - __double_as_longlong(kIntMagic);          // in [0, 2^40)
+        double sd = (which == 0 ? dxs : which == 1 ? dys : de * 0.0625) * sh.fix_scale;
+        if (!(fabs(sd) < 0x1p93)) sd = 0.0;
+        const double topm = __dadd_rd(sd * (1.0 / kLimb), kIntMagic);         // floor, as the low bits of a double near 1.5 2^52
+        const long long top = __double_as_longlong(topm) - __double_as_longlong(kIntMagic);          // in [-2^46, 2^46)
+        const double lowm = __dadd_rd(__fma_rn(-(topm - kIntMagic), kLimb, sd), kIntMagic);
+        const long long low = __double_as_longlong(lowm) - __double_as_longlong(kIntMagic);          // in [0, 2^47]
         const unsigned long long add = (unsigned long long)((sum_warp & 1) ? top + kTopBias : low) + kOneArrival;
         if (which < 2) atomicAdd(acc + sum_cell * kAccStride + sum_warp, add);
         else if (do_e && lane < 6 && which == 2) atomicAdd(acc + kCells * kAccStride + (lane - 4), add);
@@ -764,17 +766,18 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             if (lane == 0) sh.failed = 1;
         } else {
             auto total = [&](const unsigned long long (&w)[2]) {
-                const long long top = (long long)(w[1] & kLimbMask) - (long long)nblk * kTopBias;
-                const long long low = (long long)(w[0] & kLimbMask);
+                const unsigned long long sum = w[0] & kLimbMask;         // (its upper bits belong to the top limb)
+                const long long low = (long long)(sum & ((1ull << kLimbBits) - 1ull));
+                const long long top = (long long)(w[1] & kLimbMask) + (long long)(sum >> kLimbBits) - (long long)nblk * kTopBias;
                 const double t = __longlong_as_double(top + __double_as_longlong(kIntMagic)) - kIntMagic;
                 const double l = __longlong_as_double(low + __double_as_longlong(kIntMagic)) - kIntMagic;
-                return __fma_rn(t, 0x1p40, l) * sh.fix_unscale;
+                return __fma_rn(t, kLimb, l) * sh.fix_unscale;
             };
             // Eq. 11; cells of duplicate entries are empty: they keep their value
             const double sx = total(x), wt = total(y);
             double T = wt > 0.0 ? (double)S.centre[lane] + __ddiv_rn(sx, wt) : S.Td[lane];
             // the trace holds the Eq. 8 objective of each assignment step
-            if (my_e) p.err_trace[p.trace_base + round] = total(e);
+            if (my_e) p.err_trace[p.trace_base + round] = 16.0 * total(e);
             const double Tp = __shfl_up_sync(kAll, T, 1);
             if (__any_sync(kAll, (lane & 15) != 0 && Tp > T)) {
                 // ascending order within the table by rank (ties by index)

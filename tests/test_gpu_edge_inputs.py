@@ -97,3 +97,22 @@ def test_user_tables_far_outside_the_weights(far):
     assert int(r["status"].item()) == 0
     assert np.allclose(host(r["trace"]), o["trace"], rtol=1e-4)
     assert table_close(host(r["T01"]), o["T"])[0]
+
+
+def test_an_entry_of_one_weight_of_hardly_any_importance_moves():
+    """The sums over blocks are integers: their step has to lie far below every cell's weight, here 2^-60 of a channel's."""
+    N, K = 16, 256
+    rng = np.random.default_rng(8)
+    w = rng.uniform(-0.07, 0.07, (N, K)).astype(np.float32)
+    w[:, ::128] = -0.1                               # every group's largest magnitude, on the negative side ...
+    w[0, 0] = 0.1                                    # ... but one: the only weight next to the uppermost entries
+    I = np.ones(K, np.float32)
+    I[0] = 2.0 ** -60
+    T0 = np.stack([np.append(np.linspace(-7, 5, 15), 6.6), np.append(np.linspace(-6.5, 5.2, 15), 6.7)]).astype(np.float32)
+    W = synth.f32_to_bf16_bits(w)
+    o = oracle.fit_layer(W, INT4, 128, 1, I=I, init="user", T_init=T0)
+    assert (np.abs(o["T"][:, 15] - T0[:, 15]) > 0.2).sum() == 1
+    r = binding.quantize_layer(dev_bf16(W), INT4, I=torch.from_numpy(I).to(DEV), n_outer=1, init=binding.INIT_USER,
+                               T01_init=torch.from_numpy(T0).to(DEV))
+    torch.cuda.synchronize()
+    assert table_close(host(r["T01"]), o["T"])[0]
