@@ -692,7 +692,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             for (uint32_t t = 0; t < 4; ++t) {
                 const float2 a = lds_bin(cell_addr ^ (i + t * 8));
                 dx[t] += scaled_double(a.x);
-                dy[t] += __hiloint2double(__float_as_int(a.y) >> 3, __float_as_int(a.y) << 29);      // (weights are not negative)
+                dy[t] += scaled_double(a.y);
             }
         }
         sh.wsum[warp][lane] = ((dx[0] + dx[1]) + (dx[2] + dx[3])) * 0x1p896;

@@ -116,3 +116,16 @@ def test_an_entry_of_one_weight_of_hardly_any_importance_moves():
                                T01_init=torch.from_numpy(T0).to(DEV))
     torch.cuda.synchronize()
     assert table_close(host(r["T01"]), o["T"])[0]
+
+
+@pytest.mark.parametrize("mode,N,K", [(INT4, 64, 512), (NVFP4, 200, 640)])
+def test_negative_importances_of_the_callers(mode, N, K):
+    """Importances are sums of squares, but nothing checks a caller's: a few negative ones give finite, if odd, sums."""
+    g = binding.group_of(mode)
+    W, X = layer(mode, N, K, name=f"neg/{mode}")
+    I = oracle.act_stats(X)
+    I[5::97] *= -0.25
+    o = oracle.fit_layer(W, mode, g, 1, I=I, init="grid")
+    r = binding.quantize_layer(dev_bf16(W), mode, I=torch.from_numpy(I).to(DEV), n_outer=1, init=binding.INIT_GRID)
+    torch.cuda.synchronize()
+    assert table_close(host(r["T01"]), o["T"], rel=1e-4)[0]      # (terms of both signs cancel: ten times the usual bar)
