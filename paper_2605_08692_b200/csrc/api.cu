@@ -564,6 +564,7 @@ int aaac_quantize_layer_host_async(const void* W_host, int64_t N, int64_t K, int
     const size_t scale_bytes = (size_t)N * (K / g) * (mode == AAAC_INT4 ? 2 : 1);
     uint32_t* dstatus = reinterpret_cast<uint32_t*>(d + h.status);
     if ((unsigned long long)N * (unsigned long long)K >= (1ull << 32)) return AAAC_ERR_TOO_LARGE;
+    if (n_outer > (1 << 20)) return AAAC_ERR_SHAPE;
     const Workspace w = carve(d + h.ws, mode, N, K, ws_bytes - h.ws);
     const uint16_t* const W = reinterpret_cast<const uint16_t*>(d + h.W);
     const uint16_t* const X = reinterpret_cast<const uint16_t*>(d + h.X);

@@ -99,6 +99,7 @@ def test_argument_validation_happens_on_the_host(L):
     assert L.aaac_quantize_layer_host(None, 64, 256, 0, 128, ok, 8, 2, 0, ok, ok, ok, ok, ok, None, ok, big, None) == 1
     assert L.aaac_quantize_layer_host(ok, 64, 256, 0, 128, ok, 8, 2, 0, ok, ok, ok, ok, ok, None, ok,
                                       C.c_size_t(4096), None) == 5
+    assert L.aaac_quantize_layer_host(ok, 64, 256, 0, 128, ok, 8, (1 << 20) + 1, 0, ok, ok, ok, ok, ok, None, ok, big, None) == 3
 
 
 def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
