@@ -104,11 +104,13 @@ def _ptr(t):
 
 
 # The raw handle of the current stream: building a Stream object for it would take longer than all the
-# rest of a small call's host work.
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# rest of a small call's host work.  (Not a public name of torch: without it, the Stream object.)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
     return _raw_stream(torch.cuda.current_device())
 
 

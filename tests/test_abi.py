@@ -110,6 +110,17 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
         binding.workspace_bytes(0, 512, 512)
 
 
+def test_binding_needs_no_private_name_of_torch(monkeypatch):
+    import runpy
+    import types
+
+    import torch
+    from paper_2605_08692_b200 import binding
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1234))
+    assert runpy.run_path(binding.__file__)["_stream"]() == 0x1234
+
+
 def test_product_path_never_imports_the_oracle():
     pkg = os.path.join(ROOT, "paper_2605_08692_b200")
     for dirpath, _, files in os.walk(pkg):
