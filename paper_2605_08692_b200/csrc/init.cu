@@ -303,6 +303,7 @@ quantile_plan_kernel(Ctrl* ctrl, const uint32_t* __restrict__ hist, uint8_t* __r
         if (lead0) open(slot0, bin0, room - c0 - c1);
         if (lead1) open(slot1, bin1, room - c1);
     }
+    __syncwarp();                                            // lane 0 reads every lane's req_slot
     if (lane) return;
     if (!all_fit) {
         uint64_t seen = 0, fit = 0;                          // bins take their space in the order of the table entries

@@ -129,3 +129,27 @@ def test_negative_importances_of_the_callers(mode, N, K):
     r = binding.quantize_layer(dev_bf16(W), mode, I=torch.from_numpy(I).to(DEV), n_outer=1, init=binding.INIT_GRID)
     torch.cuda.synchronize()
     assert table_close(host(r["T01"]), o["T"], rel=1e-4)[0]      # (terms of both signs cancel: ten times the usual bar)
+
+
+@pytest.mark.parametrize("mode", [INT4, NVFP4])
+def test_quantile_start_with_room_for_some_of_the_bins(mode):
+    """Which bins get space in a list that cannot hold all of them goes by the requests' slots, which every lane of a warp
+    writes and one reads.  Bins of one value each are answered with or without space: the tables are those of a list that
+    holds everything, whatever fits."""
+    N, K, g = 300, 768, binding.group_of(mode)
+    rng = np.random.default_rng(6)
+    vals = (np.arange(-20, 21) * 0.33).astype(np.float32)          # 41 values in as many bins, 2 to 11 thousand weights each
+    p = np.exp(-0.5 * (np.arange(-20, 21) / 9.0) ** 2)
+    w = rng.choice(vals, size=(N, K), p=p / p.sum())
+    w[:, ::g] = 7.0                                                # one scale for all groups
+    W = dev_bf16(synth.f32_to_bf16_bits(w))
+    I = torch.ones(K, device=DEV)
+    want, status = fit_only(W, mode, I, 0, binding.INIT_QUANTILE, binding.alloc_workspace(mode, N, K, full=True))
+    assert status == 0
+    try:
+        for cap in (1000, 6000, 20000, 60000, 150000):
+            binding.debug_quantile_cap(cap)
+            got, status = fit_only(W, mode, I, 0, binding.INIT_QUANTILE, binding.alloc_workspace(mode, N, K))
+            assert status == 0 and np.array_equal(got, want), cap
+    finally:
+        binding.debug_quantile_cap(0)
