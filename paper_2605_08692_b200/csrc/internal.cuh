@@ -136,9 +136,9 @@ __device__ __forceinline__ void qbins(const uint4& v, float r, uint32_t (&bin)[8
 }
 
 // fl32(1 / s) of a positive BF16 scale, from fl32(1 / (1 + m / 128)) per mantissa m: a power of two more does
-// not change the rounding (scales are 2^-126 or more).
+// not change the rounding (scales are 2^-126 or more; that of a group with an infinite weight is infinite, and 0 here).
 __device__ __forceinline__ float bf16_rcp(const float* lut, uint32_t b) {
-    return __fmul_rn(lut[b & 0x7Fu], __uint_as_float((254u - ((b >> 7) & 0xFFu)) << 23));
+    return __fmul_rn(lut[b & 0x7Fu], __uint_as_float((uint32_t)max(254 - (int)((b >> 7) & 0xFFu), 0) << 23));
 }
 __device__ __forceinline__ float bf16_rcp_entry(uint32_t m) { return __frcp_rn(1.f + (float)m * 0.0078125f); }
 

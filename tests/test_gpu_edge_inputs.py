@@ -153,3 +153,27 @@ def test_quantile_start_with_room_for_some_of_the_bins(mode):
             assert status == 0 and np.array_equal(got, want), cap
     finally:
         binding.debug_quantile_cap(0)
+
+
+def test_quantile_start_of_a_group_with_an_infinite_weight():
+    """The group's scale is infinite, its finite weights are 0 of it and the infinite one is NaN, which sorts last: the start
+    tables are the order statistics of that."""
+    N, K = 40, 512
+    W, _ = layer(INT4, N, K, name="infgroup")
+    W[3, 140] = 0x7F80
+    zeroed = W.copy()
+    zeroed[3, 128:256] = 0
+    s, ts = oracle.scales(zeroed, INT4, 128)
+    x = oracle.normalise(zeroed, INT4, 128, s, ts).reshape(N, K).astype(np.float64)
+    x[3, 140] = np.inf
+    x = np.sort(x.reshape(-1))
+    q = np.concatenate([np.arange(16) / 15.0, 1 / 30.0 + (1 - 1 / 30.0) * np.arange(16) / 15.0])
+    pos = q * (x.size - 1)
+    lo = np.floor(pos).astype(int)
+    with np.errstate(invalid="ignore"):
+        want = (x[lo] + (pos - lo) * (x[np.minimum(lo + 1, x.size - 1)] - x[lo])).astype(np.float32).reshape(2, 16)
+    got, status = fit_only(dev_bf16(W), INT4, torch.ones(K, device=DEV), 0, binding.INIT_QUANTILE,
+                           binding.alloc_workspace(INT4, N, K, full=True))
+    assert status == binding.DEV_NONFINITE
+    assert np.isfinite(want[:, :15]).all() and np.array_equal(got[:, :15], want[:, :15])
+    assert not np.isfinite(got[:, 15]).any()
