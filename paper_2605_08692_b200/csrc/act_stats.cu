@@ -23,7 +23,7 @@ constexpr int kBlocksPerSM = 4;          // resident blocks: 64 KB of loads in f
 
 // |a| of a BF16 value as a double (upper word; the lower is zero).  A zero or a denormal reads as some
 // 2^-127 <= |a| < 2^-126, whose square is below 2^-252 and vanishes in an FP32 sum; Inf and NaN read as
-// 2^128 and more, whose square makes the FP32 sum infinite.
+// 2^128 and more, whose square is beyond an FP32 sum (see finish).
 __device__ __forceinline__ double abs_lo(uint32_t w) { return __hiloint2double((int)((w & 0x7FFFu) * 8192u + 0x38000000u), 0); }
 __device__ __forceinline__ double abs_hi(uint32_t w) { return __hiloint2double((int)(((w & 0x7FFF0000u) >> 3) + 0x38000000u), 0); }
 __device__ __forceinline__ void add_squares(double (&s)[8], uint4 v) {
@@ -38,6 +38,7 @@ __device__ __forceinline__ void add_squares(double (&s)[8], uint4 v) {
 
 __device__ __forceinline__ void finish(float* I, int64_t k, double s, int accumulate, uint32_t* dev_status) {
     float v = (float)s;
+    if (isinf(v)) v = __int_as_float(0x7FFFFFFF);          // NaN: Inf and NaN among the inputs cannot be told apart any more
     if (accumulate) v += I[k];
     I[k] = v;
     if (dev_status && !isfinite(v)) atomicOr(dev_status, AAAC_DEV_NONFINITE);

@@ -177,3 +177,19 @@ def test_quantile_start_of_a_group_with_an_infinite_weight():
     assert status == binding.DEV_NONFINITE
     assert np.isfinite(want[:, :15]).all() and np.array_equal(got[:, :15], want[:, :15])
     assert not np.isfinite(got[:, 15]).any()
+
+
+@pytest.mark.parametrize("T", [40, 1000])                   # one strip, and several
+@pytest.mark.parametrize("value", [0x7F80, 0xFF80, 0x7FC0])
+def test_importance_of_a_channel_with_a_nonfinite_activation(T, value):
+    K = 264
+    X = synth.activations(T, K, 4, f"nonfinite/{T}", kind="lognormal")
+    want = oracle.act_stats(X)
+    X[T // 2, 7] = value
+    ws, I = binding.alloc_workspace(NVFP4, 1, K), torch.ones(K, dtype=torch.float32, device=DEV)
+    for accumulate in (False, True):
+        st = torch.zeros(1, dtype=torch.int32, device=DEV)
+        binding.act_stats(dev_bf16(X), I, ws, accumulate=accumulate, dev_status=st)
+        got = host(I)
+        assert int(st.item()) == binding.DEV_NONFINITE and np.isnan(got[7])
+        assert np.allclose(np.delete(got, 7), np.delete(want, 7) * (1 + accumulate), rtol=1e-6, atol=0)
