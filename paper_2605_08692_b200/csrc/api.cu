@@ -3,6 +3,7 @@
 #include <atomic>
 #include <cstddef>
 #include <mutex>
+#include <utility>
 
 #include "internal.cuh"
 
@@ -120,8 +121,6 @@ struct SideStreams {
     bool tried = false, ok = false;
     cudaStream_t s[kSideStreams];
     cudaEvent_t fork, join[kSideStreams];
-    cudaEvent_t step;              // what one stream of a host-buffer call waits for on the other (re-recorded, see HostLanes)
-    unsigned next_copy = 0;        // the side stream the next host-buffer call copies on
 };
 std::mutex g_side_mu;                  // held while a call queues work on the side streams
 SideStreams g_side[kMaxDevices];
@@ -133,8 +132,7 @@ SideStreams* side_streams() {
     SideStreams& p = g_side[dev];
     if (!p.tried) {
         p.tried = true;
-        bool ok = cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&p.step, cudaEventDisableTiming) == cudaSuccess;
+        bool ok = cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < kSideStreams && ok; ++i)
             ok = cudaStreamCreateWithFlags(&p.s[i], cudaStreamNonBlocking) == cudaSuccess &&
                  cudaEventCreateWithFlags(&p.join[i], cudaEventDisableTiming) == cudaSuccess;
@@ -182,17 +180,45 @@ private:
     bool ok_ = true;
 };
 
-// The two streams of a host-buffer call: the caller's, with the kernels, and one for the copies (a side
-// stream, taken in turn; or the caller's own, where overlapping is not worth the events).  to_kernels() /
-// to_copies() make the one stream wait for what the other holds so far: a wait takes the event as it was
-// recorded last, so one event serves all of them.
+// The copy stream that a host-buffer call borrows, and the event that orders it against the caller's stream.
+// One call at a time has it, from its first copy to its return; no call waits for another's -- a copy from or to
+// pageable memory returns only when it is done, and the whole call may lie before it -- but takes the next free one.
+constexpr int kHostLanes = 7;
+struct HostLane {
+    std::mutex mu;
+    bool tried = false, ok = false;
+    cudaStream_t copies;
+    cudaEvent_t step;              // what one stream waits for on the other (re-recorded, see HostLanes)
+};
+HostLane g_host_lane[kMaxDevices][kHostLanes];
+std::atomic<unsigned> g_host_calls{0};
+
+// The two streams of a host-buffer call: the caller's, with the kernels, and one for the copies (or the caller's own,
+// where overlapping is not worth the events, or no copy stream is free).  to_kernels() / to_copies() make the one
+// stream wait for what the other holds so far: a wait takes the event as it was recorded last, so one event serves
+// all of them.
 class HostLanes {
 public:
-    HostLanes(cudaStream_t st, bool overlap) : lk_(g_side_mu, std::defer_lock), st_(st), cp_(st) {
-        if (!overlap) return;
-        lk_.lock();
-        side_ = side_streams();
-        if (side_) cp_ = side_->s[side_->next_copy++ % kSideStreams];
+    HostLanes(cudaStream_t st, bool overlap) : st_(st), cp_(st) {
+        int dev = -1;
+        if (!overlap || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
+        const unsigned at = g_host_calls.fetch_add(1, std::memory_order_relaxed);
+        for (unsigned i = 0; i < kHostLanes; ++i) {
+            HostLane& l = g_host_lane[dev][(at + i) % kHostLanes];
+            std::unique_lock<std::mutex> lk(l.mu, std::try_to_lock);
+            if (!lk) continue;
+            if (!l.tried) {
+                l.tried = true;
+                l.ok = cudaStreamCreateWithFlags(&l.copies, cudaStreamNonBlocking) == cudaSuccess &&
+                       cudaEventCreateWithFlags(&l.step, cudaEventDisableTiming) == cudaSuccess;
+                if (!l.ok) cudaGetLastError();
+            }
+            if (!l.ok) return;
+            lk_ = std::move(lk);
+            step_ = l.step;
+            cp_ = l.copies;
+            return;
+        }
     }
     cudaStream_t copies() const { return cp_; }
     bool overlapped() const { return cp_ != st_; }
@@ -200,10 +226,10 @@ public:
     bool to_kernels() { return pass(cp_, st_); }
 private:
     bool pass(cudaStream_t from, cudaStream_t to) {
-        return from == to || (cudaEventRecord(side_->step, from) == cudaSuccess && cudaStreamWaitEvent(to, side_->step, 0) == cudaSuccess);
+        return from == to || (cudaEventRecord(step_, from) == cudaSuccess && cudaStreamWaitEvent(to, step_, 0) == cudaSuccess);
     }
     std::unique_lock<std::mutex> lk_;
-    SideStreams* side_ = nullptr;
+    cudaEvent_t step_ = nullptr;
     cudaStream_t st_, cp_;
 };
 

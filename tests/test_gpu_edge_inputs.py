@@ -1,4 +1,7 @@
 """Inputs at the edges of what the entry points take: they are answered, or reported, and touch nothing else."""
+import threading
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -47,17 +50,18 @@ def test_quantile_start_with_nan_groups_stays_inside_its_workspace():
     assert bool((buf[size:] == 0xA5).all())
 
 
-def quantize_from_host(W, X, mode, rounds, init=binding.INIT_QUANTILE):
+def host_call(W, X, mode, rounds, init=binding.INIT_QUANTILE, pinned=True):
+    """A host-buffer call with all its buffers: a function that makes it, and the outputs it fills."""
     N, K, T = W.shape[0], W.shape[1], X.shape[0]
-    pin = lambda *a, **k: torch.empty(*a, **k).pin_memory()
-    out = dict(T01_host=pin(2, 16, dtype=torch.float32), T01_bf16_host=pin(2, 16, dtype=torch.int16),
-               scales_host=pin(N, K // binding.group_of(mode), dtype=torch.int16 if mode == INT4 else torch.uint8),
-               tensor_scale_host=pin(1, dtype=torch.float32), codes_host=pin(N, K // 2, dtype=torch.uint8),
-               err_out_host=pin(2, dtype=torch.float64))
+    pin = lambda t: t.pin_memory() if pinned else t
+    out = dict(T01_host=torch.empty(2, 16), T01_bf16_host=torch.empty(2, 16, dtype=torch.int16),
+               scales_host=torch.empty(N, K // binding.group_of(mode), dtype=torch.int16 if mode == INT4 else torch.uint8),
+               tensor_scale_host=torch.empty(1), codes_host=torch.empty(N, K // 2, dtype=torch.uint8),
+               err_out_host=torch.empty(2, dtype=torch.float64))
+    out = {k: pin(v) for k, v in out.items()}
+    Wh, Xh = pin(torch.from_numpy(W.view(np.int16))), pin(torch.from_numpy(X.view(np.int16)))
     ws = torch.empty(binding.host_workspace_bytes(mode, N, K, T), dtype=torch.uint8, device=DEV)
-    binding.quantize_layer_host(torch.from_numpy(W.view(np.int16)).pin_memory(), torch.from_numpy(X.view(np.int16)).pin_memory(), mode,
-                                n_outer=rounds, init=init, ws=ws, **out)
-    return out
+    return lambda: binding.quantize_layer_host(Wh, Xh, mode, n_outer=rounds, init=init, ws=ws, **out), out
 
 
 # (4096 x 1024 and 4096 x 512: a quarter and a half of the blocks share the column slab of the infinite importance)
@@ -71,7 +75,7 @@ def test_nonfinite_activations_are_reported_as_such(mode, N, K, value):
     torch.cuda.synchronize()
     assert int(r["status"].item()) == binding.DEV_NONFINITE
     with pytest.raises(binding.AaacError, match="Inf or NaN"):
-        quantize_from_host(W, X, mode, 5)
+        host_call(W, X, mode, 5)[0]()
 
 
 @pytest.mark.parametrize("mode", [INT4, NVFP4])
@@ -193,3 +197,55 @@ def test_importance_of_a_channel_with_a_nonfinite_activation(T, value):
         got = host(I)
         assert int(st.item()) == binding.DEV_NONFINITE and np.isnan(got[7])
         assert np.allclose(np.delete(got, 7), np.delete(want, 7) * (1 + accumulate), rtol=1e-6, atol=0)
+
+
+def batch(mode, N, K, n):
+    """n layers for quantize_layers"""
+    g, out = binding.group_of(mode), []
+    for l in range(n):
+        W, X = layer(mode, N, K, name=f"batch/{mode}/{l}")
+        out.append(dict(W=dev_bf16(W), X=dev_bf16(X), T01=torch.zeros(2, 16, device=DEV), T01_bf16=torch.zeros(2, 16, dtype=torch.bfloat16, device=DEV),
+                        scales=torch.zeros(N, K // g, dtype=torch.int16 if mode == INT4 else torch.uint8, device=DEV),
+                        tensor_scale=torch.ones(1, device=DEV), codes=torch.zeros(N, K // 2, dtype=torch.uint8, device=DEV),
+                        ws=binding.alloc_workspace(mode, N, K, X.shape[0])))
+    return out
+
+
+def test_calls_of_other_threads_do_not_wait_for_a_host_buffer_call():
+    """A host-buffer call returns when its stream is done, here behind about a second of other work; meanwhile another thread
+    queues a batch, and runs a host-buffer call of its own."""
+    W, X = layer(NVFP4, 1100, 2048, name="threads")
+    layers, streams = batch(NVFP4, 256, 512, 2), [torch.cuda.Stream(), torch.cuda.Stream()]
+    (call, mine), (slow_call, theirs) = host_call(W, X, NVFP4, 3), host_call(W, X, NVFP4, 3)
+    run_batch = lambda: binding.quantize_layers(layers, NVFP4, n_outer=2, init=binding.INIT_QUANTILE)
+    with torch.cuda.stream(streams[1]):                    # (what a first use loads or creates, every copy stream among it, is there)
+        run_batch()
+        for _ in range(8):
+            call()
+    with torch.cuda.stream(streams[0]):
+        torch.cuda._sleep(1000)
+        slow_call()
+    want = {k: v.clone() for k, v in mine.items()}
+    torch.cuda.synchronize()
+
+    t0, at = time.perf_counter(), {}
+
+    def behind_other_work():
+        with torch.cuda.stream(streams[0]):
+            torch.cuda._sleep(2_000_000_000)
+            slow_call()
+        at["slow call"] = time.perf_counter() - t0
+
+    t = threading.Thread(target=behind_other_work)
+    t.start()
+    time.sleep(0.2)
+    with torch.cuda.stream(streams[1]):
+        run_batch()
+        at["batch"] = time.perf_counter() - t0
+        call()
+        at["call"] = time.perf_counter() - t0
+    t.join()
+    torch.cuda.synchronize()
+    assert at["call"] < 0.7 * at["slow call"], at
+    for k, v in want.items():
+        assert torch.equal(mine[k], v) and torch.equal(theirs[k], v), k
