@@ -193,6 +193,13 @@ struct HostLane {
 HostLane g_host_lane[kMaxDevices][kHostLanes];
 std::atomic<unsigned> g_host_calls{0};
 
+bool page_locked(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type != cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    return false;
+}
+
 // The two streams of a host-buffer call: the caller's, with the kernels, and one for the copies (or the caller's own,
 // where overlapping is not worth the events, or no copy stream is free).  to_kernels() / to_copies() make the one
 // stream wait for what the other holds so far: a wait takes the event as it was recorded last, so one event serves
@@ -599,8 +606,10 @@ int aaac_quantize_layer_host_async(const void* W_host, int64_t N, int64_t K, int
     float* const ts = reinterpret_cast<float*>(d + h.ts);
     // Copies on a stream of their own: the scales and start passes, which need W alone, run while X arrives, X is
     // summed piece by piece as it does, and the codes of packed rows leave while the next rows are packed.  The
-    // events cost some 10 us of host time, which copies of 4 MB and more hide.
-    HostLanes lanes(st, (size_t)(N + T) * (size_t)K * 2 >= ((size_t)4 << 20));
+    // events cost some 10 us of host time, which copies of 4 MB and more hide.  Copies from and to pageable memory
+    // do not run beside anything, and the pieces then cost 2-6 %.
+    HostLanes lanes(st, (size_t)(N + T) * (size_t)K * 2 >= ((size_t)4 << 20) && page_locked(W_host) && page_locked(X_host) &&
+                            page_locked(codes_host) && page_locked(scales_host));
     cudaStream_t const cp = lanes.copies();
     cudaError_t e = cudaSuccess;
     auto run = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };

@@ -249,3 +249,16 @@ def test_calls_of_other_threads_do_not_wait_for_a_host_buffer_call():
     assert at["call"] < 0.7 * at["slow call"], at
     for k, v in want.items():
         assert torch.equal(mine[k], v) and torch.equal(theirs[k], v), k
+
+
+def test_pageable_host_buffers_give_what_page_locked_ones_do():
+    W, X = layer(NVFP4, 1100, 2048, T=100, name="pageable")
+    (pinned, want), (pageable, got) = host_call(W, X, NVFP4, 3), host_call(W, X, NVFP4, 3, pinned=False)
+    pinned()
+    before = binding.launch_count()
+    pageable()
+    assert binding.launch_count() - before == 9      # absmax, scales, plan, collect, select, importances (2), rounds, one pack of all rows
+    for k in want:
+        assert torch.equal(got[k], want[k]) or k == "err_out_host", k
+    # (a lane adds up to 16 rows' terms in FP32, other rows where the pass runs by row ranges: 16 roundings of 2^-24)
+    assert torch.allclose(got["err_out_host"], want["err_out_host"], rtol=1e-6)
