@@ -208,7 +208,10 @@ class HostLanes {
 public:
     HostLanes(cudaStream_t st, bool overlap) : st_(st), cp_(st) {
         int dev = -1;
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         if (!overlap || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) { cudaGetLastError(); return; }
+        if (capture != cudaStreamCaptureStatusNone) return;         // (the copy stream would be part of the graph until the capture ends)
         const unsigned at = g_host_calls.fetch_add(1, std::memory_order_relaxed);
         for (unsigned i = 0; i < kHostLanes; ++i) {
             HostLane& l = g_host_lane[dev][(at + i) % kHostLanes];

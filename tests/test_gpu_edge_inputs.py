@@ -50,7 +50,7 @@ def test_quantile_start_with_nan_groups_stays_inside_its_workspace():
     assert bool((buf[size:] == 0xA5).all())
 
 
-def host_call(W, X, mode, rounds, init=binding.INIT_QUANTILE, pinned=True):
+def host_call(W, X, mode, rounds, init=binding.INIT_QUANTILE, pinned=True, queue_only=False):
     """A host-buffer call with all its buffers: a function that makes it, and the outputs it fills."""
     N, K, T = W.shape[0], W.shape[1], X.shape[0]
     pin = lambda t: t.pin_memory() if pinned else t
@@ -61,6 +61,9 @@ def host_call(W, X, mode, rounds, init=binding.INIT_QUANTILE, pinned=True):
     out = {k: pin(v) for k, v in out.items()}
     Wh, Xh = pin(torch.from_numpy(W.view(np.int16))), pin(torch.from_numpy(X.view(np.int16)))
     ws = torch.empty(binding.host_workspace_bytes(mode, N, K, T), dtype=torch.uint8, device=DEV)
+    if queue_only:
+        st = pin(torch.zeros(1, dtype=torch.int32))
+        return lambda: binding.quantize_layer_host_async(Wh, Xh, mode, n_outer=rounds, init=init, ws=ws, status_host=st, **out), out
     return lambda: binding.quantize_layer_host(Wh, Xh, mode, n_outer=rounds, init=init, ws=ws, **out), out
 
 
@@ -262,3 +265,51 @@ def test_pageable_host_buffers_give_what_page_locked_ones_do():
         assert torch.equal(got[k], want[k]) or k == "err_out_host", k
     # (a lane adds up to 16 rows' terms in FP32, other rows where the pass runs by row ranges: 16 roundings of 2^-24)
     assert torch.allclose(got["err_out_host"], want["err_out_host"], rtol=1e-6)
+
+
+def test_host_buffer_calls_beside_the_capture_of_one():
+    """A captured call leaves nothing that other calls use in its graph: they go on while the capture is open, and the graph
+    gives what the call gives."""
+    W, X = layer(NVFP4, 1100, 2048, name="capture")
+    (call, want), (captured, got) = host_call(W, X, NVFP4, 3, queue_only=True), host_call(W, X, NVFP4, 3, queue_only=True)
+    beside, other = torch.cuda.Stream(), torch.cuda.Stream()
+    captured()
+    with torch.cuda.stream(beside):
+        call()
+    torch.cuda.synchronize()
+    for t in got.values():
+        t.zero_()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=other, capture_error_mode="relaxed"):
+        captured()
+        with torch.cuda.stream(beside):
+            for _ in range(8):
+                call()
+    graph.replay()
+    torch.cuda.synchronize()
+    for k, v in want.items():
+        assert torch.equal(got[k], v) or k == "err_out_host", k
+    assert torch.allclose(got["err_out_host"], want["err_out_host"], rtol=1e-6)      # (row ranges, see above)
+
+
+@pytest.mark.parametrize("mode,n_inner", [(INT4, 1), (NVFP4, 2)])
+def test_captured_batch_gives_what_the_call_gives(mode, n_inner):
+    """Side streams, the chain of dependent launches and the cooperative rounds as a graph."""
+    layers = batch(mode, 300, 768, 3)
+    run = lambda: binding.quantize_layers(layers, mode, n_outer=3, n_inner=n_inner, init=binding.INIT_QUANTILE)
+    run()
+    torch.cuda.synchronize()
+    names = ("T01", "T01_bf16", "scales", "codes")
+    want = [{k: d[k].clone() for k in names} for d in layers]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    for d in layers:
+        for k in names:
+            d[k].zero_()
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    for d, w in zip(layers, want):
+        for k in names:
+            assert torch.equal(d[k], w[k]), k
