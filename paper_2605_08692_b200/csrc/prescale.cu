@@ -14,9 +14,9 @@ namespace aaac {
 namespace {
 
 __global__ void __launch_bounds__(256)
-prescale_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, const float* __restrict__ a,
-                uint16_t* __restrict__ Wout, int64_t ldo, int rows_per_block, const float* __restrict__ I,
-                float* __restrict__ Iout, uint32_t* dev_status) {
+prescale_kernel(const uint16_t* __restrict__ W, int64_t N, int64_t K, int64_t ldw, const float* a,
+                uint16_t* __restrict__ Wout, int64_t ldo, int rows_per_block, const float* I,
+                float* Iout, uint32_t* dev_status) {
     const int64_t col = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
     if (col >= K) return;
     chain_next();
@@ -70,8 +70,14 @@ cudaError_t launch_prescale(const uint16_t* W, int64_t N, int64_t K, int64_t ldw
     int64_t rows = (N + strips - 1) / strips;
     rows = (rows + 3) / 4 * 4;
     strips = (N + rows - 1) / rows;
+    // I' written over the multipliers: by a launch of its own (no rows), once all strips have read them.
+    const bool over_a = I && Iout < a + K && a < Iout + K;
     note_launch();
-    return launch_chained(prescale_kernel, dim3(bx, (unsigned)strips), 256, 0, st, W, N, K, ldw, a, Wout, ldo, (int)rows, I, Iout, dev_status);
+    const cudaError_t e = launch_chained(prescale_kernel, dim3(bx, (unsigned)strips), 256, 0, st, W, N, K, ldw, a, Wout, ldo, (int)rows,
+                                         over_a ? nullptr : I, Iout, dev_status);
+    if (e != cudaSuccess || !over_a) return e;
+    note_launch();
+    return launch_chained(prescale_kernel, dim3(bx, 1), 256, 0, st, W, (int64_t)0, K, ldw, a, Wout, ldo, 0, I, Iout, (uint32_t*)nullptr);
 }
 
 }  // namespace aaac

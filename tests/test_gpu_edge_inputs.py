@@ -313,3 +313,18 @@ def test_captured_batch_gives_what_the_call_gives(mode, n_inner):
     for d, w in zip(layers, want):
         for k in names:
             assert torch.equal(d[k], w[k]), k
+
+
+def test_prescaled_importances_may_replace_the_multipliers():
+    N, K = 4096, 2048
+    W, _ = layer(NVFP4, N, K, name="over_a")
+    rng = np.random.default_rng(9)
+    a, I = np.exp(0.5 * rng.standard_normal(K)).astype(np.float32), np.exp(rng.standard_normal(K)).astype(np.float32)
+    Wd, a_then_I, Id = dev_bf16(W), torch.from_numpy(a).to(DEV), torch.from_numpy(I).to(DEV)
+    want, I_want = torch.empty_like(Wd), torch.empty_like(Id)
+    binding.prescale_columns(Wd, a_then_I, want, I=Id, I_out=I_want)
+    got = torch.empty_like(Wd)
+    binding.prescale_columns(Wd, a_then_I, got, I=Id, I_out=a_then_I)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want) and torch.equal(a_then_I, I_want)
+    assert np.array_equal(host(I_want), (I.astype(np.float64) / (a.astype(np.float64) ** 2)).astype(np.float32))
