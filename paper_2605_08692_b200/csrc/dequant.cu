@@ -81,7 +81,8 @@ dequant_kernel(const uint32_t* __restrict__ codes, const void* __restrict__ scal
             }
             int64_t at = w * 8;
             if (GAPS) {
-                const int64_t row = w / per_row;
+                // (with selection bytes, a 32-bit division where it will do: 14336 x 4096 38.5 -> 37.9 us; without, that is 1 % slower)
+                const int64_t row = SEP && words <= 0xFFFFFFFFll ? (int64_t)((uint32_t)w / per_row) : w / per_row;
                 at = row * ldo + (w - row * per_row) * 8;
             }
             __stcs(reinterpret_cast<uint4*>(What + at), make_uint4(o[0], o[1], o[2], o[3]));
