@@ -219,8 +219,8 @@ int aaac_dequant_sel(const uint8_t* codes, const void* scales, const uint8_t* si
  * the fitted tables agree to about 1e-7 relative and are bitwise reproducible from call to call).
  * With n_inner = 1 the rounds of up to eight layers run in one launch, each layer on its own
  * share of the blocks, so that the cost of a round that does not depend on the layer's size is
- * paid once per batch and small layers do not leave most of the GPU idle; more layers, and
- * n_inner > 1, are run in turn.  Scales, importances (from X where I is NULL) and start tables
+ * paid once per batch and small layers do not leave most of the GPU idle; more layers are run in
+ * turn.  (With n_inner > 1 a round is two launches, of up to eight layers each.)  Scales, importances (from X where I is NULL) and start tables
  * are computed per layer exactly as by aaac_fit_layer_sel, except that layers given the same
  * activations (the same X, T, K and ldx, with I == NULL) share their importances, which are
  * computed once (into the workspace of the first of them).  With more than one layer these

@@ -6,7 +6,7 @@
 // instructions (its fields moved, the exponent rebased), and one double-precision multiply-add
 // squares it -- exactly -- and adds it, so a sum is off by a few 2^-53.  That is three
 // instructions an element where error-free FP32 pairs took nine, and leaves the pass to the
-// memory (16384 x 14336: 4.2 -> 5.9 TB/s with the launch geometry below).  A second kernel adds
+// memory (16384 x 14336: 4.2 -> 5.8 TB/s with the launch geometry below).  A second kernel adds
 // the strip partials in a fixed order and rounds once to FP32.
 #include <algorithm>
 #include <mutex>

@@ -101,7 +101,7 @@ struct FitParams {
     unsigned arrivals;            // blocks whose sums a total must hold before it is read (the grid size)
     unsigned spin_limit;          // polls of a total before the wait is given up
     int rows;                     // rows per warp of an item: 4, or 2 or 1 for layers that have too few items of 4
-    int items, per_block, nrb;    // items of (16 rows) x 256 columns, items per block, row blocks per slab
+    int items, per_block, nrb;    // items of 16 * rows rows x 256 columns, items per block, row blocks per slab
     int tail_item0, tail_quarters;   // items from tail_item0 on are dealt out a quarter (one row per warp) per block
 };
 
@@ -581,7 +581,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             group_sums<LPG>(e0, e1, lane);
             const float es = e0 + e1;
             const float tau = __fmaf_ru(es, g1, isum);
-            // lanes past K carry I = 0 and w~ = 0; they need the exact path only if their slot is
+            // lanes past K carry I = 0 and the row's last weights; they need the exact path only if their slot is
             // poisoned (NaN), so that no NaN reaches a bin
             const bool near = !(fabsf(e1 - e0) > tau) && (col_ok || !(es == es));
             const bool sg = e1 < e0;

@@ -19,7 +19,7 @@ def _built():
     (INT4, 512, 512),        # items of one row per warp
     (NVFP4, 1531, 2064),     # items of two rows, ragged rows and columns
     (INT4, 4003, 512),       # items of four rows, the last one ragged
-    (NVFP4, 9479, 256),      # one whole item per block and one more
+    (NVFP4, 9479, 256),      # items of two rows, three per block (149 items of four would be one more than the blocks)
 ])
 def test_rows_per_item(mode, N, K):
     W, X = layer(mode, N, K, name=f"items/{mode}/{N}x{K}")
@@ -31,6 +31,13 @@ def test_rows_per_item(mode, N, K):
     assert table_close(host(r["T01"]), o["T"])[0]
     assert np.allclose(host(r["trace"])[:4], o["trace"], rtol=1e-4, atol=0)
     check_end_to_end_bits(r, o, f"{mode} {N}x{K}")
+
+
+@pytest.mark.parametrize("mode,extra", [(INT4, 1), (NVFP4, 1), (NVFP4, 0)])
+def test_several_items_per_block(mode, extra):
+    """Four items of four rows per block, the last one ragged; with one more than that, it is dealt out by quarters."""
+    N, K = 64 * (4 * torch.cuda.get_device_properties(0).multi_processor_count + extra) - 5, 256
+    test_rows_per_item(mode, N, K)
 
 
 @pytest.mark.parametrize("mode", [INT4, NVFP4])
