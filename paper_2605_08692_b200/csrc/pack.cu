@@ -35,11 +35,7 @@ namespace aaac {
 
 namespace {
 
-// warps per block
-#ifndef AAAC_PACK_WARPS
-#define AAAC_PACK_WARPS 8
-#endif
-constexpr int pack_warps(int) { return AAAC_PACK_WARPS; }
+constexpr int kPackWarps = 8;            // warps per block
 
 struct PackParams {
     const uint16_t* W;
@@ -445,7 +441,6 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
 template <int MODE, int SEL>
 cudaError_t launch_pack_variant(const PackParams& p, unsigned grid, cudaStream_t st) {
     constexpr size_t smem = (size_t)kLut1Bytes + kLut2Bytes;
-    constexpr int kPackWarps = pack_warps(MODE);
     auto kern = pack_kernel<MODE, SEL, kPackWarps>;
     static std::atomic<size_t> ready[kMaxDevices];
     const cudaError_t e = allow_smem(kern, smem, ready);
@@ -466,7 +461,7 @@ cudaError_t launch_pack(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, in
     const int64_t slabs = (K + 255) / 256;
     const int64_t most = std::min<int64_t>((int64_t)sm_count() * kPackBlocksPerSM, kMaxBlocks / kPackRanges);
     auto grid_of = [&](int64_t rows) {
-        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(most, (rows * slabs + pack_warps(mode) - 1) / pack_warps(mode)));
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(most, (rows * slabs + kPackWarps - 1) / kPackWarps));
     };
     const unsigned grid = grid_of(row1 - row0);
     PackParams p{};

@@ -141,11 +141,9 @@ scales_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row, int6
 // group's maximum after the butterfly, forms the scale and its reciprocal itself -- with exactly the
 // expressions the later passes use -- and bins its eight normalised weights into the block's
 // shared-memory histogram, which is merged into the global one at the end.
-#ifndef AAAC_SH_BLOCKS
-#define AAAC_SH_BLOCKS 2
-#endif
+constexpr int kHistBlocksPerSM = 2;
 template <int MODE, bool DENSE>
-__global__ void __launch_bounds__(512, AAAC_SH_BLOCKS)
+__global__ void __launch_bounds__(512, kHistBlocksPerSM)
 scales_hist_kernel(const uint16_t* __restrict__ W, unsigned n, unsigned per_row, int64_t ldw, void* __restrict__ scales,
                    float* __restrict__ rinv, float* __restrict__ tensor_scale, Ctrl* ctrl, uint32_t* dev_status,
                    uint32_t* __restrict__ hist) {
@@ -247,7 +245,7 @@ cudaError_t launch_scales(const uint16_t* W, int64_t N, int64_t K, int64_t ldw, 
     auto kern = mode == AAAC_NVFP4 ? (dense ? scales_hist_kernel<AAAC_NVFP4, true> : scales_hist_kernel<AAAC_NVFP4, false>)
                                    : (dense ? scales_hist_kernel<AAAC_INT4, true> : scales_hist_kernel<AAAC_INT4, false>);
     if ((e = allow_smem(kern, smem, ready[2 * (mode == AAAC_NVFP4) + dense])) != cudaSuccess) return e;
-    return launch_chained(kern, sm_count() * AAAC_SH_BLOCKS, 512, smem, st, W, n, per_row, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status, ws.qhist);
+    return launch_chained(kern, sm_count() * kHistBlocksPerSM, 512, smem, st, W, n, per_row, ldw, scales, rinv, tensor_scale, ws.ctrl, dev_status, ws.qhist);
 }
 
 }  // namespace aaac
