@@ -95,6 +95,7 @@ struct FitParams {
     float* T01_out;               // [2][16] or null: the tables after the launch's last pass, as FP32
     uint32_t* dev_status;         // or null
     uint32_t* sigw;               // [N][slabs]: selection bits of a row's 256-column slab, bit = lane (n_inner > 1)
+    uint32_t* kept;               // [N][K / 16]: index bits and selection per 16 weights (kKeep and the incremental rounds; the same memory)
     int n_rounds;                 // passes over W in this launch
     int trace_base;               // err_trace index of this launch's first assignment pass
     unsigned bar_base;            // passes of the layer's earlier launches (the sum buffers rotate per pass)
@@ -155,7 +156,14 @@ __device__ __forceinline__ void sts_u2(uint32_t addr, uint32_t a, uint32_t b) {
 // kAssignKeep: the same pass, which also stores the selection bits.  kInner: further inner
 // iterations with the stored selection.  With n_inner > 1 a round is one kAssignKeep launch of a
 // single pass followed by one kInner launch of n_inner - 1 passes.
-enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2 };
+// kKeep: assignment passes (n_inner = 1) of which the last also stores, per 16 columns of a row, the low bits of
+// the entries' indices and the selection (below); the rounds after it are those of fit_delta.cuh.
+// kRest: assignment passes again, as many as those have left (mostly none).
+enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4 };
+
+// What the incremental rounds keep of 16 adjacent weights of a row: bit 2 j the low bit of the index of weight j's
+// entry in the table its group has chosen, bit 1 that choice.
+
 
 // Decides the listed selection groups in double (Eq. 8: each lane adds its weights' terms in index
 // order, the lanes of the group are combined pairwise; a tie goes to table 0) and adds every weight
@@ -169,6 +177,7 @@ struct DeferArgs {                // what the routine needs of the layer (passed
     const float* rinv;
     const float* I;
     uint32_t* sigw;
+    uint32_t* kept;
 };
 template <int MODE, int SEL, int KIND>
 __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferArgs p, uint32_t list_addr, int count,
@@ -215,6 +224,7 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
         e0 = __shfl_sync(0xFFFFFFFFu, e0, 0);
         e1 = __shfl_sync(0xFFFFFFFFu, e1, 0);
         const bool sg = e1 < e0;
+        uint32_t parity = 0;
         if (lane < ACTIVE) {
 #pragma unroll
             for (int t = 0; t < WPL; ++t) {
@@ -225,7 +235,17 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
                 b.x += __fmul_rn(Is[t], __fsub_rn(xs[t], c));
                 b.y += Is[t];
                 sts_bin(a, b);
+                parity |= (__float_as_uint(c) & 1u) << (2 * t);
             }
+        }
+        if (KIND == kKeep) {
+            // the lanes of 16 weights put their bits together
+            constexpr int LPE = 16 / WPL;
+            parity <<= (lane % LPE) * WPL * 2;
+#pragma unroll
+            for (int o = 1; o < LPE; o <<= 1) parity |= __shfl_xor_sync(0xFFFFFFFFu, parity, o);
+            if (lane < ACTIVE && lane % LPE == 0)
+                p.kept[(size_t)row * (size_t)(K / 16) + (uint32_t)(cg / 16 + lane / LPE)] = parity | (sg ? 2u : 0u);
         }
         if (lane == 0) {
             esum += sg ? e1 : e0;
@@ -304,6 +324,10 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     __shared__ FitShared sh;
     FitTables& S = sh.t;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int done = KIND == kRest ? (int)p.ctrl->next_round : 0;
+    const int n_rounds = p.n_rounds - done, trace_base = p.trace_base + done;
+    const unsigned bar_base = KIND == kRest ? p.ctrl->passes : p.bar_base;
+    if (KIND == kRest && n_rounds <= 0) return;
 
     // 32-bit shared addresses.  The bin table sits at a shared address that is a multiple of its own
     // span (64 KB), so that a lookup's address -- bin bits, the lane's copy and the table base -- is one
@@ -432,7 +456,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     }
     for (int b = 0; b < kBinSlots; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
     __syncthreads();
-    write_tables<NT, true>(S, tid, kLut1At, lut2_addr);
+    write_tables<NT, true>(S, S.pq32, tid, kLut1At, lut2_addr);
     __syncthreads();
 
     // bin arithmetic: the masked mantissa of fl32(kBinsPerUnit x + kMagic) is bin * (REP * 8)
@@ -440,8 +464,9 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     constexpr float kMagic = (float)(NB / 2) + 1.5f * (float)(1 << 23) / (float)(REP * 8);
     constexpr uint32_t kBinMask = (uint32_t)(NB - 1) * (REP * 8);
 
-  for (int round = 0; round < p.n_rounds; ++round) {
-    const unsigned pass_no = p.bar_base + (unsigned)round;
+  for (int round = 0; round < n_rounds; ++round) {
+    const unsigned pass_no = bar_base + (unsigned)round;
+    const bool keep = KIND == kKeep && round + 1 == n_rounds;
     // block 0 clears the buffer of the next pass: it was the buffer of two passes ago, and every block
     // finished reading it before it added to the previous pass's buffer, whose totals block 0 has seen
     static_assert(NT >= 256 + kCells * 4 + kLimbs, "threads 256.. of block 0 clear the next buffer");
@@ -602,6 +627,14 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 const unsigned bits = __ballot_sync(0xFFFFFFFFu, sg);        // (the bits of listed groups are set when they are decided)
                 if (lane == 0) p.sigw[(size_t)row * (size_t)slabs + slab] = bits;
             }
+            if (KIND == kKeep && keep) {
+                // (the two lanes of 16 columns write a half each; the selection stands in the lower one)
+                uint32_t bits = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) bits = __funnelshift_r(bits, __float_as_uint(sg ? hi2(pq[j]) : lo2(pq[j])), 2);
+                bits = ((bits >> 16) & 0x5555u) | (sg && !(lane & 1) ? 2u : 0u);
+                if (col_ok) reinterpret_cast<uint16_t*>(p.kept)[(unsigned)row * (unsigned)(K / 8) + (unsigned)(slab * 32 + lane)] = (uint16_t)bits;
+            }
             // cell = entry index (low bits of the centre constant) under the chosen table
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -669,13 +702,13 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         Eacc += (double)eitem;
         if (!INNER && ndefer > kDeferCap - R * (32 / LPG)) {    // the next item could overflow the list
             __syncwarp();
-            Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw}, list_addr, ndefer, bins_lane, lane);
+            Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw, KIND == kKeep ? p.kept : nullptr}, list_addr, ndefer, bins_lane, lane);
             ndefer = 0;
         }
     }
     if (!INNER && ndefer > 0) {
         __syncwarp();
-        Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw}, list_addr, ndefer, bins_lane, lane);
+        Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw, KIND == kKeep ? p.kept : nullptr}, list_addr, ndefer, bins_lane, lane);
     }
 
     // ---- the warp's sums: lane c adds the 32 lane-private values of cell c (in an order of its own that
@@ -777,9 +810,12 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             const double sx = total(x), wt = total(y);
             double T = wt > 0.0 ? (double)S.centre[lane] + __ddiv_rn(sx, wt) : S.Td[lane];
             // the trace holds the Eq. 8 objective of each assignment step
-            if (my_e) p.err_trace[p.trace_base + round] = 16.0 * total(e);
+            double err = 0.0;
+            if (my_e) p.err_trace[trace_base + round] = err = 16.0 * total(e);
             const double Tp = __shfl_up_sync(kAll, T, 1);
-            if (__any_sync(kAll, (lane & 15) != 0 && Tp > T)) {
+            const double before = KIND == kKeep ? S.Td[lane] : 0.0;
+            const bool unsorted = __any_sync(kAll, (lane & 15) != 0 && Tp > T);
+            if (unsorted) {
                 // ascending order within the table by rank (ties by index)
                 int rank = 0;
 #pragma unroll 1
@@ -791,6 +827,20 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 __syncwarp();
                 T = S.Td[lane];
                 __syncwarp();
+            }
+            if (KIND == kKeep && keep && bid == 0) {
+                // what the incremental rounds start from
+                Ctrl& c = *p.ctrl;
+                c.keep_T[lane] = before;
+                c.keep_c[lane] = S.centre[lane];
+                c.keep_sx[lane] = sx;
+                c.keep_sw[lane] = wt;
+                if (lane == 0) {
+                    c.keep_q = err;
+                    c.keep_ok = !unsorted;
+                    c.next_round = (uint32_t)(trace_base + round + 1);
+                    c.passes = pass_no + 1u;
+                }
             }
             derive_tables(S, lane, T);
         }
@@ -804,8 +854,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         }
         return;
     }
-    if (round + 1 < p.n_rounds) {
-        write_tables<NT, true>(S, tid, kLut1At, lut2_addr);
+    if (round + 1 < n_rounds) {
+        write_tables<NT, true>(S, S.pq32, tid, kLut1At, lut2_addr);
         __syncthreads();
     }
   }
@@ -826,6 +876,8 @@ struct FitBatch {
     unsigned first[kMaxBatch + 1];    // first block of every layer; first[n..] = grid size
 };
 
+#include "fit_delta.cuh"
+
 template <int MODE, int SEL, int KIND>
 __global__ void __launch_bounds__(kFitWarps * 32, 1) fit_kernel(const __grid_constant__ FitBatch b) {
     // a single layer: its parameters at fixed places (1-3 % faster than picked by index, which for several
@@ -842,9 +894,8 @@ __global__ void export_tables_kernel(const Ctrl* ctrl, float* T01) {
 
 // The fit kernels place their tables at fixed shared addresses and take all the shared memory a block
 // may have beyond their static part (one block per SM either way); the kernel checks that its layout fits.
-template <int MODE, int SEL, int KIND>
+template <void (*kern)(FitBatch)>
 cudaError_t launch_variant(FitBatch& b, unsigned grid, cudaStream_t st) {
-    auto kern = fit_kernel<MODE, SEL, KIND>;
     static std::atomic<size_t> ready[kMaxDevices];          // dynamic shared memory, once it is set up on a device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -869,10 +920,11 @@ cudaError_t launch_variant(FitBatch& b, unsigned grid, cudaStream_t st) {
 
 template <int KIND>
 cudaError_t launch_kind(FitBatch& b, unsigned grid, int mode, int sel_group, cudaStream_t st) {
-    if (mode == AAAC_INT4 && sel_group == 16) return launch_variant<AAAC_INT4, 16, KIND>(b, grid, st);
-    if (mode == AAAC_INT4) return launch_variant<AAAC_INT4, 128, KIND>(b, grid, st);
-    return launch_variant<AAAC_NVFP4, 16, KIND>(b, grid, st);
+    if (mode == AAAC_INT4 && sel_group == 16) return launch_variant<fit_kernel<AAAC_INT4, 16, KIND>>(b, grid, st);
+    if (mode == AAAC_INT4) return launch_variant<fit_kernel<AAAC_INT4, 128, KIND>>(b, grid, st);
+    return launch_variant<fit_kernel<AAAC_NVFP4, 16, KIND>>(b, grid, st);
 }
+
 
 }  // namespace
 
@@ -927,10 +979,23 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
     p.ctrl = a.ws.ctrl; p.acc = a.ws.acc; p.err_trace = a.err_trace; p.T01_out = a.T01_out; p.dev_status = dev_status;
     p.n_rounds = n_outer; p.trace_base = 0; p.bar_base = 0u;
     p.spin_limit = g_spin_limit;
+    p.kept = a.ws.qlist;
     p.sigw = a.ws.qlist;            // the quantile selection's list is free once the start tables exist
     const int64_t slabs = (a.K + 255) / 256;
     const int64_t nrb = (a.N + kFitWarps - 1) / kFitWarps;
     return !(a.N > 0x7FFFFFFF || a.K > 0x7FFFFFFF || slabs * nrb > 0x7FFFFFFF);
+}
+
+// Incremental rounds (fit_delta.cuh) pay where few weights move and the passes are long.  4096 x 14336, us a pass, all
+// weights added against those that move: NVFP4 72 against 80 in the second round, 70 in the third to sixth, 56 from the
+// tenth on; INT4, whose tables move more, 74 against 112 and 95.  The two launches more cost some 20 us, and what is
+// left on a warp's lists at the end of a pass is worked off alone: a block should have 16 units of 16 x 512 weights.
+// A piece is read with one 32-byte load; its number must be divisible by more than one piece per row (row_of).
+constexpr int kFullRounds = 3, kLeastIncremental = 5, kLeastUnits = 16;
+static bool can_increment(const FitLayerArgs& a, int64_t blocks) {
+    const int64_t slabs = (a.K + kDeltaCols - 1) / kDeltaCols, units = slabs * ((a.N + kFitWarps - 1) / kFitWarps);
+    return a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 && a.ldw % 16 == 0 &&
+           units >= kLeastUnits * blocks && 8 * a.K >= 7 * kDeltaCols * slabs;
 }
 
 cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode, int sel_group, int n_outer, int n_inner,
@@ -968,8 +1033,17 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             grid += (unsigned)plan_layer(b.L[l], a.N, a.K, share[l]);
         }
         for (int l = m; l <= kMaxBatch; ++l) b.first[l] = grid;
+        bool incremental = mode == AAAC_NVFP4 && n_inner == 1 && n_outer >= kFullRounds + kLeastIncremental;
+        for (int l = 0; l < m; ++l) incremental = incremental && can_increment(layers[at + l], b.first[l + 1] - b.first[l]);
         cudaError_t e = cudaSuccess;
-        if (n_inner == 1) {
+        if (incremental) {
+            // the first rounds, the last of which stores what the incremental ones need; these; and whatever they leave undone
+            for (int l = 0; l < m; ++l) b.L[l].n_rounds = kFullRounds;
+            e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kKeep>>(b, grid, st);
+            for (int l = 0; l < m; ++l) b.L[l].n_rounds = n_outer;
+            if (e == cudaSuccess) e = launch_variant<delta_kernel<AAAC_NVFP4, 16>>(b, grid, st);
+            if (e == cudaSuccess) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);
+        } else if (n_inner == 1) {
             e = launch_kind<kRounds>(b, grid, mode, sel_group, st);
         } else {
             for (int outer = 0; outer < n_outer && e == cudaSuccess; ++outer) {

@@ -27,6 +27,12 @@ struct Ctrl {
     float s_t;                      // NVFP4 tensor scale
     uint32_t absmax_bits;           // layer max |w| as float bits (atomicMax on non-negative floats)
     uint32_t nonfinite;             // set if a non-finite weight was seen
+    // the incremental rounds: the tables and centre constants of the pass they start from, its sums, and where they end
+    double keep_T[2 * kM], keep_sx[2 * kM], keep_sw[2 * kM];
+    double keep_q;                  // that pass's objective
+    float keep_c[2 * kM];
+    uint32_t keep_ok;               // its tables were in order
+    uint32_t next_round, passes;    // the first round not done; passes made so far (the sum buffers rotate per pass)
     uint32_t abort;                 // set when a block's wait for the totals of a pass ran out
     // quantile selection
     double frac[2 * kM];            // interpolation fraction per table entry

@@ -21,6 +21,7 @@ constexpr int kPoison = kNJ * kPqRow;              // byte offset of the poisone
 constexpr int kLut1Bytes = kNBins * kRep * 8;
 constexpr int kLut2Bytes = kJSlots * kPqRow;
 constexpr int kCells = 2 * kM;                     // bins per lane: [sigma][entry]
+constexpr uint32_t kNoHint = 0xFFu;                // in the place of an interval: search for it
 constexpr uint32_t kIdxMask = 15u;                 // low mantissa bits of a centre constant = entry index
 
 // Shared-memory accesses of the hot loop with explicit 32-bit addresses.  All are volatile asm,
@@ -163,9 +164,10 @@ __device__ __forceinline__ void derive_tables(FitTables& S, const int lane, cons
 // breakpoints are sorted, so those inside a bin are the first ones not below its lower edge.  A thread
 // writes the 16 copies of its bin, two per store, in an order rotated by its lane, so that the eight
 // lanes that a 16-byte store is served for meet in no bank.
-// DIRECT: the fit rounds' form of the bins' entries.
+// rows: the constants of every interval; low, where given: the interval of every bin's lower edge (kNoHint if poisoned).  DIRECT: the fit rounds' form of the bins' entries.
 template <int NT, bool DIRECT>
-__device__ __forceinline__ void write_tables(const FitTables& S, const int tid, const uint32_t lut1_addr, const uint32_t lut2_addr) {
+__device__ __forceinline__ void write_tables(const FitTables& S, const float2* rows, const int tid, const uint32_t lut1_addr, const uint32_t lut2_addr,
+                                             uint8_t* low = nullptr) {
     static_assert(kNBins % NT == 0, "whole bins per thread");
     constexpr float h = 0.5f / (float)(kRep * 8);
     constexpr float kHalf = (float)(kNBins / 2), kWidth = 16.f / (float)kNBins;
@@ -175,12 +177,13 @@ __device__ __forceinline__ void write_tables(const FitTables& S, const int tid, 
         const int below = find_interval(S.bp, lo);
         const float v0 = S.bp[below], v1 = S.bp[below + 1];     // bp[30], bp[31] = +inf
         const bool poison = v1 <= hi;                            // two breakpoints or more
+        if (low) low[b] = (uint8_t)(poison ? kNoHint : (uint32_t)below);
         uint32_t e0, e1, c1 = 0;                                // c1: what an address grows by from copy to copy
         if (!DIRECT) {
             e0 = lut2_addr + (poison ? (uint32_t)kPoison : (uint32_t)(below * kPqRow));
             e1 = !poison && v0 <= hi ? __float_as_uint(v0) : 0x7F800000u;
         } else if (!poison && !(v0 <= hi)) {
-            const float2 v = S.pq32[below];
+            const float2 v = rows[below];
             e0 = __float_as_uint(v.x);
             e1 = __float_as_uint(v.y);
         } else {
@@ -202,7 +205,7 @@ __device__ __forceinline__ void write_tables(const FitTables& S, const int tid, 
     }
     static_assert(kLut2Bytes / 16 <= NT, "one store per thread");
     if (tid < kLut2Bytes / 16) {
-        const float2 v = S.pq32[tid >> 3];
+        const float2 v = rows[tid >> 3];
         asm volatile("st.shared.v4.f32 [%0], {%1, %2, %1, %2};" :: "r"(lut2_addr + (uint32_t)tid * 16u), "f"(v.x), "f"(v.y) : "memory");
     }
 }
@@ -214,7 +217,6 @@ __device__ __forceinline__ uint32_t pq_entry_addr(uint32_t lut2_addr, int J, int
 
 // hint[j] < kNJ names the interval of weight j where the caller knows it, else the interval is searched
 struct Row8 { float x[8]; float I[8]; uint32_t hint[8]; };
-constexpr uint32_t kNoHint = 0xFFu;
 
 // The interval of a weight from the constants {P, Q} the fast path has looked up: with no equal
 // entries inside a table, entry index = number of that table's breakpoints below the weight, and

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(NW * 32, kPackBlocksPerSM) pack_kernel(const P
         derive_tables(S, lane, T);
     }
     __syncthreads();
-    write_tables<NW * 32, false>(S, tid, (uint32_t)__cvta_generic_to_shared(dyn), (uint32_t)__cvta_generic_to_shared(dyn) + kLut1Bytes);
+    write_tables<NW * 32, false>(S, S.pq32, tid, (uint32_t)__cvta_generic_to_shared(dyn), (uint32_t)__cvta_generic_to_shared(dyn) + kLut1Bytes);
     __syncthreads();
 
     const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(dyn);

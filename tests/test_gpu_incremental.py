@@ -1,0 +1,71 @@
+"""The incremental fit rounds, at sizes and on data where they can go wrong, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_08692_b200 import binding, build, synth
+from test_gpu_parity import NVFP4, check_end_to_end_bits, dev_bf16, host, layer, table_close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def check(W, X, rounds, init, name, **kw):
+    o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, init={binding.INIT_QUANTILE: "quantile", binding.INIT_GRID: "grid"}[init])
+    before = binding.launch_count()
+    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, init=init, want_trace=True, **kw)
+    launches = binding.launch_count() - before
+    torch.cuda.synchronize()
+    assert int(r["status"].item()) == 0
+    assert table_close(host(r["T01"]), o["T"])[0], name
+    # (FP32 terms, 2^-24 each, and their sums over a lane's rows; where the entries meet every weight what is left is the
+    # distance of the constants from the entries, 8 units in the last place at most: (2^-20 * 8)^2 of sum I)
+    assert np.allclose(host(r["trace"])[:rounds], o["trace"], rtol=1e-5, atol=1e-10 * o["trace"][0]), name
+    check_end_to_end_bits(r, o, name)
+    return launches
+
+
+def rows_for(units, K):
+    """Rows of a layer of K columns with so many units of 16 rows x 512 columns per block."""
+    blocks = torch.cuda.get_device_properties(0).multi_processor_count
+    return 16 * -(-units * blocks // -(-K // 512))
+
+
+@pytest.mark.parametrize("K,extra,rounds,init", [
+    (512, 0, 8, binding.INIT_QUANTILE),         # one slab, the fewest rounds
+    (512, -3, 20, binding.INIT_QUANTILE),       # a last unit with rows missing
+    (1008, 5, 12, binding.INIT_GRID),           # lanes without columns, ranges of units that differ by one; a start with equal entries
+    (4096, 16, 9, binding.INIT_QUANTILE),       # short slabs
+])
+def test_layers_of_few_units_per_block(K, extra, rounds, init):
+    N = rows_for(16, K) + extra
+    W, X = layer(NVFP4, N, K, T=64, name=f"incremental/{K}/{extra}")
+    # (of a few rows the rounds are one launch; here they are three)
+    assert check(W, X, rounds, init, f"incremental {K} {extra}") == check(W[:64].copy(), X, rounds, init, "a few rows") + 2
+
+
+@pytest.mark.parametrize("levels", [3, 17, 40])
+def test_layers_of_few_distinct_weights(levels):
+    """Equal entries, empty cells and breakpoints that jump: the incremental rounds end early, or never begin."""
+    N, K = rows_for(16, 512), 512
+    W, X = layer(NVFP4, N, K, T=64, name=f"incremental/levels/{levels}")
+    rng = np.random.default_rng(levels)
+    values = np.sort(rng.standard_normal(levels)).astype(np.float32) * 0.02
+    W = synth.f32_to_bf16_bits(values[rng.integers(0, levels, size=(N, K))])
+    check(W, X, 12, binding.INIT_GRID, f"levels {levels}")
+
+
+def test_two_runs_give_the_same_bits():
+    N, K = rows_for(17, 2048), 2048
+    W, X = layer(NVFP4, N, K, T=64, name="incremental/twice")
+    out = []
+    for _ in range(2):
+        r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=14, init=binding.INIT_QUANTILE, want_trace=True)
+        torch.cuda.synchronize()
+        out.append([host(r[k]) for k in ("T01", "trace", "codes", "scales")])
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
