@@ -171,6 +171,7 @@ constexpr int kDeltaCols = 512;                       // columns of a slab
 // A warp's list: moves from the front, flips from the back.  Behind a pass its place holds the warp's sums (66
 // doubles); the 16 bytes spread the warps over the banks.
 constexpr int kDeltaCap = 110;
+constexpr int kLeastFlips = 20;                       // flips that are worked off before the end of a pass
 constexpr int kDeltaScales = kDeltaCap * 8;           // the entries' reciprocal scales, behind the entries
 constexpr int kDeltaWeights = kDeltaCap * 12;         // the moving weights being worked off (at most 95), two bytes each
 constexpr int kDeltaList = kDeltaWeights + 192 + 16;
@@ -290,8 +291,10 @@ __device__ __noinline__ float apply_moves(const DeltaShared* sh, const DeltaArgs
                 if (next >= count) break;
                 piece = (uint32_t)(next + lane);
                 if (next + lane < count) {
-                    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(left) : "r"(list_at + piece * 8u + 4u) : "memory");
+                    uint32_t at;
+                    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(at), "=r"(left) : "r"(list_at + piece * 8u) : "memory");
                     left &= 0x55555555u;
+                    atomicXor(p.kept + at, left);          // (nobody waits for it; the pass's loads of these words go past the L1)
                 }
                 next += 32;
                 continue;
@@ -343,9 +346,8 @@ __device__ __noinline__ float apply_moves(const DeltaShared* sh, const DeltaArgs
     }
 }
 
-// Works off the list's last `count` pieces, whose selection has changed or is open: all their weights move.  Half a warp
-// takes a piece, a weight per lane, two pieces after one another side by side.  Every lane calls; returns what the
-// lane's weights add to q.
+// Works off the list's last `count` pieces, whose selection has changed or is open: all their weights move.  A lane takes
+// a piece, four weights side by side.  Every lane calls; returns what the lane's weights add to q.
 template <int MODE, int SEL>
 __device__ __noinline__ float apply_flips(const DeltaShared* sh, const DeltaArgs p, const uint32_t list_at, const int count,
                                           const uint32_t bins_lane, const int lane) {
@@ -395,52 +397,52 @@ __device__ __noinline__ float apply_flips(const DeltaShared* sh, const DeltaArgs
         }
     }
     __syncwarp();
-    constexpr int E = 2;
-    const uint32_t j = (uint32_t)lane & 15u;
     float dq = 0.f;
-    for (int first = 0; first < count; first += 2 * E) {
-        uint32_t at[E], old[E], w[E];
-        float iv[E], x[E];
-        bool mine[E];
+    for (int first = 0; first < count; first += 32) {
+        if (first + lane >= count) continue;
+        uint32_t at, old;
+        float rinv;
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(at), "=r"(old) : "r"(list_addr + (uint32_t)(first + lane) * 8u) : "memory");
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(rinv) : "r"(scales_at + (uint32_t)(first + lane) * 4u) : "memory");
+        const uint32_t tn = (at & kSelected) ? (uint32_t)kM : 0u, to = (old & 2u) ? (uint32_t)kM : 0u;
+        at &= kPieceMask;
+        const unsigned row = row_of(at, K16, p.k16_inv), col = (at - row * K16) * 16u;
+        const uint16_t* const W = p.W + (row * (unsigned)p.ldw + col);
+        const float* const I = p.I + col;
+        uint32_t word = tn ? 2u : 0u;
+        uint2 w = __ldg(reinterpret_cast<const uint2*>(W));
+        float4 iv = __ldg(reinterpret_cast<const float4*>(I));
+#pragma unroll 1
+        for (uint32_t q = 0; q < 4; ++q) {
+            const uint2 wc = w;
+            const float4 ic = iv;
+            const uint32_t nx = min(q + 1u, 3u) * 4u;      // (the next four are asked for meanwhile)
+            w = __ldg(reinterpret_cast<const uint2*>(W + nx));
+            iv = __ldg(reinterpret_cast<const float4*>(I + nx));
+            const float x[4] = {__fmul_rn(bf16_lo(wc.x), rinv), __fmul_rn(bf16_hi(wc.x), rinv), __fmul_rn(bf16_lo(wc.y), rinv),
+                                __fmul_rn(bf16_hi(wc.y), rinv)};
+            const float Iv[4] = {ic.x, ic.y, ic.z, ic.w};
+            const uint32_t was = old >> (8u * q);
+            uint32_t from[4], into[4], bits = 0u;
+            Move m[4];
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const int e = first + 2 * k + (lane >> 4);
-            mine[k] = e < count;
-            at[k] = old[k] = w[k] = 0u;
-            iv[k] = x[k] = 0.f;
-            if (mine[k]) {
-                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(at[k]), "=r"(old[k]) : "r"(list_addr + (uint32_t)e * 8u) : "memory");
-                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[k]) : "r"(scales_at + (uint32_t)e * 4u) : "memory");
-                const unsigned a = at[k] & kPieceMask, row = row_of(a, K16, p.k16_inv), col = (a - row * K16) * 16u + j;
-                w[k] = __ldg(p.W + (row * (unsigned)p.ldw + col));
-                iv[k] = __ldg(p.I + col);
+            for (int t = 0; t < 4; ++t) {
+                const uint32_t c = entries_of(sh, x[t]);
+                const uint32_t in = (c >> (tn / 4u)) & kIdxMask;
+                uint32_t io = (c >> (to / 4u)) & kIdxMask;
+                if (((was >> (2 * t)) ^ io) & 1u) io = (x[t] > sh->mid_old[to + io] ? io + 1u : io - 1u) & kIdxMask;
+                from[t] = to + io;
+                into[t] = tn + in;
+                bits |= (in & 1u) << (2 * t);
             }
+            word |= bits << (8u * q);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) m[t] = move_terms(sh, from[t], into[t], x[t], Iv[t], dq);
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (from[t] != into[t]) move_weight(bins_lane, from[t], into[t], m[t], Iv[t]);
         }
-#pragma unroll
-        for (int k = 0; k < E; ++k) x[k] = __fmul_rn(__uint_as_float(w[k] << 16), x[k]);
-        uint32_t from[E], to[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const bool sg = (at[k] & kSelected) != 0u, so = (old[k] & 2u) != 0u;
-            const uint32_t c = entries_of(sh, x[k]);
-            const uint32_t in = (sg ? c >> 4 : c) & kIdxMask;
-            uint32_t io = (so ? c >> 4 : c) & kIdxMask;
-            if (((old[k] >> (2u * j)) ^ io) & 1u) io = (x[k] > sh->mid_old[(so ? kM : 0) + io] ? io + 1u : io - 1u) & kIdxMask;
-            from[k] = (so ? (uint32_t)kM : 0u) + io;
-            to[k] = (sg ? (uint32_t)kM : 0u) + in;
-            if (__any_sync(kAll, mine[k] && (at[k] & kUndecided) != 0u)) {      // its kept word was written before it was decided
-                uint32_t bits = (in & 1u) << (2u * j);
-#pragma unroll
-                for (int o = 8; o; o >>= 1) bits |= __shfl_xor_sync(kAll, bits, o);
-                if (mine[k] && j == 0u) p.kept[at[k] & kPieceMask] = bits | (sg ? 2u : 0u);
-            }
-        }
-        Move m[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) m[k] = move_terms(sh, from[k], to[k], x[k], iv[k], dq);
-#pragma unroll
-        for (int k = 0; k < E; ++k)
-            if (mine[k] && from[k] != to[k]) move_weight(bins_lane, from[k], to[k], m[k], iv[k]);
+        p.kept[at] = word;
     }
     return dq;
 }
@@ -511,7 +513,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
                      : "l"(p.W + wo));
         if (MODE == AAAC_NVFP4) asm volatile("ld.global.u8 %0, [%1];" : "=r"(sc[s]) : "l"(p.scales + so));
         else asm volatile("ld.global.u32 %0, [%1];" : "=r"(sc[s]) : "l"(p.rinv + so));
-        asm volatile("ld.global.u32 %0, [%1];" : "=r"(kw[s]) : "l"(p.kept + ko) : "memory");
+        asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(kw[s]) : "l"(p.kept + ko) : "memory");
         if (--lleft == 0) {
             lleft = n_units;
             lslab = slab0;
@@ -673,11 +675,10 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
                        move ? (diff & 0x55555555u) | (sg << 1) : old);
                 asm volatile("st.shared.f32 [%0], %1;" :: "r"(list_at + (uint32_t)(kDeltaScales + e * 4)), "f"(rinv_now) : "memory");
             }
-            if (flip || move) p.kept[at] = now;
             n_moves += __popc(mm);
             n_flips += __popc(fm);
             if (++rb == nrb) { rb = 0; ++slab; }
-            return n_moves + n_flips > kDeltaCap - 32;
+            return n_moves + n_flips > kDeltaCap - 32 || n_flips >= 32;
         };
         for (int i = 0; i < n_units;) {
             rinv = rinv_of(sc[0]);
@@ -701,8 +702,11 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             // (out of the loop above, whose registers would be spilled in its midst)
             __syncwarp();
             if (n_moves > 0) dq += (double)apply_moves(&sh, args, list_at, n_moves, bins_lane, lane);
-            if (n_flips > 0) dq += (double)apply_flips<MODE, SEL>(&sh, args, list_at, n_flips, bins_lane, lane);
-            n_moves = n_flips = 0;
+            n_moves = 0;
+            if (n_flips > (i < n_units ? kLeastFlips - 1 : 0)) {
+                dq += (double)apply_flips<MODE, SEL>(&sh, args, list_at, n_flips, bins_lane, lane);
+                n_flips = 0;
+            }
             __syncwarp();
         }
         __syncwarp();
@@ -715,7 +719,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             for (int s = 0; s < 2; ++s) {
                 unsigned wo, so, ko;
                 offsets(wo, so, ko);
-                asm volatile("ld.global.u32 %0, [%1];" : "=r"(kw[s]) : "l"(p.kept + ko) : "memory");
+                asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(kw[s]) : "l"(p.kept + ko) : "memory");
                 if (n_units > 1 && ++lrb == nrb) { lrb = 0; ++lslab; }
             }
             lslab = s_slab;
