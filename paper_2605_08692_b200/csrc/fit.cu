@@ -96,7 +96,10 @@ struct FitParams {
     uint32_t* dev_status;         // or null
     uint32_t* sigw;               // [N][slabs]: selection bits of a row's 256-column slab, bit = lane (n_inner > 1)
     uint32_t* kept;               // [N][K / 16]: index bits and selection per 16 weights (kKeep and the incremental rounds; the same memory)
-    int n_rounds;                 // passes over W in this launch
+    int n_rounds;                 // passes over W in this launch (of the incremental rounds: in all)
+    int n_inner;                  // incremental rounds: passes per round
+    int n_total;                  // kAssignAgain, kInnerAgain: passes of the whole fit
+    bool restart;                 // the first of those
     int trace_base;               // err_trace index of this launch's first assignment pass
     unsigned bar_base;            // passes of the layer's earlier launches (the sum buffers rotate per pass)
     unsigned arrivals;            // blocks whose sums a total must hold before it is read (the grid size)
@@ -158,8 +161,9 @@ __device__ __forceinline__ void sts_u2(uint32_t addr, uint32_t a, uint32_t b) {
 // single pass followed by one kInner launch of n_inner - 1 passes.
 // kKeep: assignment passes (n_inner = 1) of which the last also stores, per 16 columns of a row, the low bits of
 // the entries' indices and the selection (below); the rounds after it are those of fit_delta.cuh.
-// kRest: assignment passes again, as many as those have left (mostly none).
-enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4 };
+// kRest: assignment passes again, as many as those have left (mostly none).  With n_inner > 1, where they end within a
+// round, kAssignAgain and kInnerAgain do everything again, from the start tables, unless nothing is left.
+enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4, kAssignAgain = 5, kInnerAgain = 6 };
 
 // What the incremental rounds keep of 16 adjacent weights of a row: bit 2 j the low bit of the index of weight j's
 // entry in the table its group has chosen, bit 1 that choice.
@@ -249,7 +253,7 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
         }
         if (lane == 0) {
             esum += sg ? e1 : e0;
-            if (KIND == kAssignKeep) {
+            if (KIND == kAssignKeep || KIND == kAssignAgain) {
                 // the stored selection bits of the row's slab: bit = lane of the row pipeline
                 const uint32_t first = ((uint32_t)cg & 255u) >> 3;
                 const uint32_t mask = (LPG >= 32 ? 0xFFFFFFFFu : ((1u << LPG) - 1u)) << first;
@@ -326,8 +330,10 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int done = KIND == kRest ? (int)p.ctrl->next_round : 0;
     const int n_rounds = p.n_rounds - done, trace_base = p.trace_base + done;
-    const unsigned bar_base = KIND == kRest ? p.ctrl->passes : p.bar_base;
+    constexpr bool AGAIN = KIND == kAssignAgain || KIND == kInnerAgain;
+    const unsigned bar_base = KIND == kRest ? p.ctrl->passes : AGAIN ? p.ctrl->passes + p.bar_base : p.bar_base;
     if (KIND == kRest && n_rounds <= 0) return;
+    if (AGAIN && (int)p.ctrl->next_round >= p.n_total) return;
 
     // 32-bit shared addresses.  The bin table sits at a shared address that is a multiple of its own
     // span (64 KB), so that a lookup's address -- bin bits, the lane's copy and the table base -- is one
@@ -377,8 +383,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     uint4 v[R];
     uint32_t sc[R];           // NVFP4: scale byte; INT4: bits of the reciprocal scale
     uint32_t sgw[R];          // inner iteration: the row's stored selection bits
-    constexpr bool INNER = KIND == kInner;
-    constexpr bool keep_sigma = KIND == kAssignKeep;
+    constexpr bool INNER = KIND == kInner || KIND == kInnerAgain;
+    constexpr bool keep_sigma = KIND == kAssignKeep || KIND == kAssignAgain;
     // Offsets of the item being loaded (element offsets fit 32 bits: the entry points refuse layers of 2^32
     // elements and more).  Nothing guards the loads: rows past the item's last read that one again, lanes past
     // K the row's last columns (their importances are zero).
@@ -451,7 +457,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 sh.fix_unscale = scalbn(1.0, e - kSumBits);
                 sh.failed = 0;
             }
-            derive_tables(S, lane, p.ctrl->T[lane]);
+            derive_tables(S, lane, AGAIN && p.restart ? p.ctrl->keep_T[lane] : p.ctrl->T[lane]);
         }
     }
     for (int b = 0; b < kBinSlots; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
@@ -714,7 +720,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     // ---- the warp's sums: lane c adds the 32 lane-private values of cell c (in an order of its own that
     //      avoids bank conflicts, and a fixed one).  In double, 32 FP32 values are added without rounding
     //      unless they are more than 2^24 apart ----
-    const bool trace = KIND != kInner && p.err_trace != nullptr;
+    const bool trace = !INNER && p.err_trace != nullptr;
     __syncwarp();
     {
         const uint32_t cell_addr = bins_warp + lane * (kSlotBytes + 8);
@@ -926,6 +932,20 @@ cudaError_t launch_kind(FitBatch& b, unsigned grid, int mode, int sel_group, cud
 }
 
 
+// n_inner > 1: per round an assignment pass and the further inner iterations
+template <int ASSIGN, int INNER>
+cudaError_t launch_inner(FitBatch& b, int m, unsigned grid, int mode, int sel_group, int n_outer, int n_inner, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    for (int outer = 0; outer < n_outer && e == cudaSuccess; ++outer) {
+        for (int l = 0; l < m; ++l) { b.L[l].n_rounds = 1; b.L[l].trace_base = outer; }
+        e = launch_kind<ASSIGN>(b, grid, mode, sel_group, st);
+        for (int l = 0; l < m; ++l) { b.L[l].bar_base += 1u; b.L[l].n_rounds = n_inner - 1; b.L[l].restart = false; }
+        if (e == cudaSuccess) e = launch_kind<INNER>(b, grid, mode, sel_group, st);
+        for (int l = 0; l < m; ++l) b.L[l].bar_base += (unsigned)(n_inner - 1);
+    }
+    return e;
+}
+
 }  // namespace
 
 // Deals a layer's items to `blocks` blocks: whole items in contiguous ranges plus, where that is
@@ -987,15 +1007,22 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
 }
 
 // Incremental rounds (fit_delta.cuh) pay where few weights move and the passes are long.  4096 x 14336, us a pass, all
-// weights added against those that move: NVFP4 72 against 80 in the second round, 70 in the third to sixth, 56 from the
-// tenth on; INT4, whose tables move more, 74 against 112 and 95.  The two launches more cost some 20 us, and what is
-// left on a warp's lists at the end of a pass is worked off alone: a block should have 16 units of 16 x 512 weights.
+// weights added against those that move: NVFP4 70 against 93 in the second round, 70 in the third to sixth, 56 from the
+// tenth on; INT4, whose tables move more, 74 against 112 and 95.  The launches beside them cost some 20 us, and what is
+// left on a warp's lists at the end of a pass is worked off alone.  So one more round saves the more the more units of
+// 16 x 512 weights a block has, and the first eight or so save nothing: with 13.8 units (4096 x 4096) 10, 20, 30
+// rounds took 338, 569, 806 us before and 356, 570, 780 so, with 27.7 574, 993, 1410 and 584, 932, 1269, with 48.4
+// 924, 1626, 2324 and 906, 1479, 2028.
+// Further inner iterations have no flips and gain from the first: 3 rounds of 10 with 3.5, 6.9, 13.8, 48.4 units 394, 552,
+// 796, 2217 us before, 375, 495, 685, 1725 so; against that stand two more launches a round and the assignment passes.
 // A piece is read with one 32-byte load; its number must be divisible by more than one piece per row (row_of).
-constexpr int kFullRounds = 3, kLeastIncremental = 5, kLeastUnits = 16;
-static bool can_increment(const FitLayerArgs& a, int64_t blocks) {
+constexpr int kFullRounds = 3;
+static bool can_increment(const FitLayerArgs& a, int64_t blocks, int n_outer, int n_inner) {
     const int64_t slabs = (a.K + kDeltaCols - 1) / kDeltaCols, units = slabs * ((a.N + kFitWarps - 1) / kFitWarps);
-    return a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 && a.ldw % 16 == 0 &&
-           units >= kLeastUnits * blocks && 8 * a.K >= 7 * kDeltaCols * slabs;
+    const bool pays = n_inner == 1 ? units >= 12 * blocks && (n_outer - 6) * units >= 220 * blocks
+                                   : n_inner >= 4 && units >= 3 * blocks && (int64_t)n_outer * n_inner * units >= (100 + 20 * n_outer) * blocks;
+    return pays && a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 &&
+           a.ldw % 16 == 0 && 8 * a.K >= 7 * kDeltaCols * slabs;
 }
 
 cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode, int sel_group, int n_outer, int n_inner,
@@ -1033,26 +1060,26 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             grid += (unsigned)plan_layer(b.L[l], a.N, a.K, share[l]);
         }
         for (int l = m; l <= kMaxBatch; ++l) b.first[l] = grid;
-        bool incremental = mode == AAAC_NVFP4 && n_inner == 1 && n_outer >= kFullRounds + kLeastIncremental;
-        for (int l = 0; l < m; ++l) incremental = incremental && can_increment(layers[at + l], b.first[l + 1] - b.first[l]);
+        const int full = n_inner == 1 ? kFullRounds : 1;
+        bool incremental = mode == AAAC_NVFP4 && n_outer * n_inner > full;
+        for (int l = 0; l < m; ++l) incremental = incremental && can_increment(layers[at + l], b.first[l + 1] - b.first[l], n_outer, n_inner);
         cudaError_t e = cudaSuccess;
         if (incremental) {
-            // the first rounds, the last of which stores what the incremental ones need; these; and whatever they leave undone
-            for (int l = 0; l < m; ++l) b.L[l].n_rounds = kFullRounds;
+            // the first rounds (the first pass), the last of which stores what the incremental ones need; these; and
+            // whatever they leave undone
+            for (int l = 0; l < m; ++l) b.L[l].n_rounds = full;
             e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kKeep>>(b, grid, st);
-            for (int l = 0; l < m; ++l) b.L[l].n_rounds = n_outer;
+            for (int l = 0; l < m; ++l) { b.L[l].n_rounds = n_outer * n_inner; b.L[l].n_inner = n_inner; }
             if (e == cudaSuccess) e = launch_variant<delta_kernel<AAAC_NVFP4, 16>>(b, grid, st);
-            if (e == cudaSuccess) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);
+            if (e == cudaSuccess && n_inner == 1) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);
+            if (e == cudaSuccess && n_inner > 1) {
+                for (int l = 0; l < m; ++l) { b.L[l].n_total = n_outer * n_inner; b.L[l].restart = true; }
+                e = launch_inner<kAssignAgain, kInnerAgain>(b, m, grid, mode, sel_group, n_outer, n_inner, st);
+            }
         } else if (n_inner == 1) {
             e = launch_kind<kRounds>(b, grid, mode, sel_group, st);
         } else {
-            for (int outer = 0; outer < n_outer && e == cudaSuccess; ++outer) {
-                for (int l = 0; l < m; ++l) { b.L[l].n_rounds = 1; b.L[l].trace_base = outer; }
-                e = launch_kind<kAssignKeep>(b, grid, mode, sel_group, st);
-                for (int l = 0; l < m; ++l) { b.L[l].bar_base += 1u; b.L[l].n_rounds = n_inner - 1; }
-                if (e == cudaSuccess) e = launch_kind<kInner>(b, grid, mode, sel_group, st);
-                for (int l = 0; l < m; ++l) b.L[l].bar_base += (unsigned)(n_inner - 1);
-            }
+            e = launch_inner<kAssignKeep, kInner>(b, m, grid, mode, sel_group, n_outer, n_inner, st);
         }
         if (e != cudaSuccess) return e;
         at += m;

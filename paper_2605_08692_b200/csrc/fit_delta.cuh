@@ -33,6 +33,9 @@
 // Objective of a round (Eq. 8), from the same sums: with q = sum I (x - c)^2 carried along like them and d = T - c,
 // sum I (x - T)^2 = q - sum over the cells (2 d sum I (x - c) - d^2 sum I).
 //
+// Inner iterations (n_inner > 1).  All passes of the fit but the first run here; in a further inner iteration the kept
+// selection stands, and only moves within a table occur.
+//
 // Work.  A unit is 16 rows (one per warp) x 512 columns; every block takes a contiguous range of the layer's units
 // (slab by slab), all of them within one unit of the same length.
 
@@ -577,8 +580,10 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
 #pragma unroll
     for (int j = 0; j < 8; ++j) II[j] = 0ull;
 
-    int round = first_round;
+    int round = first_round;  // counts passes
+    int inner = first_round % p.n_inner;
     for (;;) {
+        const bool frozen = inner != 0;                    // a further inner iteration: the selection stands
         // (block 0 clears the buffer of the next pass, as in fit_rounds_body)
         static_assert(NT >= 256 + kCells * 4 + kLimbs, "threads 256.. of block 0 clear the next buffer");
         if (bid == 0 && tid >= 256 && tid < 256 + kCells * 4 + kLimbs) {
@@ -661,8 +666,9 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             float d = lo2(sum) + hi2(sum);
 #pragma unroll
             for (int o = LPG / 2; o; o >>= 1) d += __shfl_xor_sync(kAll, d, o);
-            const bool near = !(fabsf(d) > tau);
-            const uint32_t sg = d > 0.f ? 1u : 0u;
+            // (a NaN, from a poisoned row, counts as a flip also where the selection stands)
+            const bool near = !(fabsf(d) > tau) && !(frozen && d == d);
+            const uint32_t sg = frozen ? (old >> 1) & 1u : d > 0.f ? 1u : 0u;
             const uint32_t now = ((bits >> sg) & 0x55555555u) | (sg << 1);
             const uint32_t diff = now ^ old;
             const bool ok = row < N && piece < K16;
@@ -671,7 +677,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             const uint32_t at = (uint32_t)row * K16 + piece;
             const int e = move ? n_moves + __popc(mm & ((1u << lane) - 1u)) : kDeltaCap - n_flips - __popc(fm & ((2u << lane) - 1u));
             if (flip || move) {
-                sts_u2(list_at + (uint32_t)e * 8u, move ? at : at | (sg ? kSelected : 0u) | (near ? kUndecided : 0u),
+                sts_u2(list_at + (uint32_t)e * 8u, move ? at : at | (sg ? kSelected : 0u) | (near && !frozen ? kUndecided : 0u),
                        move ? (diff & 0x55555555u) | (sg << 1) : old);
                 asm volatile("st.shared.f32 [%0], %1;" :: "r"(list_at + (uint32_t)(kDeltaScales + e * 4)), "f"(rinv_now) : "memory");
             }
@@ -768,7 +774,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
                         for (int s = 16; s; s >>= 1) f += __shfl_xor_sync(kAll, f, s);
                         if (lane == 0) {
                             sh.q += 16.0 * total_of(t.e, nblk, sh.fix_unscale);
-                            p.err_trace[p.trace_base + round] = sh.q - f;
+                            if (!frozen) p.err_trace[round / p.n_inner] = sh.q - f;
                         }
                     }
                     sh.sx[lane] = sx;
@@ -793,6 +799,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             return;
         }
         if (sh.stop != 1) ++round;
+        if (++inner == p.n_inner) inner = 0;
         if (sh.stop || round >= p.n_rounds) break;
         write_tables<NT, false>(S, sh.ab, tid, kLut1At, lut2_addr, sh.low);
         __syncthreads();

@@ -15,10 +15,10 @@ def _built():
     build.build()
 
 
-def check(W, X, rounds, init, name, **kw):
-    o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, init={binding.INIT_QUANTILE: "quantile", binding.INIT_GRID: "grid"}[init])
+def check(W, X, rounds, init, name, inner=1):
+    o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, init={binding.INIT_QUANTILE: "quantile", binding.INIT_GRID: "grid"}[init], n_inner=inner)
     before = binding.launch_count()
-    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, init=init, want_trace=True, **kw)
+    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, n_inner=inner, init=init, want_trace=True)
     launches = binding.launch_count() - before
     torch.cuda.synchronize()
     assert int(r["status"].item()) == 0
@@ -36,28 +36,33 @@ def rows_for(units, K):
     return 16 * -(-units * blocks // -(-K // 512))
 
 
-@pytest.mark.parametrize("K,extra,rounds,init", [
-    (512, 0, 8, binding.INIT_QUANTILE),         # one slab, the fewest rounds
-    (512, -3, 20, binding.INIT_QUANTILE),       # a last unit with rows missing
-    (1008, 5, 12, binding.INIT_GRID),           # lanes without columns, ranges of units that differ by one; a start with equal entries
-    (4096, 16, 9, binding.INIT_QUANTILE),       # short slabs
+@pytest.mark.parametrize("K,units,extra,rounds,inner,init", [
+    (512, 12, 0, 25, 1, binding.INIT_QUANTILE),         # one slab, the fewest units
+    (512, 111, 16, 8, 1, binding.INIT_QUANTILE),        # the fewest rounds
+    (512, 16, -3, 20, 1, binding.INIT_QUANTILE),        # a last unit with rows missing
+    (1008, 16, 5, 21, 1, binding.INIT_GRID),            # lanes without columns, ranges of units that differ by one; a start with equal entries
+    (4096, 16, 16, 21, 1, binding.INIT_QUANTILE),       # short slabs
+    (512, 4, -3, 3, 14, binding.INIT_QUANTILE),         # inner iterations
+    (1008, 9, 5, 2, 10, binding.INIT_QUANTILE),
+    (2048, 8, 0, 3, 10, binding.INIT_GRID),             # a start with equal entries: everything is done again
 ])
-def test_layers_of_few_units_per_block(K, extra, rounds, init):
-    N = rows_for(16, K) + extra
-    W, X = layer(NVFP4, N, K, T=64, name=f"incremental/{K}/{extra}")
-    # (of a few rows the rounds are one launch; here they are three)
-    assert check(W, X, rounds, init, f"incremental {K} {extra}") == check(W[:64].copy(), X, rounds, init, "a few rows") + 2
+def test_layers_of_few_units_per_block(K, units, extra, rounds, inner, init):
+    W, X = layer(NVFP4, rows_for(units, K) + extra, K, T=64, name=f"incremental/{K}/{extra}")
+    # (of a few rows a fit is one launch, with inner iterations two a round; here they are two more)
+    few = check(W[:64].copy(), X, rounds, init, "a few rows", inner)
+    assert check(W, X, rounds, init, f"incremental {K} {units} {extra}", inner) == few + 2
 
 
+@pytest.mark.parametrize("rounds,inner", [(25, 1), (3, 10)])
 @pytest.mark.parametrize("levels", [3, 17, 40])
-def test_layers_of_few_distinct_weights(levels):
+def test_layers_of_few_distinct_weights(levels, rounds, inner):
     """Equal entries, empty cells and breakpoints that jump: the incremental rounds end early, or never begin."""
-    N, K = rows_for(16, 512), 512
+    N, K = rows_for(12, 512), 512
     W, X = layer(NVFP4, N, K, T=64, name=f"incremental/levels/{levels}")
     rng = np.random.default_rng(levels)
     values = np.sort(rng.standard_normal(levels)).astype(np.float32) * 0.02
     W = synth.f32_to_bf16_bits(values[rng.integers(0, levels, size=(N, K))])
-    check(W, X, 12, binding.INIT_GRID, f"levels {levels}")
+    check(W, X, rounds, binding.INIT_GRID, f"levels {levels}", inner)
 
 
 def test_two_runs_give_the_same_bits():
@@ -65,7 +70,7 @@ def test_two_runs_give_the_same_bits():
     W, X = layer(NVFP4, N, K, T=64, name="incremental/twice")
     out = []
     for _ in range(2):
-        r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=14, init=binding.INIT_QUANTILE, want_trace=True)
+        r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=20, init=binding.INIT_QUANTILE, want_trace=True)
         torch.cuda.synchronize()
         out.append([host(r[k]) for k in ("T01", "trace", "codes", "scales")])
     assert all(np.array_equal(a, b) for a, b in zip(*out))
