@@ -36,6 +36,13 @@
 // Inner iterations (n_inner > 1).  All passes of the fit but the first run here; in a further inner iteration the kept
 // selection stands, and only moves within a table occur.
 //
+// What bounds it.  A pass over 4096 x 14336 takes 42 us where nothing moves (full rounds: 70), 19 instructions a weight at 72 %
+// of the issue slots, the shared-memory pipe 75-80 % busy; with 9-10 % of the pieces moving, as in late rounds, 55-57 us, 11
+// SM cycles for each of them: an address per lane, so a wavefront per lane and load, and eight for a weight's two bins.
+// Measured against it: list work inside the row loop (its registers spill, 103 us), by all warps at a time between barriers
+// (66 us: nothing runs beside it), two, four and eight weights of a flip side by side in half-warps (57, 57, 63 us), the full rounds' form of
+// the table (a second lookup for some weights only: 57.8 against 56.5 us), importances from shared memory (56.8 against 55.0 us: less room for the lists).
+//
 // Work.  A unit is 16 rows (one per warp) x 512 columns; every block takes a contiguous range of the layer's units
 // (slab by slab), all of them within one unit of the same length.
 
@@ -176,8 +183,9 @@ constexpr int kDeltaCols = 512;                       // columns of a slab
 constexpr int kDeltaCap = 110;
 constexpr int kLeastFlips = 20;                       // flips that are worked off before the end of a pass
 constexpr int kDeltaScales = kDeltaCap * 8;           // the entries' reciprocal scales, behind the entries
-constexpr int kDeltaWeights = kDeltaCap * 12;         // the moving weights being worked off (at most 95), two bytes each
+constexpr int kDeltaWeights = kDeltaCap * 12;         // the moving weights being worked off (63 at most), two bytes each
 constexpr int kDeltaList = kDeltaWeights + 192 + 16;
+static_assert(192 >= 2 * 63, "room for the moving weights");
 static_assert(kDeltaList % 8 == 0, "the sums are doubles");
 constexpr int kDeltaBins = kCells * kSlotBytes;       // a warp's bins (no spare slot)
 // a flip's entry is {piece | flags, old word}, a move's {piece, changed bits | selection in bit 1}; a piece's number is
@@ -276,12 +284,11 @@ struct DeltaArgs {                // what the list work needs of the layer
 };
 
 // Works off the list's first `count` pieces, in which weights move within their table: first the moving weights are put
-// into a row (most pieces have one, few more than two), then a lane takes two of them side by side.  Every lane calls;
-// returns what the lane's weights add to q.
+// into a row (most pieces have one, few more than two), then every lane takes one of them.  Every lane calls; returns what the lane's weights add to q.
 __device__ __noinline__ float apply_moves(const DeltaShared* sh, const DeltaArgs p, const uint32_t list_at, const int count,
                                           const uint32_t bins_lane, const int lane) {
     constexpr unsigned kAll = 0xFFFFFFFFu;
-    constexpr int E = 2;
+    constexpr int E = 1;                                   // weights per lane (two: 1 % slower, the code is longer)
     const unsigned K16 = (unsigned)p.K / 16u;
     const uint32_t row_at = list_at + kDeltaWeights, below = (1u << lane) - 1u;
     float dq = 0.f;
@@ -413,37 +420,38 @@ __device__ __noinline__ float apply_flips(const DeltaShared* sh, const DeltaArgs
         const uint16_t* const W = p.W + (row * (unsigned)p.ldw + col);
         const float* const I = p.I + col;
         uint32_t word = tn ? 2u : 0u;
-        uint2 w = __ldg(reinterpret_cast<const uint2*>(W));
-        float4 iv = __ldg(reinterpret_cast<const float4*>(I));
+        uint4 w = __ldg(reinterpret_cast<const uint4*>(W));
 #pragma unroll 1
-        for (uint32_t q = 0; q < 4; ++q) {
-            const uint2 wc = w;
-            const float4 ic = iv;
-            const uint32_t nx = min(q + 1u, 3u) * 4u;      // (the next four are asked for meanwhile)
-            w = __ldg(reinterpret_cast<const uint2*>(W + nx));
-            iv = __ldg(reinterpret_cast<const float4*>(I + nx));
-            const float x[4] = {__fmul_rn(bf16_lo(wc.x), rinv), __fmul_rn(bf16_hi(wc.x), rinv), __fmul_rn(bf16_lo(wc.y), rinv),
-                                __fmul_rn(bf16_hi(wc.y), rinv)};
-            const float Iv[4] = {ic.x, ic.y, ic.z, ic.w};
-            const uint32_t was = old >> (8u * q);
-            uint32_t from[4], into[4], bits = 0u;
-            Move m[4];
+        for (uint32_t q = 0; q < 2; ++q) {
+            const uint4 wc = w;
+            if (q == 0) w = __ldg(reinterpret_cast<const uint4*>(W + 8));      // (the next eight are asked for meanwhile)
+            const uint32_t ws[4] = {wc.x, wc.y, wc.z, wc.w}, was = old >> (16u * q);
+            const float4 i0 = __ldg(reinterpret_cast<const float4*>(I + 8u * q)), i1 = __ldg(reinterpret_cast<const float4*>(I + 8u * q + 4u));
+            const float Iv[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+            uint32_t bits = 0u;
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const uint32_t c = entries_of(sh, x[t]);
-                const uint32_t in = (c >> (tn / 4u)) & kIdxMask;
-                uint32_t io = (c >> (to / 4u)) & kIdxMask;
-                if (((was >> (2 * t)) ^ io) & 1u) io = (x[t] > sh->mid_old[to + io] ? io + 1u : io - 1u) & kIdxMask;
-                from[t] = to + io;
-                into[t] = tn + in;
-                bits |= (in & 1u) << (2 * t);
+            for (int h = 0; h < 8; h += 4) {
+                uint32_t from[4], into[4];
+                float x[4];
+                Move m[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    x[t] = __fmul_rn((t & 1) ? bf16_hi(ws[(h + t) / 2]) : bf16_lo(ws[(h + t) / 2]), rinv);
+                    const uint32_t c = entries_of(sh, x[t]);
+                    const uint32_t in = (c >> (tn / 4u)) & kIdxMask;
+                    uint32_t io = (c >> (to / 4u)) & kIdxMask;
+                    if (((was >> (2 * (h + t))) ^ io) & 1u) io = (x[t] > sh->mid_old[to + io] ? io + 1u : io - 1u) & kIdxMask;
+                    from[t] = to + io;
+                    into[t] = tn + in;
+                    bits |= (in & 1u) << (2 * (h + t));
+                }
+#pragma unroll
+                for (int t = 0; t < 4; ++t) m[t] = move_terms(sh, from[t], into[t], x[t], Iv[h + t], dq);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (from[t] != into[t]) move_weight(bins_lane, from[t], into[t], m[t], Iv[h + t]);
             }
-            word |= bits << (8u * q);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) m[t] = move_terms(sh, from[t], into[t], x[t], Iv[t], dq);
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (from[t] != into[t]) move_weight(bins_lane, from[t], into[t], m[t], Iv[t]);
+            word |= bits << (16u * q);
         }
         p.kept[at] = word;
     }
