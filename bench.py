@@ -457,8 +457,8 @@ def main():
     achieved = bytes_alg / (fit_ms * 1e-3) / 1e9 if fit_ms > 0 else 0.0
     peak, peak_kind = peaks()
     tpw = measured_traffic_per_weight()
-    roofline = {"kernel": "fit_kernel (one launch = the 20 k-means rounds of the step's layers, each layer on its share "
-                          "of the blocks)" if len(layers) > 1 else "fit_kernel (one launch = the 20 k-means rounds of the layer)",
+    roofline = {"kernel": "fit_kernel and delta_kernel (the launches of the 20 k-means rounds of the step's layers, each layer on its "
+                          "share of the blocks)" if len(layers) > 1 else "fit_kernel and delta_kernel (the 20 k-means rounds of the layer)",
                 "bound": "hbm",
                 "binding_units": "by the ncu counters the kernel is held by the shared-memory data pipe and instruction "
                                  "issue, not by HBM; the HBM fraction is reported because it is the metric",
