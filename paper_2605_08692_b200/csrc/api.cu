@@ -33,7 +33,8 @@ size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // Candidate list of the quantile start: by default a sixteenth of the layer's weights (what the
 // <= 64 histogram bins of the requested order statistics hold is usually 1-3 %), never less than
-// the fit's selection words [N][ceil(K/256)] that later reuse the space.
+// the fit's selection words [N][ceil(K/256)] that later reuse the space (as do, where they fit, the words that the incremental
+// rounds keep, one per 16 weights).
 size_t g_debug_qcap = 0;         // aaac_debug_quantile_cap: a forced list capacity (0 = none)
 
 size_t default_qcap(int64_t N, int64_t K) {

@@ -13,6 +13,8 @@
 // lookups and conversions chosen for it (see below), and by having the first rows of the next pass
 // in flight, and the bins being cleared, meanwhile.  A pass of a 512 x 512 layer took 11.4 us with 19k cycles of it and whole
 // items, 5.2 us now; 4096 x 4096, 27.4 -> 23.3 us.
+// (NVFP4 layers of enough units and rounds leave most of their rounds to the incremental ones of fit_delta.cuh; see
+// can_increment.)
 // With n_inner > 1 the assignment pass (which is also the first inner iteration) stores the
 // selection bits, one word per row and 256-column slab, and the remaining n_inner - 1 inner
 // iterations are passes of a second instance of the kernel that reads those bits instead of
@@ -95,11 +97,7 @@ struct FitParams {
     float* T01_out;               // [2][16] or null: the tables after the launch's last pass, as FP32
     uint32_t* dev_status;         // or null
     uint32_t* sigw;               // [N][slabs]: selection bits of a row's 256-column slab, bit = lane (n_inner > 1)
-    uint32_t* kept;               // [N][K / 16]: index bits and selection per 16 weights (kKeep and the incremental rounds; the same memory)
     int n_rounds;                 // passes over W in this launch (of the incremental rounds: in all)
-    int n_inner;                  // incremental rounds: passes per round
-    int n_total;                  // kAssignAgain, kInnerAgain: passes of the whole fit
-    bool restart;                 // the first of those
     int trace_base;               // err_trace index of this launch's first assignment pass
     unsigned bar_base;            // passes of the layer's earlier launches (the sum buffers rotate per pass)
     unsigned arrivals;            // blocks whose sums a total must hold before it is read (the grid size)
@@ -107,6 +105,10 @@ struct FitParams {
     int rows;                     // rows per warp of an item: 4, or 2 or 1 for layers that have too few items of 4
     int items, per_block, nrb;    // items of 16 * rows rows x 256 columns, items per block, row blocks per slab
     int tail_item0, tail_quarters;   // items from tail_item0 on are dealt out a quarter (one row per warp) per block
+    uint32_t* kept;               // [N][K / 16]: index bits and selection per 16 weights (kKeep and the incremental rounds; the same memory)
+    int n_inner;                  // incremental rounds: passes per round
+    int n_total;                  // kAssignAgain, kInnerAgain: passes of the whole fit
+    bool restart;                 // the first of those
 };
 
 constexpr uint32_t kLut1At = 65536;                    // shared address of the bin table (see fit_rounds_body)
