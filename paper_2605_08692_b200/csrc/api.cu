@@ -396,7 +396,7 @@ int aaac_fit_layers(const aaac_layer* layers, int n_layers, int mode, int group,
                                                : carve(layers[owner].ws, mode, layers[owner].N, layers[owner].K, layers[owner].ws_bytes).I;
             rc = prepare_fit_layer(L, mode, init, dev_status, w, lanes.of(l), shared_I, &I);
             args[l] = FitLayerArgs{static_cast<const uint16_t*>(L.W), L.N, L.K, L.ldw, L.scales, I, L.err_trace, L.T01, w,
-                                   init == AAAC_INIT_USER ? &w.ctrl->reach : nullptr};
+                                   init == AAAC_INIT_USER ? &w.ctrl->reach : nullptr, mode == AAAC_NVFP4 && init == AAAC_INIT_GRID};
         }
         if (!lanes.join() && rc == AAAC_OK) rc = AAAC_ERR_CUDA;
     }

@@ -1017,13 +1017,15 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
 // 924, 1626, 2324 and 906, 1479, 2028.
 // Further inner iterations have no flips and gain from the first: 3 rounds of 10 with 3.5, 6.9, 13.8, 48.4 units 394, 552,
 // 796, 2217 us before, 375, 495, 685, 1725 so; against that stand two more launches a round and the assignment passes.
+// They start from the first pass's tables, though, and do not begin where these hold one value twice, as the NVFP4 grid
+// does (tried and made again, 4096 x 4096 took 778 us for 743, and 312 for 274 in one round of 10).
 // A piece is read with one 32-byte load; its number must be divisible by more than one piece per row (row_of).
 constexpr int kFullRounds = 3;
 static bool can_increment(const FitLayerArgs& a, int64_t blocks, int n_outer, int n_inner) {
     const int64_t slabs = (a.K + kDeltaCols - 1) / kDeltaCols, units = slabs * ((a.N + kFitWarps - 1) / kFitWarps);
     const bool pays = n_inner == 1 ? units >= 12 * blocks && (n_outer - 6) * units >= 220 * blocks
                                    : n_inner >= 4 && units >= 3 * blocks && (int64_t)n_outer * n_inner * units >= (100 + 20 * n_outer) * blocks;
-    return pays && a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 &&
+    return pays && !(n_inner > 1 && a.twin_entries) && a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 &&
            a.ldw % 16 == 0 && 8 * a.K >= 7 * kDeltaCols * slabs;
 }
 

@@ -189,6 +189,7 @@ struct FitLayerArgs {
     float* T01_out;          // where the fitted tables go as FP32 (written by the last launch), or null
     Workspace ws;
     const float* reach = nullptr;   // Ctrl::reach where the start tables are the caller's, else null
+    bool twin_entries = false;      // a start table holds one value twice (the NVFP4 grid: 0)
 };
 cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode, int sel_group, int n_outer, int n_inner,
                                     uint32_t* dev_status, cudaStream_t st);

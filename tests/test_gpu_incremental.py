@@ -44,13 +44,19 @@ def rows_for(units, K):
     (4096, 16, 16, 21, 1, binding.INIT_QUANTILE),       # short slabs
     (512, 4, -3, 3, 14, binding.INIT_QUANTILE),         # inner iterations
     (1008, 9, 5, 2, 10, binding.INIT_QUANTILE),
-    (2048, 8, 0, 3, 10, binding.INIT_GRID),             # a start with equal entries: everything is done again
 ])
 def test_layers_of_few_units_per_block(K, units, extra, rounds, inner, init):
     W, X = layer(NVFP4, rows_for(units, K) + extra, K, T=64, name=f"incremental/{K}/{extra}")
     # (of a few rows a fit is one launch, with inner iterations two a round; here they are two more)
     few = check(W[:64].copy(), X, rounds, init, "a few rows", inner)
     assert check(W, X, rounds, init, f"incremental {K} {units} {extra}", inner) == few + 2
+
+
+def test_inner_iterations_from_equal_entries_are_not_tried():
+    """The NVFP4 grid holds 0 twice: such a fit could not begin, and runs the launches of a small one."""
+    W, X = layer(NVFP4, rows_for(8, 2048), 2048, T=64, name="incremental/2048/0")
+    few = check(W[:64].copy(), X, 3, binding.INIT_GRID, "a few rows", 10)
+    assert check(W, X, 3, binding.INIT_GRID, "grid start, 3 x 10", 10) == few
 
 
 @pytest.mark.parametrize("rounds,inner", [(25, 1), (3, 10)])
