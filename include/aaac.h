@@ -358,6 +358,13 @@ int aaac_debug_fit_wait(int extra_arrivals, unsigned spin_limit);
 int aaac_debug_quantile_cap(size_t entries);
 
 /*
+ * Diagnostics for the incremental fit rounds (passes that carry the sums of the cells and add only the weights that
+ * move): passes *first .. *end - 1 of the last fit that ran with the workspace ws were such passes (first = end = 0:
+ * none), counted over the whole fit from 0, n_inner passes a round.  Waits for the device.
+ */
+int aaac_debug_incremental(const void* ws, int* first, int* end);
+
+/*
  * Number of kernels this library has launched in the calling process so far (all entry points,
  * all devices and streams; a process-wide counter, diagnostics only).  The benchmark reports
  * the difference across its timed region.

@@ -25,7 +25,7 @@ EXPORTS = ["aaac_status_string", "aaac_workspace_bytes", "aaac_act_stats", "aaac
            "aaac_dequant", "aaac_act_stats_noalloc", "aaac_host_workspace_bytes", "aaac_quantize_layer_host", "aaac_timing_begin",
            "aaac_timing_end", "aaac_fit_layer_sel", "aaac_pack_sel", "aaac_dequant_sel", "aaac_prescale_columns",
            "aaac_quantize_layer_host_async", "aaac_launch_count", "aaac_debug_fit_wait", "aaac_fit_layers", "aaac_workspace_bytes_full", "aaac_debug_quantile_cap",
-           "aaac_quantize_layers"]
+           "aaac_quantize_layers", "aaac_debug_incremental"]
 
 
 class AaacError(RuntimeError):
@@ -82,6 +82,8 @@ def lib():
         L.aaac_debug_quantile_cap.restype = ci
         L.aaac_debug_fit_wait.argtypes = [ci, C.c_uint]
         L.aaac_debug_fit_wait.restype = ci
+        L.aaac_debug_incremental.argtypes = [vp, vp, vp]
+        L.aaac_debug_incremental.restype = ci
         L.aaac_launch_count.restype = C.c_ulonglong
         L.aaac_launch_count.argtypes = []
         L.aaac_timing_begin.argtypes = [ci]
@@ -273,6 +275,13 @@ def debug_fit_wait(extra_arrivals: int = 0, spin_limit: int = 0):
 def debug_quantile_cap(entries: int = 0):
     """Test hook: cap the quantile start's candidate list at `entries` (0 restores the normal size)."""
     _check(lib().aaac_debug_quantile_cap(entries))
+
+
+def debug_incremental(ws) -> tuple[int, int]:
+    """First and end of the passes that the last fit with this workspace made incrementally (0, 0: none)."""
+    first, end = C.c_int(), C.c_int()
+    _check(lib().aaac_debug_incremental(_ptr(ws), C.byref(first), C.byref(end)))
+    return first.value, end.value
 
 
 def launch_count() -> int:

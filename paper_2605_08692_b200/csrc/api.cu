@@ -673,6 +673,16 @@ int aaac_debug_fit_wait(int extra_arrivals, unsigned spin_limit) {
     return AAAC_OK;
 }
 
+int aaac_debug_incremental(const void* ws, int* first, int* end) {
+    if (!ws || !first || !end) return AAAC_ERR_NULL;
+    uint32_t at[2];
+    const char* from = static_cast<const char*>(ws) + offsetof(Ctrl, first_incremental);
+    if (cudaMemcpy(at, from, sizeof(at), cudaMemcpyDeviceToHost) != cudaSuccess) return AAAC_ERR_CUDA;
+    *first = (int)at[0];
+    *end = (int)at[1];
+    return AAAC_OK;
+}
+
 unsigned long long aaac_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 // ---- timing of the fit-round kernel ----

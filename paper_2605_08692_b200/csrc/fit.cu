@@ -105,10 +105,11 @@ struct FitParams {
     int rows;                     // rows per warp of an item: 4, or 2 or 1 for layers that have too few items of 4
     int items, per_block, nrb;    // items of 16 * rows rows x 256 columns, items per block, row blocks per slab
     int tail_item0, tail_quarters;   // items from tail_item0 on are dealt out a quarter (one row per warp) per block
-    uint32_t* kept;               // [N][K / 16]: index bits and selection per 16 weights (kKeep and the incremental rounds; the same memory)
+    uint32_t* kept;               // [N][K / 16], the same memory (kKeep and the incremental rounds): per 16 adjacent weights, bit 2 j the low bit
+                                  // of the index of weight j's entry in the table its group has chosen, bit 1 that choice
     int n_inner;                  // incremental rounds: passes per round
-    int n_total;                  // kAssignAgain, kInnerAgain: passes of the whole fit
-    bool restart;                 // the first of those
+    int n_total;                  // kInnerRest: passes of the whole fit
+    bool from_kept;               // kInnerRest: the selection stands in the kept words, and the round that they belong to is finished
 };
 
 constexpr uint32_t kLut1At = 65536;                    // shared address of the bin table (see fit_rounds_body)
@@ -163,13 +164,10 @@ __device__ __forceinline__ void sts_u2(uint32_t addr, uint32_t a, uint32_t b) {
 // single pass followed by one kInner launch of n_inner - 1 passes.
 // kKeep: assignment passes (n_inner = 1) of which the last also stores, per 16 columns of a row, the low bits of
 // the entries' indices and the selection (below); the rounds after it are those of fit_delta.cuh.
-// kRest: assignment passes again, as many as those have left (mostly none).  With n_inner > 1, where they end within a
-// round, kAssignAgain and kInnerAgain do everything again, from the start tables, unless nothing is left.
-enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4, kAssignAgain = 5, kInnerAgain = 6 };
-
-// What the incremental rounds keep of 16 adjacent weights of a row: bit 2 j the low bit of the index of weight j's
-// entry in the table its group has chosen, bit 1 that choice.
-
+// kRest: assignment passes again, as many as those have left (mostly none).  With n_inner > 1 kInnerRest finishes the
+// round in which they ended, with the selection that they kept, and one kAssignRest and one kInnerRest launch per further
+// round make it, unless it is done.
+enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4, kAssignRest = 5, kInnerRest = 6 };
 
 // Decides the listed selection groups in double (Eq. 8: each lane adds its weights' terms in index
 // order, the lanes of the group are combined pairwise; a tie goes to table 0) and adds every weight
@@ -255,7 +253,7 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
         }
         if (lane == 0) {
             esum += sg ? e1 : e0;
-            if (KIND == kAssignKeep || KIND == kAssignAgain) {
+            if (KIND == kAssignKeep || KIND == kAssignRest) {
                 // the stored selection bits of the row's slab: bit = lane of the row pipeline
                 const uint32_t first = ((uint32_t)cg & 255u) >> 3;
                 const uint32_t mask = (LPG >= 32 ? 0xFFFFFFFFu : ((1u << LPG) - 1u)) << first;
@@ -330,12 +328,20 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     __shared__ FitShared sh;
     FitTables& S = sh.t;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int done = KIND == kRest ? (int)p.ctrl->next_round : 0;
-    const int n_rounds = p.n_rounds - done, trace_base = p.trace_base + done;
-    constexpr bool AGAIN = KIND == kAssignAgain || KIND == kInnerAgain;
-    const unsigned bar_base = KIND == kRest ? p.ctrl->passes : AGAIN ? p.ctrl->passes + p.bar_base : p.bar_base;
-    if (KIND == kRest && n_rounds <= 0) return;
-    if (AGAIN && (int)p.ctrl->next_round >= p.n_total) return;
+    constexpr bool REST = KIND == kRest || KIND == kAssignRest || KIND == kInnerRest;
+    const int passed = REST ? (int)p.ctrl->next_round : 0;
+    int n_rounds = p.n_rounds, trace_base = p.trace_base;
+    if (KIND == kRest) {
+        n_rounds -= passed;
+        trace_base += passed;
+    }
+    if (KIND == kAssignRest && passed != p.trace_base * p.n_inner) return;
+    if (KIND == kInnerRest) {
+        if (p.from_kept) n_rounds = passed < p.n_total && passed % p.n_inner ? p.n_inner - passed % p.n_inner : 0;
+        else if (passed != p.trace_base * p.n_inner + 1) return;
+    }
+    if (REST && n_rounds <= 0) return;
+    const unsigned bar_base = REST ? p.ctrl->passes : p.bar_base;
 
     // 32-bit shared addresses.  The bin table sits at a shared address that is a multiple of its own
     // span (64 KB), so that a lookup's address -- bin bits, the lane's copy and the table base -- is one
@@ -385,8 +391,13 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     uint4 v[R];
     uint32_t sc[R];           // NVFP4: scale byte; INT4: bits of the reciprocal scale
     uint32_t sgw[R];          // inner iteration: the row's stored selection bits
-    constexpr bool INNER = KIND == kInner || KIND == kInnerAgain;
-    constexpr bool keep_sigma = KIND == kAssignKeep || KIND == kAssignAgain;
+    constexpr bool INNER = KIND == kInner || KIND == kInnerRest;
+    constexpr bool keep_sigma = KIND == kAssignKeep || KIND == kAssignRest;
+    // (the selection's words per row, and a lane's bit: see FitParams)
+    const bool from_kept = KIND == kInnerRest && p.from_kept;
+    const uint32_t* const sel = from_kept ? p.kept : p.sigw;
+    const unsigned sel_row = from_kept ? (unsigned)K / 16u : (unsigned)slabs;
+    const int sel_bit = from_kept ? 1 : lane;
     // Offsets of the item being loaded (element offsets fit 32 bits: the entry points refuse layers of 2^32
     // elements and more).  Nothing guards the loads: rows past the item's last read that one again, lanes past
     // K the row's last columns (their importances are zero).
@@ -397,7 +408,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         const unsigned col = (unsigned)min(slab * 256 + lane * 8, K - 8);
         nwo = (unsigned)row * (unsigned)p.ldw + col;
         ngo = (unsigned)row * (unsigned)Gr + col / G;
-        if (INNER) nso = (unsigned)row * (unsigned)slabs + (unsigned)slab;
+        if (INNER) nso = (unsigned)row * sel_row + (from_kept ? col / 16u : (unsigned)slab);
         nlast = min(N - row, rows) - 1;
     };
     // (volatile: the compiler would move these loads down to where the row is worked on, to save registers)
@@ -407,7 +418,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                      : "l"(p.W + (nwo + m * (unsigned)p.ldw)));
         if (MODE == AAAC_NVFP4) asm volatile("ld.global.u8 %0, [%1];" : "=r"(sc[u]) : "l"(p.scales + (ngo + m * (unsigned)Gr)));   // masked at use
         else asm volatile("ld.global.u32 %0, [%1];" : "=r"(sc[u]) : "l"(p.rinv + (ngo + m * (unsigned)Gr)));
-        if (INNER) asm volatile("ld.global.u32 %0, [%1];" : "=r"(sgw[u]) : "l"(p.sigw + (nso + m * (unsigned)slabs)));
+        if (INNER) asm volatile("ld.global.u32 %0, [%1];" : "=r"(sgw[u]) : "l"(sel + (nso + m * sel_row)));
     };
     int cur_slab = -1;
     uint64_t II[4];           // importances of the lane's eight columns, in pairs
@@ -459,7 +470,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 sh.fix_unscale = scalbn(1.0, e - kSumBits);
                 sh.failed = 0;
             }
-            derive_tables(S, lane, AGAIN && p.restart ? p.ctrl->keep_T[lane] : p.ctrl->T[lane]);
+            derive_tables(S, lane, p.ctrl->T[lane]);
         }
     }
     for (int b = 0; b < kBinSlots; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
@@ -543,7 +554,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         uint32_t ba[2][8];                                 // its bin address
         bool sg_row = false;                               // inner iteration: this lane's stored selection bit
         auto L1 = [&](int u) {
-            if (INNER) sg_row = (sgw[u] >> lane) & 1u;
+            if (INNER) sg_row = (sgw[u] >> sel_bit) & 1u;
             const float rinv = MODE == AAAC_NVFP4 ? S.rlut[sc[u] & 0x7Fu] : __uint_as_float(sc[u]);
             const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
             const uint64_t rr = pack2(rinv, rinv);
@@ -870,6 +881,10 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     if (bid == 0 && tid < 2 * kM) {
         p.ctrl->T[tid] = S.Td[tid];
         if (p.T01_out) p.T01_out[tid] = (float)S.Td[tid];
+        if (REST && tid == 0) {
+            p.ctrl->next_round = (uint32_t)(passed + n_rounds);
+            p.ctrl->passes = bar_base + (unsigned)n_rounds;
+        }
     }
 }
 
@@ -935,14 +950,14 @@ cudaError_t launch_kind(FitBatch& b, unsigned grid, int mode, int sel_group, cud
 
 
 // n_inner > 1: per round an assignment pass and the further inner iterations
-template <int ASSIGN, int INNER>
-cudaError_t launch_inner(FitBatch& b, int m, unsigned grid, int mode, int sel_group, int n_outer, int n_inner, cudaStream_t st) {
+template <typename Assign, typename Inner>
+cudaError_t launch_inner(FitBatch& b, int m, int first, int n_outer, int n_inner, Assign assign, Inner inner) {
     cudaError_t e = cudaSuccess;
-    for (int outer = 0; outer < n_outer && e == cudaSuccess; ++outer) {
+    for (int outer = first; outer < n_outer && e == cudaSuccess; ++outer) {
         for (int l = 0; l < m; ++l) { b.L[l].n_rounds = 1; b.L[l].trace_base = outer; }
-        e = launch_kind<ASSIGN>(b, grid, mode, sel_group, st);
-        for (int l = 0; l < m; ++l) { b.L[l].bar_base += 1u; b.L[l].n_rounds = n_inner - 1; b.L[l].restart = false; }
-        if (e == cudaSuccess) e = launch_kind<INNER>(b, grid, mode, sel_group, st);
+        e = assign();
+        for (int l = 0; l < m; ++l) { b.L[l].bar_base += 1u; b.L[l].n_rounds = n_inner - 1; }
+        if (e == cudaSuccess) e = inner();
         for (int l = 0; l < m; ++l) b.L[l].bar_base += (unsigned)(n_inner - 1);
     }
     return e;
@@ -1077,13 +1092,19 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             if (e == cudaSuccess) e = launch_variant<delta_kernel<AAAC_NVFP4, 16>>(b, grid, st);
             if (e == cudaSuccess && n_inner == 1) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);
             if (e == cudaSuccess && n_inner > 1) {
-                for (int l = 0; l < m; ++l) { b.L[l].n_total = n_outer * n_inner; b.L[l].restart = true; }
-                e = launch_inner<kAssignAgain, kInnerAgain>(b, m, grid, mode, sel_group, n_outer, n_inner, st);
+                auto inner_rest = [&] { return launch_variant<fit_kernel<AAAC_NVFP4, 16, kInnerRest>>(b, grid, st); };
+                for (int l = 0; l < m; ++l) { b.L[l].n_total = n_outer * n_inner; b.L[l].from_kept = true; }
+                e = inner_rest();
+                for (int l = 0; l < m; ++l) b.L[l].from_kept = false;
+                if (e == cudaSuccess)
+                    e = launch_inner(b, m, 1, n_outer, n_inner, [&] { return launch_variant<fit_kernel<AAAC_NVFP4, 16, kAssignRest>>(b, grid, st); },
+                                     inner_rest);
             }
         } else if (n_inner == 1) {
             e = launch_kind<kRounds>(b, grid, mode, sel_group, st);
         } else {
-            e = launch_inner<kAssignKeep, kInner>(b, m, grid, mode, sel_group, n_outer, n_inner, st);
+            e = launch_inner(b, m, 0, n_outer, n_inner, [&] { return launch_kind<kAssignKeep>(b, grid, mode, sel_group, st); },
+                             [&] { return launch_kind<kInner>(b, grid, mode, sel_group, st); });
         }
         if (e != cudaSuccess) return e;
         at += m;

@@ -816,7 +816,8 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
         ctl.T[tid] = S.Td[tid];
         if (p.T01_out) p.T01_out[tid] = (float)S.Td[tid];
         if (tid == 0) {
-            ctl.next_round = (uint32_t)round;
+            ctl.first_incremental = (uint32_t)first_round;
+            ctl.next_round = ctl.end_incremental = (uint32_t)round;
             ctl.passes = pass_no;
         }
     }

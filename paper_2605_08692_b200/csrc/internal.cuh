@@ -32,7 +32,8 @@ struct Ctrl {
     double keep_q;                  // that pass's objective
     float keep_c[2 * kM];
     uint32_t keep_ok;               // its tables were in order
-    uint32_t next_round, passes;    // the first round not done; passes made so far (the sum buffers rotate per pass)
+    uint32_t next_round, passes;    // the first pass of the fit not done; passes made so far (the sum buffers rotate per pass)
+    uint32_t first_incremental, end_incremental;    // passes first .. end - 1 of the fit were incremental
     uint32_t abort;                 // set when a block's wait for the totals of a pass ran out
     // quantile selection
     double frac[2 * kM];            // interpolation fraction per table entry

@@ -15,11 +15,13 @@ def _built():
     build.build()
 
 
-def check(W, X, rounds, init, name, inner=1):
-    o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, init={binding.INIT_QUANTILE: "quantile", binding.INIT_GRID: "grid"}[init], n_inner=inner)
-    before = binding.launch_count()
-    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, n_inner=inner, init=init, want_trace=True)
-    launches = binding.launch_count() - before
+def check(W, X, rounds, init, name, inner=1, T01=None):
+    """Compares a fit with the oracle's; returns the passes that were incremental, (first, end)."""
+    o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, n_inner=inner, T_init=T01,
+                         init={binding.INIT_QUANTILE: "quantile", binding.INIT_GRID: "grid", binding.INIT_USER: "user"}[init])
+    ws = binding.alloc_workspace(NVFP4, W.shape[0], W.shape[1], X.shape[0])
+    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, n_inner=inner, init=init, want_trace=True, ws=ws,
+                               T01_init=None if T01 is None else torch.from_numpy(T01))
     torch.cuda.synchronize()
     assert int(r["status"].item()) == 0
     assert table_close(host(r["T01"]), o["T"])[0], name
@@ -27,7 +29,7 @@ def check(W, X, rounds, init, name, inner=1):
     # distance of the constants from the entries, 8 units in the last place at most: (2^-20 * 8)^2 of sum I)
     assert np.allclose(host(r["trace"])[:rounds], o["trace"], rtol=1e-5, atol=1e-10 * o["trace"][0]), name
     check_end_to_end_bits(r, o, name)
-    return launches
+    return binding.debug_incremental(ws)
 
 
 def rows_for(units, K):
@@ -47,16 +49,39 @@ def rows_for(units, K):
 ])
 def test_layers_of_few_units_per_block(K, units, extra, rounds, inner, init):
     W, X = layer(NVFP4, rows_for(units, K) + extra, K, T=64, name=f"incremental/{K}/{extra}")
-    # (of a few rows a fit is one launch, with inner iterations two a round; here they are two more)
-    few = check(W[:64].copy(), X, rounds, init, "a few rows", inner)
-    assert check(W, X, rounds, init, f"incremental {K} {units} {extra}", inner) == few + 2
+    assert check(W, X, rounds, init, f"incremental {K} {units} {extra}", inner) == (3 if inner == 1 else 1, rounds * inner)
 
 
 def test_inner_iterations_from_equal_entries_are_not_tried():
     """The NVFP4 grid holds 0 twice: such a fit could not begin, and runs the launches of a small one."""
     W, X = layer(NVFP4, rows_for(8, 2048), 2048, T=64, name="incremental/2048/0")
-    few = check(W[:64].copy(), X, 3, binding.INIT_GRID, "a few rows", 10)
-    assert check(W, X, 3, binding.INIT_GRID, "grid start, 3 x 10", 10) == few
+    counts = []
+    for rows in (64, len(W)):
+        before = binding.launch_count()
+        assert check(W[:rows].copy(), X, 3, binding.INIT_GRID, f"grid start, 3 x 10, {rows} rows", 10) == (0, 0)
+        counts.append(binding.launch_count() - before)
+    assert counts[0] == counts[1]
+
+
+def tables(t0, t1):
+    return np.stack([t0, t1]).astype(np.float32)
+
+
+@pytest.mark.parametrize("start,rounds,inner", [
+    ("far", 3, 10), ("far", 1, 30), ("apart", 25, 1), ("apart", 2, 14), ("twins", 3, 10)])
+def test_fits_that_end_early_are_finished(start, rounds, inner):
+    """Start tables beside the weights, whose entries jump: a cell's weight changes too much, or a breakpoint passes its
+    neighbour, within the fit and within a round.  Equal entries: it cannot begin where it starts from the first pass."""
+    N, K = rows_for(12, 512), 512
+    W, X = layer(NVFP4, N, K, T=64, name="incremental/early")
+    even = np.linspace(-6, 6, 16)
+    T01 = {"far": tables(np.linspace(0.5, 1.5, 16), np.linspace(0.52, 1.52, 16)), "apart": tables(np.linspace(-6, -1, 16), np.linspace(1, 6, 16)),
+           "twins": tables(np.where(np.arange(16) == 8, even[7], even), even)}[start]
+    first, end = check(W, X, rounds, binding.INIT_USER, f"{start} {rounds} x {inner}", inner, T01)
+    if start == "twins":
+        assert (first, end) == (0, 0)
+    else:
+        assert first == (3 if inner == 1 else 1) and first < end < rounds * inner - 1
 
 
 @pytest.mark.parametrize("rounds,inner", [(25, 1), (3, 10)])
