@@ -162,8 +162,9 @@ __device__ __forceinline__ void sts_u2(uint32_t addr, uint32_t a, uint32_t b) {
 // kAssignKeep: the same pass, which also stores the selection bits.  kInner: further inner
 // iterations with the stored selection.  With n_inner > 1 a round is one kAssignKeep launch of a
 // single pass followed by one kInner launch of n_inner - 1 passes.
-// kKeep: assignment passes (n_inner = 1) of which the last also stores, per 16 columns of a row, the low bits of
-// the entries' indices and the selection (below); the rounds after it are those of fit_delta.cuh.
+// kKeep: one assignment pass with exact weight sums (collect_counts) that also stores, per 16 columns of a row, the low
+// bits of the entries' indices and the selection; the passes after it are those of fit_delta.cuh.  (A launch of its own:
+// with the first rounds in it, their bin updates paid for the choice of what to add, 14 us a pass of 16432 x 8192.)
 // kRest: assignment passes again, as many as those have left (mostly none).  With n_inner > 1 kInnerRest finishes the
 // round in which they ended, with the selection that they kept, and one kAssignRest and one kInnerRest launch per further
 // round make it, unless it is done.
@@ -174,6 +175,14 @@ enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4, 
 // to the calling lane's bins under the chosen table, with the arithmetic of the row pipeline
 // (centred term I (x - c), c the chosen entry's centre constant).  Every lane of the warp calls;
 // returns the sum of the groups' smaller errors in lane 0 (0 elsewhere).
+__device__ __forceinline__ void add_term(uint32_t addr, float v) {
+    float a;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(addr) : "memory");
+    asm volatile("st.shared.f32 [%0], %1;" :: "r"(addr), "f"(a + v) : "memory");
+}
+__device__ __forceinline__ void count_weight(uint32_t addr, uint32_t one) {
+    asm volatile("red.shared.add.u32 [%0], %1;" :: "r"(addr), "r"(one) : "memory");
+}
 struct DeferArgs {                // what the routine needs of the layer (passed by value: the kernel's
     const uint16_t* W;            // parameters themselves stay where they are)
     int64_t K, ldw;
@@ -235,10 +244,19 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
                 const float2 c2 = S->pq32[Js[t]];
                 const float c = sg ? c2.y : c2.x;
                 const uint32_t a = bins_lane + ((sg ? (uint32_t)kM : 0u) + (__float_as_uint(c) & kIdxMask)) * kSlotBytes;
-                float2 b = lds_bin(a);
-                b.x += __fmul_rn(Is[t], __fsub_rn(xs[t], c));
-                b.y += Is[t];
-                sts_bin(a, b);
+                const float term = __fmul_rn(Is[t], __fsub_rn(xs[t], c));
+                if (KIND == kKeep) {
+                    // (the count belongs to the lane that has the column in the row pipeline)
+                    static_assert(KIND != kKeep || WPL == 1, "a weight per lane");
+                    const uint32_t col = (uint32_t)(cg + lane) & 255u;
+                    add_term(a, term);
+                    count_weight(a + ((col >> 3) - (uint32_t)lane) * 8u + 4u, 1u << (4 * (col & 7u)));
+                } else {
+                    float2 b = lds_bin(a);
+                    b.x += term;
+                    b.y += Is[t];
+                    sts_bin(a, b);
+                }
                 parity |= (__float_as_uint(c) & 1u) << (2 * t);
             }
         }
@@ -308,6 +326,57 @@ __device__ __forceinline__ void group_sums(float& e0, float& e1, int lane) {
             e1 += __shfl_xor_sync(kAll, e1, s);
         }
     }
+}
+
+// The weight sums of the pass that the incremental rounds start from.  They carry a cell's sum of I from round to round,
+// and an error of it counts times the way its entry has gone since, where one of any other pass counts times the entry's
+// movement in that pass.  FP32 sums in a lane's bins are not good enough for that: a lane's eight importances are the same
+// in every row, so are their rounding errors (those of a massive channel's neighbours above all), and no number of rows
+// averages them out: -1e-8 of the sum in every cell.  In this pass a bin's second word therefore counts the weights of the
+// lane's eight columns, four bits each.  After every 12 rows, and before the slab changes, the block adds its warps'
+// counts and multiplies them by the importances in double: warp w takes the cells 2 w and 2 w + 1, and their residuals
+// too.  The bins are zero again behind it.  Every thread calls.
+// Tables of one pass against 64-bit sums, 2-norm, 35520 x 1024 Student-t weights, pass 25: 3.4e-9 -> 1.7e-10 (a full
+// pass: 1.2e-10); bins emptied into doubles after every item instead: 2.4e-10 to 5.6e-10.
+constexpr int kCountedItems = 3;                      // items of four rows: 12 rows, a count has room for 15
+static_assert(kCountedItems * kRowsPerWarp < 16, "four bits a count");
+struct CountedSums { double x[2], y[2]; };            // a lane's part of two cells' sums, 2^-896 times
+__device__ __noinline__ void collect_counts(CountedSums* const sums, const uint32_t low_at, const uint32_t high_at, const int n_low,
+                                            const uint32_t warp_bytes, const float4 I0, const float4 I1, const int warp, const int lane) {
+    const float I[8] = {I0.x, I0.y, I0.z, I0.w, I1.x, I1.y, I1.z, I1.w};
+    __syncthreads();
+    const uint32_t at = (uint32_t)(2 * warp) * kSlotBytes + (uint32_t)lane * 8u;
+    double x[2] = {0.0, 0.0}, y[2] = {0.0, 0.0};
+    uint32_t even[2] = {0u, 0u}, odd[2] = {0u, 0u};   // counts over the warps, a byte each (16 times 12 at most)
+#pragma unroll 4
+    for (int w = 0; w < kFitWarps; ++w) {
+        const uint32_t a = at + (w < n_low ? low_at + (uint32_t)w * warp_bytes : high_at + (uint32_t)(w - n_low) * warp_bytes);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float2 b = lds_bin(a + c * kSlotBytes);
+            sts_bin(a + c * kSlotBytes, make_float2(0.f, 0.f));
+            x[c] += scaled_double(b.x);
+            const uint32_t n = __float_as_uint(b.y);
+            even[c] += n & 0x0F0F0F0Fu;
+            odd[c] += (n >> 4) & 0x0F0F0F0Fu;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const double Id = scaled_double(I[j]);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const uint32_t n = (((j & 1) ? odd[c] : even[c]) >> (8 * (j >> 1))) & 255u;
+            // (n as a double: 2^52 + n has it in its low bits; no 0 * Inf in cells without the column)
+            if (n) y[c] = __fma_rn(Id, __hiloint2double(0x43300000, (int)n) - 0x1p52, y[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        sums->x[c] += x[c];
+        sums->y[c] += y[c];
+    }
+    __syncthreads();
 }
 
 // SEL is the selection group size S (Sec. 3.1): the weights that share one codebook choice; the
@@ -485,7 +554,6 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
 
   for (int round = 0; round < n_rounds; ++round) {
     const unsigned pass_no = bar_base + (unsigned)round;
-    const bool keep = KIND == kKeep && round + 1 == n_rounds;
     // block 0 clears the buffer of the next pass: it was the buffer of two passes ago, and every block
     // finished reading it before it added to the previous pass's buffer, whose totals block 0 has seen
     static_assert(NT >= 256 + kCells * 4 + kLimbs, "threads 256.. of block 0 clear the next buffer");
@@ -499,6 +567,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     const float g1 = 0x1p-24f * __fmaf_ru(S.tmax283, 4.f, 16.f), g2 = 0x1p-24f * __fmul_ru(S.tmax283, 0.0625f);
     double Eacc = 0.0;
 
+    CountedSums collected{};
+    int counted = 0;          // items since the last collect_counts
     int ndefer = 0;           // groups on the warp's list (the same in every lane)
     float isum = __fmul_ru(isum_raw, g2);
     for (int i = 0; i < n_items; ++i) {
@@ -646,7 +716,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 const unsigned bits = __ballot_sync(0xFFFFFFFFu, sg);        // (the bits of listed groups are set when they are decided)
                 if (lane == 0) p.sigw[(size_t)row * (size_t)slabs + slab] = bits;
             }
-            if (KIND == kKeep && keep) {
+            if (KIND == kKeep) {
                 // (the two lanes of 16 columns write a half each; the selection stands in the lower one)
                 uint32_t bits = 0;
 #pragma unroll
@@ -667,7 +737,8 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             for (int j = j0; j < j1; ++j) {
                 float2 a = lds_bin(ba_i[j]);
                 a.x += mt_i[j];
-                a.y += Ic(j);
+                if (KIND == kKeep) a.y = __uint_as_float(__float_as_uint(a.y) + (1u << (4 * j)));
+                else a.y += Ic(j);
                 sts_bin(ba_i[j], a);
             }
         };
@@ -719,15 +790,21 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             for (int t = 0; t < R; ++t) load_row(t);
         }
         Eacc += (double)eitem;
-        if (!INNER && ndefer > kDeferCap - R * (32 / LPG)) {    // the next item could overflow the list
+        const bool collect = KIND == kKeep && (++counted == kCountedItems || i + 1 == n_items || nslab != slab);
+        if (!INNER && (ndefer > kDeferCap - R * (32 / LPG) || (collect && ndefer > 0))) {    // the next item could overflow the list, or the counts
             __syncwarp();
-            Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw, KIND == kKeep ? p.kept : nullptr}, list_addr, ndefer, bins_lane, lane);
+            Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw, p.kept}, list_addr, ndefer, bins_lane, lane);
             ndefer = 0;
+        }
+        if (collect) {
+            collect_counts(&collected, sm_base, hi_base, n_low, kBinBytes, make_float4(Ic(0), Ic(1), Ic(2), Ic(3)),
+                           make_float4(Ic(4), Ic(5), Ic(6), Ic(7)), warp, lane);
+            counted = 0;
         }
     }
     if (!INNER && ndefer > 0) {
         __syncwarp();
-        Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw, KIND == kKeep ? p.kept : nullptr}, list_addr, ndefer, bins_lane, lane);
+        Eacc += resolve_deferred<MODE, SEL, KIND>(&S, DeferArgs{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.sigw, p.kept}, list_addr, ndefer, bins_lane, lane);
     }
 
     // ---- the warp's sums: lane c adds the 32 lane-private values of cell c (in an order of its own that
@@ -735,7 +812,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     //      unless they are more than 2^24 apart ----
     const bool trace = !INNER && p.err_trace != nullptr;
     __syncwarp();
-    {
+    if (KIND != kKeep) {
         const uint32_t cell_addr = bins_warp + lane * (kSlotBytes + 8);
         double dx[4] = {0.0, 0.0, 0.0, 0.0}, dy[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
@@ -749,11 +826,28 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
         }
         sh.wsum[warp][lane] = ((dx[0] + dx[1]) + (dx[2] + dx[3])) * 0x1p896;
         sh.wsum[warp][kCells + lane] = ((dy[0] + dy[1]) + (dy[2] + dy[3])) * 0x1p896;
-        if (trace) {
+    } else {
+        // the block's sums of two cells, which the others' rows add nothing to
+        sh.wsum[warp][lane] = sh.wsum[warp][kCells + lane] = 0.0;
+        __syncwarp();
 #pragma unroll
-            for (int s = 16; s; s >>= 1) Eacc += __shfl_xor_sync(kAll, Eacc, s);
-            if (lane == 0) sh.wsum[warp][2 * kCells] = Eacc;
+        for (int c = 0; c < 2; ++c) {
+            double x = collected.x[c], y = collected.y[c];
+#pragma unroll
+            for (int s = 16; s; s >>= 1) {
+                x += __shfl_xor_sync(kAll, x, s);
+                y += __shfl_xor_sync(kAll, y, s);
+            }
+            if (lane == 0) {
+                sh.wsum[warp][2 * warp + c] = x * 0x1p896;
+                sh.wsum[warp][kCells + 2 * warp + c] = y * 0x1p896;
+            }
         }
+    }
+    if (trace) {
+#pragma unroll
+        for (int s = 16; s; s >>= 1) Eacc += __shfl_xor_sync(kAll, Eacc, s);
+        if (lane == 0) sh.wsum[warp][2 * kCells] = Eacc;
     }
     __syncthreads();                                       // every warp is done with the lookup tables, its sums are there
     unsigned long long* const acc = p.acc + (size_t)(pass_no % 3u) * kAccBuffer;
@@ -847,7 +941,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
                 T = S.Td[lane];
                 __syncwarp();
             }
-            if (KIND == kKeep && keep && bid == 0) {
+            if (KIND == kKeep && bid == 0) {
                 // what the incremental rounds start from
                 Ctrl& c = *p.ctrl;
                 c.keep_T[lane] = before;
@@ -1035,7 +1129,7 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
 // They start from the first pass's tables, though, and do not begin where these hold one value twice, as the NVFP4 grid
 // does (tried and made again, 4096 x 4096 took 778 us for 743, and 312 for 274 in one round of 10).
 // A piece is read with one 32-byte load; its number must be divisible by more than one piece per row (row_of).
-constexpr int kFullRounds = 3;
+constexpr int kFullRounds = 3;                        // the last of them the keeping one
 static bool can_increment(const FitLayerArgs& a, int64_t blocks, int n_outer, int n_inner) {
     const int64_t slabs = (a.K + kDeltaCols - 1) / kDeltaCols, units = slabs * ((a.N + kFitWarps - 1) / kFitWarps);
     const bool pays = n_inner == 1 ? units >= 12 * blocks && (n_outer - 6) * units >= 220 * blocks
@@ -1085,9 +1179,15 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
         cudaError_t e = cudaSuccess;
         if (incremental) {
             // the first rounds (the first pass), the last of which stores what the incremental ones need; these; and
-            // whatever they leave undone
-            for (int l = 0; l < m; ++l) b.L[l].n_rounds = full;
-            e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kKeep>>(b, grid, st);
+            // whatever they leave undone.  (16432 x 8192: the keeping pass takes 41 us more than a full one, 18 of them
+            // the counts, the rest its launch; 4096 x 14336: 33 and 19.)
+            if (n_inner == 1) {
+                for (int l = 0; l < m; ++l) b.L[l].n_rounds = full - 1;
+                e = launch_kind<kRounds>(b, grid, mode, sel_group, st);
+            }
+            for (int l = 0; l < m; ++l) { b.L[l].n_rounds = 1; b.L[l].trace_base = full - 1; b.L[l].bar_base = (unsigned)(full - 1); }
+            if (e == cudaSuccess) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kKeep>>(b, grid, st);
+            for (int l = 0; l < m; ++l) b.L[l].trace_base = 0;
             for (int l = 0; l < m; ++l) { b.L[l].n_rounds = n_outer * n_inner; b.L[l].n_inner = n_inner; }
             if (e == cudaSuccess) e = launch_variant<delta_kernel<AAAC_NVFP4, 16>>(b, grid, st);
             if (e == cudaSuccess && n_inner == 1) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);

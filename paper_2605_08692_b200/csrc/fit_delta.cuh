@@ -24,8 +24,12 @@
 // lane, and change the lane's bins.
 //
 // Accuracy.  The sums start from a full pass (kKeep), centred on that pass's constants c, and stay centred on them:
-// sum I (x - c) and sum I.  T = c + sum I (x - c) / sum I, so an error of sum I counts times T - c only, as in a full
-// pass, and what a pass adds is the FP32 rounding of the terms that move.  A cell that has lost three quarters
+// sum I (x - c) and sum I.  T = c + sum I (x - c) / sum I, so an error of sum I counts times T - c, which is the way the
+// entry has gone since that pass (0.2 to 0.6 at the end, where a full pass has the 0.01 of a round): the sums of I start
+// exact (collect_counts).  A weight leaves a cell with the very term it came with, rounding included, so what is left is one
+// FP32 rounding per weight of a cell, as in a full pass, of terms that are larger by |x - c| over |x - T|, and the
+// roundings of the few that meet in a bin within a pass.  Tables of one pass against 64-bit sums, 2-norm, mean over 24
+// fits of four sizes: 1.2e-10, a full pass 1.0e-10.  A cell that has lost three quarters
 // of the weight it started with (what is left of the first pass's rounding would weigh four times as much in it), or gains
 // weight from nothing, ends the incremental rounds before its sum is used.  So do a table out of order, equal entries and a breakpoint
 // that passes a neighbour; the rounds that are left are then made by fit_rounds_body.

@@ -96,6 +96,32 @@ def test_layers_of_few_distinct_weights(levels, rounds, inner):
     check(W, X, rounds, binding.INIT_GRID, f"levels {levels}", inner)
 
 
+@pytest.mark.parametrize("K,units,extra,rounds,inner", [(512, 12, 0, 25, 1), (1008, 16, 5, 21, 1), (4096, 24, -3, 17, 1), (512, 4, -3, 3, 14), (1008, 9, 5, 2, 10)])
+def test_weight_sums_that_are_carried_are_exact(K, units, extra, rounds, inner):
+    """The sums of I that the incremental passes start from, against 64-bit sums over the cells of the same tables: counts
+    times importances, rounded a few dozen times to 2^-53.  (FP32 sums erred by 1e-8 in every cell.)"""
+    N = rows_for(units, K) + extra
+    W, X = layer(NVFP4, N, K, T=64, name=f"incremental/sums/{K}/{extra}", dist="student5")
+    Wd, ws = dev_bf16(W), binding.alloc_workspace(NVFP4, N, K)
+    r = binding.quantize_layer(Wd, NVFP4, X=dev_bf16(X), n_outer=rounds, n_inner=inner, init=binding.INIT_QUANTILE, ws=ws)
+    torch.cuda.synchronize()
+    assert binding.debug_incremental(ws)[0] == (3 if inner == 1 else 1)
+    T, _, got = ws[272:272 + 768].clone().view(torch.float64).view(3, 2, 16)      # Ctrl::keep_T, keep_sx, keep_sw
+    scale = torch.arange(128, dtype=torch.uint8, device="cuda").view(torch.float8_e4m3fn).float()[r["scales_pos"].long()] * r["tensor_scale"]
+    I = r["I"].double().view(1, -1, 16)
+    want = torch.zeros(2, 16, dtype=torch.float64, device="cuda")
+    for r0 in range(0, N, 4096):
+        x = (Wd[r0:r0 + 4096].float().view(-1, K // 16, 16) * (1.0 / scale[r0:r0 + 4096])[..., None]).double()
+        cell = [torch.searchsorted((0.5 * (t[1:] + t[:-1])).contiguous(), x) for t in T]
+        err = [(I * (x - t[c]) ** 2).sum(-1) for t, c in zip(T, cell)]
+        second = (err[1] < err[0])[..., None]
+        for t in range(2):
+            mine = second if t else ~second
+            for c in range(16):
+                want[t, c] += (I * ((cell[t] == c) & mine)).sum()
+    assert torch.allclose(got, want, rtol=1e-12, atol=0)
+
+
 def test_two_runs_give_the_same_bits():
     N, K = rows_for(17, 2048), 2048
     W, X = layer(NVFP4, N, K, T=64, name="incremental/twice")
