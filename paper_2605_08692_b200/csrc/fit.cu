@@ -97,7 +97,7 @@ struct FitParams {
     float* T01_out;               // [2][16] or null: the tables after the launch's last pass, as FP32
     uint32_t* dev_status;         // or null
     uint32_t* sigw;               // [N][slabs]: selection bits of a row's 256-column slab, bit = lane (n_inner > 1)
-    int n_rounds;                 // passes over W in this launch (of the incremental rounds: in all)
+    int n_rounds;                 // passes over W in this launch (incremental rounds, kRest: of the fit so far, with this launch's)
     int trace_base;               // err_trace index of this launch's first assignment pass
     unsigned bar_base;            // passes of the layer's earlier launches (the sum buffers rotate per pass)
     unsigned arrivals;            // blocks whose sums a total must hold before it is read (the grid size)
@@ -165,7 +165,8 @@ __device__ __forceinline__ void sts_u2(uint32_t addr, uint32_t a, uint32_t b) {
 // kKeep: one assignment pass with exact weight sums (collect_counts) that also stores, per 16 columns of a row, the low
 // bits of the entries' indices and the selection; the passes after it are those of fit_delta.cuh.  (A launch of its own:
 // with the first rounds in it, their bin updates paid for the choice of what to add, 14 us a pass of 16432 x 8192.)
-// kRest: assignment passes again, as many as those have left (mostly none).  With n_inner > 1 kInnerRest finishes the
+// kRest: assignment passes again, as many as those have left: the last of the fit, whose sums are made anew for the
+// tables that are handed out, and mostly no other.  With n_inner > 1 kInnerRest finishes the
 // round in which they ended, with the selection that they kept, and one kAssignRest and one kInnerRest launch per further
 // round make it, unless it is done.
 enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4, kAssignRest = 5, kInnerRest = 6 };
@@ -1174,12 +1175,12 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
         }
         for (int l = m; l <= kMaxBatch; ++l) b.first[l] = grid;
         const int full = n_inner == 1 ? kFullRounds : 1;
-        bool incremental = mode == AAAC_NVFP4 && n_outer * n_inner > full;
+        bool incremental = mode == AAAC_NVFP4 && n_outer * n_inner > full + 1;
         for (int l = 0; l < m; ++l) incremental = incremental && can_increment(layers[at + l], b.first[l + 1] - b.first[l], n_outer, n_inner);
         cudaError_t e = cudaSuccess;
         if (incremental) {
-            // the first rounds (the first pass), the last of which stores what the incremental ones need; these; and
-            // whatever they leave undone.  (16432 x 8192: the keeping pass takes 41 us more than a full one, 18 of them
+            // the first rounds (the first pass), the last of which stores what the incremental ones need; these; and the
+            // last pass, or whatever they leave undone.  (16432 x 8192: the keeping pass takes 41 us more than a full one, 18 of them
             // the counts, the rest its launch; 4096 x 14336: 33 and 19.)
             if (n_inner == 1) {
                 for (int l = 0; l < m; ++l) b.L[l].n_rounds = full - 1;
@@ -1188,8 +1189,9 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             for (int l = 0; l < m; ++l) { b.L[l].n_rounds = 1; b.L[l].trace_base = full - 1; b.L[l].bar_base = (unsigned)(full - 1); }
             if (e == cudaSuccess) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kKeep>>(b, grid, st);
             for (int l = 0; l < m; ++l) b.L[l].trace_base = 0;
-            for (int l = 0; l < m; ++l) { b.L[l].n_rounds = n_outer * n_inner; b.L[l].n_inner = n_inner; }
+            for (int l = 0; l < m; ++l) { b.L[l].n_rounds = n_outer * n_inner - 1; b.L[l].n_inner = n_inner; }
             if (e == cudaSuccess) e = launch_variant<delta_kernel<AAAC_NVFP4, 16>>(b, grid, st);
+            for (int l = 0; l < m; ++l) b.L[l].n_rounds = n_outer * n_inner;
             if (e == cudaSuccess && n_inner == 1) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);
             if (e == cudaSuccess && n_inner > 1) {
                 auto inner_rest = [&] { return launch_variant<fit_kernel<AAAC_NVFP4, 16, kInnerRest>>(b, grid, st); };

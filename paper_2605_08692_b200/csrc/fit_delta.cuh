@@ -29,7 +29,8 @@
 // exact (collect_counts).  A weight leaves a cell with the very term it came with, rounding included, so what is left is one
 // FP32 rounding per weight of a cell, as in a full pass, of terms that are larger by |x - c| over |x - T|, and the
 // roundings of the few that meet in a bin within a pass.  Tables of one pass against 64-bit sums, 2-norm, mean over 24
-// fits of four sizes: 1.2e-10, a full pass 1.0e-10.  A cell that has lost three quarters
+// fits of four sizes: 1.2e-10, a full pass 1.0e-10.  The last pass of a fit is a full one, so the tables that are handed
+// out have a full pass's error.  A cell that has lost three quarters
 // of the weight it started with (what is left of the first pass's rounding would weigh four times as much in it), or gains
 // weight from nothing, ends the incremental rounds before its sum is used.  So do a table out of order, equal entries and a breakpoint
 // that passes a neighbour; the rounds that are left are then made by fit_rounds_body.
@@ -37,7 +38,7 @@
 // Objective of a round (Eq. 8), from the same sums: with q = sum I (x - c)^2 carried along like them and d = T - c,
 // sum I (x - T)^2 = q - sum over the cells (2 d sum I (x - c) - d^2 sum I).
 //
-// Inner iterations (n_inner > 1).  All passes of the fit but the first run here; in a further inner iteration the kept
+// Inner iterations (n_inner > 1).  All passes of the fit but the first and the last run here; in a further inner iteration the kept
 // selection stands, and only moves within a table occur.
 //
 // What bounds it.  A pass over 4096 x 14336 takes 42 us where nothing moves (full rounds: 70), 19 instructions a weight at 72 %
@@ -462,7 +463,7 @@ __device__ __noinline__ float apply_flips(const DeltaShared* sh, const DeltaArgs
     return dq;
 }
 
-// The incremental rounds of one layer, from the first after the kKeep launch to p.n_rounds, run by the blocks
+// The incremental passes of one layer, from the first after the kKeep launch to p.n_rounds, run by the blocks
 // bid = 0 .. nblk - 1.  Layout in shared memory as in fit_rounds_body.
 template <int MODE, int SEL>
 __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsigned bid, const unsigned nblk) {
