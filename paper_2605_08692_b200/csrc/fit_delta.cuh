@@ -31,8 +31,8 @@
 // roundings of the few that meet in a bin within a pass.  Tables of one pass against 64-bit sums, 2-norm, mean over 24
 // fits of four sizes: 1.2e-10, a full pass 1.0e-10.  The last pass of a fit is a full one, so the tables that are handed
 // out have a full pass's error.  A cell that has lost three quarters
-// of the weight it started with (what is left of the first pass's rounding would weigh four times as much in it), or gains
-// weight from nothing, ends the incremental rounds before its sum is used.  So do a table out of order, equal entries and a breakpoint
+// of the most weight it has had (the roundings of all that passed through its bins would weigh four times as much in what
+// is left), or gains weight from nothing, ends the incremental rounds before its sum is used.  So do a table out of order, equal entries and a breakpoint
 // that passes a neighbour; the rounds that are left are then made by fit_rounds_body.
 //
 // Objective of a round (Eq. 8), from the same sums: with q = sum I (x - c)^2 carried along like them and d = T - c,
@@ -199,7 +199,7 @@ constexpr uint32_t kPieceMask = (1u << 28) - 1u, kSelected = 1u << 28, kUndecide
 
 struct DeltaShared {
     FitTables t;
-    double sx[kCells], sw[kCells], sw0[kCells];   // the cells' sums, and the weight sums at the start
+    double sx[kCells], sw[kCells], sw_most[kCells];   // the cells' sums, and the largest weight sums that they have had
     double q;
     double fix_scale, fix_unscale;
     float2 ab[kJSlots];                           // {A, B} of every interval
@@ -564,7 +564,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             const double bp = __shfl_up_sync(kAll, before, 1);
             good = interlaced(sh.mid_old, S.tmp_b, lane) && good && S.no_dup && !__any_sync(kAll, (lane & 15) != 0 && !(bp <= before));
             sh.sx[lane] = ctl.keep_sx[lane];
-            sh.sw[lane] = sh.sw0[lane] = ctl.keep_sw[lane];
+            sh.sw[lane] = sh.sw_most[lane] = ctl.keep_sw[lane];
             sh.c[lane] = ctl.keep_c[lane];
             if (lane == 0) {
                 sh.q = ctl.keep_q;
@@ -774,8 +774,8 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
                 if (lane == 0) sh.failed = 1;
             } else {
                 const double sx = sh.sx[lane] + total_of(t.x, nblk, sh.fix_unscale), sw = sh.sw[lane] + total_of(t.y, nblk, sh.fix_unscale);
-                const double sw0 = sh.sw0[lane];
-                if (!__all_sync(kAll, sw0 > 0.0 ? sw > 0.25 * sw0 : sw0 == 0.0 && sw == 0.0)) {
+                const double most = sh.sw_most[lane];
+                if (!__all_sync(kAll, most > 0.0 ? sw > 0.25 * most : most == 0.0 && sw == 0.0)) {
                     if (lane == 0) sh.stop = 1;                    // this round is not used
                 } else {
                     const double c = (double)sh.c[lane], before = S.Td[lane];
@@ -792,6 +792,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
                     }
                     sh.sx[lane] = sx;
                     sh.sw[lane] = sw;
+                    sh.sw_most[lane] = fmax(most, sw);
                     sh.mid_old[lane] = S.tmp_b[lane];
                     const bool moved = sort_tables(S, T, lane);
                     __syncwarp();

@@ -96,6 +96,47 @@ def test_layers_of_few_distinct_weights(levels, rounds, inner):
     check(W, X, rounds, binding.INIT_GRID, f"levels {levels}", inner)
 
 
+def followed(W, I, T, rounds):
+    """The first pass behind the third at which a cell's weight falls below a quarter of the most it has had since, from a
+    plain 64-bit run; the passes that can be incremental if there is none."""
+    s, ts = oracle.scales(W, NVFP4, 16)
+    x, w = oracle.normalise(W, NVFP4, 16, s, ts).astype(np.float64), np.broadcast_to(I.astype(np.float64), W.shape)
+    T, most = T.astype(np.float64), None
+    for r in range(rounds - 1):
+        at = [np.searchsorted(0.5 * (t[1:] + t[:-1]), x) for t in T]
+        err = [(w * (x - t[a]) ** 2).reshape(len(W), -1, 16).sum(-1) for t, a in zip(T, at)]
+        cell = np.where(np.repeat(err[1] < err[0], 16, axis=1), at[1] + 16, at[0]).ravel()
+        sw, sx = (np.bincount(cell, v.ravel(), minlength=32) for v in (w, w * x))
+        if most is not None and (sw <= 0.25 * most)[most > 0].any():
+            return r
+        if r >= 2:
+            most = sw if most is None else np.maximum(most, sw)
+        T = np.sort(np.divide(sx, sw, out=T.ravel().copy(), where=sw > 0).reshape(2, 16), axis=1)
+    return rounds - 1
+
+
+@pytest.mark.parametrize("seed", [132, 163, 251])
+def test_a_cell_that_loses_what_it_has_gained_ends_the_incremental_rounds(seed):
+    """Cells that grow behind the third round and shrink again, though never below a quarter of their weight there."""
+    rng = np.random.default_rng(seed)
+    W = synth.f32_to_bf16_bits((rng.standard_normal((64, 512)) * 0.02).astype(np.float32))
+    I = np.exp(rng.uniform(0.5, 3.0) * rng.standard_normal(512)).astype(np.float32)
+    T01 = tables(*(np.linspace(*np.sort(rng.uniform(-6, 6, 2)), 16) for _ in range(2)))
+    rounds = 28
+    end = followed(W, I, T01, rounds)
+    assert 3 < end < rounds - 1
+    W = np.tile(W, (rows_for(12, 512) // 64, 1))
+    ws = binding.alloc_workspace(NVFP4, *W.shape)
+    o = oracle.fit_layer(W, NVFP4, 16, rounds, I=I, init="user", T_init=T01)
+    r = binding.quantize_layer(dev_bf16(W), NVFP4, I=torch.from_numpy(I).cuda(), n_outer=rounds, init=binding.INIT_USER, ws=ws, want_trace=True,
+                               T01_init=torch.from_numpy(T01))
+    torch.cuda.synchronize()
+    assert binding.debug_incremental(ws) == (3, end)
+    assert int(r["status"].item()) == 0 and table_close(host(r["T01"]), o["T"])[0]
+    assert np.allclose(host(r["trace"]), o["trace"], rtol=1e-5, atol=0)
+    check_end_to_end_bits(r, o, f"seed {seed}")
+
+
 @pytest.mark.parametrize("K,units,extra,rounds,inner", [(512, 12, 0, 25, 1), (1008, 16, 5, 21, 1), (4096, 24, -3, 17, 1), (512, 4, -3, 3, 14), (1008, 9, 5, 2, 10)])
 def test_weight_sums_that_are_carried_are_exact(K, units, extra, rounds, inner):
     """The sums of I that the incremental passes start from, against 64-bit sums over the cells of the same tables: counts
