@@ -811,7 +811,7 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
     // ---- the warp's sums: lane c adds the 32 lane-private values of cell c (in an order of its own that
     //      avoids bank conflicts, and a fixed one).  In double, 32 FP32 values are added without rounding
     //      unless they are more than 2^24 apart ----
-    const bool trace = !INNER && p.err_trace != nullptr;
+    const bool trace = KIND == kKeep || (!INNER && p.err_trace != nullptr);
     __syncwarp();
     if (KIND != kKeep) {
         const uint32_t cell_addr = bins_warp + lane * (kSlotBytes + 8);
@@ -925,7 +925,10 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             double T = wt > 0.0 ? (double)S.centre[lane] + __ddiv_rn(sx, wt) : S.Td[lane];
             // the trace holds the Eq. 8 objective of each assignment step
             double err = 0.0;
-            if (my_e) p.err_trace[trace_base + round] = err = 16.0 * total(e);
+            if (my_e) {
+                err = 16.0 * total(e);
+                if (KIND != kKeep || p.err_trace) p.err_trace[trace_base + round] = err;
+            }
             const double Tp = __shfl_up_sync(kAll, T, 1);
             const double before = KIND == kKeep ? S.Td[lane] : 0.0;
             const bool unsorted = __any_sync(kAll, (lane & 15) != 0 && Tp > T);

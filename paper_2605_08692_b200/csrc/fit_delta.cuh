@@ -36,7 +36,11 @@
 // that passes a neighbour; the rounds that are left are then made by fit_rounds_body.
 //
 // Objective of a round (Eq. 8), from the same sums: with q = sum I (x - c)^2 carried along like them and d = T - c,
-// sum I (x - T)^2 = q - sum over the cells (2 d sum I (x - c) - d^2 sum I).
+// sum I (x - T)^2 = q - sum over the cells (2 d sum I (x - c) - d^2 sum I).  Where that falls below a sixteenth of the
+// largest q there has been, the incremental rounds end, whether a trace is wanted or not, and the round is made in full:
+// the difference would have lost four bits, and the terms of the cells' sums are then larger than a full pass's by more
+// than four.  (From the third round's constants it is 0.24 to 0.95 of q over 30 rounds, from the first pass's 0.15 to 0.4;
+// start tables far from the weights come to 0.01.)
 //
 // Inner iterations (n_inner > 1).  All passes of the fit but the first and the last run here; in a further inner iteration the kept
 // selection stands, and only moves within a table occur.
@@ -57,14 +61,14 @@
 // ---- a block's sums: half-warp h of warp v adds cell 2 v + h, a lane per warp, pairwise.  wsum: one row of `stride`
 //      doubles per warp (residuals, weights, objective) ----
 __device__ __forceinline__ void put_block_sums(const double* wsum, const int stride, unsigned long long* acc, const double fix_scale,
-                                               const int warp, const int lane, const bool trace) {
+                                               const int warp, const int lane) {
     constexpr unsigned kAll = 0xFFFFFFFFu;
     static_assert(kFitWarps == 16 && 2 * kFitWarps == kCells, "a half-warp per cell, a lane per warp");
     const int sum_warp = lane & 15, sum_cell = 2 * warp + (lane >> 4);
     const double* row = wsum + sum_warp * stride;
     double dxs = row[sum_cell], dys = row[kCells + sum_cell];
     double de = 0.0;
-    const bool do_e = trace && warp == kFitWarps - 1;
+    const bool do_e = warp == kFitWarps - 1;
     if (do_e) de = row[2 * kCells];
 #pragma unroll
     for (int s = 8; s; s >>= 1) {
@@ -89,11 +93,12 @@ __device__ __forceinline__ void put_block_sums(const double* wsum, const int str
     else if (do_e && lane < 6 && which == 2) atomicAdd(acc + kCells * kAccStride + (lane - 4), add);
 }
 
-// The totals of a pass, lane c those of cell c, as one warp waits for them (my_e: a lane that wants the objective's
-// too).  False: the wait ran out, here or in another block.
+// The totals of a pass, lane c those of cell c, lane 0 that of the objective too, as one warp waits for them.  False: the
+// wait ran out, here or in another block.
 struct Totals { unsigned long long x[2], y[2], e[2]; };
-__device__ __forceinline__ bool await_totals(Totals& t, const unsigned long long* acc, const FitParams& p, const int lane, const bool my_e) {
+__device__ __forceinline__ bool await_totals(Totals& t, const unsigned long long* acc, const FitParams& p, const int lane) {
     constexpr unsigned kAll = 0xFFFFFFFFu;
+    const bool my_e = lane == 0;
     const unsigned long long want = (unsigned long long)p.arrivals;
     t.e[0] = t.e[1] = 0;
     for (unsigned spins = 0;; ++spins) {
@@ -200,7 +205,7 @@ constexpr uint32_t kPieceMask = (1u << 28) - 1u, kSelected = 1u << 28, kUndecide
 struct DeltaShared {
     FitTables t;
     double sx[kCells], sw[kCells], sw_most[kCells];   // the cells' sums, and the largest weight sums that they have had
-    double q;
+    double q, q_most;
     double fix_scale, fix_unscale;
     float2 ab[kJSlots];                           // {A, B} of every interval
     uint2 row[kJSlots];                           // {its upper breakpoint, the entries' indices in T0, T1 on it and on the next (four bits each)}
@@ -567,7 +572,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             sh.sw[lane] = sh.sw_most[lane] = ctl.keep_sw[lane];
             sh.c[lane] = ctl.keep_c[lane];
             if (lane == 0) {
-                sh.q = ctl.keep_q;
+                sh.q = sh.q_most = ctl.keep_q;
                 sh.fix_scale = fix.x;
                 sh.fix_unscale = fix.y;
                 sh.failed = 0;
@@ -584,7 +589,6 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
     constexpr float kBinsPerUnit = (float)(NB / 16);
     constexpr float kMagic = (float)(NB / 2) + 1.5f * (float)(1 << 23) / (float)(REP * 8);
     constexpr uint32_t kBinMask = (uint32_t)(NB - 1) * (REP * 8);
-    const bool trace = p.err_trace != nullptr;
     const DeltaArgs args{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.kept, (unsigned)((1ull << 32) / (unsigned long long)K16)};
 
     uint64_t II[8];           // importances of the lane's columns, in pairs
@@ -749,15 +753,13 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             double* const row = wsums + warp * kSumStride;
             row[lane] = ws.x;
             row[kCells + lane] = ws.y;
-            if (trace) {
 #pragma unroll
-                for (int s = 16; s; s >>= 1) dq += __shfl_xor_sync(kAll, dq, s);
-                if (lane == 0) row[2 * kCells] = dq;
-            }
+            for (int s = 16; s; s >>= 1) dq += __shfl_xor_sync(kAll, dq, s);
+            if (lane == 0) row[2 * kCells] = dq;
         }
         __syncthreads();
         unsigned long long* const acc = p.acc + (size_t)(pass_no % 3u) * kAccBuffer;
-        put_block_sums(wsums, kSumStride, acc, sh.fix_scale, warp, lane, trace);
+        put_block_sums(wsums, kSumStride, acc, sh.fix_scale, warp, lane);
         if (warp) {
 #pragma unroll 8
             for (int b = 0; b < kCells; ++b) sts_bin(bins_lane + b * kSlotBytes, make_float2(0.f, 0.f));
@@ -768,27 +770,25 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
         }
         ++pass_no;
         if (warp == 0) {
-            const bool my_e = trace && bid == 0 && lane == 0;
             Totals t;
-            if (!await_totals(t, acc, p, lane, my_e)) {
+            if (!await_totals(t, acc, p, lane)) {
                 if (lane == 0) sh.failed = 1;
             } else {
                 const double sx = sh.sx[lane] + total_of(t.x, nblk, sh.fix_unscale), sw = sh.sw[lane] + total_of(t.y, nblk, sh.fix_unscale);
-                const double most = sh.sw_most[lane];
-                if (!__all_sync(kAll, most > 0.0 ? sw > 0.25 * most : most == 0.0 && sw == 0.0)) {
+                const double most = sh.sw_most[lane], c = (double)sh.c[lane], before = S.Td[lane], d = before - c;
+                double f = d * (2.0 * sx - d * sw);
+#pragma unroll
+                for (int s = 16; s; s >>= 1) f += __shfl_xor_sync(kAll, f, s);
+                const double q = sh.q + 16.0 * total_of(t.e, nblk, sh.fix_unscale), q_most = fmax(sh.q_most, q), err = q - f;
+                const bool used = (most > 0.0 ? sw > 0.25 * most : most == 0.0 && sw == 0.0) && (lane || err >= 0.0625 * q_most);
+                if (!__all_sync(kAll, used)) {
                     if (lane == 0) sh.stop = 1;                    // this round is not used
                 } else {
-                    const double c = (double)sh.c[lane], before = S.Td[lane];
                     double T = sw > 0.0 ? c + __ddiv_rn(sx, sw) : before;
-                    if (trace && bid == 0) {
-                        const double d = before - c;
-                        double f = d * (2.0 * sx - d * sw);
-#pragma unroll
-                        for (int s = 16; s; s >>= 1) f += __shfl_xor_sync(kAll, f, s);
-                        if (lane == 0) {
-                            sh.q += 16.0 * total_of(t.e, nblk, sh.fix_unscale);
-                            if (!frozen) p.err_trace[round / p.n_inner] = sh.q - f;
-                        }
+                    if (lane == 0) {
+                        sh.q = q;
+                        sh.q_most = q_most;
+                        if (bid == 0 && !frozen && p.err_trace) p.err_trace[round / p.n_inner] = err;
                     }
                     sh.sx[lane] = sx;
                     sh.sw[lane] = sw;
