@@ -39,13 +39,14 @@ def rows_for(units, K):
 
 
 @pytest.mark.parametrize("K,units,extra,rounds,inner,init", [
-    (512, 12, 0, 25, 1, binding.INIT_QUANTILE),         # one slab, the fewest units
-    (512, 111, 16, 8, 1, binding.INIT_QUANTILE),        # the fewest rounds
-    (512, 16, -3, 20, 1, binding.INIT_QUANTILE),        # a last unit with rows missing
-    (1008, 16, 5, 21, 1, binding.INIT_GRID),            # lanes without columns, ranges of units that differ by one; a start with equal entries
-    (4096, 16, 16, 21, 1, binding.INIT_QUANTILE),       # short slabs
-    (512, 4, -3, 3, 14, binding.INIT_QUANTILE),         # inner iterations
-    (1008, 9, 5, 2, 10, binding.INIT_QUANTILE),
+    (512, 20, 0, 29, 1, binding.INIT_QUANTILE),         # one slab, the fewest units
+    (512, 100, 16, 17, 1, binding.INIT_QUANTILE),       # few rounds
+    (512, 24, -3, 27, 1, binding.INIT_QUANTILE),        # a last unit with rows missing
+    (1008, 20, 5, 29, 1, binding.INIT_GRID),            # lanes without columns, ranges of units that differ by one; a start with equal entries
+    (4096, 20, 16, 29, 1, binding.INIT_QUANTILE),       # short slabs
+    (512, 6, -3, 3, 14, binding.INIT_QUANTILE),         # inner iterations
+    (512, 7, 0, 1, 30, binding.INIT_QUANTILE),
+    (1008, 11, 5, 2, 10, binding.INIT_QUANTILE),
 ])
 def test_layers_of_few_units_per_block(K, units, extra, rounds, inner, init):
     W, X = layer(NVFP4, rows_for(units, K) + extra, K, T=64, name=f"incremental/{K}/{extra}")
@@ -63,16 +64,26 @@ def test_inner_iterations_from_equal_entries_are_not_tried():
     assert counts[0] == counts[1]
 
 
+@pytest.mark.parametrize("units,rounds,inner,incremental", [
+    (20, 28, 1, False), (19, 40, 1, False), (40, 21, 1, False), (40, 22, 1, True),
+    (30, 5, 6, False), (19, 1, 10, False), (20, 1, 10, True), (10, 2, 10, False), (9, 3, 7, False), (12, 3, 7, True)])
+def test_the_rule_takes_what_pays(units, rounds, inner, incremental):
+    """(Layers may use some blocks fewer than there are, so that a block has a tenth more units.)"""
+    W, X = layer(NVFP4, rows_for(units, 512), 512, T=64, name="incremental/rule")
+    got = check(W, X, rounds, binding.INIT_QUANTILE, f"{units} units, {rounds} x {inner}", inner)
+    assert got == ((3 if inner == 1 else 1, rounds * inner - 1) if incremental else (0, 0))
+
+
 def tables(t0, t1):
     return np.stack([t0, t1]).astype(np.float32)
 
 
 @pytest.mark.parametrize("start,rounds,inner", [
-    ("far", 3, 10), ("far", 1, 30), ("apart", 25, 1), ("apart", 2, 14), ("twins", 3, 10)])
+    ("far", 3, 10), ("far", 1, 30), ("apart", 29, 1), ("apart", 2, 14), ("twins", 3, 10)])
 def test_fits_that_end_early_are_finished(start, rounds, inner):
     """Start tables beside the weights, whose entries jump: a cell's weight changes too much, or a breakpoint passes its
     neighbour, within the fit and within a round.  Equal entries: it cannot begin where it starts from the first pass."""
-    N, K = rows_for(12, 512), 512
+    N, K = rows_for(20, 512), 512
     W, X = layer(NVFP4, N, K, T=64, name="incremental/early")
     even = np.linspace(-6, 6, 16)
     T01 = {"far": tables(np.linspace(0.5, 1.5, 16), np.linspace(0.52, 1.52, 16)), "apart": tables(np.linspace(-6, -1, 16), np.linspace(1, 6, 16)),
@@ -84,11 +95,11 @@ def test_fits_that_end_early_are_finished(start, rounds, inner):
         assert first == (3 if inner == 1 else 1) and first < end < rounds * inner - 1
 
 
-@pytest.mark.parametrize("rounds,inner", [(25, 1), (3, 10)])
+@pytest.mark.parametrize("rounds,inner", [(29, 1), (3, 10)])
 @pytest.mark.parametrize("levels", [3, 17, 40])
 def test_layers_of_few_distinct_weights(levels, rounds, inner):
     """Equal entries, empty cells and breakpoints that jump: the incremental rounds end early, or never begin."""
-    N, K = rows_for(12, 512), 512
+    N, K = rows_for(20, 512), 512
     W, X = layer(NVFP4, N, K, T=64, name=f"incremental/levels/{levels}")
     rng = np.random.default_rng(levels)
     values = np.sort(rng.standard_normal(levels)).astype(np.float32) * 0.02
@@ -130,7 +141,7 @@ def test_sums_that_have_lost_their_accuracy_end_the_incremental_rounds(seed):
     rounds = 28
     end = followed(W, I, T01, rounds)
     assert 3 < end < rounds - 1
-    W = np.tile(W, (rows_for(12, 512) // 64, 1))
+    W = np.tile(W, (rows_for(24, 512) // 64, 1))
     ws = binding.alloc_workspace(NVFP4, *W.shape)
     o = oracle.fit_layer(W, NVFP4, 16, rounds, I=I, init="user", T_init=T01)
     r = binding.quantize_layer(dev_bf16(W), NVFP4, I=torch.from_numpy(I).cuda(), n_outer=rounds, init=binding.INIT_USER, ws=ws, want_trace=True,
@@ -142,7 +153,7 @@ def test_sums_that_have_lost_their_accuracy_end_the_incremental_rounds(seed):
     check_end_to_end_bits(r, o, f"seed {seed}")
 
 
-@pytest.mark.parametrize("K,units,extra,rounds,inner", [(512, 12, 0, 25, 1), (1008, 16, 5, 21, 1), (4096, 24, -3, 17, 1), (512, 4, -3, 3, 14), (1008, 9, 5, 2, 10)])
+@pytest.mark.parametrize("K,units,extra,rounds,inner", [(512, 20, 0, 29, 1), (1008, 20, 5, 29, 1), (4096, 28, -3, 25, 1), (512, 6, -3, 3, 14), (1008, 11, 5, 2, 10)])
 def test_weight_sums_that_are_carried_are_exact(K, units, extra, rounds, inner):
     """The sums of I that the incremental passes start from, against 64-bit sums over the cells of the same tables: counts
     times importances, rounded a few dozen times to 2^-53.  (FP32 sums erred by 1e-8 in every cell.)"""
@@ -169,11 +180,11 @@ def test_weight_sums_that_are_carried_are_exact(K, units, extra, rounds, inner):
 
 
 def test_two_runs_give_the_same_bits():
-    N, K = rows_for(17, 2048), 2048
+    N, K = rows_for(30, 2048), 2048
     W, X = layer(NVFP4, N, K, T=64, name="incremental/twice")
     out = []
     for _ in range(2):
-        r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=20, init=binding.INIT_QUANTILE, want_trace=True)
+        r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=25, init=binding.INIT_QUANTILE, want_trace=True)
         torch.cuda.synchronize()
         out.append([host(r[k]) for k in ("T01", "trace", "codes", "scales")])
     assert all(np.array_equal(a, b) for a, b in zip(*out))
