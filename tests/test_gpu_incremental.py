@@ -15,12 +15,12 @@ def _built():
     build.build()
 
 
-def check(W, X, rounds, init, name, inner=1, T01=None):
-    """Compares a fit with the oracle's; returns the passes that were incremental, (first, end)."""
+def check(W, X, rounds, init, name, inner=1, T01=None, place=dev_bf16):
+    """Compares a fit with the oracle's (place: puts the weights on the device); returns the passes that were incremental, (first, end)."""
     o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, n_inner=inner, T_init=T01,
                          init={binding.INIT_QUANTILE: "quantile", binding.INIT_GRID: "grid", binding.INIT_USER: "user"}[init])
     ws = binding.alloc_workspace(NVFP4, W.shape[0], W.shape[1], X.shape[0])
-    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, n_inner=inner, init=init, want_trace=True, ws=ws,
+    r = binding.quantize_layer(place(W), NVFP4, X=dev_bf16(X), n_outer=rounds, n_inner=inner, init=init, want_trace=True, ws=ws,
                                T01_init=None if T01 is None else torch.from_numpy(T01))
     torch.cuda.synchronize()
     assert int(r["status"].item()) == 0
@@ -51,6 +51,59 @@ def rows_for(units, K):
 def test_layers_of_few_units_per_block(K, units, extra, rounds, inner, init):
     W, X = layer(NVFP4, rows_for(units, K) + extra, K, T=64, name=f"incremental/{K}/{extra}")
     assert check(W, X, rounds, init, f"incremental {K} {units} {extra}", inner) == (3 if inner == 1 else 1, rounds * inner - 1)
+
+
+def with_stride(ldw, offset):
+    """Puts weights into a buffer of rows of ldw elements, the first one `offset` elements behind a 256-byte boundary."""
+    def place(W):
+        N, K = W.shape
+        buf = torch.full((N * ldw + offset + 128,), float("nan"), dtype=torch.bfloat16, device="cuda")
+        Wd = buf[offset:offset + N * ldw].view(N, ldw)[:, :K]
+        Wd.copy_(dev_bf16(W))
+        return Wd
+    return place
+
+
+@pytest.mark.parametrize("rounds,inner", [(29, 1), (3, 10)])
+@pytest.mark.parametrize("ldw,offset,incremental", [(528, 0, True), (640, 16, True), (520, 0, False), (528, 8, False)])
+def test_rows_apart_and_weights_off_32_bytes(ldw, offset, incremental, rounds, inner):
+    """A piece is one 32-byte load: rows further apart than their width are taken, addresses that are not multiples of 32
+    bytes are left to the full rounds."""
+    W, X = layer(NVFP4, rows_for(20, 512) - 5, 512, T=64, name="incremental/stride")
+    got = check(W, X, rounds, binding.INIT_QUANTILE, f"ldw {ldw} + {offset}", inner, place=with_stride(ldw, offset))
+    assert got == ((3 if inner == 1 else 1, rounds * inner - 1) if incremental else (0, 0))
+
+
+@pytest.mark.parametrize("rounds,inner", [(29, 1), (3, 10)])
+def test_columns_without_importance(rounds, inner):
+    """Whole groups of importance 0, undecided in every pass, and single columns of it."""
+    W, X = layer(NVFP4, rows_for(20, 512), 512, T=64, name="incremental/zero")
+    X[:, 64:192] = 0
+    X[:, 200:512:7] = 0
+    assert check(W, X, rounds, binding.INIT_QUANTILE, "zero importances", inner) == (3 if inner == 1 else 1, rounds * inner - 1)
+
+
+@pytest.mark.parametrize("rounds,inner", [(29, 1), (3, 10)])
+def test_wait_that_runs_out_is_reported(rounds, inner):
+    """As of the full rounds: the status word says so, and the next fit with the workspace is what it was."""
+    W, X = layer(NVFP4, rows_for(20, 512), 512, T=64, name="incremental/wait")
+    Wd, Xd, ws = dev_bf16(W), dev_bf16(X), binding.alloc_workspace(NVFP4, *W.shape, X.shape[0])
+
+    def fit():
+        r = binding.quantize_layer(Wd, NVFP4, X=Xd, n_outer=rounds, n_inner=inner, init=binding.INIT_QUANTILE, ws=ws, want_trace=True)
+        torch.cuda.synchronize()
+        return r
+    good = fit()
+    assert int(good["status"].item()) == 0
+    try:
+        binding.debug_fit_wait(1, 1000)
+        assert int(fit()["status"].item()) & binding.DEV_TIMEOUT and binding.debug_incremental(ws) == (0, 0)
+    finally:
+        binding.debug_fit_wait(0, 0)
+    again = fit()
+    assert int(again["status"].item()) == 0
+    for k in ("T01", "codes", "scales", "trace", "err"):
+        assert torch.equal(again[k], good[k]), k
 
 
 def test_inner_iterations_from_equal_entries_are_not_tried():
