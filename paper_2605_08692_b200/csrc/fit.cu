@@ -171,11 +171,6 @@ __device__ __forceinline__ void sts_u2(uint32_t addr, uint32_t a, uint32_t b) {
 // round make it, unless it is done.
 enum PassKind { kRounds = 0, kAssignKeep = 1, kInner = 2, kKeep = 3, kRest = 4, kAssignRest = 5, kInnerRest = 6 };
 
-// Decides the listed selection groups in double (Eq. 8: each lane adds its weights' terms in index
-// order, the lanes of the group are combined pairwise; a tie goes to table 0) and adds every weight
-// to the calling lane's bins under the chosen table, with the arithmetic of the row pipeline
-// (centred term I (x - c), c the chosen entry's centre constant).  Every lane of the warp calls;
-// returns the sum of the groups' smaller errors in lane 0 (0 elsewhere).
 __device__ __forceinline__ void add_term(uint32_t addr, float v) {
     float a;
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(addr) : "memory");
@@ -184,6 +179,12 @@ __device__ __forceinline__ void add_term(uint32_t addr, float v) {
 __device__ __forceinline__ void count_weight(uint32_t addr, uint32_t one) {
     asm volatile("red.shared.add.u32 [%0], %1;" :: "r"(addr), "r"(one) : "memory");
 }
+
+// Decides the listed selection groups in double (Eq. 8: each lane adds its weights' terms in index
+// order, the lanes of the group are combined pairwise; a tie goes to table 0) and adds every weight
+// to the calling lane's bins under the chosen table, with the arithmetic of the row pipeline
+// (centred term I (x - c), c the chosen entry's centre constant).  Every lane of the warp calls;
+// returns the sum of the groups' smaller errors in lane 0 (0 elsewhere).
 struct DeferArgs {                // what the routine needs of the layer (passed by value: the kernel's
     const uint16_t* W;            // parameters themselves stay where they are)
     int64_t K, ldw;
@@ -258,17 +259,15 @@ __device__ __noinline__ double resolve_deferred(const FitTables* S, const DeferA
                     b.y += Is[t];
                     sts_bin(a, b);
                 }
-                parity |= (__float_as_uint(c) & 1u) << (2 * t);
+                if (KIND == kKeep) parity = __float_as_uint(c) & 1u;
             }
         }
         if (KIND == kKeep) {
-            // the lanes of 16 weights put their bits together
-            constexpr int LPE = 16 / WPL;
-            parity <<= (lane % LPE) * WPL * 2;
+            // the group's lanes put their bits together
+            parity <<= 2 * (lane & 15);
 #pragma unroll
-            for (int o = 1; o < LPE; o <<= 1) parity |= __shfl_xor_sync(0xFFFFFFFFu, parity, o);
-            if (lane < ACTIVE && lane % LPE == 0)
-                p.kept[(size_t)row * (size_t)(K / 16) + (uint32_t)(cg / 16 + lane / LPE)] = parity | (sg ? 2u : 0u);
+            for (int o = 1; o < 16; o <<= 1) parity |= __shfl_xor_sync(0xFFFFFFFFu, parity, o);
+            if (lane == 0) p.kept[(size_t)row * (size_t)(K / 16) + (uint32_t)(cg / 16)] = parity | (sg ? 2u : 0u);
         }
         if (lane == 0) {
             esum += sg ? e1 : e0;
@@ -1201,7 +1200,7 @@ cudaError_t launch_fit_rounds_batch(const FitLayerArgs* layers, int n, int mode,
             if (e == cudaSuccess) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kKeep>>(b, grid, st);
             for (int l = 0; l < m; ++l) b.L[l].trace_base = 0;
             for (int l = 0; l < m; ++l) { b.L[l].n_rounds = n_outer * n_inner - 1; b.L[l].n_inner = n_inner; }
-            if (e == cudaSuccess) e = launch_variant<delta_kernel<AAAC_NVFP4, 16>>(b, grid, st);
+            if (e == cudaSuccess) e = launch_variant<delta_kernel>(b, grid, st);
             for (int l = 0; l < m; ++l) b.L[l].n_rounds = n_outer * n_inner;
             if (e == cudaSuccess && n_inner == 1) e = launch_variant<fit_kernel<AAAC_NVFP4, 16, kRest>>(b, grid, st);
             if (e == cudaSuccess && n_inner > 1) {

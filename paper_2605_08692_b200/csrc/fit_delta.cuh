@@ -6,7 +6,7 @@
 // the sums of the cells are carried from round to round, and a pass takes the weights that move out of their old
 // cell and adds them to their new one.  The assignment itself is made for every weight in every round, exactly as there.
 //
-// Assignment.  A lane holds 16 adjacent weights of a row (a whole group where S = 16: no exchange between lanes, and
+// Assignment.  A lane holds 16 adjacent weights of a row (a whole selection group: no exchange between lanes, and
 // what a row costs besides its weights is paid once per 16).  Only the difference of the two errors decides, and
 // (x - P)^2 - (x - Q)^2 = x A + B with A = 2 (Q - P), B = P^2 - Q^2 constant on an interval, so the tables hold
 // {A, B} and a weight costs one multiply-add and half of a two-wide one where the two errors cost six instructions.
@@ -287,18 +287,17 @@ struct DeltaArgs {                // what the list work needs of the layer
     const uint16_t* W;
     int64_t K, ldw;
     const uint8_t* scales;
-    const float* rinv;
     const float* I;
     uint32_t* kept;
     unsigned k16_inv;             // floor(2^32 / (K / 16))
 };
 
 // Works off the list's first `count` pieces, in which weights move within their table: first the moving weights are put
-// into a row (most pieces have one, few more than two), then every lane takes one of them.  Every lane calls; returns what the lane's weights add to q.
+// into a row (most pieces have one, few more than two), then every lane takes one of them (two: 1 % slower).  Every lane
+// calls; returns what the lane's weights add to q.
 __device__ __noinline__ float apply_moves(const DeltaShared* sh, const DeltaArgs p, const uint32_t list_at, const int count,
                                           const uint32_t bins_lane, const int lane) {
     constexpr unsigned kAll = 0xFFFFFFFFu;
-    constexpr int E = 1;                                   // weights per lane (two: 1 % slower, the code is longer)
     const unsigned K16 = (unsigned)p.K / 16u;
     const uint32_t row_at = list_at + kDeltaWeights, below = (1u << lane) - 1u;
     float dq = 0.f;
@@ -325,92 +324,67 @@ __device__ __noinline__ float apply_moves(const DeltaShared* sh, const DeltaArgs
                 asm volatile("st.shared.u16 [%0], %1;" :: "r"(row_at + (uint32_t)(n + __popc(some & below)) * 2u), "h"((uint16_t)(piece | (j << 8))) : "memory");
             }
             n += __popc(some);
-            if (n >= 32 * E) break;
+            if (n >= 32) break;
         }
         if (n == 0) return dq;
-        const int take = min(n, 32 * E);
+        const int take = min(n, 32);
         n -= take;
         __syncwarp();
-        uint32_t w[E], table[E];
-        float iv[E], x[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            w[k] = table[k] = 0u;
-            iv[k] = x[k] = 0.f;
-            if (lane + 32 * k < take) {
-                uint32_t ej, at, word;
-                asm volatile("ld.shared.u16 %0, [%1];" : "=r"(ej) : "r"(row_at + (uint32_t)(n + lane + 32 * k) * 2u) : "memory");
-                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(at), "=r"(word) : "r"(list_at + (ej & 255u) * 8u) : "memory");
-                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[k]) : "r"(list_at + kDeltaScales + (ej & 255u) * 4u) : "memory");
-                const unsigned row = row_of(at, K16, p.k16_inv), col = (at - row * K16) * 16u + (ej >> 8);
-                w[k] = __ldg(p.W + (row * (unsigned)p.ldw + col));
-                iv[k] = __ldg(p.I + col);
-                table[k] = (word & 2u) ? (uint32_t)kM : 0u;
-            }
+        uint32_t w = 0u, table = 0u;
+        float iv = 0.f, x = 0.f;
+        if (lane < take) {
+            uint32_t ej, at, word;
+            asm volatile("ld.shared.u16 %0, [%1];" : "=r"(ej) : "r"(row_at + (uint32_t)(n + lane) * 2u) : "memory");
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(at), "=r"(word) : "r"(list_at + (ej & 255u) * 8u) : "memory");
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(list_at + kDeltaScales + (ej & 255u) * 4u) : "memory");
+            const unsigned row = row_of(at, K16, p.k16_inv), col = (at - row * K16) * 16u + (ej >> 8);
+            w = __ldg(p.W + (row * (unsigned)p.ldw + col));
+            iv = __ldg(p.I + col);
+            table = (word & 2u) ? (uint32_t)kM : 0u;
         }
-        uint32_t from[E], to[E];
-        Move m[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            x[k] = __fmul_rn(__uint_as_float(w[k] << 16), x[k]);
-            const uint32_t in = (entries_of(sh, x[k]) >> (table[k] / 4u)) & kIdxMask;
-            to[k] = table[k] + in;
-            from[k] = table[k] + ((x[k] > sh->mid_old[to[k]] ? in + 1u : in - 1u) & kIdxMask);
-        }
-#pragma unroll
-        for (int k = 0; k < E; ++k) m[k] = move_terms(sh, from[k], to[k], x[k], iv[k], dq);
-#pragma unroll
-        for (int k = 0; k < E; ++k)
-            if (lane + 32 * k < take) move_weight(bins_lane, from[k], to[k], m[k], iv[k]);
+        x = __fmul_rn(__uint_as_float(w << 16), x);
+        const uint32_t in = (entries_of(sh, x) >> (table / 4u)) & kIdxMask, to = table + in;
+        const uint32_t from = table + ((x > sh->mid_old[to] ? in + 1u : in - 1u) & kIdxMask);
+        const Move m = move_terms(sh, from, to, x, iv, dq);
+        if (lane < take) move_weight(bins_lane, from, to, m, iv);
         __syncwarp();
     }
 }
 
 // Works off the list's last `count` pieces, whose selection has changed or is open: all their weights move.  A lane takes
 // a piece, four weights side by side.  Every lane calls; returns what the lane's weights add to q.
-template <int MODE, int SEL>
 __device__ __noinline__ float apply_flips(const DeltaShared* sh, const DeltaArgs p, const uint32_t list_at, const int count,
                                           const uint32_t bins_lane, const int lane) {
-    constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
-    constexpr int WPL = SEL >= 32 ? SEL / 32 : 1, ACTIVE = SEL / WPL;
     constexpr unsigned kAll = 0xFFFFFFFFu;
     const FitTables& S = sh->t;
-    const unsigned K16 = (unsigned)p.K / 16u, Gr = (unsigned)p.K / G;
+    const unsigned K16 = (unsigned)p.K / 16u;
     const uint32_t list_addr = list_at + (uint32_t)(kDeltaCap - count) * 8u, scales_at = list_at + (uint32_t)(kDeltaScales + (kDeltaCap - count) * 4);
-    // the open ones: Eq. 8 in double, a weight or four per lane, in the order of resolve_deferred
+    // the open ones: Eq. 8 in double, a weight per lane, in the order of resolve_deferred
     for (int first = 0; first < count; first += 32) {
         uint32_t at = 0u;
         if (first + lane < count) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(at) : "r"(list_addr + (uint32_t)(first + lane) * 8u) : "memory");
         unsigned open = __ballot_sync(kAll, (at & kUndecided) != 0u);
-        while (open) {
+        for (; open; open &= open - 1u) {
             const int who = __ffs(open) - 1;
             const unsigned a = __shfl_sync(kAll, at, who) & kPieceMask;
-            // (the pieces of a group stand next to one another)
-            const bool same = (at & kUndecided) != 0u && ((at & kPieceMask) ^ a) < (unsigned)(SEL / 16);
-            open &= ~__ballot_sync(kAll, same);
-            const unsigned r = row_of(a, K16, p.k16_inv), c0 = (a - r * K16) * 16u / SEL * SEL;
             double e0 = 0.0, e1 = 0.0;
-            if (lane < ACTIVE) {
-#pragma unroll
-                for (int t = 0; t < WPL; ++t) {
-                    const unsigned cc = c0 + (unsigned)(lane * WPL + t);
-                    const uint32_t wb = p.W[r * (unsigned)p.ldw + cc];
-                    const unsigned gi = r * Gr + cc / G;
-                    const float x = __fmul_rn(__uint_as_float(wb << 16), MODE == AAAC_NVFP4 ? S.rlut[p.scales[gi] & 0x7Fu] : __ldg(p.rinv + gi));
-                    const double2 pq = S.PQ[find_interval(S.bp, x)];
-                    const double xd = (double)x, id = (double)__ldg(p.I + cc);
-                    const double d0 = __dsub_rn(xd, pq.x), d1 = __dsub_rn(xd, pq.y);
-                    e0 = __dadd_rn(e0, __dmul_rn(id, __dmul_rn(d0, d0)));
-                    e1 = __dadd_rn(e1, __dmul_rn(id, __dmul_rn(d1, d1)));
-                }
+            if (lane < 16) {
+                const unsigned r = row_of(a, K16, p.k16_inv), col = (a - r * K16) * 16u + (unsigned)lane;
+                const uint32_t wb = p.W[r * (unsigned)p.ldw + col];
+                const float x = __fmul_rn(__uint_as_float(wb << 16), S.rlut[p.scales[a] & 0x7Fu]);
+                const double2 pq = S.PQ[find_interval(S.bp, x)];
+                const double xd = (double)x, id = (double)__ldg(p.I + col);
+                const double d0 = __dsub_rn(xd, pq.x), d1 = __dsub_rn(xd, pq.y);
+                e0 = __dmul_rn(id, __dmul_rn(d0, d0));
+                e1 = __dmul_rn(id, __dmul_rn(d1, d1));
             }
 #pragma unroll
-            for (int o = ACTIVE / 2; o; o >>= 1) {
+            for (int o = 8; o; o >>= 1) {
                 e0 = __dadd_rn(e0, __shfl_xor_sync(kAll, e0, o));
                 e1 = __dadd_rn(e1, __shfl_xor_sync(kAll, e1, o));
             }
             const bool second = __shfl_sync(kAll, (int)(e1 < e0), 0) != 0;
-            if (same) {
+            if (lane == who) {
                 at = second ? at | kSelected : at & ~kSelected;
                 asm volatile("st.shared.u32 [%0], %1;" :: "r"(list_addr + (uint32_t)(first + lane) * 8u), "r"(at) : "memory");
             }
@@ -470,12 +444,9 @@ __device__ __noinline__ float apply_flips(const DeltaShared* sh, const DeltaArgs
 
 // The incremental passes of one layer, from the first after the kKeep launch to p.n_rounds, run by the blocks
 // bid = 0 .. nblk - 1.  Layout in shared memory as in fit_rounds_body.
-template <int MODE, int SEL>
 __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsigned bid, const unsigned nblk) {
     constexpr int NW = kFitWarps, NB = kNBins, REP = kRep, NT = NW * 32;
     constexpr unsigned kAll = 0xFFFFFFFFu;
-    constexpr int G = MODE == AAAC_INT4 ? 128 : 16;
-    constexpr int LPG = SEL / 16;                          // lanes per selection group
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ DeltaShared sh;
     FitTables& S = sh.t;
@@ -507,7 +478,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
     unsigned pass_no = ctl.passes;
 
     const int N = (int)p.N, K = (int)p.K;
-    const unsigned K16 = (unsigned)K / 16u, Gr = (unsigned)K / G;
+    const unsigned K16 = (unsigned)K / 16u;
     const int nrb = (N + NW - 1) / NW, slabs = (K + kDeltaCols - 1) / kDeltaCols;
     const int64_t units = (int64_t)slabs * nrb;
     const int t0 = (int)(units * bid / nblk), n_units = (int)(units * (bid + 1) / nblk) - t0;
@@ -518,22 +489,20 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
     uint4 v[2][2];
     uint32_t sc[2], kw[2];
     int lslab = slab0, lrb = rb0, lleft = n_units;         // the unit to be loaded next
-    auto offsets = [&](unsigned& wo, unsigned& so, unsigned& ko) {
+    auto offsets = [&](unsigned& wo, unsigned& ko) {       // elements of W; scales and kept words
         const unsigned row = (unsigned)min(lrb * NW + warp, N - 1);
         const unsigned piece = min((unsigned)(lslab * 32 + lane), K16 - 1u);
         wo = row * (unsigned)p.ldw + piece * 16u;
         ko = row * K16 + piece;
-        so = MODE == AAAC_NVFP4 ? ko : row * Gr + piece / 8u;
     };
     auto load_unit = [&](int s) {
-        unsigned wo, so, ko;
-        offsets(wo, so, ko);
+        unsigned wo, ko;
+        offsets(wo, ko);
         asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                      : "=r"(v[s][0].x), "=r"(v[s][0].y), "=r"(v[s][0].z), "=r"(v[s][0].w), "=r"(v[s][1].x), "=r"(v[s][1].y), "=r"(v[s][1].z),
                        "=r"(v[s][1].w)
                      : "l"(p.W + wo));
-        if (MODE == AAAC_NVFP4) asm volatile("ld.global.u8 %0, [%1];" : "=r"(sc[s]) : "l"(p.scales + so));
-        else asm volatile("ld.global.u32 %0, [%1];" : "=r"(sc[s]) : "l"(p.rinv + so));
+        asm volatile("ld.global.u8 %0, [%1];" : "=r"(sc[s]) : "l"(p.scales + ko));
         asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(kw[s]) : "l"(p.kept + ko) : "memory");
         if (--lleft == 0) {
             lleft = n_units;
@@ -549,7 +518,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
         load_unit(1);
     }
 
-    if (MODE == AAAC_NVFP4 && tid >= 64 && tid < 192) {
+    if (tid >= 64 && tid < 192) {
         const int c = tid - 64;
         const float sv = __fmul_rn(e4m3_value((uint32_t)c), ctl.s_t);
         S.rlut[c] = c ? __frcp_rn(sv) : 0.f;
@@ -589,7 +558,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
     constexpr float kBinsPerUnit = (float)(NB / 16);
     constexpr float kMagic = (float)(NB / 2) + 1.5f * (float)(1 << 23) / (float)(REP * 8);
     constexpr uint32_t kBinMask = (uint32_t)(NB - 1) * (REP * 8);
-    const DeltaArgs args{p.W, p.K, p.ldw, p.scales, p.rinv, p.I, p.kept, (unsigned)((1ull << 32) / (unsigned long long)K16)};
+    const DeltaArgs args{p.W, p.K, p.ldw, p.scales, p.I, p.kept, (unsigned)((1ull << 32) / (unsigned long long)K16)};
 
     uint64_t II[8];           // importances of the lane's columns, in pairs
     float isum = 0.f;         // sum of |I| over the lane's group (rounded up a little)
@@ -645,7 +614,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
 #pragma unroll
             for (int j = 0; j < 8; ++j) bits = __funnelshift_r(bits, __float_as_uint(lo2(ab[b][j])), 2);
         };
-        auto rinv_of = [&](uint32_t s) { return MODE == AAAC_NVFP4 ? S.rlut[s & 0x7Fu] : __uint_as_float(s); };
+        auto rinv_of = [&](uint32_t s) { return S.rlut[s & 0x7Fu]; };
 
         int slab = slab0, rb = rb0;
         float rinv = 0.f;
@@ -662,8 +631,6 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
                     II[2 * j + 1] = pack2(a.z, a.w);
                     isum += (fabsf(a.x) + fabsf(a.y)) + (fabsf(a.z) + fabsf(a.w));
                 }
-#pragma unroll
-                for (int o = LPG / 2; o; o >>= 1) isum += __shfl_xor_sync(kAll, isum, o);
                 isum *= 1.0001f;
                 tau = __fmul_ru(isum, margin);
             }
@@ -680,9 +647,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             L1(v[s ^ 1][0], rinv, 0);                      // (for nothing at the end of a pass, or before the lists are worked off)
             L2(1);
             E(1);
-            float d = lo2(sum) + hi2(sum);
-#pragma unroll
-            for (int o = LPG / 2; o; o >>= 1) d += __shfl_xor_sync(kAll, d, o);
+            const float d = lo2(sum) + hi2(sum);
             // (a NaN, from a poisoned row, counts as a flip also where the selection stands)
             const bool near = !(fabsf(d) > tau) && !(frozen && d == d);
             const uint32_t sg = frozen ? (old >> 1) & 1u : d > 0.f ? 1u : 0u;
@@ -727,7 +692,7 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             if (n_moves > 0) dq += (double)apply_moves(&sh, args, list_at, n_moves, bins_lane, lane);
             n_moves = 0;
             if (n_flips > (i < n_units ? kLeastFlips - 1 : 0)) {
-                dq += (double)apply_flips<MODE, SEL>(&sh, args, list_at, n_flips, bins_lane, lane);
+                dq += (double)apply_flips(&sh, args, list_at, n_flips, bins_lane, lane);
                 n_flips = 0;
             }
             __syncwarp();
@@ -740,8 +705,8 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
             lrb = rb0;
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
-                unsigned wo, so, ko;
-                offsets(wo, so, ko);
+                unsigned wo, ko;
+                offsets(wo, ko);
                 asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(kw[s]) : "l"(p.kept + ko) : "memory");
                 if (n_units > 1 && ++lrb == nrb) { lrb = 0; ++lslab; }
             }
@@ -829,10 +794,9 @@ __device__ __forceinline__ void delta_rounds_body(const FitParams& p, const unsi
     }
 }
 
-template <int MODE, int SEL>
 __global__ void __launch_bounds__(kFitWarps * 32, 1) delta_kernel(const __grid_constant__ FitBatch b) {
-    if (b.first[1] == gridDim.x) { delta_rounds_body<MODE, SEL>(b.L[0], blockIdx.x, gridDim.x); return; }
+    if (b.first[1] == gridDim.x) { delta_rounds_body(b.L[0], blockIdx.x, gridDim.x); return; }
     int l = 0;
     while (l + 1 < kMaxBatch && blockIdx.x >= b.first[l + 1]) ++l;
-    delta_rounds_body<MODE, SEL>(b.L[l], blockIdx.x - b.first[l], b.first[l + 1] - b.first[l]);
+    delta_rounds_body(b.L[l], blockIdx.x - b.first[l], b.first[l + 1] - b.first[l]);
 }
