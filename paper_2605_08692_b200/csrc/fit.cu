@@ -923,9 +923,18 @@ __device__ __forceinline__ void fit_rounds_body(const FitParams& p, const unsign
             const double sx = total(x), wt = total(y);
             double T = wt > 0.0 ? (double)S.centre[lane] + __ddiv_rn(sx, wt) : S.Td[lane];
             // the trace holds the Eq. 8 objective of each assignment step
-            double err = 0.0;
+            double err = 0.0, about = 0.0;
+            if (KIND == kRest && trace) {
+                // (the errors were formed about the constants, up to 8 units in the last place from the entries: sum I (x - T)^2 is
+                // sum I (x - c)^2 less this.  Behind incremental rounds, whose objective has no such error: 1e-7 of it -> 1e-9)
+                const double d = S.Td[lane] - (double)S.centre[lane];
+                about = d * (2.0 * sx - d * wt);
+#pragma unroll
+                for (int s = 16; s; s >>= 1) about += __shfl_xor_sync(kAll, about, s);
+            }
             if (my_e) {
                 err = 16.0 * total(e);
+                if (about < 0.5 * err) err -= about;
                 if (KIND != kKeep || p.err_trace) p.err_trace[trace_base + round] = err;
             }
             const double Tp = __shfl_up_sync(kAll, T, 1);

@@ -232,6 +232,16 @@ def test_weight_sums_that_are_carried_are_exact(K, units, extra, rounds, inner):
     assert torch.allclose(got, want, rtol=1e-12, atol=0)
 
 
+@pytest.mark.parametrize("K,units,extra,rounds,dist", [(512, 20, 0, 29, "normal"), (1008, 24, 5, 27, "student5"), (4096, 40, -3, 22, "student5")])
+def test_objectives_behind_the_third_round_are_the_entries(K, units, extra, rounds, dist):
+    """The objective of the incremental rounds and of the last, full one is that of the entries, not of the constants beside
+    them (1e-7 of it): the FP32 roundings of millions of terms, 2^-24 each and of either sign, leave less than a sixth of one."""
+    W, X = layer(NVFP4, rows_for(units, K) + extra, K, T=64, name=f"incremental/trace/{K}", dist=dist)
+    o = oracle.fit_layer(W, NVFP4, 16, rounds, X=X, init="quantile")
+    r = binding.quantize_layer(dev_bf16(W), NVFP4, X=dev_bf16(X), n_outer=rounds, init=binding.INIT_QUANTILE, want_trace=True)
+    assert np.allclose(host(r["trace"])[3:], o["trace"][3:], rtol=1e-8, atol=0)
+
+
 def test_two_runs_give_the_same_bits():
     N, K = rows_for(30, 2048), 2048
     W, X = layer(NVFP4, N, K, T=64, name="incremental/twice")
