@@ -58,9 +58,9 @@ TRAFFIC_FILE = os.path.join("profiles", "fit_batch_cfg2_full_step.md")
 
 
 def measured_traffic_per_weight():
-    """DRAM bytes per weight and round of the fit-rounds kernel, from the line
+    """DRAM bytes per weight and round over the launches of the fit rounds, from the line
     `dram_bytes_per_weight_round = X` of the committed ncu summary (None if absent).  It is a
-    constant taken from one earlier capture on one layer, not a measurement of this run."""
+    constant taken from one earlier capture, not a measurement of this run."""
     p = os.path.join(ROOT, TRAFFIC_FILE)
     try:
         for line in open(p):
@@ -256,7 +256,7 @@ def run_stack(args, which, emit=True):
     status = torch.zeros(1, dtype=torch.int32, device=dev)
 
     # the seven linears of a decoder layer are independent: one aaac_quantize_layers call (importances -- once per
-    # distinct input: q, k, v share theirs, gate and up too --, scales, start, rounds in one launch, pack)
+    # distinct input: q, k, v share theirs, gate and up too --, scales, start, rounds in common launches, pack)
     descs = [dict(W=Ws[n], X=X[xin], T01=out[n]["T01"], scales=out[n]["scales"], tensor_scale=out[n]["ts"], ws=out[n]["ws"],
                   T01_bf16=out[n]["Tb"], codes=out[n]["codes"], err_out=out[n]["err"], sigma_bits=out[n]["bits"])
              for n, N, K, xin in lin]
@@ -394,7 +394,7 @@ def main():
 
     def step():
         # the layers of a step are independent problems: one aaac_quantize_layers call takes them through the
-        # whole path (importances from X, scales, start tables, the 20 rounds of all of them in one launch,
+        # whole path (importances from X, scales, start tables, the 20 rounds of all of them in common launches,
         # pack, reconstruction)
         if args.with_prescale:
             for X, W, o in zip(Xd, Wd, outs):
@@ -450,7 +450,7 @@ def main():
     ms_step = ms_total / args.steps
     value = sharding.job_throughput(weights_per_step, ROUNDS, ms_step, world)
 
-    # roofline of the dominant kernel: algorithmic bytes of every timed fit-round launch / its device time
+    # roofline of the dominant kernels: algorithmic bytes of every step's fit rounds / the device time of their launches
     per_launch_w = [weights_per_step * ROUNDS] * args.steps
     bytes_alg = sum(per_launch_w[:len(round_ms)]) * BYTES_PER_WEIGHT
     fit_ms = float(sum(round_ms))
@@ -466,7 +466,7 @@ def main():
                 "unit": "GB/s", "frac": achieved / peak, "peak_source": f"of {peak_kind}",
                 "traffic": None if tpw is None else tpw * float(np.mean(per_launch_w)),
                 "traffic_source": None if tpw is None else f"{TRAFFIC_FILE} (a constant per weight and round from one "
-                                                           "earlier ncu capture of this workload's launch; not measured "
+                                                           "earlier ncu capture of this workload's fit launches; not measured "
                                                            "in this run)",
                 "algorithmic_bytes_per_launch": float(np.mean(per_launch_w)) * BYTES_PER_WEIGHT,
                 "avg_launch_ms": fit_ms / max(len(round_ms), 1),

@@ -133,6 +133,11 @@ int aaac_act_stats_noalloc(const void* X, int64_t T, int64_t K, int64_t ldx, flo
  * before the iteration, an entry whose cell has no weight keeping its value; sort }.  With
  * n_inner = 1 a round is a single pass over W (the cells of the update are the nearest-entry
  * indices of the assignment step); every further inner iteration is one more, cheaper pass.
+ * NVFP4 layers of many weights and rounds make most of their passes with sums that are carried from
+ * pass to pass, to which only the weights that move are added: decisions are made as in any pass, and the
+ * last pass forms its sums anew, so that the tables are as exact as without (2-norm of the error
+ * before they are rounded to FP32 about 1e-10; fits made either way agree to about 1e-7, as a group
+ * whose errors under the two tables nearly meet may go either way by such a difference).
  * n_inner >= 1 and n_outer * n_inner <= 2^20, else AAAC_ERR_SHAPE.  A layer must span fewer than
  * 2^32 elements (N * ldw < 2^32; the fit kernels index it with 32 bits), else AAAC_ERR_TOO_LARGE.
  *
@@ -142,7 +147,8 @@ int aaac_act_stats_noalloc(const void* X, int64_t T, int64_t K, int64_t ldx, flo
  *   tensor_scale  out  [1] FP32 (1.0 for INT4)
  *   T01           in (AAAC_INIT_USER) / out  [2][16] FP32 tables after the last round, sorted
  *   err_trace     out  [n_outer] double or NULL: Eq. 8 objective (sum over groups of the
- *                      smaller weighted error, normalised units) of each round's assignment
+ *                      smaller weighted error, normalised units) of each round's assignment, to
+ *                      about 1e-6 of it (the rounds that carry their sums, below: 1e-8)
  *   dev_status    out  device word or NULL
  */
 int aaac_fit_layer(const void* W, int64_t N, int64_t K, int64_t ldw, int mode, int group,
@@ -220,7 +226,8 @@ int aaac_dequant_sel(const uint8_t* codes, const void* scales, const uint8_t* si
  * With n_inner = 1 the rounds of up to eight layers run in one launch, each layer on its own
  * share of the blocks, so that the cost of a round that does not depend on the layer's size is
  * paid once per batch and small layers do not leave most of the GPU idle; more layers are run in
- * turn.  (With n_inner > 1 a round is two launches, of up to eight layers each.)  Scales, importances (from X where I is NULL) and start tables
+ * turn.  (With n_inner > 1 a round is two launches, of up to eight layers each.  Where all of
+ * them carry their sums, the rounds are four launches, or 2 n_outer + 1 with n_inner > 1.)  Scales, importances (from X where I is NULL) and start tables
  * are computed per layer exactly as by aaac_fit_layer_sel, except that layers given the same
  * activations (the same X, T, K and ldx, with I == NULL) share their importances, which are
  * computed once (into the workspace of the first of them).  With more than one layer these

@@ -13,8 +13,8 @@
 // lookups and conversions chosen for it (see below), and by having the first rows of the next pass
 // in flight, and the bins being cleared, meanwhile.  A pass of a 512 x 512 layer took 11.4 us with 19k cycles of it and whole
 // items, 5.2 us now; 4096 x 4096, 27.4 -> 23.3 us.
-// (NVFP4 layers of enough units and rounds leave most of their rounds to the incremental ones of fit_delta.cuh; see
-// can_increment.)
+// (NVFP4 layers of enough units and rounds leave most of their rounds to the incremental ones of fit_delta.cuh, and run as
+// four launches: see can_increment.)
 // With n_inner > 1 the assignment pass (which is also the first inner iteration) stores the
 // selection bits, one word per row and 256-column slab, and the remaining n_inner - 1 inner
 // iterations are passes of a second instance of the kernel that reads those bits instead of

@@ -5,7 +5,7 @@ import torch
 
 import oracle
 from paper_2605_08692_b200 import binding, build, synth
-from test_gpu_parity import NVFP4, check_end_to_end_bits, dev_bf16, host, layer, table_close
+from test_gpu_parity import NVFP4, check_end_to_end_bits, dev_bf16, host, layer, run_fit_batch, table_close
 
 pytestmark = pytest.mark.gpu
 
@@ -230,6 +230,22 @@ def test_weight_sums_that_are_carried_are_exact(K, units, extra, rounds, inner):
             for c in range(16):
                 want[t, c] += (I * ((cell[t] == c) & mine)).sum()
     assert torch.allclose(got, want, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("rounds,inner,small", [(29, 1, False), (3, 10, False), (29, 1, True)])
+def test_layers_that_share_a_launch(rounds, inner, small):
+    """Two layers, each on its share of the blocks; with a small one in their launch all rounds of all three are full ones."""
+    shapes = [(rows_for(12, 512), 512), (rows_for(14, 1008) + 5, 1008)] + [(70, 640)] * small
+    cases, oracles = [], []
+    for N, K in shapes:
+        W, X = layer(NVFP4, N, K, T=64, name=f"incremental/batch/{K}")
+        oracles.append(oracle.fit_layer(W, NVFP4, 16, rounds, X=X, n_inner=inner, init="quantile"))
+        cases.append((W, oracles[-1]["I"]))
+    for d, o in zip(run_fit_batch(cases, NVFP4, rounds, binding.INIT_QUANTILE, n_inner=inner), oracles):
+        assert binding.debug_incremental(d["ws"]) == ((0, 0) if small else (3 if inner == 1 else 1, rounds * inner - 1))
+        assert table_close(host(d["T01"]), o["T"])[0]
+        assert np.allclose(host(d["err_trace"]), o["trace"], rtol=1e-5, atol=0)
+        assert np.array_equal(host(d["scales"]), o["scales_unsigned"])
 
 
 @pytest.mark.parametrize("K,units,extra,rounds,dist", [(512, 20, 0, 29, "normal"), (1008, 24, 5, 27, "student5"), (4096, 40, -3, 22, "student5")])
