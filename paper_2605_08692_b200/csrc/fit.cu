@@ -1135,25 +1135,25 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
 // is left on the warps' lists cost 60 to 100 us, and the early rounds gain nothing.  How many weights move is not known here: the
 // more even the importances, the more (and with heavier tails more from quantiles, fewer from the grid).  Time of all full rounds /
 // time so, the lowest and highest of normal and Student-t weights from the quantile and the grid start (units are 16 x 512 weights a block):
-//   units x rounds             12 x 30    20 x 20    20 x 30    28 x 20    48 x 16    48 x 20    48 x 30    98 x 10    98 x 20    98 x 30
-//   massive channels          .96- .98   .97-1.02  1.00-1.08  1.00-1.05   .99-1.01  1.01-1.04  1.05-1.09   .95- .98  1.02-1.07  1.07-1.12
-//   log-normal, deviation 1.2 .91- .95   .91- .95   .95-1.00   .93- .98   .92- .96   .93- .98   .98-1.03   .91- .95   .95-1.01   .99-1.06
-//   equal                     .90- .94   .86- .94   .94- .98   .92- .96   .90- .95   .91- .97   .96-1.02   .87- .93   .94- .99   .98-1.04
-// The line lies where the mean of the first two rows is 1: about 20 x 29, 28 x 25, 48 x 21, 98 x 18.
-// Further inner iterations have no flips and gain from the first pass on, the assignments between them lose (massive channels / equal, quantile start):
-//   rounds x inner        1 x 10               2 x 4                2 x 7                2 x 10               3 x 7                3 x 10
-//   12 units       .98- .99 / .94- .97  .92- .93 / .88- .91  1.00-1.01 / .93- .96  1.06-1.07 / .97-1.00  1.06-1.07 / .96-1.01  1.12 / 1.00-1.05
-//   20 units      1.02      / .96-1.00  .94      / .90- .93  1.04-1.05 / .95- .99  1.12-1.13 / .99-1.04  1.12      / 1.00-1.03  1.18-1.19 / 1.04-1.09
-//   48 units      1.06      / .96-1.01  .94      / .89- .92  1.06-1.07 / .94- .99  1.15      / .99-1.04  1.13-1.14 / .98-1.03  1.22 / 1.03-1.08
-// and 1 x 30, 3 x 10 (log-normal importances) with 5 units .97-.98, .96-.97, with 7 1.04-1.05, 1.01-1.04.
+//   units x rounds             12 x 30    20 x 21    20 x 30    28 x 19    48 x 16    48 x 20    48 x 30    98 x 10    98 x 14    98 x 20    98 x 30
+//   massive channels          .96- .98   .97-1.03  1.00-1.08  1.00-1.04   .99-1.02  1.01-1.04  1.05-1.09   .95- .98   .99-1.03  1.02-1.07  1.07-1.12
+//   log-normal, deviation 1.2 .91- .95   .91- .95   .95-1.00   .93- .97   .92- .96   .93- .98   .98-1.03   .91- .95   .93- .98   .95-1.01   .99-1.06
+//   equal                     .90- .94   .86- .94   .94- .98   .92- .96   .90- .95   .91- .97   .96-1.02   .87- .93   .92- .96   .94- .99   .98-1.04
+// Activations have massive channels, so the first row counts double against the second: the line is about 20 x 26, 28 x 23, 48 x 19, 98 x 16.
+// Further inner iterations have no flips and gain from the first pass on, the assignments between them lose.  Mean of normal and Student-t
+// weights from the quantile start, massive channels / log-normal:
+//   3 x 10   6 units 1.08 / 1.03, 9 1.08 / 1.02        2 x 10   7 units 1.03 / .99, 16 1.09 / 1.04        1 x 10   13 units .99 / .98, 16 1.01 / .99, 20 1.03 / 1.02
+//   3 x 7    9 units 1.04 / .98                        2 x 7   13 units 1.01 / .97                        1 x 8   48 units 1.01 / 1.01, 98 1.02 / 1.01
+//   3 x 6   13 units 1.05 / 1.00, 28 1.12 / 1.05       2 x 6   16 units 1.00 / .97, 20 1.02 / .99, 48 1.04 / .99
+//   2 x 5   20 units  .99 / .96                        2 x 4   12 to 98 units .92-.96 / .91-.94
 // They start from the first pass's tables, though, and do not begin where these hold one value twice, as the NVFP4 grid
 // does (tried and made again, 4096 x 4096 took 778 us for 743, and 312 for 274 in one round of 10).
 // A piece is read with one 32-byte load; its number must be divisible by more than one piece per row (row_of).
 constexpr int kFullRounds = 3;                        // the last of them the keeping one
 static bool can_increment(const FitLayerArgs& a, int64_t blocks, int n_outer, int n_inner) {
     const int64_t slabs = (a.K + kDeltaCols - 1) / kDeltaCols, units = slabs * ((a.N + kFitWarps - 1) / kFitWarps);
-    const bool pays = n_inner == 1 ? units >= 20 * blocks && (n_outer - 14) * units >= 300 * blocks
-                                   : n_inner >= 7 && (int64_t)n_outer * n_inner * units >= (180 + 20 * n_outer) * blocks;
+    const bool pays = n_inner == 1 ? units >= 20 * blocks && (n_outer - 13) * units >= 260 * blocks
+                                   : n_inner >= 6 && (int64_t)n_outer * n_inner >= 8 && (int64_t)n_outer * (n_inner - 4) * units >= 100 * blocks;
     return pays && !(n_inner > 1 && a.twin_entries) && a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 &&
            a.ldw % 16 == 0 && 8 * a.K >= 7 * kDeltaCols * slabs;
 }

@@ -118,8 +118,8 @@ def test_inner_iterations_from_equal_entries_are_not_tried():
 
 
 @pytest.mark.parametrize("units,rounds,inner,incremental", [
-    (20, 28, 1, False), (19, 40, 1, False), (40, 21, 1, False), (40, 22, 1, True),
-    (30, 5, 6, False), (19, 1, 10, False), (20, 1, 10, True), (10, 2, 10, False), (9, 3, 7, False), (12, 3, 7, True)])
+    (20, 25, 1, False), (20, 26, 1, True), (19, 40, 1, False), (40, 19, 1, False),
+    (30, 5, 5, False), (30, 1, 7, False), (14, 1, 10, False), (18, 1, 10, True), (7, 2, 10, False), (9, 2, 10, True), (9, 3, 7, False), (12, 3, 7, True)])
 def test_the_rule_takes_what_pays(units, rounds, inner, incremental):
     """(Layers may use some blocks fewer than there are, so that a block has a tenth more units.)"""
     W, X = layer(NVFP4, rows_for(units, 512), 512, T=64, name="incremental/rule")
