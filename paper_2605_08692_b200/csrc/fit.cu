@@ -1145,15 +1145,17 @@ static bool fill_params(FitParams& p, const FitLayerArgs& a, int n_outer, uint32
 //   3 x 10   6 units 1.08 / 1.03, 9 1.08 / 1.02        2 x 10   7 units 1.03 / .99, 16 1.09 / 1.04        1 x 10   13 units .99 / .98, 16 1.01 / .99, 20 1.03 / 1.02
 //   3 x 7    9 units 1.04 / .98                        2 x 7   13 units 1.01 / .97                        1 x 8   48 units 1.01 / 1.01, 98 1.02 / 1.01
 //   3 x 6   13 units 1.05 / 1.00, 28 1.12 / 1.05       2 x 6   16 units 1.00 / .97, 20 1.02 / .99, 48 1.04 / .99
-//   2 x 5   20 units  .99 / .96                        2 x 4   12 to 98 units .92-.96 / .91-.94
+//   3 x 5   16 units 1.04 / .98, 20 1.05 / 1.00        2 x 5   20 units  .99 / .96                        2 x 4   12 to 98 units .92-.96 / .91-.94
+// Roughly the units times these iterations tell.
 // They start from the first pass's tables, though, and do not begin where these hold one value twice, as the NVFP4 grid
 // does (tried and made again, 4096 x 4096 took 778 us for 743, and 312 for 274 in one round of 10).
 // A piece is read with one 32-byte load; its number must be divisible by more than one piece per row (row_of).
 constexpr int kFullRounds = 3;                        // the last of them the keeping one
 static bool can_increment(const FitLayerArgs& a, int64_t blocks, int n_outer, int n_inner) {
     const int64_t slabs = (a.K + kDeltaCols - 1) / kDeltaCols, units = slabs * ((a.N + kFitWarps - 1) / kFitWarps);
+    const int64_t frozen = (int64_t)n_outer * (n_inner - 1);      // further inner iterations
     const bool pays = n_inner == 1 ? units >= 20 * blocks && (n_outer - 13) * units >= 260 * blocks
-                                   : n_inner >= 6 && (int64_t)n_outer * n_inner >= 8 && (int64_t)n_outer * (n_inner - 4) * units >= 100 * blocks;
+                                   : n_inner >= 5 && frozen >= 9 && frozen * units >= 165 * blocks;
     return pays && !(n_inner > 1 && a.twin_entries) && a.ws.qcap >= (size_t)a.N * (size_t)a.K / 16 && a.K >= 64 && reinterpret_cast<uintptr_t>(a.W) % 32 == 0 &&
            a.ldw % 16 == 0 && 8 * a.K >= 7 * kDeltaCols * slabs;
 }

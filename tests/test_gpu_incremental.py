@@ -119,7 +119,8 @@ def test_inner_iterations_from_equal_entries_are_not_tried():
 
 @pytest.mark.parametrize("units,rounds,inner,incremental", [
     (20, 25, 1, False), (20, 26, 1, True), (19, 40, 1, False), (40, 19, 1, False),
-    (30, 5, 5, False), (30, 1, 7, False), (14, 1, 10, False), (18, 1, 10, True), (7, 2, 10, False), (9, 2, 10, True), (9, 3, 7, False), (12, 3, 7, True)])
+    (30, 2, 5, False), (30, 5, 4, False), (30, 1, 7, False), (14, 1, 10, False), (20, 1, 10, True), (7, 2, 10, False), (10, 2, 10, True), (8, 3, 7, False),
+    (12, 3, 7, True), (16, 3, 5, True)])
 def test_the_rule_takes_what_pays(units, rounds, inner, incremental):
     """(Layers may use some blocks fewer than there are, so that a block has a tenth more units.)"""
     W, X = layer(NVFP4, rows_for(units, 512), 512, T=64, name="incremental/rule")
